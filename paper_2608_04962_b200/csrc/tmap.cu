@@ -8,37 +8,47 @@
 
 namespace specroll {
 
-// A tensor map is a pure function of (base pointer, extents, strides, box): the last few are remembered, so that
+// A tensor map is a pure function of (base pointer, extents, strides, box): the ones met lately are remembered, so that
 // the calls of a step (the same caches, weights and activations layer after layer, step after step) do not encode
-// theirs again (encoding costs a few microseconds of host time per map, five maps per attention call).
+// theirs again (encoding costs about a microsecond of host time per map, five maps per attention call).  A step of 48
+// layers has some 250 maps and a host may alternate between several sets of buffers: 512 sets of 8 entries, the
+// oldest of a set replaced.  (128 entries replaced in turn were too few: 28 layers have 140 maps, so every one of
+// them was encoded anew in every step.)
 namespace {
 struct MapKey {
     const void *base;
     uint64_t a, b, c;
-    uint32_t box1, box2, rank;
+    uint32_t box1, box2, rank, pad;
 };
 struct MapEntry {
     MapKey key;
     CUtensorMap map;
     bool used;
 };
-constexpr int MAP_CACHE = 128;
+constexpr int MAP_SETS = 512, MAP_WAYS = 8;
 std::mutex map_mu;
-MapEntry map_cache[MAP_CACHE];
-unsigned map_next = 0;
+MapEntry map_cache[MAP_SETS][MAP_WAYS];
+uint8_t map_next[MAP_SETS];
 
+unsigned map_set(const MapKey &k) {
+    uint64_t h = reinterpret_cast<uintptr_t>(k.base) >> 4;
+    for (uint64_t v : {k.a, k.b, k.c, (uint64_t)k.box1 << 32 | k.box2}) h = (h ^ v) * 0x9E3779B97F4A7C15ull;
+    return (unsigned)(h >> 40) % MAP_SETS;
+}
 bool map_lookup(const MapKey &k, CUtensorMap *out) {
+    MapEntry *set = map_cache[map_set(k)];
     std::lock_guard<std::mutex> lock(map_mu);
-    for (int i = 0; i < MAP_CACHE; ++i)
-        if (map_cache[i].used && memcmp(&map_cache[i].key, &k, sizeof(MapKey)) == 0) {
-            *out = map_cache[i].map;
+    for (int i = 0; i < MAP_WAYS; ++i)
+        if (set[i].used && memcmp(&set[i].key, &k, sizeof(MapKey)) == 0) {
+            *out = set[i].map;
             return true;
         }
     return false;
 }
 void map_store(const MapKey &k, const CUtensorMap &m) {
+    const unsigned s = map_set(k);
     std::lock_guard<std::mutex> lock(map_mu);
-    MapEntry &e = map_cache[map_next++ % MAP_CACHE];
+    MapEntry &e = map_cache[s][map_next[s]++ % MAP_WAYS];
     e.key = k;
     e.map = m;
     e.used = true;
