@@ -96,6 +96,10 @@ attn_prep_kernel(const int32_t *__restrict__ kv_indptr, const int32_t *__restric
     __shared__ int sh_tmp[PREP_MAX_B];
     __shared__ int warp_tot[33];
     const int t = threadIdx.x;
+    // (the attention kernel behind this one may be set up meanwhile; it waits for this kernel's completion before it
+    // lets anything behind itself start)
+    pdl_launch_dependents();
+    pdl_wait();
     if (t == 0) *status = 0;
     for (int i = t; i < n_counters; i += PREP_THREADS) counters[i] = 0;
     if (B > PREP_MAX_B) {
@@ -461,17 +465,34 @@ __global__ void __launch_bounds__(128) attn_combine_kernel(AttnArgs a) {
 
 constexpr int PLAN_SMS = 148;  // SMs the chunking is planned for
 
-// Estimated finishing time, in quarter tiles, of the persistent tcgen05 kernel when sequences of the given tile
-// counts (sorted, longest first) are cut into chunks of at most ct tiles: work units go, in the order the device
-// uses, to whichever of PLAN_SMS CTAs is free first.  A unit costs its K/V tiles, one more for the tree tile of a
-// sequence's last chunk, one for the hand-over between units; a chunk of a split sequence adds one for its
-// partial, and the last one the merge when the attention kernel does it (fewer than 5 chunks per sequence).
+// Chunks of the sequences (tile counts) when none may hold more than ct tiles, and the most a sequence has.
+static long long count_chunks(const std::vector<int> &tiles, int ct, int *max_ns) {
+    long long n = 0;
+    *max_ns = 1;
+    for (int t : tiles) {
+        const int ns = std::max(1, (t + ct - 1) / ct);
+        n += ns;
+        *max_ns = std::max(*max_ns, ns);
+    }
+    return n;
+}
+
+// Who merges the chunks of a split sequence: the CTA that finishes its last chunk, while the others keep streaming, or
+// (true) a kernel of its own over the whole GPU.  The latter for many chunks (the last CTA would sit on a long chain of
+// dependent loads), and when all work units run side by side, so that nothing streams beside that CTA.
+static bool merge_by_kernel(long long units, int max_ns) { return max_ns >= 5 || (max_ns >= 2 && units <= PLAN_SMS); }
+
+// Estimated finishing time, in quarter tiles (about a third of a microsecond), of the persistent tcgen05 kernel when
+// sequences of the given tile counts (sorted, longest first) are cut into chunks of at most ct tiles: work units go, in
+// the order the device uses, to whichever of PLAN_SMS CTAs is free first.  A unit costs its K/V tiles, one more for the
+// tree tile of a sequence's last chunk, one for the hand-over between units; a chunk of a split sequence adds one
+// for its partial, and the last one the merge when the attention kernel does it, else the merge kernel follows.
 static long long estimate_makespan(const std::vector<int> &tiles, int ct, int copies) {
     struct Chunk { int tps, cost; };
     std::vector<Chunk> chunks;
     int max_ns = 1;
-    for (int t : tiles) max_ns = std::max(max_ns, (t + ct - 1) / ct);
-    const bool merge_inline = max_ns < 5;
+    const long long units = count_chunks(tiles, ct, &max_ns) * copies;
+    const bool merge_inline = !merge_by_kernel(units, max_ns);
     for (int t : tiles) {
         const int ns = std::max(1, (t + ct - 1) / ct), tps = (t + ns - 1) / ns;
         for (int s = 0; s < ns; ++s) {
@@ -493,7 +514,7 @@ static long long estimate_makespan(const std::vector<int> &tiles, int ct, int co
             sms.push(t);
             end = std::max(end, t);
         }
-    return end;
+    return end + ((max_ns > 1 && !merge_inline) ? 8 + max_ns / 2 : 0);
 }
 
 struct AttnPlan {
@@ -559,18 +580,24 @@ static int compute_attn_plan(const specroll_attn_desc *d, const int32_t *indptr_
         std::sort(tiles.begin(), tiles.end(), std::greater<int>());
         static const int pcts[] = {75, 100, 125, 150, 200, 300};
         long long best = -1;
-        int seen[6], n_seen = 0;
-        for (int pct : pcts) {
-            const int c = chunk_for(pct);
-            bool dup = false;
-            for (int i = 0; i < n_seen; ++i) dup |= (seen[i] == c);
-            if (dup) continue;
+        int seen[9], n_seen = 0;
+        auto consider = [&](int c) {
+            for (int i = 0; i < n_seen; ++i)
+                if (seen[i] == c) return;
             seen[n_seen++] = c;
             const long long m = estimate_makespan(tiles, c, (int)ctas_per_tile);
             if (best < 0 || m < best) {
                 best = m;
                 ct = c;
             }
+        };
+        for (int pct : pcts) consider(chunk_for(pct));
+        // Chunks below 512 tokens only where every unit still gets an SM of its own: there the layer lasts as long as
+        // its longest unit (two sequences of 900 and 2400 tokens: 26 us in chunks of four tiles, attention and
+        // merge), and the partials that this adds pass through L2 on an otherwise idle GPU.
+        for (int c = 1; c < 512 / TT; ++c) {
+            int ns = 1;
+            if (c <= max_tiles && count_chunks(tiles, c, &ns) * ctas_per_tile <= PLAN_SMS) consider(c);
         }
     }
     p->chunk_tiles = (int)ct;
@@ -583,9 +610,8 @@ static int compute_attn_plan(const specroll_attn_desc *d, const int32_t *indptr_
     }
     p->items = items;
     if (max_tiles / p->chunk_tiles + 1 > 65535) return SPECROLL_EINVAL;
-    // A sequence cut into many chunks is merged by a kernel of its own, over the whole GPU; with few chunks the
-    // CTA that finishes a sequence's last chunk merges them while the others keep streaming.
-    p->merge_mode = (p->use_tc && (max_tiles + p->chunk_tiles - 1) / p->chunk_tiles >= 5) ? 2 : 0;
+    p->merge_mode = (p->use_tc && merge_by_kernel((long long)items * ctas_per_tile, (max_tiles + p->chunk_tiles - 1) / p->chunk_tiles)) ? 2 : 0;
+    if (p->use_tc && items == d->B) p->merge_mode = 2;  // (nothing is split: nothing is merged anywhere)
     p->n_counters = 64 + d->B * d->Hkv * p->n_rb;  // [0]: work counter, [1]: CTAs that have left; [64 ...]: per (b, hkv, rb) arrivals
     size_t o = 0;
     p->off_status = o;
@@ -744,17 +770,17 @@ static int run_tree_attn(const specroll_attn_desc *d, const void *Q, const void 
     a.total_work = p.items * d->Hkv * p.n_rb;
     a.merge_mode = p.merge_mode;
     a.nodes_per_block = p.nodes_per_block;
+    a.plan_fresh = 0;
     a.no_pdl = (d->flags & SPECROLL_ATTN_NO_PDL) ? 1 : 0;
     // early cache loads need a plan that is not being made by the kernel just before the attention kernel
     a.early_cache = ((d->flags & SPECROLL_ATTN_CACHE_SETTLED) && (d->flags & SPECROLL_ATTN_REUSE_PLAN)) ? 1 : 0;
     if (!(p.use_tc && (d->flags & SPECROLL_ATTN_REUSE_PLAN))) {
         // (the tcgen05 kernel leaves its scheduling counters cleared, so a kept plan can be run again as is)
-        attn_prep_kernel<<<1, PREP_THREADS, 0, st>>>(kv_indptr_dev, paged ? kv_len_dev : nullptr, page_indptr_dev, d->B,
-                                                     p.chunk_tiles, p.tile_tokens,
-                                                     reinterpret_cast<int32_t *>(ws + p.off_items),
-                                                     p.use_tc ? sorted_start : nullptr, seq_at_rank,
-                                                     p.use_tc ? unit_tab : nullptr, status, counters, p.n_counters);
-        SR_LAUNCH_CHECK();
+        SR_CUDA_TRY(launch_dependent(true, attn_prep_kernel, dim3(1), dim3(PREP_THREADS), 0, st, kv_indptr_dev,
+                                     paged ? kv_len_dev : nullptr, page_indptr_dev, d->B, p.chunk_tiles, p.tile_tokens,
+                                     reinterpret_cast<int32_t *>(ws + p.off_items), p.use_tc ? sorted_start : nullptr,
+                                     seq_at_rank, p.use_tc ? unit_tab : nullptr, status, counters, p.n_counters));
+        a.plan_fresh = 1;
     }
     const size_t n_out = (size_t)d->B * d->N * d->Hq;
     if (p.use_tc) {

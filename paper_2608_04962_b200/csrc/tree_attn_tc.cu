@@ -156,7 +156,12 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     volatile int *tickets = reinterpret_cast<volatile int *>(extra + 8);
     unsigned char *xch_base = extra + 16;
     volatile UnitDesc *ring = reinterpret_cast<volatile UnitDesc *>(extra + 16 + C::XCH_BYTES);  // 2 slots of 64 bytes
-    float *hand = a.hand + (size_t)blockIdx.x * C::HAND_FLOATS;  // [l of team 0 | l of team 1 | m of team 0 | m of team 1][128 rows]
+    // Every CTA has one unit at most (few sequences): the second Q buffer is free for the hand-over area, and nothing
+    // is counted - the merge, if any, is a kernel of its own - so the CTA leaves without a round trip to memory.
+    const bool one_wave = a.total_work <= (int)gridDim.x && a.merge_mode != 0;
+    // [l of team 0 | l of team 1 | m of team 0 | m of team 1][128 rows]
+    float *hand = a.hand + (size_t)blockIdx.x * C::HAND_FLOATS;
+    volatile float *hand_s = reinterpret_cast<volatile float *>(aligned + C::Q_BYTES);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int N = a.N, G = a.G;
@@ -215,12 +220,14 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // Launched as a programmatic dependent of the kernel before it in the stream, this CTA may have done all
     // of the above while that kernel was still finishing.  From here on it reads what earlier kernels wrote
     // (the plan, the counters the launch before cleared, Q and the tree's K/V), so it waits for them to be
-    // complete.  The kernel after this one may be set up as early as its CTAs find room.
+    // complete.  The kernel after this one may be set up as early as its CTAs find room - except behind a plan that
+    // is only being made: that kernel may read the plan before it waits, so this one waits for the plan first.
     // Exception: when the caller has said that the plan and the cache were complete before that kernel was
     // even launched, the loading thread fetches its first cache tiles right away and waits just before it
     // needs Q (below).
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const bool early = a.early_cache != 0;
+    if (a.plan_fresh) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (!(early && warp == 0)) asm volatile("griddepcontrol.wait;" ::: "memory");
 
     // Sums the partials of all chunks of one (sequence, kv head, row block) for columns [col0, col0 + ncols) of one row;
@@ -307,7 +314,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 }
                 // the first unit of a CTA is its own index (no round trip before the first loads); the counter
                 // hands out the units after those
-                const int w = u == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(a.work_counter, 1);
+                const int w = u == 0 ? (int)blockIdx.x : (one_wave ? a.total_work : (int)gridDim.x + atomicAdd(a.work_counter, 1));
                 volatile UnitDesc *d = ring + slot;
                 if (w >= a.total_work) {
                     d->valid = 0;
@@ -552,8 +559,18 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             // each team's share of the sum is relative to the reference as that team last knew it
-            const float l0 = __ldcg(hand + row), l1 = __ldcg(hand + 128 + row);
-            const float m0 = __ldcg(hand + 256 + row), m1 = __ldcg(hand + 384 + row);
+            float l0, l1, m0, m1;
+            if (one_wave) {
+                l0 = hand_s[row];
+                l1 = hand_s[128 + row];
+                m0 = hand_s[256 + row];
+                m1 = hand_s[384 + row];
+            } else {
+                l0 = __ldcg(hand + row);
+                l1 = __ldcg(hand + 128 + row);
+                m0 = __ldcg(hand + 256 + row);
+                m1 = __ldcg(hand + 384 + row);
+            }
             const float m_used = fmaxf(m0, m1);
             const float lt = (m0 == -INFINITY ? 0.f : l0 * ex2_approx(m0 - m_used)) +
                              (m1 == -INFINITY ? 0.f : l1 * ex2_approx(m1 - m_used));
@@ -839,8 +856,13 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 ok = twait(3, bar(C::B_HFREE), (u & 1u) ^ 1u);  // the values of the unit before have been taken
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                hand[team * 128 + row] = l;
-                hand[256 + team * 128 + row] = m_used;
+                if (one_wave) {
+                    hand_s[team * 128 + row] = l;
+                    hand_s[256 + team * 128 + row] = m_used;
+                } else {
+                    hand[team * 128 + row] = l;
+                    hand[256 + team * 128 + row] = m_used;
+                }
                 mbar_arrive(bar(C::B_HFULL));
             }
         } else {
@@ -1048,8 +1070,13 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                 ok = twait(3, bar(C::B_HFREE), (u & 1u) ^ 1u);  // the values of the unit before have been taken
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                hand[half * 128 + row] = l;
-                hand[256 + half * 128 + row] = m_used;  // the same value from both threads of the pair
+                if (one_wave) {
+                    hand_s[half * 128 + row] = l;
+                    hand_s[256 + half * 128 + row] = m_used;
+                } else {
+                    hand[half * 128 + row] = l;
+                    hand[256 + half * 128 + row] = m_used;
+                }
                 mbar_arrive(bar(C::B_HFULL));
             }
         }
@@ -1066,8 +1093,11 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
                             (int)(blockIdx.x << 16);
         }
         // the CTA that leaves last clears the scheduling counters, so the same plan can be launched again
-        __threadfence();
-        tickets[0] = (atomicAdd(a.work_counter + 1, 1) == (int)gridDim.x - 1) ? 1 : 0;
+        tickets[0] = 0;
+        if (!one_wave) {
+            __threadfence();
+            tickets[0] = (atomicAdd(a.work_counter + 1, 1) == (int)gridDim.x - 1) ? 1 : 0;
+        }
     }
     if (warp == 1) {
         tc_fence_after();
@@ -1124,66 +1154,103 @@ static int launch_tc(const AttnArgs &a, const TopoMask &mask, long long T_kv, in
 
 // Sums the chunks of every split sequence (the plan uses this instead of merging inside the attention kernel
 // when some sequence has many chunks: there the last chunk's CTA would sit on a long chain of dependent loads).
-// grid = (chunks in work order, Hkv * n_rb, D / 32); only the block of a split sequence's first chunk works.
-// 256 threads: 128 rows x 2 groups of 4 float4 columns.
+// grid = (chunks in work order, Hkv * n_rb, D / 8); only the blocks of a split sequence's first chunk work: 128 rows x
+// 2 halves of the chunks, two float4 columns each.  What bounds it is round trips to L2, not bytes: the chunks of a
+// half are taken eight at a time with all their loads in flight, and the halves meet in shared memory (one thread per
+// row for all chunks, four at a time: 7.5 us between the end of the attention kernel and the end of this one for
+// 19 chunks).
+// Launched as a programmatic dependent of the attention kernel: its blocks are in place (on SMs that the attention
+// leaves idle or has finished on) when the partials are complete; nothing is read before.
 template <int D>
 __global__ void __launch_bounds__(256) attn_merge_tc_kernel(AttnArgs a) {
+    constexpr int STEP = 8;
+    __shared__ float sh_m[2][128];
+    __shared__ float4 sh_acc[2][128];
+    __shared__ float sh_l[128];
+    pdl_launch_dependents();
+    pdl_wait();
     const int4 e0 = __ldg(reinterpret_cast<const int4 *>(a.unit_tab) + 2 * (size_t)blockIdx.x);
     const int b = e0.x, n_splits = e0.z, item0 = e0.w;
     if (e0.y != 0 || n_splits < 2) return;
     const int hkv = blockIdx.y / a.n_rb, rb = blockIdx.y % a.n_rb;
-    const int row = threadIdx.x & 127, cg = threadIdx.x >> 7;
+    const int row = threadIdx.x & 127, half = threadIdx.x >> 7;
     const int gr = rb * a.rows_per_block + row;
-    if (row >= a.rows_per_block || gr >= a.rows) return;
-    const int c4 = blockIdx.z * 8 + cg * 4;  // first of this thread's 4 float4 columns
+    const bool ok = row < a.rows_per_block && gr < a.rows;
+    const int c4 = blockIdx.z * 2;  // first of this block's float4 columns
     const size_t unit_ml = (size_t)a.Hkv * a.rows_pad, unit_o = (size_t)a.Hkv * (D / 4) * a.rows_pad;
-    const float *ml = a.part_ml + 2 * (((size_t)item0 * a.Hkv + hkv) * a.rows_pad + gr);
+    const float2 *ml = reinterpret_cast<const float2 *>(a.part_ml) + ((size_t)item0 * a.Hkv + hkv) * a.rows_pad + (ok ? gr : 0);
     const float4 *po = reinterpret_cast<const float4 *>(a.part_o) + ((size_t)item0 * a.Hkv + hkv) * (size_t)(D / 4) * a.rows_pad +
-                       (size_t)c4 * a.rows_pad + gr;
+                       (size_t)c4 * a.rows_pad + (ok ? gr : 0);
+    // this thread's chunks: half, half + 2, ...
+    const int n_mine = (n_splits - half + 1) / 2;
     float Mx = -INFINITY;
-    for (int s = 0; s < n_splits; ++s) Mx = fmaxf(Mx, __ldcg(ml + 2 * s * unit_ml));
+#pragma unroll 1
+    for (int i0 = 0; i0 < n_mine; i0 += STEP) {
+        float v[STEP];
+#pragma unroll
+        for (int i = 0; i < STEP; ++i) v[i] = i0 + i < n_mine ? __ldcg(&ml[(size_t)(half + 2 * (i0 + i)) * unit_ml].x) : -INFINITY;
+#pragma unroll
+        for (int i = 0; i < STEP; ++i) Mx = fmaxf(Mx, v[i]);
+    }
+    sh_m[half][row] = Mx;
+    __syncthreads();
+    Mx = fmaxf(sh_m[0][row], sh_m[1][row]);
     float lsum = 0.f;
-    float4 acc[4];
+    float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+#pragma unroll 1
+    for (int i0 = 0; i0 < n_mine; i0 += STEP) {
+        float2 v[STEP];
+        float4 x[STEP][2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-    for (int s = 0; s < n_splits; ++s) {
-        const float ms = __ldcg(ml + 2 * s * unit_ml), ls = __ldcg(ml + 2 * s * unit_ml + 1);
-        const float wgt = (ms == -INFINITY) ? 0.f : ex2_approx(ms - Mx);
-        lsum += wgt * ls;
+        for (int i = 0; i < STEP; ++i) {
+            const size_t s = (size_t)(half + 2 * min(i0 + i, n_mine - 1));  // (a chunk beyond the last: weight zero below)
+            v[i] = __ldcg(&ml[s * unit_ml]);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float4 x = __ldcg(po + s * unit_o + (size_t)i * a.rows_pad);
-            acc[i].x += wgt * x.x;
-            acc[i].y += wgt * x.y;
-            acc[i].z += wgt * x.z;
-            acc[i].w += wgt * x.w;
+            for (int c = 0; c < 2; ++c) x[i][c] = __ldcg(po + s * unit_o + (size_t)c * a.rows_pad);
+        }
+#pragma unroll
+        for (int i = 0; i < STEP; ++i) {
+            const float wgt = (i0 + i >= n_mine || v[i].x == -INFINITY) ? 0.f : ex2_approx(v[i].x - Mx);
+            lsum += wgt * v[i].y;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                acc[c].x += wgt * x[i][c].x;
+                acc[c].y += wgt * x[i][c].y;
+                acc[c].z += wgt * x[i][c].z;
+                acc[c].w += wgt * x[i][c].w;
+            }
         }
     }
+    if (half == 1) {
+        sh_acc[0][row] = acc[0];
+        sh_acc[1][row] = acc[1];
+        sh_l[row] = lsum;
+    }
+    __syncthreads();
+    if (half == 1 || !ok) return;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const float4 y = sh_acc[c][row];
+        acc[c].x += y.x;
+        acc[c].y += y.y;
+        acc[c].z += y.z;
+        acc[c].w += y.w;
+    }
+    lsum += sh_l[row];
     const float inv = lsum > 0.f ? 1.0f / lsum : 0.f;
     const int n = gr / a.G, g = gr % a.G;
-    __nv_bfloat16 *dst = a.O + (((size_t)b * a.N + n) * a.Hq + hkv * a.G + g) * D + c4 * 4;
-    uint4 q0, q1;
-    q0.x = pack_bf16x2(acc[0].x * inv, acc[0].y * inv);
-    q0.y = pack_bf16x2(acc[0].z * inv, acc[0].w * inv);
-    q0.z = pack_bf16x2(acc[1].x * inv, acc[1].y * inv);
-    q0.w = pack_bf16x2(acc[1].z * inv, acc[1].w * inv);
-    q1.x = pack_bf16x2(acc[2].x * inv, acc[2].y * inv);
-    q1.y = pack_bf16x2(acc[2].z * inv, acc[2].w * inv);
-    q1.z = pack_bf16x2(acc[3].x * inv, acc[3].y * inv);
-    q1.w = pack_bf16x2(acc[3].z * inv, acc[3].w * inv);
-    reinterpret_cast<uint4 *>(dst)[0] = q0;
-    reinterpret_cast<uint4 *>(dst)[1] = q1;
+    uint4 q;
+    q.x = pack_bf16x2(acc[0].x * inv, acc[0].y * inv);
+    q.y = pack_bf16x2(acc[0].z * inv, acc[0].w * inv);
+    q.z = pack_bf16x2(acc[1].x * inv, acc[1].y * inv);
+    q.w = pack_bf16x2(acc[1].z * inv, acc[1].w * inv);
+    *reinterpret_cast<uint4 *>(a.O + (((size_t)b * a.N + n) * a.Hq + hkv * a.G + g) * D + c4 * 4) = q;
     if (a.lse && c4 == 0) a.lse[((size_t)b * a.N + n) * a.Hq + hkv * a.G + g] = (Mx + log2f(lsum)) * 0.6931471805599453f;
 }
 
 int launch_attn_merge_tc(const AttnArgs &a, int D, int items, cudaStream_t st) {
-    const dim3 grid((unsigned)items, (unsigned)(a.Hkv * a.n_rb), (unsigned)(D / 32));
-    if (D == 128)
-        attn_merge_tc_kernel<128><<<grid, 256, 0, st>>>(a);
-    else
-        attn_merge_tc_kernel<64><<<grid, 256, 0, st>>>(a);
-    SR_LAUNCH_CHECK();
+    const dim3 grid((unsigned)items, (unsigned)(a.Hkv * a.n_rb), (unsigned)(D / 8));
+    SR_CUDA_TRY(launch_dependent(!a.no_pdl, D == 128 ? attn_merge_tc_kernel<128> : attn_merge_tc_kernel<64>, grid, dim3(256), 0, st, a));
     return SPECROLL_OK;
 }
 

@@ -78,9 +78,11 @@ __host__ __device__ inline int rs_run_of_vec(int nvec, int vi) {
 __global__ void __launch_bounds__(RS_THREADS, 8)
 row_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, float *__restrict__ row_max,
                  float *__restrict__ row_sum, float2 *__restrict__ run_tab) {
-    // a kernel launched behind this one as its programmatic dependent may start its own prologue as SMs free up; it
-    // waits for this grid's completion before it reads the statistics
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // Set up under the tail of the kernel before, which may have written the logits.  The kernel launched behind this
+    // one as its programmatic dependent reads the call's other inputs before it waits for the statistics: it may only
+    // start once everything in front of this kernel is complete.
+    pdl_wait();
+    pdl_launch_dependents();
     const size_t row = blockIdx.x;
     const uint4 *p = reinterpret_cast<const uint4 *>(logits + row * (size_t)V);
     const int nvec = V >> 3;
@@ -1743,9 +1745,8 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     const int rows = d->B * d->N;
     float2 *run_tab = use_runs ? reinterpret_cast<float2 *>(ws) : nullptr;  // (behind the hand-over area; no nucleus arrays in this form)
     if (!lazy) {
-        row_stats_kernel<<<rows, RS_THREADS, 0, st>>>(static_cast<const uint16_t *>(logits), d->V, c, row_max,
-                                                      row_sum, run_tab);
-        SR_LAUNCH_CHECK();
+        SR_CUDA_TRY(launch_dependent(true, row_stats_kernel, dim3((unsigned)rows), dim3(RS_THREADS), 0, st,
+                                     static_cast<const uint16_t *>(logits), d->V, c, row_max, row_sum, run_tab));
     }
 
     WalkArgs wa;

@@ -250,3 +250,33 @@ def test_plan_reuse_across_layers():
                         x["parent"], workspace=ws, flags=S.ATTN_REUSE_PLAN if layer > 0 else 0, check_status=True)
         diff = np.abs(host(O.float()) - o["O64"])
         assert (diff <= O_ATOL * np.maximum(1.0, np.abs(o["O64"]))).all(), (layer, diff.max())
+
+
+@pytest.mark.parametrize("lengths,N", [((937, 2404), 10), ((129,), 1), ((5000, 1, 128), 40)])
+def test_few_units_in_short_chunks_merged_behind_the_layer(lengths, N):
+    """Few work units: chunks of one to three tiles, the merge in a kernel of its own, and layers after the first that
+    reuse the plan and load their cache while that kernel may still be running.  Bound: the one of every other shape."""
+    if FLAGS["v"] != 0:
+        pytest.skip("plans are reused by the tcgen05 kernel only")
+    w = I.scaled(I.WORKLOADS["qwen1.5b"], B=len(lengths), N=N)
+    ip = np.zeros(w.B + 1, np.int32)
+    np.cumsum(lengths, out=ip[1:])
+    ws = S.alloc(S.tree_attn_workspace_bytes(w.B, N, w.Hq, w.Hkv, w.D, ip), dtype=torch.uint8, device="cuda")
+    dip, outs, refs = dev(ip), [], []
+    layers = []
+    for layer in range(3):
+        x = I.attn_inputs(I.scaled(w, kv_kind="uniform", kv_a=1, kv_b=1), layer=layer)
+        g = I.rng(99 + layer)
+        for n in ("Kc", "Vc"):
+            x[n] = I.f32_to_bf16_bits(g.standard_normal((int(ip[-1]), w.Hkv, w.D), dtype=np.float32))
+        layers.append(x)
+        refs.append(ref.tree_attn(x["Q"], x["Kc"], x["Vc"], ip, x["Kt"], x["Vt"], x["parent"], want_lse=True))
+    d = [[dev_bf16(x[n]) for n in ("Q", "Kc", "Vc", "Kt", "Vt")] for x in layers]
+    torch.cuda.synchronize()
+    for layer, t in enumerate(d):
+        flags = FLAGS["v"] | (S.ATTN_REUSE_PLAN | S.ATTN_CACHE_SETTLED if layer else 0)
+        outs.append(S.tree_attn(t[0], t[1], t[2], dip, ip, t[3], t[4], layers[layer]["parent"], want_lse=True,
+                                workspace=ws, flags=flags))
+    assert S.workspace_status(ws) == 0
+    for o, (O, lse) in zip(refs, outs):
+        check(o, host(O.float()).astype(np.float64), host(lse).astype(np.float64), edge=True)
