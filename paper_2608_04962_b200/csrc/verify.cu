@@ -28,6 +28,7 @@ constexpr int RS_THREADS = 256;
 constexpr int WALK_WARPS = 4;
 constexpr int TERM_THREADS = 512;  // two CTAs per SM
 constexpr int TERM_WARPS = TERM_THREADS / 32;
+constexpr int TERM_SMEM_LIMIT = 200 * 1024;  // slice masses of the terminal draw
 constexpr float NEG_INF = -INFINITY;
 
 // ------------------------------------------------------------------------------ row statistics
@@ -145,32 +146,30 @@ constexpr int NUC_THREADS = 512;
 // Nucleus of one row (sampling configuration of the experiments: threshold 0.95): tokens are taken in order of
 // decreasing probability until their mass first reaches top_p, and every token that ties with the last one
 // taken is kept too.  Equal probabilities are equal bf16 logits, so the kept set is "key >= threshold key".
-// Run by all NUC_THREADS threads of a CTA; the row comes from HBM once and from L2 after.  Result: st->prefix =
-// threshold key (a token is kept iff ord_key(logit) >= key), st->keep = sum of the kept exp((l - M)/T).
+// Run by all NUC_THREADS threads of a CTA; the row comes from HBM or L2 once.  Result: st->prefix = threshold key (a
+// token is kept iff ord_key(logit) >= key), st->keep = sum of the kept exp((l - M)/T).
 //
-// The threshold is searched from coarse to exact:
-//   A  256 bins of the distance below the maximum, e = (M - l) c in log2 units, 1/8 unit wide, 32 units in all:
-//      one pass, fixed-point masses added to counters in shared memory; the bin where the mass from the
-//      top reaches top_p * S is selected;
-//   C  the keys of the tokens in the selected bin are collected in shared memory (a few thousand at most);
-//   D  a radix search over the 16 key bits, four per pass, on that list alone finds the exact key.
-// A costs about a dozen instructions per token, C half of that; the bin index is the argument of the
-// exponential, which is needed anyway.  If the threshold lies beyond the bins or the list overflows, the
-// radix search runs over the whole row instead (nucleus_row_radix; same result, four full passes).
-// (Two passes of sixteen private bins per thread in place of A, every token a load, an add and a store in
-// shared memory in each: 0.80 ms for the verification of the 1.5B shape against 0.28 without a nucleus.)
-constexpr int NUC_LIST = 8192;
-constexpr int NUC_BINS = 256;
-constexpr float NUC_WB = 0.125f;
+// A token's mass depends on its 16 bits alone, so one pass COUNTS the tokens of every bf16 value in shared memory and
+// the cut is found by a scan over the values, largest first, with the masses count * exp((l - M)/T): exact key, exact
+// integer counts, no order of additions.  Two tables (the signs), one counter per value from 2^-13 up to 2^15 in
+// magnitude; the values nearer to zero share a counter.  Only tokens at or above a bound are counted: all tokens below
+// M - T ln(V / ((1 - top_p) S)) together weigh at most (1 - top_p) S, so the cut lies at or above it.  (Peaked rows
+// then count a few tokens, and the count, an atomic per token, is what the pass waits for.)  Where a counter does not
+// tell the values apart, or the counted mass stays below the target by rounding, the radix search over the whole row
+// gives the same result in four passes (nucleus_row_radix).
+constexpr int NUC_OCT_LO = (127 - 13) << 7;              // bf16 bits of 2^-13
+constexpr int NUC_VALUES = ((127 + 15) << 7) - NUC_OCT_LO;  // counters per sign; 0: nearer to zero than 2^-13
+constexpr int NUC_SIGN = 4096;                           // offset of the negative values' table
+static_assert(NUC_VALUES <= NUC_SIGN, "a table per sign");
 
 struct NucleusSmem {
-    float bins[16][NUC_THREADS];
+    union {
+        uint32_t count[2 * NUC_SIGN];
+        float bins[16][NUC_THREADS];
+    };
     float wsum[NUC_THREADS / 32][16];
-    uint32_t c_lo, c_hi;  // bf16 bits of the ends of the interval of logits that fall into the selected bin
-    uint32_t fine_lo[NUC_BINS], fine_hi[NUC_BINS];  // 64-bit fixed-point masses of the fine bins, in two words
-    unsigned short list[NUC_LIST];
-    int n_list;
-    int sel;  // bin selected by the last level
+    double wtot[NUC_THREADS / 32];
+    int sel;  // bin selected by the last level; count search: 1 found, 0 not
     float above, keep;
     uint32_t prefix;
 };
@@ -237,22 +236,6 @@ __device__ __forceinline__ void nucleus_key_bin(NucleusSmem *st, uint32_t bits, 
         st->bins[(key >> shift) & 15u][threadIdx.x] += ex2_approx((__uint_as_float(bits << 16) - M) * c);
 }
 
-// Four vectors of a row, NUC_THREADS apart, for one thread.  All four in range (every round but the last): plain
-// loads one after the other, so that all four are in flight together; a load under a condition of its own ends up
-// behind the use of the one before it.  Absent vectors read as -inf.
-__device__ __forceinline__ void nucleus_load4(const uint4 *__restrict__ p, int i0, int nvec, uint4 (&vv)[4]) {
-    if (i0 + 3 * NUC_THREADS < nvec) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) vv[q] = ld_nc_v4(p + i0 + q * NUC_THREADS);
-    } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int i = i0 + q * NUC_THREADS;
-            vv[q] = i < nvec ? ld_nc_v4(p + i) : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
-        }
-    }
-}
-
 // Exact search over the whole row (fallback): four passes, four key bits each.
 __device__ void nucleus_row_radix(const uint4 *__restrict__ p, int nvec, float c, float M, float target,
                                   NucleusSmem *st) {
@@ -279,198 +262,117 @@ __device__ void nucleus_row_radix(const uint4 *__restrict__ p, int nvec, float c
     }
 }
 
-__device__ void nucleus_row(const uint16_t *__restrict__ row_logits, int V, float c, float M, float target,
+// One counter more for the tokens of a pair of bf16 logits that are at or above the bound (lo2: the bound, twice);
+// base2: the shared-memory address of the tables, twice.
+__device__ __forceinline__ void nucleus_count2(uint32_t w, const __nv_bfloat162 &lo2, uint32_t base2) {
+    const uint32_t keep = __hge2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&w), lo2);
+    // the magnitude's steps above 2^-13, within the table (a counted token lies below 2^15), and the sign above it
+    const uint32_t mag = __viaddmin_s16x2_relu(w & 0x7fff7fffu, (uint32_t)(-NUC_OCT_LO & 0xffff) * 0x10001u, (NUC_VALUES - 1) * 0x10001u);
+    const uint32_t at = (mag | ((w >> 3) & 0x10001000u)) * 4u + base2;
+    if (keep & 0xffffu) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at & 0xffffu) : "memory");
+    if (keep >> 16) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at >> 16) : "memory");
+}
+
+__device__ void nucleus_row(const uint16_t *__restrict__ row_logits, int V, float c, float M, float S, float top_p,
                             NucleusSmem *st) {
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint4 *p = reinterpret_cast<const uint4 *>(row_logits);
     const int nvec = V >> 3;
-    const float Mc = M * c;
-    if (tid == 0) {
-        st->above = 0.f;
-        st->n_list = 0;
-    }
-    // the distance below the maximum, in log2 units, and the mass: e >= 0, mass = 2^-e
-    auto dist = [&](uint32_t bits) { return Mc - __uint_as_float(bits << 16) * c; };
-    // bin = e / width rounded to nearest, taken from the mantissa of e / width + 1.5 * 2^23 (float-to-int
-    // conversions share the special-function unit with the exponentials; this stays on the FMA and integer
-    // pipes).  Any monotone rule would do: the same one is used in every pass.
-    auto to_int = [](float x) { return (int)(__float_as_uint(x + 12582912.0f) - 0x4B400000u); };
-    // ---- A: one pass, 256 bins of 1/8 unit over the first 32 units below the maximum, masses as 32-bit fixed point
-    //      (round to nearest; the row's largest element is 2^32) added to counters in shared memory: integer
-    //      sums do not depend on the order of the atomics, so the result is the same from run to run.  Tokens
-    //      further down fall outside the bins; a cut among them goes to the exact search below.
-    auto bin_ab = [&](float e) { return to_int(e * (1.0f / NUC_WB)); };  // (>= 0; >= NUC_BINS: outside)
-    // (one copy of the counters per warp, in the storage of the private bins of the later steps: only the lanes
-    // of a warp can meet at a counter.  Rows of more than 2^20 tokens could overflow a counter: exact search.)
-    if (nvec > (1 << 17)) {
+    const float target = top_p * S;
+    const uint32_t base = smem_u32(st->count);
+    // the bound, one bf16 step below its value (the rest of its rounding does not matter: a cut that the counted
+    // tokens do not reach is searched over the whole row)
+    float bound = fmaxf(M - (log2f((float)V) - log2f(S - target)) / c, -32000.0f);
+    bound = fminf(bound, M);  // (top_p near 0)
+    bound -= 0.008f * fabsf(bound);
+    const uint32_t lo_bits = __bfloat16_as_ushort(__float2bfloat16_rd(bound));
+    const bool counted = fabsf(M) < 32000.0f && bound == bound && bound <= M && base + sizeof(st->count) <= 0x10000u;
+    if (!counted) {  // (uniform over the CTA)
         nucleus_row_radix(p, nvec, c, M, target, st);
         return;
     }
-    static_assert(sizeof(st->bins) >= (NUC_THREADS / 32) * 2 * NUC_BINS * sizeof(uint32_t), "per-warp fine bins fit");
-    uint32_t *wfine = reinterpret_cast<uint32_t *>(&st->bins[0][0]) + (tid >> 5) * 2 * NUC_BINS;
-    for (int j = tid; j < (NUC_THREADS / 32) * 2 * NUC_BINS; j += NUC_THREADS) reinterpret_cast<uint32_t *>(&st->bins[0][0])[j] = 0u;
-    __syncthreads();
-    for (int i0 = tid; i0 < nvec; i0 += 4 * NUC_THREADS) {
-        uint4 vv[4];  // four independent loads in flight; an absent one reads as -inf (no mass)
-        nucleus_load4(p, i0, nvec, vv);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t w[4] = {vv[q].x, vv[q].y, vv[q].z, vv[q].w};
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                const float e = dist((t & 1) ? (w[t >> 1] >> 16) : (w[t >> 1] & 0xffffu));
-                const int j = bin_ab(e);
-                if (j < NUC_BINS) {
-                    // the two halves of the 32-bit mass go to counters of their own: a warp's share of the row is at
-                    // most 2^16 tokens, so neither can overflow, and the additions need no result back
-                    const uint32_t v = __float2uint_rn(ex2_approx(-e) * 4294967296.0f);
-                    atomicAdd(&wfine[j], v & 0xffffu);
-                    if (v >> 16) atomicAdd(&wfine[NUC_BINS + j], v >> 16);  // (most tokens are far below the maximum)
-                }
-            }
-        }
-    }
-    __syncthreads();
-    for (int j = tid; j < NUC_BINS; j += NUC_THREADS) {
-        unsigned long long tot = 0ull;
-        for (int w2 = 0; w2 < NUC_THREADS / 32; ++w2) {
-            const uint32_t *wf = reinterpret_cast<const uint32_t *>(&st->bins[0][0]) + w2 * 2 * NUC_BINS;
-            tot += ((unsigned long long)wf[NUC_BINS + j] << 16) + wf[j];
-        }
-        st->fine_lo[j] = (uint32_t)tot;
-        st->fine_hi[j] = (uint32_t)(tot >> 32);
-    }
-    __syncthreads();
-    if (tid < 32) {
-        // the bin at which the mass from the top reaches the target: every lane takes eight consecutive bins
-        const unsigned long long tgt = (unsigned long long)((double)target * 4294967296.0);
-        unsigned long long mine = 0ull;
-        auto fine = [&](int j) { return ((unsigned long long)st->fine_hi[j] << 32) | st->fine_lo[j]; };
-#pragma unroll
-        for (int q = 0; q < NUC_BINS / 32; ++q) mine += fine(tid * (NUC_BINS / 32) + q);
-        unsigned long long incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long x = __shfl_up_sync(0xffffffffu, incl, o);
-            if (tid >= o) incl += x;
-        }
-        const unsigned hit = __ballot_sync(0xffffffffu, incl >= tgt);
-        if (hit == 0u) {
-            if (tid == 0) st->sel = -1;  // the cut lies further down than the bins reach
-        } else if (tid == __ffs(hit) - 1) {
-            unsigned long long cum = incl - mine;
-            int j = tid * (NUC_BINS / 32);
-            while (cum + fine(j) < tgt) cum += fine(j++);  // (ends inside this lane's bins)
-            st->sel = j;
-            st->above = (float)((double)cum * (1.0 / 4294967296.0));
-            st->keep = (float)((double)(cum + fine(j)) * (1.0 / 4294967296.0));
-        }
-    }
-    __syncthreads();
-    const int jb = st->sel;
-    if (jb < 0) {  // exact search over the whole row
-        nucleus_row_radix(p, nvec, c, M, target, st);
-        return;
-    }
-    // ---- C: the tokens of bin jb.  The bin index does not increase with the logit, so they are the logits of an
-    //      interval, whose two ends thread 0 finds by bisection over the 16-bit keys (between the most negative finite
-    //      value and the row's maximum) with the very rule of pass A; the pass then compares packed bf16 pairs with
-    //      the two ends and looks closer only at vectors that hold a member (a few per cent).
-    if (tid == 0) {
-        auto bits_of_key = [](uint32_t key) { return (key & 0x8000u) ? (key & 0x7fffu) : (~key & 0xffffu); };
-        auto bin_of_key = [&](uint32_t key) { return bin_ab(dist(bits_of_key(key))); };
-        const uint32_t k_min = ord_key(0xff7fu), k_max = ord_key(__float_as_uint(M) >> 16);
-        // smallest key whose bin is <= jb (the bins fall as the keys rise; bin(k_max) = 0 <= jb)
-        uint32_t lo = k_min, hi = k_max;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (bin_of_key(mid) <= jb)
-                hi = mid;
-            else
-                lo = mid + 1;
-        }
-        const uint32_t k_lo = lo;
-        // largest key whose bin is >= jb (bin(k_lo) = jb: pass A found a token there)
-        lo = k_lo;
-        hi = k_max;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi + 1) >> 1;
-            if (bin_of_key(mid) >= jb)
-                lo = mid;
-            else
-                hi = mid - 1;
-        }
-        st->c_lo = bits_of_key(k_lo);
-        st->c_hi = bits_of_key(lo);
-    }
+    for (int j = 0; j < 2 * NUC_SIGN / (4 * NUC_THREADS); ++j)
+        reinterpret_cast<uint4 *>(st->count)[j * NUC_THREADS + tid] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) st->sel = 0;
     __syncthreads();
     {
-        auto as_bf162 = [](uint32_t w_) { return *reinterpret_cast<const __nv_bfloat162 *>(&w_); };
-        const __nv_bfloat162 lo2 = as_bf162(st->c_lo | (st->c_lo << 16)), hi2 = as_bf162(st->c_hi | (st->c_hi << 16));
-        // (the loop bound is the same for all lanes of a warp: the body votes and scans over the whole warp; an
-        // absent vector reads as -inf, which no interval of finite ends holds)
-        for (int ib = tid & ~31; ib < nvec; ib += 4 * NUC_THREADS) {
-            const int i0 = ib + (tid & 31);
-            uint4 vv[4];
-            nucleus_load4(p, i0, nvec, vv);
-            // the members among this thread's 32 logits, as one bit each; one reservation in the list per warp and
-            // round: the lanes' counts are scanned over the warp
-            uint32_t member = 0u;
+        const uint32_t base2 = base * 0x10001u, lob2 = lo_bits * 0x10001u;
+        const __nv_bfloat162 lo2 = *reinterpret_cast<const __nv_bfloat162 *>(&lob2);
+        auto count8 = [&](const uint4 &v) {
+            nucleus_count2(v.x, lo2, base2);
+            nucleus_count2(v.y, lo2, base2);
+            nucleus_count2(v.z, lo2, base2);
+            nucleus_count2(v.w, lo2, base2);
+        };
+        int i = tid;
+        for (; i + 3 * NUC_THREADS < nvec; i += 4 * NUC_THREADS) {
+            uint4 v[4];  // four independent loads in flight
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t w[4] = {vv[q].x, vv[q].y, vv[q].z, vv[q].w};
+            for (int q = 0; q < 4; ++q) v[q] = ld_nc_v4(p + i + q * NUC_THREADS);
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const uint32_t mk = __hge2_mask(as_bf162(w[t]), lo2) & __hle2_mask(as_bf162(w[t]), hi2);
-                    member |= ((mk & 1u) | ((mk >> 15) & 2u)) << (8 * q + 2 * t);
-                }
-            }
-            if (__ballot_sync(0xffffffffu, member != 0u) == 0u) continue;
-            const int cnt = __popc(member);
-            int incl = cnt;
+            for (int q = 0; q < 4; ++q) count8(v[q]);
+        }
+        for (; i < nvec; i += NUC_THREADS) count8(ld_nc_v4(p + i));
+    }
+    __syncthreads();
+    // place r of the scan: values in falling order, 0 = the largest positive one, ZERO = the counter around zero
+    constexpr int ZERO = NUC_VALUES - 1;
+    auto place = [&](uint32_t bits) {
+        const int m = max((int)(bits & 0x7fffu) - NUC_OCT_LO, 0);
+        return (bits & 0x8000u) ? ZERO + m : ZERO - m;
+    };
+    auto value_bits = [&](int r) {  // (the counter around zero: 0)
+        return r < ZERO ? (uint32_t)(ZERO - r + NUC_OCT_LO) : r > ZERO ? (uint32_t)(r - ZERO + NUC_OCT_LO) | 0x8000u : 0u;
+    };
+    auto count_at = [&](int r) {
+        return r < ZERO ? st->count[ZERO - r] : r > ZERO ? st->count[NUC_SIGN + r - ZERO] : st->count[0] + st->count[NUC_SIGN];
+    };
+    auto mass_at = [&](int r) {
+        const uint32_t n = count_at(r);
+        return n ? (double)n * (double)ex2_approx((bf16_bits_to_float(value_bits(r)) - M) * c) : 0.0;
+    };
+    const int r0 = place(__float_as_uint(M) >> 16), r1 = place(lo_bits);
+    const int per = (r1 - r0 + NUC_THREADS) / NUC_THREADS;
+    const int my0 = r0 + tid * per, my1 = min(r1 + 1, my0 + per);
+    double mine = 0.0;
+    for (int r = my0; r < my1; ++r) mine += mass_at(r);
+    double incl = mine;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int x = __shfl_up_sync(0xffffffffu, incl, o);
-                if ((tid & 31) >= o) incl += x;
-            }
-            int base = 0;
-            if ((tid & 31) == 31) base = atomicAdd(&st->n_list, incl);
-            base = __shfl_sync(0xffffffffu, base, 31);
-            int pos = base + incl - cnt;
-            if (cnt) {  // (element 8 q + 2 t + half of this round)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint32_t w[4] = {vv[q].x, vv[q].y, vv[q].z, vv[q].w};
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) {
-                        if ((member >> (8 * q + t)) & 1u) {
-                            if (pos < NUC_LIST) st->list[pos] = (unsigned short)((t & 1) ? (w[t >> 1] >> 16) : (w[t >> 1] & 0xffffu));
-                            ++pos;
-                        }
-                    }
-                }
-            }
+    for (int o = 1; o < 32; o <<= 1) {
+        const double x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+    }
+    if (lane == 31) st->wtot[warp] = incl;
+    __syncthreads();
+    // (a thread's end is formed as its successor's beginning, so that one thread at most holds the target)
+    double before = 0.0;
+    for (int w = 0; w < warp; ++w) before += st->wtot[w];
+    const double up = __shfl_up_sync(0xffffffffu, incl, 1);
+    const double excl = lane ? before + up : before, end = before + incl;
+    if (excl < (double)target && end >= (double)target) {
+        double cum = excl;
+        int r = my0, last = my0;
+        for (; r < my1; ++r) {
+            const double m = mass_at(r);
+            if (m > 0.0) last = r;
+            cum += m;
+            if (cum >= (double)target) break;
+        }
+        // The counter around zero: it must not be the cut, and its values must not differ by more than their mass's
+        // rounding if it lies above the cut.
+        bool ok = last != ZERO;
+        if (last > ZERO && r0 <= ZERO) ok = ok && mass_at(ZERO) * (double)(c * 0.6931472f) * 0x1p-13 <= 0x1p-24 * (double)S;
+        if (ok) {
+            st->prefix = ord_key(value_bits(last));
+            st->keep = (float)cum;
+            st->sel = 1;
         }
     }
     __syncthreads();
-    const int n_list = st->n_list;
-    if (n_list > NUC_LIST) {  // more tokens in one sub-bin than the list holds: exact search over the whole row
-        __syncthreads();
-        nucleus_row_radix(p, nvec, c, M, target, st);
-        return;
-    }
-    // ---- D: st->above is the mass above the sub-bin; the key search runs on the list
-    if (tid == 0) st->prefix = 0u;
+    const int sel = st->sel;
     __syncthreads();
-    for (int level = 0; level < 4; ++level) {
-        const uint32_t prefix = st->prefix;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) st->bins[j][tid] = 0.f;
-        for (int i = tid; i < n_list; i += NUC_THREADS) nucleus_key_bin(st, st->list[i], level, prefix, M, c);
-        nucleus_pick(st, target, true);
-        if (tid == 0) st->prefix = (prefix << 4) | (uint32_t)st->sel;
-        __syncthreads();
-    }
+    if (sel == 0) nucleus_row_radix(p, nvec, c, M, target, st);
 }
 
 // ------------------------------------------------------------------------------ walk
@@ -942,119 +844,6 @@ __device__ void row_stats_row(const uint16_t *__restrict__ row_logits, int V, fl
     *S_out = sb;
 }
 
-// One CTA per sequence, for the two variants in which something has to be computed per visited node before the
-// node can be walked, and which nodes are visited is known only as the walk goes:
-//   LAZY  the softmax statistics of a row are computed when the walk reaches it (at most K + 1 rows per
-//         sequence instead of all N), and written to row_max / row_sum for those rows only;
-//   NUC   the target distributions are their nuclei: the row's threshold is searched (nucleus_row) and left
-//         in thr_key / keep_sum (the terminal draw reads those of the last node).
-// Before each node all threads do that work, then warp 0 does the node.
-template <bool LAZY, bool NUC>
-__global__ void __launch_bounds__(NUC_THREADS)
-walk_cta_kernel(WalkArgs a, Topo topo, float c, float top_p, float *__restrict__ row_max_w,
-                float *__restrict__ row_sum_w, uint32_t *__restrict__ thr_key, float *__restrict__ keep_sum,
-                float *__restrict__ out_thr, float *__restrict__ out_sum, int thr_ready) {
-    extern __shared__ __align__(16) unsigned char nuc_raw[];  // NucleusSmem (NUC only): above the static limit
-    NucleusSmem &nuc = *reinterpret_cast<NucleusSmem *>(nuc_raw);
-    __shared__ WalkSmem sm;
-    __shared__ float sm_m[NUC_THREADS / 32], sm_s[NUC_THREADS / 32];
-    __shared__ int sh_next;  // next node, or -1 when the walk is over
-    const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WalkState st;
-    if (warp == 0) walk_begin(a, b, lane, &st);
-    int u = 0;
-    for (;;) {
-        const size_t row = (size_t)b * a.N + u;
-        float M, S;
-        if constexpr (LAZY) {
-            row_stats_row(a.logits + row * a.V, a.V, c, sm_m, sm_s, &M, &S);
-            if (threadIdx.x == 0) {
-                row_max_w[row] = M;
-                row_sum_w[row] = S;
-            }
-        } else {
-            M = a.row_max[row];
-            S = a.row_sum[row];
-        }
-        uint32_t thr = 0u;
-        float norm = S;
-        if constexpr (NUC) {
-            if (thr_ready && topo.n_child[u] > 0) {  // (left by nucleus_rows_kernel for every node with children)
-                thr = thr_key[row];
-                norm = keep_sum[row];
-            } else {
-                nucleus_row(a.logits + row * a.V, a.V, c, M, top_p * S, &nuc);
-                thr = nuc.prefix;
-                norm = nuc.keep;
-            }
-            if (threadIdx.x == 0 && !(thr_ready && topo.n_child[u] > 0)) {
-                thr_key[row] = thr;
-                keep_sum[row] = norm;
-                if (out_sum) out_sum[row] = norm;
-                if (out_thr) {  // the threshold as a logit: undo the key
-                    const uint32_t bits = (thr & 0x8000u) ? (thr & 0x7fffu) : (~thr & 0xffffu);
-                    out_thr[row] = __uint_as_float(bits << 16);
-                }
-            }
-        }
-        if (warp == 0) {
-            int next = -1;
-            if (topo.n_child[u] == 0) {
-                st.kind = (u != 0) ? 1 : 0;
-                st.have_residual = false;
-            } else {
-                next = walk_node(a, topo, b, u, (double)M, (double)norm, thr, lane, &sm, &st);
-                if (next < 0) {
-                    st.kind = 0;
-                    st.have_residual = true;
-                }
-            }
-            if (next < 0) walk_end(a, b, u, (double)norm, lane, &sm, &st);
-            if (lane == 0) sh_next = next;
-        }
-        __syncthreads();
-        const int next = sh_next;
-        __syncthreads();
-        if (next < 0) break;
-        u = next;
-    }
-}
-
-// The nucleus thresholds of every node with children, one CTA per (sequence, such node), all at once: which of
-// them the walk visits is not known yet, but a row's threshold depends on the row alone, and one pass of all
-// of them over the machine costs less than the visited ones one after the other inside a sequence's walk.  (A
-// sequence that ends at a leaf still needs that leaf's threshold for its last token: the walk kernel finds it.)
-#ifndef NUC_AHEAD_ROWS_PER_SM
-#define NUC_AHEAD_ROWS_PER_SM 5
-#endif
-struct NodeList {
-    int32_t n;
-    int8_t node[SPECROLL_MAX_NODES];
-};
-
-__global__ void __launch_bounds__(NUC_THREADS)
-nucleus_rows_kernel(const uint16_t *__restrict__ logits, int V, int N, NodeList nodes, float c, float top_p,
-                    const float *__restrict__ row_max, const float *__restrict__ row_sum,
-                    uint32_t *__restrict__ thr_key, float *__restrict__ keep_sum, float *__restrict__ out_thr,
-                    float *__restrict__ out_sum) {
-    extern __shared__ __align__(16) unsigned char nuc_raw[];
-    NucleusSmem &nuc = *reinterpret_cast<NucleusSmem *>(nuc_raw);
-    const int b = blockIdx.x / nodes.n, u = nodes.node[blockIdx.x - b * nodes.n];
-    const size_t row = (size_t)b * N + u;
-    const float M = row_max[row], S = row_sum[row];
-    nucleus_row(logits + row * V, V, c, M, top_p * S, &nuc);
-    if (threadIdx.x == 0) {
-        const uint32_t thr = nuc.prefix;
-        thr_key[row] = thr;
-        keep_sum[row] = nuc.keep;
-        if (out_sum) out_sum[row] = nuc.keep;
-        if (out_thr) {  // the threshold as a logit: undo the key
-            const uint32_t bits = (thr & 0x8000u) ? (thr & 0x7fffu) : (~thr & 0xffffu);
-            out_thr[row] = __uint_as_float(bits << 16);
-        }
-    }
-}
-
 // ------------------------------------------------------------------------------ terminal draw
 
 struct TermArgs {
@@ -1064,11 +853,9 @@ struct TermArgs {
     const int32_t *n_acc, *term_node;
     const int32_t *ws_nov, *ws_ovid;
     const double *ws_ovm;
-    const uint32_t *thr_key;  // nucleus threshold per row (NULL: no truncation)
     int32_t *out_tok;
     int32_t B, N, K, k, V;
     float c;  // log2(e) / T
-    int32_t row_per_seq;  // logits holds one row per sequence (that of its terminal node) instead of [B, N, V]
 };
 
 // Plain softmax masses of eight tokens; tokens below the nucleus threshold (thr = 0: none) weigh nothing.
@@ -1251,21 +1038,17 @@ __host__ __device__ inline int term_slices(int V) {
     return (vpw + 31) / 32;
 }
 
-__global__ void __launch_bounds__(TERM_THREADS) terminal_kernel(TermArgs a) {
-    extern __shared__ double sh_slice[];  // [TERM_WARPS][n_sl]
+// By all TERM_THREADS threads of a CTA; sh_slice: TERM_WARPS * term_slices(V) doubles.  (M, thr: the row's maximum and
+// nucleus threshold key, 0 for none; the walk's results of sequence b are read from where walk_end left them.)
+__device__ void terminal_draw(const TermArgs &a, int b, const uint16_t *__restrict__ lg, float M, uint32_t thr, double *sh_slice) {
     __shared__ double sh_seg[32];
     __shared__ double sh_ovm[SPECROLL_MAX_TOPK];
     __shared__ int32_t sh_ovid[SPECROLL_MAX_TOPK];
     __shared__ int sh_pick[2];     // target warp, -1 if none
     __shared__ double sh_base[2];  // mass before the target warp's segment; target
 
-    const int b = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int node = a.term_node[b];
     const int nov = a.ws_nov[b];
-    const float M = a.row_max[(size_t)b * a.N + node];
-    const uint32_t thr = a.thr_key ? a.thr_key[(size_t)b * a.N + node] : 0u;
-    const uint16_t *lg = a.logits + (a.row_per_seq ? (size_t)b : (size_t)b * a.N + node) * a.V;
     const uint4 *p = reinterpret_cast<const uint4 *>(lg);
     const int nvec = a.V >> 3;
     const int vpw = (nvec + TERM_WARPS - 1) / TERM_WARPS;  // vectors per warp segment
@@ -1332,6 +1115,133 @@ __global__ void __launch_bounds__(TERM_THREADS) terminal_kernel(TermArgs a) {
 
     term_pick(p, sh_slice + warp * n_sl, n_sl, v_lo, v_hi, sh_base[0], sh_base[1], M, a.c, thr, nov, sh_ovid, sh_ovm, dst,
               lane);
+}
+
+// One CTA per sequence, for rows that were made after the walk (one per sequence).
+__global__ void __launch_bounds__(TERM_THREADS) terminal_kernel(TermArgs a) {
+    extern __shared__ double sh_slice[];  // [TERM_WARPS][n_sl]
+    const int b = blockIdx.x;
+    terminal_draw(a, b, a.logits + (size_t)b * a.V, a.row_max[(size_t)b * a.N + a.term_node[b]], 0u, sh_slice);
+}
+
+// ------------------------------------------------------------------------------ walk, a CTA per sequence
+
+// One CTA per sequence, for the two variants in which something has to be computed per visited node before the
+// node can be walked, and which nodes are visited is known only as the walk goes:
+//   LAZY  the softmax statistics of a row are computed when the walk reaches it (at most K + 1 rows per
+//         sequence instead of all N), and written to row_max / row_sum for those rows only;
+//   NUC   the target distributions are their nuclei: the row's threshold is searched (nucleus_row) and left
+//         in thr_key / keep_sum.
+// Before each node all threads do that work, then warp 0 does the node.  The terminal draw from the last node's row,
+// which the CTA has just read, follows in the same launch.
+template <bool LAZY, bool NUC>
+__global__ void __launch_bounds__(NUC_THREADS, 2)
+walk_cta_kernel(WalkArgs a, Topo topo, float c, float top_p, float *__restrict__ row_max_w,
+                float *__restrict__ row_sum_w, uint32_t *__restrict__ thr_key, float *__restrict__ keep_sum,
+                float *__restrict__ out_thr, float *__restrict__ out_sum, int thr_ready, TermArgs ta) {
+    extern __shared__ __align__(16) unsigned char nuc_raw[];  // NucleusSmem (NUC only), then the draw's slice masses
+    NucleusSmem &nuc = *reinterpret_cast<NucleusSmem *>(nuc_raw);
+    __shared__ WalkSmem sm;
+    __shared__ float sm_m[NUC_THREADS / 32], sm_s[NUC_THREADS / 32];
+    __shared__ int sh_next;  // next node, or -1 when the walk is over
+    const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    WalkState st;
+    pdl_wait();  // (set up under the tail of the kernel before, which made the statistics or the thresholds)
+    if (warp == 0) walk_begin(a, b, lane, &st);
+    int u = 0;
+    float M, S;
+    uint32_t thr;
+    for (;;) {
+        const size_t row = (size_t)b * a.N + u;
+        if constexpr (LAZY) {
+            row_stats_row(a.logits + row * a.V, a.V, c, sm_m, sm_s, &M, &S);
+            if (threadIdx.x == 0) {
+                row_max_w[row] = M;
+                row_sum_w[row] = S;
+            }
+        } else {
+            M = a.row_max[row];
+            S = a.row_sum[row];
+        }
+        thr = 0u;
+        float norm = S;
+        if constexpr (NUC) {
+            if (thr_ready && topo.n_child[u] > 0) {  // (left by nucleus_rows_kernel for every node with children)
+                thr = thr_key[row];
+                norm = keep_sum[row];
+            } else {
+                nucleus_row(a.logits + row * a.V, a.V, c, M, S, top_p, &nuc);
+                thr = nuc.prefix;
+                norm = nuc.keep;
+            }
+            if (threadIdx.x == 0 && !(thr_ready && topo.n_child[u] > 0)) {
+                thr_key[row] = thr;
+                keep_sum[row] = norm;
+                if (out_sum) out_sum[row] = norm;
+                if (out_thr) {  // the threshold as a logit: undo the key
+                    const uint32_t bits = (thr & 0x8000u) ? (thr & 0x7fffu) : (~thr & 0xffffu);
+                    out_thr[row] = __uint_as_float(bits << 16);
+                }
+            }
+        }
+        if (warp == 0) {
+            int next = -1;
+            if (topo.n_child[u] == 0) {
+                st.kind = (u != 0) ? 1 : 0;
+                st.have_residual = false;
+            } else {
+                next = walk_node(a, topo, b, u, (double)M, (double)norm, thr, lane, &sm, &st);
+                if (next < 0) {
+                    st.kind = 0;
+                    st.have_residual = true;
+                }
+            }
+            if (next < 0) walk_end(a, b, u, (double)norm, lane, &sm, &st);
+            if (lane == 0) sh_next = next;
+        }
+        __syncthreads();
+        const int next = sh_next;
+        __syncthreads();
+        if (next < 0) break;
+        u = next;
+    }
+    terminal_draw(ta, b, a.logits + ((size_t)b * a.N + u) * a.V, M, thr, reinterpret_cast<double *>(nuc_raw));
+}
+
+// The nucleus thresholds of every node with children, one CTA per (sequence, such node), all at once: which of
+// them the walk visits is not known yet, but a row's threshold depends on the row alone, and one pass of all
+// of them over the machine costs less than the visited ones one after the other inside a sequence's walk.  (A
+// sequence that ends at a leaf still needs that leaf's threshold for its last token: the walk kernel finds it.)
+#ifndef NUC_AHEAD_ROWS_PER_SM
+#define NUC_AHEAD_ROWS_PER_SM 5
+#endif
+struct NodeList {
+    int32_t n;
+    int8_t node[SPECROLL_MAX_NODES];
+};
+
+__global__ void __launch_bounds__(NUC_THREADS, 3)
+nucleus_rows_kernel(const uint16_t *__restrict__ logits, int V, int N, NodeList nodes, float c, float top_p,
+                    const float *__restrict__ row_max, const float *__restrict__ row_sum,
+                    uint32_t *__restrict__ thr_key, float *__restrict__ keep_sum, float *__restrict__ out_thr,
+                    float *__restrict__ out_sum) {
+    extern __shared__ __align__(16) unsigned char nuc_raw[];
+    NucleusSmem &nuc = *reinterpret_cast<NucleusSmem *>(nuc_raw);
+    pdl_wait();
+    const int b = blockIdx.x / nodes.n, u = nodes.node[blockIdx.x - b * nodes.n];
+    const size_t row = (size_t)b * N + u;
+    const float M = row_max[row], S = row_sum[row];
+    nucleus_row(logits + row * V, V, c, M, S, top_p, &nuc);
+    if (threadIdx.x == 0) {
+        const uint32_t thr = nuc.prefix;
+        thr_key[row] = thr;
+        keep_sum[row] = nuc.keep;
+        if (out_sum) out_sum[row] = nuc.keep;
+        if (out_thr) {  // the threshold as a logit: undo the key
+            const uint32_t bits = (thr & 0x8000u) ? (thr & 0x7fffu) : (~thr & 0xffffu);
+            out_thr[row] = __uint_as_float(bits << 16);
+        }
+    }
 }
 
 // ------------------------------------------------------------------------------ walk + terminal draw in one launch
@@ -1658,9 +1568,9 @@ static int walk_term_split(int B) {
 
 static int launch_terminal(const TermArgs &ta, cudaStream_t st) {
     const size_t smem = (size_t)TERM_WARPS * term_slices(ta.V) * sizeof(double);
-    if (smem > 200 * 1024) return SPECROLL_ELIMIT;
-    if (smem > 40 * 1024)
-        SR_CUDA_TRY(cudaFuncSetAttribute(terminal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > (size_t)TERM_SMEM_LIMIT) return SPECROLL_ELIMIT;
+    const int rc = device_setup(reinterpret_cast<const void *>(terminal_kernel), TERM_SMEM_LIMIT, nullptr);
+    if (rc != SPECROLL_OK) return rc;
     terminal_kernel<<<ta.B, TERM_THREADS, smem, st>>>(ta);
     SR_LAUNCH_CHECK();
     return SPECROLL_OK;
@@ -1774,15 +1684,32 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     wa.k = d->k;
     wa.V = d->V;
     wa.T = (double)d->temperature;
-    if (truncate) {
-        int rc_ = device_setup(reinterpret_cast<const void *>(walk_cta_kernel<false, true>), (int)sizeof(NucleusSmem), nullptr);
-        if (rc_ == SPECROLL_OK)
-            rc_ = device_setup(reinterpret_cast<const void *>(walk_cta_kernel<true, true>), (int)sizeof(NucleusSmem), nullptr);
+    if (truncate || lazy) {
+        TermArgs ta;
+        ta.logits = wa.logits;
+        ta.u_fin = u_fin;
+        ta.row_max = row_max;
+        ta.n_acc = n_acc;
+        ta.term_node = term_node;
+        ta.ws_nov = ws_nov;
+        ta.ws_ovid = ws_ovid;
+        ta.ws_ovm = ws_ovm;
+        ta.out_tok = out_tok;
+        ta.B = d->B;
+        ta.N = d->N;
+        ta.K = d->K;
+        ta.k = d->k;
+        ta.V = d->V;
+        ta.c = c;
+        // (the draw's slice masses take the threshold search's place once the walk is over)
+        const size_t slices = (size_t)TERM_WARPS * term_slices(d->V) * sizeof(double);
+        if (slices > (size_t)TERM_SMEM_LIMIT) return SPECROLL_ELIMIT;
+        const size_t smem = truncate && sizeof(NucleusSmem) > slices ? sizeof(NucleusSmem) : slices;
+        auto *const kern = truncate ? (lazy ? walk_cta_kernel<true, true> : walk_cta_kernel<false, true>) : walk_cta_kernel<true, false>;
+        int rc_ = device_setup(reinterpret_cast<const void *>(kern), TERM_SMEM_LIMIT, nullptr);
         if (rc_ != SPECROLL_OK) return rc_;
-        if (lazy) {
-            walk_cta_kernel<true, true><<<d->B, NUC_THREADS, sizeof(NucleusSmem), st>>>(
-                wa, topo, c, top_p, row_max, row_sum, thr_key, keep_sum, nucleus_thr, nucleus_sum, 0);
-        } else {
+        bool ahead = false;
+        if (truncate && !lazy) {
             NodeList nodes;
             nodes.n = 0;
             for (int u = 0; u < d->N; ++u)
@@ -1793,70 +1720,45 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
             int n_sm = 0;
             rc_ = device_setup(reinterpret_cast<const void *>(nucleus_rows_kernel), (int)sizeof(NucleusSmem), &n_sm);
             if (rc_ != SPECROLL_OK) return rc_;
-            const bool ahead = nodes.n > 0 && d->B * nodes.n <= NUC_AHEAD_ROWS_PER_SM * n_sm;
-            if (ahead) {
-                nucleus_rows_kernel<<<d->B * nodes.n, NUC_THREADS, sizeof(NucleusSmem), st>>>(
-                    static_cast<const uint16_t *>(logits), d->V, d->N, nodes, c, top_p, row_max, row_sum, thr_key, keep_sum,
-                    nucleus_thr, nucleus_sum);
-                SR_LAUNCH_CHECK();
-            }
-            walk_cta_kernel<false, true><<<d->B, NUC_THREADS, sizeof(NucleusSmem), st>>>(
-                wa, topo, c, top_p, row_max, row_sum, thr_key, keep_sum, nucleus_thr, nucleus_sum, ahead ? 1 : 0);
+            ahead = nodes.n > 0 && d->B * nodes.n <= NUC_AHEAD_ROWS_PER_SM * n_sm;
+            if (ahead)
+                SR_CUDA_TRY(launch_dependent(true, nucleus_rows_kernel, dim3((unsigned)(d->B * nodes.n)), dim3(NUC_THREADS),
+                                             sizeof(NucleusSmem), st, static_cast<const uint16_t *>(logits), d->V, d->N, nodes, c,
+                                             top_p, row_max, row_sum, thr_key, keep_sum, nucleus_thr, nucleus_sum));
         }
-    } else if (lazy) {
-        walk_cta_kernel<true, false><<<d->B, NUC_THREADS, 0, st>>>(wa, topo, c, 1.0f, row_max, row_sum, nullptr, nullptr,
-                                                                    nullptr, nullptr, 0);
-    } else {
-        // plain verification: the walk and the terminal draw in one launch, overlapping the statistics kernel's tail
-        constexpr int WT_SMEM_LIMIT = 160 * 1024;
-        const int S = use_runs ? 1 : walk_term_split(d->B);
-        const WtLayout L = wt_layout(d->N, d->K, d->k, d->V, S);
-        if (L.total > (size_t)WT_SMEM_LIMIT) return SPECROLL_ELIMIT;
-        const int rc_ = device_setup(reinterpret_cast<const void *>(walk_term_kernel), WT_SMEM_LIMIT, nullptr);
-        if (rc_ != SPECROLL_OK) return rc_;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(d->B * S));
-        cfg.blockDim = dim3(WT_THREADS);
-        cfg.dynamicSmemBytes = L.total;
-        cfg.stream = st;
-        cudaLaunchAttribute attrs[2];
-        int na = 0;
-        attrs[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attrs[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-        if (S > 1) {
-            attrs[na].id = cudaLaunchAttributeClusterDimension;
-            attrs[na].val.clusterDim.x = (unsigned)S;
-            attrs[na].val.clusterDim.y = 1;
-            attrs[na].val.clusterDim.z = 1;
-            ++na;
-        }
-        cfg.attrs = attrs;
-        cfg.numAttrs = na;
-        SR_CUDA_TRY(cudaLaunchKernelEx(&cfg, walk_term_kernel, wa, topo, u_fin, c, S, (const float2 *)run_tab));
+        SR_CUDA_TRY(launch_dependent(true, kern, dim3((unsigned)d->B), dim3(NUC_THREADS), smem, st, wa, topo, c,
+                                     truncate ? top_p : 1.0f, row_max, row_sum, thr_key, keep_sum, truncate ? nucleus_thr : nullptr,
+                                     truncate ? nucleus_sum : nullptr, ahead ? 1 : 0, ta));
         return SPECROLL_OK;
     }
-    SR_LAUNCH_CHECK();
-
-    TermArgs ta;
-    ta.logits = wa.logits;
-    ta.u_fin = u_fin;
-    ta.row_max = row_max;
-    ta.n_acc = n_acc;
-    ta.term_node = term_node;
-    ta.ws_nov = ws_nov;
-    ta.ws_ovid = ws_ovid;
-    ta.ws_ovm = ws_ovm;
-    ta.thr_key = thr_key;
-    ta.out_tok = out_tok;
-    ta.B = d->B;
-    ta.N = d->N;
-    ta.K = d->K;
-    ta.k = d->k;
-    ta.V = d->V;
-    ta.c = c;
-    ta.row_per_seq = 0;
-    return launch_terminal(ta, st);
+    // plain verification: the walk and the terminal draw in one launch, overlapping the statistics kernel's tail
+    constexpr int WT_SMEM_LIMIT = 160 * 1024;
+    const int S = use_runs ? 1 : walk_term_split(d->B);
+    const WtLayout L = wt_layout(d->N, d->K, d->k, d->V, S);
+    if (L.total > (size_t)WT_SMEM_LIMIT) return SPECROLL_ELIMIT;
+    const int rc_ = device_setup(reinterpret_cast<const void *>(walk_term_kernel), WT_SMEM_LIMIT, nullptr);
+    if (rc_ != SPECROLL_OK) return rc_;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(d->B * S));
+    cfg.blockDim = dim3(WT_THREADS);
+    cfg.dynamicSmemBytes = L.total;
+    cfg.stream = st;
+    cudaLaunchAttribute attrs[2];
+    int na = 0;
+    attrs[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attrs[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+    if (S > 1) {
+        attrs[na].id = cudaLaunchAttributeClusterDimension;
+        attrs[na].val.clusterDim.x = (unsigned)S;
+        attrs[na].val.clusterDim.y = 1;
+        attrs[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    cfg.attrs = attrs;
+    cfg.numAttrs = na;
+    SR_CUDA_TRY(cudaLaunchKernelEx(&cfg, walk_term_kernel, wa, topo, u_fin, c, S, (const float2 *)run_tab));
+    return SPECROLL_OK;
 }
 
 // The hand-over area between the walk and the terminal draw inside a workspace (the layout of run_verify).
@@ -1962,7 +1864,6 @@ extern "C" int specroll_verify_terminal_rows(const specroll_verify_desc *d, cons
     ta.ws_nov = nov;
     ta.ws_ovid = ovid;
     ta.ws_ovm = ovm;
-    ta.thr_key = nullptr;
     ta.out_tok = out_tok;
     ta.B = d->B;
     ta.N = d->N;
@@ -1970,7 +1871,6 @@ extern "C" int specroll_verify_terminal_rows(const specroll_verify_desc *d, cons
     ta.k = d->k;
     ta.V = d->V;
     ta.c = (float)(1.4426950408889634 / (double)d->temperature);
-    ta.row_per_seq = 1;
     return launch_terminal(ta, static_cast<cudaStream_t>(cuda_stream));
 }
 

@@ -107,3 +107,42 @@ def test_threshold_of_one_is_the_plain_verification():
         assert torch.equal(a[key], b[key])
     with pytest.raises(S.SpecrollError):
         S.verify_nucleus(*args, 0.0)
+
+
+@pytest.mark.parametrize("top_p", [0.95, 0.5, 0.03, 0.9995])
+@pytest.mark.parametrize("kind,V", [("gauss", 4104), ("gauss", 64), ("negative", 16392), ("peaked", 32776), ("masked", 4104),
+                                    ("zeros", 4104), ("near_zero", 4104), ("straddle", 4104), ("huge", 4104)])
+def test_values_at_the_ends_of_the_counters(kind, V, top_p):
+    """Rows whose cut lies among values that the counters resolve, around zero where one counter holds many values,
+    beyond the largest counted magnitude, below a bound that masks most of the row, and rows with -inf entries."""
+    w = I.scaled(I.WORKLOADS["tiny"], B=9, V=V, K=3, k=4, N=8)
+    parent = I.topology(w)
+    cid, cl = I.synthetic_candidates(w)
+    d = ref.tree_draw(parent, np.zeros(w.B, np.int32), cid, cl, I.uniforms24(5, (w.B, w.N)))
+    x = I.rng(4000 + V).standard_normal((w.B, w.N, V)).astype(np.float32)
+    if kind == "negative":
+        x = 2 * x - 21.0
+    elif kind == "peaked":
+        x = x - 5.0
+        x[:, :, 7] = 18.0
+    elif kind == "masked":
+        x[:, :, V // 3:] = -np.inf
+    elif kind == "zeros":
+        x[:] = 0.0
+    elif kind == "near_zero":
+        x *= 1e-4
+    elif kind == "straddle":
+        x = np.where(x > 1.0, x, np.copysign(np.abs(x) * 1e-5, x)).astype(np.float32)
+    elif kind == "huge":
+        x = 40000.0 + 300.0 * x
+    lg = torch.from_numpy(x).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+    u_acc, u_fin = I.verify_uniforms(w)
+    o, g = run_both(w, parent, lg, d, cid, cl, u_acc, u_fin, top_p)
+    if kind == "huge":
+        # (bf16 values 256 apart: the largest alone carries the mass.  The sums are of 2^(x c - M c) with M c rounded to
+        # fp32, so a relative error of M c ln 2 * 2^-24 = 2.5e-3 is their arithmetic's own bound.)
+        vis = np.isfinite(o["nucleus_thr"])
+        assert np.array_equal(g["nucleus_thr"][vis], o["nucleus_thr"][vis])
+        assert np.abs(g["nucleus_sum"][vis] / o["nucleus_sum"][vis] - 1).max() < 2.5e-3
+        return
+    check(w, o, g)
