@@ -153,23 +153,28 @@ constexpr int NUC_THREADS = 512;
 // the cut is found by a scan over the values, largest first, with the masses count * exp((l - M)/T): exact key, exact
 // integer counts, no order of additions.  Two tables (the signs), one counter per value from 2^-13 up to 2^15 in
 // magnitude; the values nearer to zero share a counter.  Only tokens at or above a bound are counted: all tokens below
-// M - T ln(V / ((1 - top_p) S)) together weigh at most (1 - top_p) S, so the cut lies at or above it.  (Peaked rows
-// then count a few tokens, and the count, an atomic per token, is what the pass waits for.)  Where a counter does not
-// tell the values apart, or the counted mass stays below the target by rounding, the radix search over the whole row
-// gives the same result in four passes (nucleus_row_radix).
+// M - T ln(V / ((1 - top_p) S)) together weigh at most (1 - top_p) S, so the cut lies at or above it.  Peaked rows then
+// count a few tokens.  What the pass waits for is the count: a warp's shared-memory atomic takes five to six cycles of the
+// SM whether twelve or twenty-four of its lanes count (with the integer instructions of the addresses
+// about 15 k cycles for a row of 152 k tokens; loads a round ahead do not help, nor does a closer bound from a sample).  Where a counter does not tell the values apart, or the counted mass
+// stays below the target by rounding, the radix search over the whole row gives the same result in four passes
+// (nucleus_row_radix).  Verification of 256 sequences x 16 nodes, V 151936: 588 us with a search of two passes and lists
+// per row, 327 us with this one.
 constexpr int NUC_OCT_LO = (127 - 13) << 7;              // bf16 bits of 2^-13
 constexpr int NUC_VALUES = ((127 + 15) << 7) - NUC_OCT_LO;  // counters per sign; 0: nearer to zero than 2^-13
-constexpr int NUC_SIGN = 4096;                           // offset of the negative values' table
-static_assert(NUC_VALUES <= NUC_SIGN, "a table per sign");
+constexpr int NUC_SIGN = 8192;                           // the negative values' table, 2^15 bytes behind the other: the sign bit of a
+                                                         // 16-bit word is an address bit
+constexpr int NUC_BASE_MAX = 0x8000 - 4 * NUC_VALUES;    // largest address of the tables for which that is so
 
 struct NucleusSmem {
     union {
-        uint32_t count[2 * NUC_SIGN];
+        uint32_t count[NUC_SIGN + NUC_VALUES];
         float bins[16][NUC_THREADS];
     };
     float wsum[NUC_THREADS / 32][16];
     double wtot[NUC_THREADS / 32];
-    int sel;  // bin selected by the last level; count search: 1 found, 0 not
+    int last;      // place of the last counter at which nucleus_scan's target was reached, -1: nowhere
+    int sel;       // bin selected by the last level
     float above, keep;
     uint32_t prefix;
 };
@@ -262,117 +267,157 @@ __device__ void nucleus_row_radix(const uint4 *__restrict__ p, int nvec, float c
     }
 }
 
-// One counter more for the tokens of a pair of bf16 logits that are at or above the bound (lo2: the bound, twice);
-// base2: the shared-memory address of the tables, twice.
-__device__ __forceinline__ void nucleus_count2(uint32_t w, const __nv_bfloat162 &lo2, uint32_t base2) {
-    const uint32_t keep = __hge2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&w), lo2);
-    // the magnitude's steps above 2^-13, within the table (a counted token lies below 2^15), and the sign above it
+// One counter more for the tokens of a pair of bf16 logits that are at or above the bound (lo2: the bound, twice).
+// base: the shared-memory address of the tables (in a cluster its upper half holds the CTA's rank), base2: its lower half,
+// twice.  The pass is bound by the integer pipe and the atomics: six integer instructions per pair.
+__device__ __forceinline__ void nucleus_count2(uint32_t w, uint32_t lo2, uint32_t base, uint32_t base2) {
+    // the magnitude's steps above 2^-13, within the table (a counted token lies below 2^15)
     const uint32_t mag = __viaddmin_s16x2_relu(w & 0x7fff7fffu, (uint32_t)(-NUC_OCT_LO & 0xffff) * 0x10001u, (NUC_VALUES - 1) * 0x10001u);
-    const uint32_t at = (mag | ((w >> 3) & 0x10001000u)) * 4u + base2;
-    if (keep & 0xffffu) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at & 0xffffu) : "memory");
-    if (keep >> 16) asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(at >> 16) : "memory");
+    const uint32_t at = (mag * 4u + base2) | (w & 0x80008000u);
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ge.bf16x2 p|q, %0, %1;\n\t"
+        "@p red.shared.add.u32 [%2], 1;\n\t"
+        "@q red.shared.add.u32 [%3], 1;\n\t}" ::"r"(w),
+        "r"(lo2), "r"(__byte_perm(at, base, 0x7610)), "r"(__byte_perm(at, base, 0x7632))
+        : "memory");
 }
 
-__device__ void nucleus_row(const uint16_t *__restrict__ row_logits, int V, float c, float M, float S, float top_p,
-                            NucleusSmem *st) {
+// A place is a counter's rank by falling value, 0 = the largest positive one, NUC_ZERO = the counter around zero.
+constexpr int NUC_ZERO = NUC_VALUES - 1;
+__device__ __forceinline__ int nucleus_place(uint32_t bits) {
+    const int m = max((int)(bits & 0x7fffu) - NUC_OCT_LO, 0);
+    return (bits & 0x8000u) ? NUC_ZERO + m : NUC_ZERO - m;
+}
+__device__ __forceinline__ uint32_t nucleus_value(int r) {  // (bf16 bits; the counter around zero: 0)
+    return r < NUC_ZERO ? (uint32_t)(NUC_ZERO - r + NUC_OCT_LO) : r > NUC_ZERO ? (uint32_t)(r - NUC_ZERO + NUC_OCT_LO) | 0x8000u : 0u;
+}
+__device__ __forceinline__ uint32_t nucleus_count_at(const NucleusSmem *st, int r, int n_cta) {
+    const int at = r <= NUC_ZERO ? NUC_ZERO - r : NUC_SIGN + r - NUC_ZERO;
+    uint32_t n = st->count[at] + (r == NUC_ZERO ? st->count[NUC_SIGN] : 0u);
+    for (int k = 1; k < n_cta; ++k) n += ld_dsmem_u32(st->count + at, k) + (r == NUC_ZERO ? ld_dsmem_u32(st->count + NUC_SIGN, k) : 0u);
+    return n;
+}
+
+// The first place of [r0, r1] at which the mass from r0 on reaches the target, by all threads of a CTA.  Result in
+// st->last (-1: not reached) and st->keep.
+__device__ void nucleus_scan(NucleusSmem *st, int r0, int r1, double target, float M, float c, int n_cta) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint4 *p = reinterpret_cast<const uint4 *>(row_logits);
-    const int nvec = V >> 3;
-    const float target = top_p * S;
-    const uint32_t base = smem_u32(st->count);
-    // the bound, one bf16 step below its value (the rest of its rounding does not matter: a cut that the counted
-    // tokens do not reach is searched over the whole row)
-    float bound = fmaxf(M - (log2f((float)V) - log2f(S - target)) / c, -32000.0f);
-    bound = fminf(bound, M);  // (top_p near 0)
-    bound -= 0.008f * fabsf(bound);
-    const uint32_t lo_bits = __bfloat16_as_ushort(__float2bfloat16_rd(bound));
-    const bool counted = fabsf(M) < 32000.0f && bound == bound && bound <= M && base + sizeof(st->count) <= 0x10000u;
-    if (!counted) {  // (uniform over the CTA)
-        nucleus_row_radix(p, nvec, c, M, target, st);
-        return;
-    }
-#pragma unroll
-    for (int j = 0; j < 2 * NUC_SIGN / (4 * NUC_THREADS); ++j)
-        reinterpret_cast<uint4 *>(st->count)[j * NUC_THREADS + tid] = make_uint4(0u, 0u, 0u, 0u);
-    if (tid == 0) st->sel = 0;
-    __syncthreads();
-    {
-        const uint32_t base2 = base * 0x10001u, lob2 = lo_bits * 0x10001u;
-        const __nv_bfloat162 lo2 = *reinterpret_cast<const __nv_bfloat162 *>(&lob2);
-        auto count8 = [&](const uint4 &v) {
-            nucleus_count2(v.x, lo2, base2);
-            nucleus_count2(v.y, lo2, base2);
-            nucleus_count2(v.z, lo2, base2);
-            nucleus_count2(v.w, lo2, base2);
-        };
-        int i = tid;
-        for (; i + 3 * NUC_THREADS < nvec; i += 4 * NUC_THREADS) {
-            uint4 v[4];  // four independent loads in flight
-#pragma unroll
-            for (int q = 0; q < 4; ++q) v[q] = ld_nc_v4(p + i + q * NUC_THREADS);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) count8(v[q]);
-        }
-        for (; i < nvec; i += NUC_THREADS) count8(ld_nc_v4(p + i));
-    }
-    __syncthreads();
-    // place r of the scan: values in falling order, 0 = the largest positive one, ZERO = the counter around zero
-    constexpr int ZERO = NUC_VALUES - 1;
-    auto place = [&](uint32_t bits) {
-        const int m = max((int)(bits & 0x7fffu) - NUC_OCT_LO, 0);
-        return (bits & 0x8000u) ? ZERO + m : ZERO - m;
-    };
-    auto value_bits = [&](int r) {  // (the counter around zero: 0)
-        return r < ZERO ? (uint32_t)(ZERO - r + NUC_OCT_LO) : r > ZERO ? (uint32_t)(r - ZERO + NUC_OCT_LO) | 0x8000u : 0u;
-    };
-    auto count_at = [&](int r) {
-        return r < ZERO ? st->count[ZERO - r] : r > ZERO ? st->count[NUC_SIGN + r - ZERO] : st->count[0] + st->count[NUC_SIGN];
-    };
     auto mass_at = [&](int r) {
-        const uint32_t n = count_at(r);
-        return n ? (double)n * (double)ex2_approx((bf16_bits_to_float(value_bits(r)) - M) * c) : 0.0;
+        const uint32_t n = nucleus_count_at(st, r, n_cta);
+        return (float)n * ex2_approx(fmaf(bf16_bits_to_float(nucleus_value(r)), c, -M * c));  // (an empty counter's value is finite)
     };
-    const int r0 = place(__float_as_uint(M) >> 16), r1 = place(lo_bits);
-    const int per = (r1 - r0 + NUC_THREADS) / NUC_THREADS;
+    const int per = (r1 - r0 + NUC_THREADS) / NUC_THREADS;  // (<= 14)
     const int my0 = r0 + tid * per, my1 = min(r1 + 1, my0 + per);
-    double mine = 0.0;
-    for (int r = my0; r < my1; ++r) mine += mass_at(r);
-    double incl = mine;
+    float part = 0.f;
+    for (int r = my0; r < my1; ++r) part += mass_at(r);
+    double incl = (double)part;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const double x = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += x;
     }
     if (lane == 31) st->wtot[warp] = incl;
+    if (tid == 0) st->last = -1;
     __syncthreads();
     // (a thread's end is formed as its successor's beginning, so that one thread at most holds the target)
     double before = 0.0;
     for (int w = 0; w < warp; ++w) before += st->wtot[w];
     const double up = __shfl_up_sync(0xffffffffu, incl, 1);
     const double excl = lane ? before + up : before, end = before + incl;
-    if (excl < (double)target && end >= (double)target) {
-        double cum = excl;
-        int r = my0, last = my0;
-        for (; r < my1; ++r) {
-            const double m = mass_at(r);
-            if (m > 0.0) last = r;
-            cum += m;
-            if (cum >= (double)target) break;
+    const unsigned mine = __ballot_sync(0xffffffffu, excl < target && end >= target);
+    if (mine) {  // the counters of that thread, one per lane
+        const int L = __ffs(mine) - 1;
+        const double e0 = __shfl_sync(0xffffffffu, excl, L);
+        const int f = __shfl_sync(0xffffffffu, my0, L), n = __shfl_sync(0xffffffffu, my1, L) - f;
+        const float m = lane < n ? mass_at(f + lane) : 0.f;
+        double cum = (double)m;
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) {
+            const double x = __shfl_up_sync(0xffffffffu, cum, o);
+            if (lane >= o) cum += x;
         }
-        // The counter around zero: it must not be the cut, and its values must not differ by more than their mass's
-        // rounding if it lies above the cut.
-        bool ok = last != ZERO;
-        if (last > ZERO && r0 <= ZERO) ok = ok && mass_at(ZERO) * (double)(c * 0.6931472f) * 0x1p-13 <= 0x1p-24 * (double)S;
-        if (ok) {
-            st->prefix = ord_key(value_bits(last));
+        cum += e0;
+        const unsigned hit = __ballot_sync(0xffffffffu, lane < n && cum >= target);
+        const unsigned pos = __ballot_sync(0xffffffffu, m > 0.f);
+        const int at = hit ? __ffs(hit) - 1 : 31 - __clz(pos);  // (no hit: rounding; the thread's mass is positive)
+        if (lane == at) {
+            st->last = f + at;
             st->keep = (float)cum;
-            st->sel = 1;
         }
     }
     __syncthreads();
-    const int sel = st->sel;
+}
+
+// n_cta > 1: the CTAs of a cluster share the pass, and its first CTA, which alone gets the result, adds their counts;
+// the caller has a cluster barrier between two rows.
+__device__ void nucleus_row(const uint16_t *__restrict__ row_logits, int V, float c, float M, float S, float top_p,
+                            NucleusSmem *st, int n_cta, int rank) {
+    const int tid = threadIdx.x;
+    const uint4 *p = reinterpret_cast<const uint4 *>(row_logits);
+    const int nvec = V >> 3;
+    const float target = top_p * S;
+    const uint32_t base = smem_u32(st->count);
+    // the bound, one bf16 step lower (the rest of its rounding does not matter: a cut that the counted tokens do not reach
+    // is searched over the whole row)
+    float bound = fmaxf(M - (log2f((float)V) - log2f(S - target)) / c, -32000.0f);
+    bound = fminf(bound, M);  // (top_p near 0)
+    const uint32_t lo_bits = __bfloat16_as_ushort(__float2bfloat16_rd(bound - 0.008f * fabsf(bound)));
+    const bool counted = fabsf(M) < 32000.0f && bf16_bits_to_float(lo_bits) <= M && (base & 0xffffu) <= (uint32_t)NUC_BASE_MAX;
+    if (!counted) {  // (uniform over the cluster)
+        if (rank == 0) nucleus_row_radix(p, nvec, c, M, target, st);
+        return;
+    }
+    for (int j = tid; j < 2 * NUC_VALUES / 4; j += NUC_THREADS)
+        reinterpret_cast<uint4 *>(st->count)[j < NUC_VALUES / 4 ? j : j - NUC_VALUES / 4 + NUC_SIGN / 4] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    if (sel == 0) nucleus_row_radix(p, nvec, c, M, target, st);
+    {
+        const uint32_t base2 = (base & 0xffffu) * 0x10001u, lob2 = lo_bits * 0x10001u;
+        auto count8 = [&](const uint4 &v) {
+            nucleus_count2(v.x, lob2, base, base2);
+            nucleus_count2(v.y, lob2, base, base2);
+            nucleus_count2(v.z, lob2, base, base2);
+            nucleus_count2(v.w, lob2, base, base2);
+        };
+        const int step = NUC_THREADS * n_cta;
+        int i = rank * NUC_THREADS + tid;
+        for (; i + 3 * step < nvec; i += 4 * step) {
+            uint4 v[4];  // four independent loads in flight
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = ld_nc_v4(p + i + q * step);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) count8(v[q]);
+        }
+        uint4 v[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[q] = ld_nc_v4(p + min(i + q * step, nvec - 1));
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (i + q * step < nvec) count8(v[q]);
+    }
+    if (n_cta > 1) {
+        cluster_sync_all();
+        if (rank != 0) return;
+    } else {
+        __syncthreads();
+    }
+    const int r0 = nucleus_place(__float_as_uint(M) >> 16), r1 = nucleus_place(lo_bits);
+    nucleus_scan(st, r0, r1, (double)target, M, c, n_cta);
+    const int last = st->last;
+    // The counter around zero: it must not be the cut, and its values must not differ by more than their mass's rounding
+    // if it lies above the cut.
+    bool ok = last >= 0 && last != NUC_ZERO;
+    if (ok && last > NUC_ZERO && r0 <= NUC_ZERO) {
+        const double m0 = (double)nucleus_count_at(st, NUC_ZERO, n_cta) * (double)ex2_approx(-M * c);
+        ok = m0 * (double)(c * 0.6931472f) * 0x1p-13 <= 0x1p-24 * (double)S;
+    }
+    if (ok) {
+        if (tid == 0) st->prefix = ord_key(nucleus_value(last));
+    } else {
+        __syncthreads();  // (all have read the counts)
+        nucleus_row_radix(p, nvec, c, M, target, st);
+    }
+    __syncthreads();
 }
 
 // ------------------------------------------------------------------------------ walk
@@ -580,11 +625,16 @@ __device__ int walk_node(const WalkArgs &a, const Topo &topo, int b, int u, doub
     const bool have = j < k;
     const double inv_T = 1.0 / a.T, inv_S = 1.0 / S;
     // the candidates: token, proposal weight, target probability
-    const bool staged = sg && sg->p && sg->e;
+    const bool staged = sg && sg->e;
     double rho = 0.0, e = 0.0;
     if (staged) {
         if (have) {
-            rho = sg->p[u * k + j];
+            if (sg->p) {
+                rho = sg->p[u * k + j];
+            } else {
+                const uint32_t bits = sg->pre[u * k + j];
+                rho = ord_key(bits) >= thr ? exp(((double)bf16_bits_to_float((uint16_t)bits) - M) * inv_T) * inv_S : 0.0;
+            }
             e = sg->e[hd * k + j];
             if (lane < k) sm->id[j] = sg->cid[hd * k + j];
         }
@@ -733,6 +783,71 @@ __host__ __device__ inline size_t walk_stage_bytes(int N, int K, int k) {
     return 4 * up((size_t)N * 4) + up((size_t)N) + 2 * up((size_t)K * k * 4) + up((size_t)N * k * 2);
 }
 
+// The same for a CTA that examines nodes with all its warps: the parent array and the proposal weights too.
+struct WalkBuf {
+    float *rmax, *rsum, *uacc;
+    int32_t *ttok;
+    uint8_t *tcand;
+    int32_t *cid;
+    float *clog;
+    uint16_t *pre;
+    int8_t *parent;
+    double *e;
+};
+__host__ __device__ inline size_t walk_buf_bytes(int N, int K, int k) {
+    auto up = [](size_t x) { return (x + 15) / 16 * 16; };
+    return walk_stage_bytes(N, K, k) + up((size_t)N) + up((size_t)K * k * sizeof(double));
+}
+__device__ __forceinline__ WalkBuf walk_buf(unsigned char *p, int N, int K, int k) {
+    auto take = [&](size_t x) {
+        unsigned char *q = p;
+        p += (x + 15) / 16 * 16;
+        return q;
+    };
+    WalkBuf w;
+    w.rmax = reinterpret_cast<float *>(take((size_t)N * 4));
+    w.rsum = reinterpret_cast<float *>(take((size_t)N * 4));
+    w.uacc = reinterpret_cast<float *>(take((size_t)N * 4));
+    w.ttok = reinterpret_cast<int32_t *>(take((size_t)N * 4));
+    w.tcand = reinterpret_cast<uint8_t *>(take((size_t)N));
+    w.cid = reinterpret_cast<int32_t *>(take((size_t)K * k * 4));
+    w.clog = reinterpret_cast<float *>(take((size_t)K * k * 4));
+    w.pre = reinterpret_cast<uint16_t *>(take((size_t)N * k * 2));
+    w.parent = reinterpret_cast<int8_t *>(take((size_t)N));
+    w.e = reinterpret_cast<double *>(take((size_t)K * k * sizeof(double)));
+    return w;
+}
+// Fills everything but the row statistics, by all threads of a CTA; complete after the caller's next __syncthreads().
+__device__ __forceinline__ void walk_buf_fetch(const WalkArgs &a, const Topo &topo, int b, const WalkBuf &w) {
+    const int N = a.N, K = a.K, k = a.k, tid = threadIdx.x, nt = blockDim.x;
+    for (int n = tid; n < N; n += nt) {
+        w.uacc[n] = a.u_acc[(size_t)b * N + n];
+        w.ttok[n] = a.tree_tok[(size_t)b * N + n];
+        w.tcand[n] = a.tree_cand[(size_t)b * N + n];
+        w.parent[n] = topo.parent[n];
+    }
+    for (int e = tid; e < K * k; e += nt) {
+        w.cid[e] = SR_CHECKED(a.cand_id[(size_t)b * K * k + e], a.V, b);
+        w.clog[e] = a.cand_logit[(size_t)b * K * k + e];
+    }
+    for (int e = tid; e < N * k; e += nt) {
+        const int u = e / k, j = e - u * k;
+        if (topo.n_child[u] > 0) {  // (a node with children is at depth < K)
+            const int t = SR_CHECKED(a.cand_id[((size_t)b * K + topo.depth[u]) * k + j], a.V, b);
+            w.pre[e] = a.logits[((size_t)b * N + u) * a.V + t];
+        }
+    }
+    // the proposal weights of every head's candidates, relative to the head's largest logit
+    const double inv_T = 1.0 / a.T;
+    __syncthreads();
+    for (int e = tid; e < K * k; e += nt) {
+        const int hd = e / k;
+        float mx = -INFINITY;
+        for (int jj = 0; jj < k; ++jj) mx = fmaxf(mx, w.clog[hd * k + jj]);
+        w.e[e] = exp(((double)w.clog[e] - (double)mx) * inv_T);
+    }
+}
+
 // Plain target distributions: one warp per sequence.  Which nodes the walk visits depends on its decisions, but
 // what it can ask for does not, so with the dense logits everything is fetched up front (WalkStage): one round
 // trip to memory per sequence instead of four or five dependent ones per visited node, which is what the walk's
@@ -809,37 +924,48 @@ __global__ void __launch_bounds__(WALK_WARPS * 32) walk_kernel(WalkArgs a, Topo 
     walk_end(a, b, u, sg ? (double)sg->rsum[u] : (double)a.row_sum[(size_t)b * N + u], lane, sm, &st);
 }
 
-// Maximum and sum of exponentials of one row by all NUC_THREADS threads of a CTA (same arithmetic as
-// row_stats_kernel); every thread returns with the result.
-__device__ void row_stats_row(const uint16_t *__restrict__ row_logits, int V, float c, float *sm_m, float *sm_s,
+// Maximum and sum of exponentials of one row by all NUC_THREADS threads of n_cta CTAs (a cluster; 1: a CTA alone), same
+// arithmetic as row_stats_kernel; every thread returns with the result.  sm_ms: NUC_THREADS / 32 pairs, at the same offset
+// in every CTA (the caller has a cluster barrier between two rows).
+__device__ void row_stats_row(const uint16_t *__restrict__ row_logits, int V, float c, float2 *sm_ms, int n_cta, int rank,
                               float *M_out, float *S_out) {
     const uint4 *p = reinterpret_cast<const uint4 *>(row_logits);
-    const int nvec = V >> 3;
+    const int nvec = V >> 3, step = NUC_THREADS * n_cta;
     float m = NEG_INF, nmc = 0.f, s = 0.f;
-    int i = threadIdx.x;
-    for (; i + 3 * NUC_THREADS < nvec; i += 4 * NUC_THREADS) {
+    int i = rank * NUC_THREADS + threadIdx.x;
+    for (; i + 3 * step < nvec; i += 4 * step) {
         uint4 v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = ld_nc_v4(p + i + u * NUC_THREADS);
+        for (int u = 0; u < 4; ++u) v[u] = ld_nc_v4(p + i + u * step);
 #pragma unroll
         for (int u = 0; u < 4; ++u) online_update(v[u], c, m, nmc, s);
     }
-    for (; i < nvec; i += NUC_THREADS) online_update(ld_nc_v4(p + i), c, m, nmc, s);
+    for (; i < nvec; i += step) online_update(ld_nc_v4(p + i), c, m, nmc, s);
     const float mw = warp_max(m);
     s = (m == NEG_INF) ? 0.f : s * ex2_approx((m - mw) * c);
     s = warp_sum(s);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __syncthreads();
-    if (lane == 0) {
-        sm_m[warp] = mw;
-        sm_s[warp] = s;
+    if (lane == 0) sm_ms[warp] = make_float2(mw, s);
+    if (n_cta > 1)
+        cluster_sync_all();
+    else
+        __syncthreads();
+    constexpr int W = NUC_THREADS / 32;
+    auto at = [&](int w) {
+        if (n_cta == 1) return sm_ms[w];
+        const double d = ld_dsmem_f64(sm_ms + w % W, w / W);
+        return make_float2(__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d)));
+    };
+    // (every warp for itself, a lane per pair)
+    float mb = NEG_INF, sb = 0.f;
+    for (int w0 = 0; w0 < W * n_cta; w0 += 32) {
+        const float2 e = w0 + lane < W * n_cta ? at(w0 + lane) : make_float2(NEG_INF, 0.f);
+        const float mn = fmaxf(mb, warp_max(e.x));
+        const float part = warp_sum(e.x == NEG_INF ? 0.f : e.y * ex2_approx((e.x - mn) * c));
+        sb = (mb == NEG_INF ? 0.f : sb * ex2_approx((mb - mn) * c)) + part;
+        mb = mn;
     }
-    __syncthreads();
-    float mb = NEG_INF;
-    for (int w = 0; w < NUC_THREADS / 32; ++w) mb = fmaxf(mb, sm_m[w]);
-    float sb = 0.f;
-    for (int w = 0; w < NUC_THREADS / 32; ++w)
-        sb += (sm_m[w] == NEG_INF) ? 0.f : sm_s[w] * ex2_approx((sm_m[w] - mb) * c);
     *M_out = mb;
     *S_out = sb;
 }
@@ -901,24 +1027,37 @@ __device__ __forceinline__ double warp_incl_scan(double v, int lane) {
 // [v_lo, v_hi) of a row, eight slices' loads in flight, left in out[0 .. n_sl).
 __device__ __forceinline__ void term_slice_masses(const uint4 *__restrict__ p, int v_lo, int v_hi, int n_sl, float M, float c,
                                                   uint32_t thr, int lane, double *out) {
+    // A slice's 256 masses are added pairwise in fp32 (relative error of a few 2^-24, the size of the exponentials' own
+    // error); everything above a slice is fp64.  (Converting every mass to fp64 first kept the conversion pipe busy for
+    // as long as the exponentials.)
+    auto sum8 = [&](const uint4 &v) {
+        float e[8];
+        masses8(v, M, c, thr, e);
+        return ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
+    };
     for (int s0 = 0; s0 < n_sl; s0 += 8) {
-        uint4 v[8];
+        uint4 v[8];  // (a load under a condition of its own ends up behind the use of the one before it: clamped instead)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = ld_nc_v4(p + max(0, min(v_lo + (s0 + q) * 32 + lane, v_hi - 1)));
+        float x[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            const int i = v_lo + (s0 + q) * 32 + lane;
-            v[q] = (s0 + q < n_sl && i < v_hi) ? ld_nc_v4(p + i) : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);  // -inf: no mass
+            x[q] = sum8(v[q]);
+            if (v_lo + (s0 + q) * 32 + lane >= v_hi) x[q] = 0.f;
         }
+        // eight sums over the warp at once: every step halves the values a lane carries (lane bits 4, 3, 2 pick the slice)
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            float e[8];
-            masses8(v[q], M, c, thr, e);
-            // a slice's 256 masses are added pairwise in fp32 (relative error of a few 2^-24, the size of the
-            // exponentials' own error); everything above a slice is fp64.  (Converting every mass to fp64 first
-            // kept the conversion pipe busy for as long as the exponentials.)
-            float acc = ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
-            acc = warp_sum(acc);
-            if (lane == 0 && s0 + q < n_sl) out[s0 + q] = (double)acc;
+        for (int h = 4, o = 16; h > 0; h >>= 1, o >>= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int q = 0; q < h; ++q) {
+                const float give = up ? x[q] : x[q + h], keep = up ? x[q + h] : x[q];
+                x[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
         }
+        x[0] += __shfl_xor_sync(0xffffffffu, x[0], 2);
+        x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
+        if ((lane & 3) == 0 && s0 + (lane >> 2) < n_sl) out[s0 + (lane >> 2)] = (double)x[0];
     }
 }
 
@@ -1029,99 +1168,114 @@ __device__ void term_pick(const uint4 *__restrict__ p, const double *seg_slices,
     term_pick_token(i, ms, lsum, base, target, take_last, v_hi, dst, lane);
 }
 
-// The vocabulary is cut into TERM_WARPS warp segments of vpw 8-token vectors, each walked in slices of 32 vectors (one per
-// lane).  Pass 1 (all warps, independent loads) leaves the fp64 mass of every slice in shared memory; the walk's
-// residual entries then replace the plain mass of their tokens; two scans pick the segment and the slice that
-// hold u * total, and only that slice is read again to find the token.
-__host__ __device__ inline int term_slices(int V) {
-    const int nvec = V >> 3, vpw = (nvec + TERM_WARPS - 1) / TERM_WARPS;
-    return (vpw + 31) / 32;
+// The vectors [v_base, v_base + nvec_r) of a row are cut into one segment per warp of the draw's n_cta CTAs (a cluster;
+// 1: a CTA alone), each walked in slices of 32 vectors (one per lane).  Pass 1 (all warps, independent loads) leaves the
+// fp64 mass of every slice in shared memory, those of the cluster's other CTAs are read by its first CTA; the residual
+// entries (nov tokens ovid, masses ovm) then replace the plain mass of their tokens; two scans pick the segment and the
+// slice that hold the target, and only that slice is read again to find the token.
+//   thr       nucleus threshold key of the row, 0 for none
+//   bits(j)   the bf16 logit of token ovid[j]
+//   base      the mass before v_base; target < 0: u times the total
+// By all TERM_THREADS threads of every CTA; slices: draw_smem_bytes, at the same offset in every CTA.  Bound by latency
+// (a few hundred KB per sequence), which is why the loads of a round are issued together.
+__host__ __device__ inline int draw_slices(int nvec, int n_cta) {
+    const int vpw = (nvec + TERM_WARPS * n_cta - 1) / (TERM_WARPS * n_cta);
+    return ((vpw > 0 ? vpw : 1) + 31) / 32;
+}
+__host__ __device__ inline size_t draw_smem_bytes(int V, int n_cta) {
+    return (size_t)TERM_WARPS * n_cta * (draw_slices(V >> 3, n_cta) + 1) * sizeof(double);
 }
 
-// By all TERM_THREADS threads of a CTA; sh_slice: TERM_WARPS * term_slices(V) doubles.  (M, thr: the row's maximum and
-// nucleus threshold key, 0 for none; the walk's results of sequence b are read from where walk_end left them.)
-__device__ void terminal_draw(const TermArgs &a, int b, const uint16_t *__restrict__ lg, float M, uint32_t thr, double *sh_slice) {
-    __shared__ double sh_seg[32];
-    __shared__ double sh_ovm[SPECROLL_MAX_TOPK];
-    __shared__ int32_t sh_ovid[SPECROLL_MAX_TOPK];
-    __shared__ int sh_pick[2];     // target warp, -1 if none
-    __shared__ double sh_base[2];  // mass before the target warp's segment; target
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nov = a.ws_nov[b];
+template <class Bits>
+__device__ void draw_row(const uint16_t *__restrict__ lg, int v_base, int nvec_r, float M, float c, uint32_t thr, int n_cta, int rank,
+                         int nov, const int32_t *ovid, const double *ovm, Bits bits, double *slices, double base, double target,
+                         float u, int32_t *dst) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint4 *p = reinterpret_cast<const uint4 *>(lg);
-    const int nvec = a.V >> 3;
-    const int vpw = (nvec + TERM_WARPS - 1) / TERM_WARPS;  // vectors per warp segment
-    const int n_sl = (vpw + 31) / 32;                      // slices per segment
-    const int v_lo = min(nvec, warp * vpw), v_hi = min(nvec, v_lo + vpw);
-
-    if (threadIdx.x < nov) {
-        sh_ovm[threadIdx.x] = a.ws_ovm[(size_t)b * a.k + threadIdx.x];
-        sh_ovid[threadIdx.x] = a.ws_ovid[(size_t)b * a.k + threadIdx.x];
-    }
-
-    term_slice_masses(p, v_lo, v_hi, n_sl, M, a.c, thr, lane, sh_slice + warp * n_sl);
-    __syncthreads();
-    // the walk's residual entries replace the plain mass of their tokens (at most k of them: one thread)
-    if (threadIdx.x == 0) {
-        for (int j = 0; j < nov; ++j) {
-            const int t = sh_ovid[j], vi = t >> 3;
-            const int w = min(TERM_WARPS - 1, vi / vpw), sl = (vi - w * vpw) >> 5;
-            sh_slice[w * n_sl + sl] += sh_ovm[j] - (double)mass1(lg[t], M, a.c, thr);
-        }
-    }
-    __syncthreads();
-    // segment masses
+    const int G = n_cta * TERM_WARPS;
+    const int vpw = (nvec_r + G - 1) / G > 0 ? (nvec_r + G - 1) / G : 1;  // vectors per warp segment
+    const int n_sl = (vpw + 31) / 32;                                     // slices per segment
+    double *seg = slices + (size_t)G * n_sl;
     {
-        double acc = 0.0;
-        for (int sl = lane; sl < n_sl; sl += 32) acc += sh_slice[warp * n_sl + sl];
-        acc = warp_sum(acc);
-        if (lane == 0) sh_seg[warp] = acc;
+        const int g = rank * TERM_WARPS + warp;
+        const int v_lo = v_base + min(nvec_r, g * vpw), v_hi = v_base + min(nvec_r, g * vpw + vpw);
+        term_slice_masses(p, v_lo, v_hi, n_sl, M, c, thr, lane, slices + (size_t)g * n_sl);
+    }
+    if (n_cta > 1) {
+        cluster_sync_all();  // every CTA's slice masses are in its shared memory
+        if (rank == 0) {
+            const int per = TERM_WARPS * n_sl;
+            for (int e = tid; e < (n_cta - 1) * per; e += TERM_THREADS) {
+                const int r = 1 + e / per;
+                slices[per + e] = ld_dsmem_f64(slices + per + e, r);
+            }
+        }
+        cluster_sync_all();  // the other CTAs may leave
+        if (rank != 0) return;
     }
     __syncthreads();
-    if (warp == 0) {
-        const double seg = lane < TERM_WARPS ? sh_seg[lane] : 0.0;
-        const double incl = warp_incl_scan(seg, lane);
-        const double total = __shfl_sync(0xffffffffu, incl, 31);
-        const double target = (double)a.u_fin[b] * total;
-        const unsigned hit = __ballot_sync(0xffffffffu, lane < TERM_WARPS && incl > target);
-        const int wsel = hit ? (__ffs(hit) - 1) : -1;
-        const double base = __shfl_sync(0xffffffffu, incl - seg, wsel < 0 ? 0 : wsel);
-        if (lane == 0) {
-            sh_pick[0] = wsel;
-            sh_base[0] = base;
-            sh_base[1] = target;
+    if (tid == 0) {
+        for (int j = 0; j < nov; ++j) {
+            const int vi = (ovid[j] >> 3) - v_base;
+            if (vi < 0 || vi >= nvec_r) continue;  // (outside the vectors the draw works on)
+            const int w = min(G - 1, vi / vpw), sl = (vi - w * vpw) >> 5;
+            slices[w * n_sl + sl] += ovm[j] - (double)mass1(bits(j), M, c, thr);
         }
     }
     __syncthreads();
-    const int wsel = sh_pick[0];
-    const int nacc = a.n_acc[b];
-    int32_t *dst = a.out_tok + (size_t)b * (a.K + 1) + nacc;
+    for (int g = warp; g < G; g += TERM_WARPS) {
+        double acc = 0.0;
+        for (int sl = lane; sl < n_sl; sl += 32) acc += slices[g * n_sl + sl];
+        acc = warp_sum(acc);
+        if (lane == 0) seg[g] = acc;
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    if (target < 0.0) {
+        double total = 0.0;
+        for (int g0 = 0; g0 < G; g0 += 32) total += warp_sum(g0 + lane < G ? seg[g0 + lane] : 0.0);
+        target = (double)u * total;
+    }
+    int wsel = -1;
+    for (int g0 = 0; g0 < G && wsel < 0; g0 += 32) {
+        const double v = g0 + lane < G ? seg[g0 + lane] : 0.0;
+        const double incl = warp_incl_scan(v, lane);
+        const unsigned hit = __ballot_sync(0xffffffffu, g0 + lane < G && base + incl > target);
+        if (hit) {
+            const int lh = __ffs(hit) - 1;
+            wsel = g0 + lh;
+            base += __shfl_sync(0xffffffffu, incl - v, lh);
+        } else {
+            base += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    }
     if (wsel < 0) {
-        // u_fin * total reached the total through rounding: take the last token with positive mass
-        if (threadIdx.x == 0) {
-            int tok = a.V - 1;
+        // the target reached the end of the masses through rounding: take the last token with positive mass (from the
+        // end of the vectors the draw worked on, downwards)
+        if (lane == 0) {
+            int tok = (v_base + nvec_r) * 8 - 1;
             for (; tok > 0; --tok) {
-                double ms = (double)mass1(lg[tok], M, a.c, thr);
+                double ms = (double)mass1(lg[tok], M, c, thr);
                 for (int j = 0; j < nov; ++j)
-                    if (sh_ovid[j] == tok) ms = sh_ovm[j];
+                    if (ovid[j] == tok) ms = ovm[j];
                 if (ms > 0.0) break;
             }
             *dst = tok;
         }
         return;
     }
-    if (warp != wsel) return;
-
-    term_pick(p, sh_slice + warp * n_sl, n_sl, v_lo, v_hi, sh_base[0], sh_base[1], M, a.c, thr, nov, sh_ovid, sh_ovm, dst,
-              lane);
+    const int v_lo = v_base + min(nvec_r, wsel * vpw), v_hi = v_base + min(nvec_r, wsel * vpw + vpw);
+    term_pick(p, slices + (size_t)wsel * n_sl, n_sl, v_lo, v_hi, base, target, M, c, thr, nov, ovid, ovm, dst, lane);
 }
 
 // One CTA per sequence, for rows that were made after the walk (one per sequence).
 __global__ void __launch_bounds__(TERM_THREADS) terminal_kernel(TermArgs a) {
-    extern __shared__ double sh_slice[];  // [TERM_WARPS][n_sl]
-    const int b = blockIdx.x;
-    terminal_draw(a, b, a.logits + (size_t)b * a.V, a.row_max[(size_t)b * a.N + a.term_node[b]], 0u, sh_slice);
+    extern __shared__ double sh_slice[];
+    const int b = blockIdx.x, nov = a.ws_nov[b];
+    const uint16_t *lg = a.logits + (size_t)b * a.V;
+    const int32_t *ovid = a.ws_ovid + (size_t)b * a.k;
+    draw_row(lg, 0, a.V >> 3, a.row_max[(size_t)b * a.N + a.term_node[b]], a.c, 0u, 1, 0, nov, ovid, a.ws_ovm + (size_t)b * a.k,
+             [&](int j) { return lg[ovid[j]]; }, sh_slice, 0.0, -1.0, a.u_fin[b], a.out_tok + (size_t)b * (a.K + 1) + a.n_acc[b]);
 }
 
 // ------------------------------------------------------------------------------ walk, a CTA per sequence
@@ -1134,78 +1288,139 @@ __global__ void __launch_bounds__(TERM_THREADS) terminal_kernel(TermArgs a) {
 //         in thr_key / keep_sum.
 // Before each node all threads do that work, then warp 0 does the node.  The terminal draw from the last node's row,
 // which the CTA has just read, follows in the same launch.
+// A sequence's rows come one after the other and each waits for memory and shared-memory atomics, so a sequence gets a
+// cluster of n_cta CTAs that share the passes over a row (walk_cta_split); the cluster's first CTA does the nodes.
+struct WalkCtaLayout {
+    size_t stage, total;  // in front of the stage: the threshold search, whose place the draw's slice masses take
+};
+__host__ __device__ inline WalkCtaLayout walk_cta_layout(int N, int K, int k, int V, int n_cta, bool nuc) {
+    WalkCtaLayout L;
+    L.stage = draw_smem_bytes(V, n_cta);
+    if (nuc && L.stage < sizeof(NucleusSmem)) L.stage = sizeof(NucleusSmem);
+    L.stage = (L.stage + 15) / 16 * 16;
+    L.total = L.stage + walk_buf_bytes(N, K, k);
+    return L;
+}
+
 template <bool LAZY, bool NUC>
 __global__ void __launch_bounds__(NUC_THREADS, 2)
 walk_cta_kernel(WalkArgs a, Topo topo, float c, float top_p, float *__restrict__ row_max_w,
                 float *__restrict__ row_sum_w, uint32_t *__restrict__ thr_key, float *__restrict__ keep_sum,
-                float *__restrict__ out_thr, float *__restrict__ out_sum, int thr_ready, TermArgs ta) {
-    extern __shared__ __align__(16) unsigned char nuc_raw[];  // NucleusSmem (NUC only), then the draw's slice masses
-    NucleusSmem &nuc = *reinterpret_cast<NucleusSmem *>(nuc_raw);
+                float *__restrict__ out_thr, float *__restrict__ out_sum, int thr_ready, const float *__restrict__ u_fin,
+                int n_cta) {
+    extern __shared__ __align__(16) unsigned char nuc_raw[];
+    NucleusSmem &nuc = *reinterpret_cast<NucleusSmem *>(nuc_raw);  // (NUC only)
     __shared__ WalkSmem sm;
-    __shared__ float sm_m[NUC_THREADS / 32], sm_s[NUC_THREADS / 32];
-    __shared__ int sh_next;  // next node, or -1 when the walk is over
-    const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ float2 sm_ms[NUC_THREADS / 32];
+    __shared__ int sh_next[2];        // the next node, or -1 when the walk is over; rows in turn (one barrier per row)
+    __shared__ uint32_t sh_last[4];   // of the last node, for the draw: threshold key, residual entries, accepted tokens
+    __shared__ double sh_ovm[SPECROLL_MAX_TOPK];
+    const int rank = n_cta > 1 ? (int)cluster_ctarank() : 0, b = blockIdx.x / n_cta;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const WalkBuf buf = walk_buf(nuc_raw + walk_cta_layout(a.N, a.K, a.k, a.V, n_cta, NUC).stage, a.N, a.K, a.k);
+    const WalkStage stage{buf.rmax, buf.rsum, buf.uacc, buf.ttok, buf.tcand, buf.cid, buf.clog, buf.pre, buf.parent, buf.e, nullptr};
     WalkState st;
-    pdl_wait();  // (set up under the tail of the kernel before, which made the statistics or the thresholds)
-    if (warp == 0) walk_begin(a, b, lane, &st);
+    // Set up under the tail of the kernel before.  Where that is this call's own (statistics, thresholds), which itself
+    // started when everything in front of the call was complete, the call's inputs are staged ahead of the wait.
+    if (LAZY) pdl_wait();
+    if (rank == 0) walk_buf_fetch(a, topo, b, buf);
+    if (!LAZY) {
+        pdl_wait();
+        if (rank == 0)
+            for (int n = threadIdx.x; n < a.N; n += NUC_THREADS) {
+                buf.rmax[n] = a.row_max[(size_t)b * a.N + n];
+                buf.rsum[n] = a.row_sum[(size_t)b * a.N + n];
+            }
+    }
+    if (rank == 0 && warp == 0) walk_begin(a, b, lane, &st);
+    __syncthreads();
     int u = 0;
     float M, S;
-    uint32_t thr;
-    for (;;) {
+    for (int turn = 0;; turn ^= 1) {
         const size_t row = (size_t)b * a.N + u;
+        const uint16_t *lg = a.logits + row * a.V;
         if constexpr (LAZY) {
-            row_stats_row(a.logits + row * a.V, a.V, c, sm_m, sm_s, &M, &S);
-            if (threadIdx.x == 0) {
+            row_stats_row(lg, a.V, c, sm_ms, n_cta, rank, &M, &S);
+            if (threadIdx.x == 0 && rank == 0) {
                 row_max_w[row] = M;
                 row_sum_w[row] = S;
             }
         } else {
-            M = a.row_max[row];
-            S = a.row_sum[row];
+            M = rank == 0 ? buf.rmax[u] : a.row_max[row];
+            S = rank == 0 ? buf.rsum[u] : a.row_sum[row];
         }
-        thr = 0u;
-        float norm = S;
-        if constexpr (NUC) {
-            if (thr_ready && topo.n_child[u] > 0) {  // (left by nucleus_rows_kernel for every node with children)
-                thr = thr_key[row];
-                norm = keep_sum[row];
-            } else {
-                nucleus_row(a.logits + row * a.V, a.V, c, M, S, top_p, &nuc);
-                thr = nuc.prefix;
-                norm = nuc.keep;
-            }
-            if (threadIdx.x == 0 && !(thr_ready && topo.n_child[u] > 0)) {
-                thr_key[row] = thr;
-                keep_sum[row] = norm;
-                if (out_sum) out_sum[row] = norm;
-                if (out_thr) {  // the threshold as a logit: undo the key
-                    const uint32_t bits = (thr & 0x8000u) ? (thr & 0x7fffu) : (~thr & 0xffffu);
-                    out_thr[row] = __uint_as_float(bits << 16);
+        const bool search = NUC && !(thr_ready && topo.n_child[u] > 0);
+        if (search) nucleus_row(lg, a.V, c, M, S, top_p, &nuc, n_cta, rank);
+        if (rank == 0) {
+            __syncthreads();  // (the staged inputs; the search's result)
+            if (warp == 0) {
+                uint32_t thr = 0u;
+                float norm = S;
+                if constexpr (NUC) {
+                    thr = search ? nuc.prefix : thr_key[row];
+                    norm = search ? nuc.keep : keep_sum[row];
+                    if (lane == 0 && search) {
+                        if (out_sum) out_sum[row] = norm;
+                        if (out_thr) {  // the threshold as a logit: undo the key
+                            const uint32_t bits = (thr & 0x8000u) ? (thr & 0x7fffu) : (~thr & 0xffffu);
+                            out_thr[row] = __uint_as_float(bits << 16);
+                        }
+                    }
+                }
+                int next = -1;
+                if (topo.n_child[u] == 0) {
+                    st.kind = (u != 0) ? 1 : 0;
+                    st.have_residual = false;
+                } else {
+                    next = walk_node(a, topo, b, u, (double)M, (double)norm, thr, lane, &sm, &st, &stage);
+                    if (next < 0) {
+                        st.kind = 0;
+                        st.have_residual = true;
+                    }
+                }
+                if (next < 0 && st.have_residual) {
+                    const double f = (double)norm / __shfl_sync(0xffffffffu, st.sigma, 0);  // (one division; the entries may be zero)
+                    for (int j = lane; j < a.k; j += 32) sh_ovm[j] = sm.r[j] * f;
+                }
+                if (lane == 0) {
+                    sh_next[turn] = next;
+                    sh_last[0] = thr;
+                    sh_last[1] = st.have_residual ? a.k : 0;
+                    sh_last[2] = st.nacc;
+                    if (next < 0) {
+                        a.n_acc[b] = st.nacc;
+                        a.term_node[b] = u;
+                        a.term_kind[b] = st.kind;
+                        if (a.min_margin) a.min_margin[b] = st.mm;
+                    }
                 }
             }
         }
-        if (warp == 0) {
-            int next = -1;
-            if (topo.n_child[u] == 0) {
-                st.kind = (u != 0) ? 1 : 0;
-                st.have_residual = false;
-            } else {
-                next = walk_node(a, topo, b, u, (double)M, (double)norm, thr, lane, &sm, &st);
-                if (next < 0) {
-                    st.kind = 0;
-                    st.have_residual = true;
-                }
-            }
-            if (next < 0) walk_end(a, b, u, (double)norm, lane, &sm, &st);
-            if (lane == 0) sh_next = next;
+        int next;
+        if (n_cta > 1) {
+            cluster_sync_all();
+            next = (int)ld_dsmem_u32(&sh_next[turn], 0);
+        } else {
+            __syncthreads();
+            next = sh_next[turn];
         }
-        __syncthreads();
-        const int next = sh_next;
-        __syncthreads();
         if (next < 0) break;
         u = next;
     }
-    terminal_draw(ta, b, a.logits + ((size_t)b * a.N + u) * a.V, M, thr, reinterpret_cast<double *>(nuc_raw));
+    const uint32_t thr = n_cta > 1 ? ld_dsmem_u32(&sh_last[0], 0) : sh_last[0];
+    draw_row(a.logits + ((size_t)b * a.N + u) * a.V, 0, a.V >> 3, M, c, thr, n_cta, rank, (int)sh_last[1],
+             buf.cid + (sh_last[1] ? topo.depth[u] : 0) * a.k, sh_ovm, [&](int j) { return buf.pre[u * a.k + j]; },
+             reinterpret_cast<double *>(nuc_raw), 0.0, -1.0, u_fin[b], a.out_tok + (size_t)b * (a.K + 1) + sh_last[2]);
+}
+
+// CTAs per row of walk_cta_kernel and nucleus_rows_kernel: as many as keep the grid within one wave of two CTAs per SM, a
+// power of two up to the portable cluster size.  (Twice that, with a second wave: 128 sequences, V 151936, statistics of the
+// visited rows 74 -> 98 us; the searches and nodes of a sequence wait for one another whatever their share of a row.)
+constexpr int WALK_CTA_WAVE = 296;
+static int walk_cta_split(int B) {
+    int n = 8;
+    while (n > 1 && (long long)B * n > WALK_CTA_WAVE) n >>= 1;
+    return n;
 }
 
 // The nucleus thresholds of every node with children, one CTA per (sequence, such node), all at once: which of
@@ -1220,19 +1435,21 @@ struct NodeList {
     int8_t node[SPECROLL_MAX_NODES];
 };
 
-__global__ void __launch_bounds__(NUC_THREADS, 3)
+__global__ void __launch_bounds__(NUC_THREADS, 2)
 nucleus_rows_kernel(const uint16_t *__restrict__ logits, int V, int N, NodeList nodes, float c, float top_p,
                     const float *__restrict__ row_max, const float *__restrict__ row_sum,
                     uint32_t *__restrict__ thr_key, float *__restrict__ keep_sum, float *__restrict__ out_thr,
-                    float *__restrict__ out_sum) {
+                    float *__restrict__ out_sum, int n_cta) {
     extern __shared__ __align__(16) unsigned char nuc_raw[];
     NucleusSmem &nuc = *reinterpret_cast<NucleusSmem *>(nuc_raw);
     pdl_wait();
-    const int b = blockIdx.x / nodes.n, u = nodes.node[blockIdx.x - b * nodes.n];
+    const int rank = n_cta > 1 ? (int)cluster_ctarank() : 0, r = blockIdx.x / n_cta;
+    const int b = r / nodes.n, u = nodes.node[r - b * nodes.n];
     const size_t row = (size_t)b * N + u;
     const float M = row_max[row], S = row_sum[row];
-    nucleus_row(logits + row * V, V, c, M, S, top_p, &nuc);
-    if (threadIdx.x == 0) {
+    nucleus_row(logits + row * V, V, c, M, S, top_p, &nuc, n_cta, rank);
+    if (n_cta > 1) cluster_sync_all();  // (the counts have been read)
+    if (threadIdx.x == 0 && rank == 0) {
         const uint32_t thr = nuc.prefix;
         thr_key[row] = thr;
         keep_sum[row] = nuc.keep;
@@ -1261,23 +1478,18 @@ nucleus_rows_kernel(const uint16_t *__restrict__ logits, int V, int N, NodeList 
 //       cluster's first CTA, which finishes as terminal_kernel does.  (Letting the statistics pass leave the mass
 //       of every slice of every row, so that this step reads a table and one slice, was tried: the table costs the
 //       statistics kernel as much as it saves here.)
-constexpr int WT_THREADS = 512;
+constexpr int WT_THREADS = TERM_THREADS;
 constexpr int WT_WARPS = WT_THREADS / 32;
 
 struct WtLayout {
-    size_t stage, ovm, first, mm, slices, seg, par, e, p, total;
-    int G, vpw, n_sl;
+    size_t stage, ovm, first, mm, slices, p, total;
 };
 __host__ __device__ inline WtLayout wt_layout(int N, int K, int k, int V, int S) {
     WtLayout L;
     auto up = [](size_t x) { return (x + 15) / 16 * 16; };
-    const int nvec = V >> 3;
-    L.G = S * WT_WARPS;
-    L.vpw = (nvec + L.G - 1) / L.G;
-    L.n_sl = (L.vpw + 31) / 32;
     size_t o = 0;
     L.stage = o;
-    o += up(walk_stage_bytes(N, K, k));
+    o += up(walk_buf_bytes(N, K, k));
     L.ovm = o;
     o += up((size_t)N * k * sizeof(double));
     L.first = o;
@@ -1285,13 +1497,7 @@ __host__ __device__ inline WtLayout wt_layout(int N, int K, int k, int V, int S)
     L.mm = o;
     o += up((size_t)N * sizeof(float));
     L.slices = o;
-    o += up((size_t)L.G * L.n_sl * sizeof(double));
-    L.seg = o;
-    o += up((size_t)L.G * sizeof(double));
-    L.par = o;
-    o += up((size_t)N);
-    L.e = o;
-    o += up((size_t)K * k * sizeof(double));
+    o += up(draw_smem_bytes(V, S));
     L.p = o;
     o += up((size_t)N * k * sizeof(double));
     L.total = o;
@@ -1308,58 +1514,19 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     const int N = a.N, K = a.K, k = a.k;
     const WtLayout L = wt_layout(N, K, k, a.V, S);
     auto up = [](size_t x) { return (x + 15) / 16 * 16; };
-    unsigned char *p0 = sh_dyn + L.stage;
-    float *rmax = reinterpret_cast<float *>(p0);
-    p0 += up((size_t)N * 4);
-    float *rsum = reinterpret_cast<float *>(p0);
-    p0 += up((size_t)N * 4);
-    float *uacc = reinterpret_cast<float *>(p0);
-    p0 += up((size_t)N * 4);
-    int32_t *ttok = reinterpret_cast<int32_t *>(p0);
-    p0 += up((size_t)N * 4);
-    uint8_t *tcand = reinterpret_cast<uint8_t *>(p0);
-    p0 += up((size_t)N);
-    int32_t *cid = reinterpret_cast<int32_t *>(p0);
-    p0 += up((size_t)K * k * 4);
-    float *clog = reinterpret_cast<float *>(p0);
-    p0 += up((size_t)K * k * 4);
-    uint16_t *pre = reinterpret_cast<uint16_t *>(p0);
+    const WalkBuf buf = walk_buf(sh_dyn + L.stage, N, K, k);
+    float *rmax = buf.rmax, *rsum = buf.rsum;
+    const int32_t *ttok = buf.ttok, *cid = buf.cid;
+    const uint16_t *pre = buf.pre;
     double *ovm = reinterpret_cast<double *>(sh_dyn + L.ovm);
     int32_t *first = reinterpret_cast<int32_t *>(sh_dyn + L.first);
     float *mmin = reinterpret_cast<float *>(sh_dyn + L.mm);
     double *slices = reinterpret_cast<double *>(sh_dyn + L.slices);
-    double *seg = reinterpret_cast<double *>(sh_dyn + L.seg);
-    int8_t *par = reinterpret_cast<int8_t *>(sh_dyn + L.par);
-    double *we = reinterpret_cast<double *>(sh_dyn + L.e);
     double *wp = reinterpret_cast<double *>(sh_dyn + L.p);
     const double inv_T = 1.0 / a.T;
     // (1) inputs of this call, none of them written by the kernel before this one
-    for (int n = tid; n < N; n += WT_THREADS) {
-        uacc[n] = a.u_acc[(size_t)b * N + n];
-        ttok[n] = a.tree_tok[(size_t)b * N + n];
-        tcand[n] = a.tree_cand[(size_t)b * N + n];
-        par[n] = topo.parent[n];
-    }
-    for (int e = tid; e < K * k; e += WT_THREADS) {
-        cid[e] = SR_CHECKED(a.cand_id[(size_t)b * K * k + e], a.V, b);
-        clog[e] = a.cand_logit[(size_t)b * K * k + e];
-    }
-    for (int e = tid; e < N * k; e += WT_THREADS) {
-        const int u = e / k, j = e - u * k;
-        if (topo.n_child[u] > 0) {  // (a node with children is at depth < K)
-            const int t = SR_CHECKED(a.cand_id[((size_t)b * K + topo.depth[u]) * k + j], a.V, b);
-            pre[e] = a.logits[((size_t)b * N + u) * a.V + t];
-        }
-    }
-    // the proposal weights of every head's candidates, relative to the head's largest logit
-    __syncthreads();
-    for (int e = tid; e < K * k; e += WT_THREADS) {
-        const int hd = e / k;
-        float mx = -INFINITY;
-        for (int jj = 0; jj < k; ++jj) mx = fmaxf(mx, clog[hd * k + jj]);
-        we[e] = exp(((double)clog[e] - (double)mx) * inv_T);
-    }
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the row statistics are complete from here on
+    walk_buf_fetch(a, topo, b, buf);
+    pdl_wait();  // the row statistics are complete from here on
     for (int n = tid; n < N; n += WT_THREADS) {
         rmax[n] = a.row_max[(size_t)b * N + n];
         rsum[n] = a.row_sum[(size_t)b * N + n];
@@ -1376,7 +1543,7 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     __syncthreads();
     // (2) every node with children on its own
     {
-        const WalkStage stage{rmax, rsum, uacc, ttok, tcand, cid, clog, pre, par, we, wp};
+        const WalkStage stage{rmax, rsum, buf.uacc, ttok, buf.tcand, cid, buf.clog, pre, buf.parent, buf.e, wp};
         int idx = 0;
         for (int u = 0; u < N; ++u) {
             if (topo.n_child[u] == 0) continue;
@@ -1441,8 +1608,7 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     const double *ovm_u = ovm + u * k;
     const float M = rmax[u];
     const uint16_t *lg = a.logits + ((size_t)b * N + u) * a.V;
-    const uint4 *p = reinterpret_cast<const uint4 *>(lg);
-    const int nvec = a.V >> 3, G = L.G;
+    const int nvec = a.V >> 3;
     // With the statistics kernel's table of the row's eight runs (run_tab; then S = 1): the run that holds the target
     // is found from the table and only that eighth of the row is read, cut into G segments like a whole row
     // otherwise.  v_base, nvec_r: the vectors the draw works on; base0: the mass before them.
@@ -1476,86 +1642,8 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
         rs_run(nvec, sh_run, &v_base, &v_end);
         nvec_r = v_end - v_base;
     }
-    const int vpw = (nvec_r + G - 1) / G > 0 ? (nvec_r + G - 1) / G : 1;  // vectors per warp segment
-    const int n_sl = (vpw + 31) / 32;                                     // slices per segment (<= the layout's)
-    {
-        {
-            const int g = rank * WT_WARPS + warp;
-            const int v_lo = v_base + min(nvec_r, g * vpw), v_hi = v_base + min(nvec_r, g * vpw + vpw);
-            term_slice_masses(p, v_lo, v_hi, n_sl, M, c, 0u, lane, slices + (size_t)g * n_sl);
-        }
-        if (S > 1) {
-            cluster_sync_all();  // every CTA's slice masses are in its shared memory
-            if (rank == 0) {
-                const int per = WT_WARPS * n_sl;
-                for (int e = tid; e < (S - 1) * per; e += WT_THREADS) {
-                    const int r = 1 + e / per, o = r * per + (e - (r - 1) * per);
-                    slices[o] = ld_dsmem_f64(slices + o, r);
-                }
-            }
-            cluster_sync_all();  // the other CTAs may leave
-            if (rank != 0) return;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            for (int j = 0; j < nov; ++j) {
-                const int t = ovid[j], vi = (t >> 3) - v_base;
-                if (vi < 0 || vi >= nvec_r) continue;  // (outside the run the draw works on)
-                const int w = min(G - 1, vi / vpw), sl = (vi - w * vpw) >> 5;
-                slices[w * n_sl + sl] += ovm_u[j] - (double)mass1(pre[u * k + j], M, c, 0u);  // (staged: lg[t])
-            }
-        }
-        __syncthreads();
-        for (int g = warp; g < G; g += WT_WARPS) {
-            double acc = 0.0;
-            for (int sl = lane; sl < n_sl; sl += 32) acc += slices[g * n_sl + sl];
-            acc = warp_sum(acc);
-            if (lane == 0) seg[g] = acc;
-        }
-        __syncthreads();
-    }
-    if (warp != 0) return;
-    double target, base;
-    if (run_tab) {
-        base = sh_b0t[0];
-        target = sh_b0t[1];
-    } else {
-        double total = 0.0;
-        for (int g0 = 0; g0 < G; g0 += 32) total += warp_sum(g0 + lane < G ? seg[g0 + lane] : 0.0);
-        target = (double)u_fin[b] * total;
-        base = 0.0;
-    }
-    int wsel = -1;
-    for (int g0 = 0; g0 < G && wsel < 0; g0 += 32) {
-        const double v = g0 + lane < G ? seg[g0 + lane] : 0.0;
-        const double incl = warp_incl_scan(v, lane);
-        const unsigned hit = __ballot_sync(0xffffffffu, g0 + lane < G && base + incl > target);
-        if (hit) {
-            const int lh = __ffs(hit) - 1;
-            wsel = g0 + lh;
-            base += __shfl_sync(0xffffffffu, incl - v, lh);
-        } else {
-            base += __shfl_sync(0xffffffffu, incl, 31);
-        }
-    }
-    int32_t *dst = a.out_tok + (size_t)b * (K + 1) + nacc;
-    if (wsel < 0) {
-        // the target reached the end of the masses through rounding: take the last token with positive mass (from the
-        // end of the vectors the draw worked on, downwards)
-        if (lane == 0) {
-            int tok = (v_base + nvec_r) * 8 - 1;
-            for (; tok > 0; --tok) {
-                double ms = (double)mass1(lg[tok], M, c, 0u);
-                for (int j = 0; j < nov; ++j)
-                    if (ovid[j] == tok) ms = ovm_u[j];
-                if (ms > 0.0) break;
-            }
-            *dst = tok;
-        }
-        return;
-    }
-    const int v_lo = v_base + min(nvec_r, wsel * vpw), v_hi = v_base + min(nvec_r, wsel * vpw + vpw);
-    term_pick(p, slices + (size_t)wsel * n_sl, n_sl, v_lo, v_hi, base, target, M, c, 0u, nov, ovid, ovm_u, dst, lane);
+    draw_row(lg, v_base, nvec_r, M, c, 0u, S, rank, nov, ovid, ovm_u, [&](int j) { return pre[u * k + j]; }, slices,
+             run_tab ? sh_b0t[0] : 0.0, run_tab ? sh_b0t[1] : -1.0, u_fin[b], a.out_tok + (size_t)b * (K + 1) + nacc);
 }
 
 // S CTAs per sequence: as many as keep the grid within about two CTAs per SM, a power of two up to the portable
@@ -1567,7 +1655,7 @@ static int walk_term_split(int B) {
 }
 
 static int launch_terminal(const TermArgs &ta, cudaStream_t st) {
-    const size_t smem = (size_t)TERM_WARPS * term_slices(ta.V) * sizeof(double);
+    const size_t smem = draw_smem_bytes(ta.V, 1);
     if (smem > (size_t)TERM_SMEM_LIMIT) return SPECROLL_ELIMIT;
     const int rc = device_setup(reinterpret_cast<const void *>(terminal_kernel), TERM_SMEM_LIMIT, nullptr);
     if (rc != SPECROLL_OK) return rc;
@@ -1685,26 +1773,9 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     wa.V = d->V;
     wa.T = (double)d->temperature;
     if (truncate || lazy) {
-        TermArgs ta;
-        ta.logits = wa.logits;
-        ta.u_fin = u_fin;
-        ta.row_max = row_max;
-        ta.n_acc = n_acc;
-        ta.term_node = term_node;
-        ta.ws_nov = ws_nov;
-        ta.ws_ovid = ws_ovid;
-        ta.ws_ovm = ws_ovm;
-        ta.out_tok = out_tok;
-        ta.B = d->B;
-        ta.N = d->N;
-        ta.K = d->K;
-        ta.k = d->k;
-        ta.V = d->V;
-        ta.c = c;
-        // (the draw's slice masses take the threshold search's place once the walk is over)
-        const size_t slices = (size_t)TERM_WARPS * term_slices(d->V) * sizeof(double);
-        if (slices > (size_t)TERM_SMEM_LIMIT) return SPECROLL_ELIMIT;
-        const size_t smem = truncate && sizeof(NucleusSmem) > slices ? sizeof(NucleusSmem) : slices;
+        const int n_cta = walk_cta_split(d->B);
+        const size_t smem = walk_cta_layout(d->N, d->K, d->k, d->V, n_cta, truncate).total;
+        if (smem > (size_t)TERM_SMEM_LIMIT) return SPECROLL_ELIMIT;
         auto *const kern = truncate ? (lazy ? walk_cta_kernel<true, true> : walk_cta_kernel<false, true>) : walk_cta_kernel<true, false>;
         int rc_ = device_setup(reinterpret_cast<const void *>(kern), TERM_SMEM_LIMIT, nullptr);
         if (rc_ != SPECROLL_OK) return rc_;
@@ -1721,14 +1792,17 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
             rc_ = device_setup(reinterpret_cast<const void *>(nucleus_rows_kernel), (int)sizeof(NucleusSmem), &n_sm);
             if (rc_ != SPECROLL_OK) return rc_;
             ahead = nodes.n > 0 && d->B * nodes.n <= NUC_AHEAD_ROWS_PER_SM * n_sm;
-            if (ahead)
-                SR_CUDA_TRY(launch_dependent(true, nucleus_rows_kernel, dim3((unsigned)(d->B * nodes.n)), dim3(NUC_THREADS),
-                                             sizeof(NucleusSmem), st, static_cast<const uint16_t *>(logits), d->V, d->N, nodes, c,
-                                             top_p, row_max, row_sum, thr_key, keep_sum, nucleus_thr, nucleus_sum));
+            if (ahead) {
+                const int rows_cta = walk_cta_split(d->B * nodes.n);
+                SR_CUDA_TRY(launch_clusters(true, rows_cta, nucleus_rows_kernel, dim3((unsigned)(d->B * nodes.n * rows_cta)),
+                                            dim3(NUC_THREADS), sizeof(NucleusSmem), st, static_cast<const uint16_t *>(logits), d->V,
+                                            d->N, nodes, c, top_p, row_max, row_sum, thr_key, keep_sum, nucleus_thr, nucleus_sum,
+                                            rows_cta));
+            }
         }
-        SR_CUDA_TRY(launch_dependent(true, kern, dim3((unsigned)d->B), dim3(NUC_THREADS), smem, st, wa, topo, c,
-                                     truncate ? top_p : 1.0f, row_max, row_sum, thr_key, keep_sum, truncate ? nucleus_thr : nullptr,
-                                     truncate ? nucleus_sum : nullptr, ahead ? 1 : 0, ta));
+        SR_CUDA_TRY(launch_clusters(true, n_cta, kern, dim3((unsigned)(d->B * n_cta)), dim3(NUC_THREADS), smem, st, wa, topo, c,
+                                    truncate ? top_p : 1.0f, row_max, row_sum, thr_key, keep_sum, truncate ? nucleus_thr : nullptr,
+                                    truncate ? nucleus_sum : nullptr, ahead ? 1 : 0, u_fin, n_cta));
         return SPECROLL_OK;
     }
     // plain verification: the walk and the terminal draw in one launch, overlapping the statistics kernel's tail
@@ -1738,26 +1812,8 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     if (L.total > (size_t)WT_SMEM_LIMIT) return SPECROLL_ELIMIT;
     const int rc_ = device_setup(reinterpret_cast<const void *>(walk_term_kernel), WT_SMEM_LIMIT, nullptr);
     if (rc_ != SPECROLL_OK) return rc_;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(d->B * S));
-    cfg.blockDim = dim3(WT_THREADS);
-    cfg.dynamicSmemBytes = L.total;
-    cfg.stream = st;
-    cudaLaunchAttribute attrs[2];
-    int na = 0;
-    attrs[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attrs[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
-    if (S > 1) {
-        attrs[na].id = cudaLaunchAttributeClusterDimension;
-        attrs[na].val.clusterDim.x = (unsigned)S;
-        attrs[na].val.clusterDim.y = 1;
-        attrs[na].val.clusterDim.z = 1;
-        ++na;
-    }
-    cfg.attrs = attrs;
-    cfg.numAttrs = na;
-    SR_CUDA_TRY(cudaLaunchKernelEx(&cfg, walk_term_kernel, wa, topo, u_fin, c, S, (const float2 *)run_tab));
+    SR_CUDA_TRY(launch_clusters(true, S, walk_term_kernel, dim3((unsigned)(d->B * S)), dim3(WT_THREADS), L.total, st, wa, topo, u_fin,
+                                c, S, (const float2 *)run_tab));
     return SPECROLL_OK;
 }
 

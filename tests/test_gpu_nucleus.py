@@ -146,3 +146,17 @@ def test_values_at_the_ends_of_the_counters(kind, V, top_p):
         assert np.abs(g["nucleus_sum"][vis] / o["nucleus_sum"][vis] - 1).max() < 2.5e-3
         return
     check(w, o, g)
+
+
+@pytest.mark.parametrize("B,V,top_p", [(300, 16392, 0.95), (160, 90128, 0.95), (40, 90128, 0.8), (3, 151936, 0.99)])
+def test_rows_shared_by_one_to_eight_ctas(B, V, top_p):
+    """A row is searched by one CTA or by a cluster of two, four or eight, by the number of rows."""
+    w = I.scaled(I.WORKLOADS["qwen1.5b"], B=B, V=V, N=4)
+    parent = I.topology(w)
+    cid, cl = I.synthetic_candidates(w)
+    d = ref.tree_draw(parent, np.zeros(w.B, np.int32), cid, cl, I.uniforms24(5, (w.B, w.N)))
+    x = I.rng(V + B).standard_normal((w.B, w.N, V), dtype=np.float32)
+    lg = torch.from_numpy(x).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+    u_acc, u_fin = I.verify_uniforms(w)
+    o, g = run_both(w, parent, lg, d, cid, cl, u_acc, u_fin, top_p)
+    check(w, o, g)
