@@ -12,9 +12,9 @@
 //
 // Two kernels, one CTA per record each:
 //   feedback_topk_kernel   exact Top_kS of the record's logits row, ordered by (logit desc, id asc), on the 16-bit
-//                          order-preserving keys of the bf16 logits.  Two passes: a lower bound of the kS-th largest
-//                          key from the threads' own maxima, then the few elements at or above it ranked in shared
-//                          memory.  Fallback for rows with thousands of equal large values: a radix search by
+//                          order-preserving keys of the bf16 logits.  One pass keeps the maximum of every few vectors;
+//                          the threads' own maxima give a lower bound of the kS-th largest key, the few groups
+//                          that reach it are read again and their elements ranked in shared memory.  Fallback for rows with thousands of equal large values: a radix search by
 //                          COUNT (four bits per pass) for the key of the kS-th largest value, a pass for the ids
 //                          above it, an ordered pass for the first ids that tie with it, a rank sort.
 //   feedback_vec_kernel    the small quantities (q, p on S, the coefficient of every support row; repeated tokens
@@ -66,16 +66,19 @@ __device__ __forceinline__ float block_sum_f(float v, float *red) {
     for (int w = 0; w < THREADS / 32; ++w) t += red[w];
     return t;
 }
-// the same for a CTA of any whole number of warps
-__device__ __forceinline__ float block_sum_rt(float v, float *red) {
+// two sums at once, for a CTA of any whole number of warps
+__device__ __forceinline__ void block_sum_rt(float &a, float &b, float2 *red) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    v = warp_sum(v);
+    a = warp_sum(a);
+    b = warp_sum(b);
     __syncthreads();
-    if (lane == 0) red[warp] = v;
+    if (lane == 0) red[warp] = make_float2(a, b);
     __syncthreads();
-    float t = 0.f;
-    for (int w = 0; w < nw; ++w) t += red[w];
-    return t;
+    a = b = 0.f;
+    for (int w = 0; w < nw; ++w) {
+        a += red[w].x;
+        b += red[w].y;
+    }
 }
 }  // namespace fb
 
@@ -87,11 +90,15 @@ struct TopkRadixSmem {
     int sel_id[SPECROLL_MAX_TOPK];
     uint32_t sel_key[SPECROLL_MAX_TOPK];
 };
+constexpr int TOPK_SLOTS = 16;  // groups per thread whose maxima are kept
 struct TopkListSmem {
-    uint32_t best[fb::TOPK_THREADS];     // every thread's largest key
-    // candidates (elements at or above the bound): key in the upper word, the complement of the id in the lower one,
-    // so that "larger" is (key desc, id asc) and a rank is a count of one comparison per entry
-    unsigned long long ent[fb::TOPK_LIST_CAP];
+    union {
+        uint16_t gmax[TOPK_SLOTS][fb::TOPK_THREADS];  // largest key of every group
+        // candidates (elements at or above the bound): key in the upper word, the complement of the id in the lower
+        // one, so that "larger" is (key desc, id asc) and a rank is a count of one comparison per entry
+        unsigned long long ent[fb::TOPK_LIST_CAP];
+    };
+    uint16_t hit[TOPK_SLOTS * fb::TOPK_THREADS];  // groups that reach the bound: slot * TOPK_THREADS + thread
 };
 
 // Exact Top_kS by a radix search over the counts (any row, also one with tens of thousands of equal values);
@@ -220,13 +227,14 @@ __device__ void topk_radix(TopkRadixSmem &sm, int &sh_above, int &sh_prefix, int
 }
 
 // top_id[r, 0..kS): ids of the kS largest logits of row rec_row[r], by (logit desc, id asc).
-// List method, two passes over the row: (1) every thread finds the largest key of its strided share of the row; the
-// kS-th largest of those 512 values is a lower bound of the kS-th largest key of the row (there are at least kS
-// elements at or above it); (2) the elements at or above the bound, a few more than kS unless the large values
-// sit in few threads' shares, go into a list in shared memory, and an entry's rank in the list by (key desc, id
-// asc) is its place in the result.  A list longer than its capacity (a row with thousands of equal large values)
-// falls back to the radix search.
-__global__ void __launch_bounds__(fb::TOPK_THREADS)
+// List method, one pass over the row.  A thread takes four vectors per round and keeps the largest key of every
+// rounds_per_slot rounds (a group); the kS-th largest of the threads' own maxima is a lower bound of the kS-th largest key
+// of the row (there are at least kS elements at or above it).  The groups that reach it, about kS of several thousand,
+// are read again, a thread per vector, and their elements at or above the bound ranked by (key desc, id asc): the rank
+// is the place in the result.  More elements than the list holds (a row with thousands of equal large values): the radix
+// search.  Bound by the one stream of the rows.  512 rows of 152064 tokens: 27 us (5.8 TB/s); reading the row twice and
+// ranking the 512 maxima against one another, as before, 76 us.
+__global__ void __launch_bounds__(fb::TOPK_THREADS, 4)
 feedback_topk_kernel(const uint16_t *__restrict__ logits, const int32_t *__restrict__ rec_row, int V, int kS,
                      int32_t *__restrict__ top_id) {
     using namespace fb;
@@ -234,77 +242,67 @@ feedback_topk_kernel(const uint16_t *__restrict__ logits, const int32_t *__restr
         TopkRadixSmem radix;
         TopkListSmem list;
     } sm;
-    __shared__ int sh_above, sh_prefix, sh_n;
-    __shared__ uint32_t sh_bound;
+    __shared__ int sh_above, sh_prefix, sh_n, sh_hits;
+    pdl_wait();
+    pdl_launch_dependents();
     const int r = blockIdx.x, tid = threadIdx.x;
     const uint16_t *row = logits + (size_t)rec_row[r] * V;
     const uint4 *p = reinterpret_cast<const uint4 *>(row);
     const int nvec = V >> 3;
     int32_t *out = top_id + (size_t)r * kS;
     const int n_sel = min(kS, V);
-    if (tid == 0) sh_n = 0;
-    // ---- pass 1: the largest key of this thread's share.  The order of the keys is the order of the values (with
-    //      -0 = +0), so the maximum is taken on the bf16 pairs as they come, one instruction per two logits, and
-    //      turned into a key once.
+    if (tid == 0) sh_n = sh_hits = 0;
+    // ---- the groups' maxima.  The order of the keys is the order of the values (with -0 = +0), so the maximum is taken on
+    //      the bf16 pairs as they come, one instruction per two logits, and turned into a key once per group.
     auto as_bf162 = [](uint32_t w_) { return *reinterpret_cast<const __nv_bfloat162 *>(&w_); };
-    __nv_bfloat162 mx2 = as_bf162(0xff80ff80u);  // (-inf, -inf)
-    // (Taking the bound from the head of the row only, to read the row once, was tried: the bound is lower, the list
-    // several hundred entries long, and ranking it costs more than the second pass over a row that sits in L2.)
-    const int nvec1 = nvec;
-    for (int i = tid; i < nvec1; i += 4 * TOPK_THREADS) {  // four loads in flight per thread
-        uint4 v[4];
+    const int rounds = (nvec + 4 * TOPK_THREADS - 1) / (4 * TOPK_THREADS);
+    const int per = (rounds + TOPK_SLOTS - 1) / TOPK_SLOTS, slots = (rounds + per - 1) / per;
+    uint32_t best = 0u;
+    for (int s = 0; s < slots; ++s) {
+        __nv_bfloat162 mx2 = as_bf162(0xff80ff80u);  // (-inf, -inf)
+        for (int j = s * per; j < min(rounds, (s + 1) * per); ++j) {
+            const int i = j * 4 * TOPK_THREADS + tid;
+            uint4 v[4];  // (beyond the row: its last vector again, which changes no maximum but its own thread's: masked)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int iu = i + u * TOPK_THREADS;
-            v[u] = iu < nvec1 ? ld_nc_v4(p + iu) : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
+            for (int u = 0; u < 4; ++u) v[u] = ld_nc_v4(p + min(i + u * TOPK_THREADS, nvec - 1));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const __nv_bfloat162 m = __hmax2(__hmax2(as_bf162(v[u].x), as_bf162(v[u].y)), __hmax2(as_bf162(v[u].z), as_bf162(v[u].w)));
+                if (i + u * TOPK_THREADS < nvec) mx2 = __hmax2(mx2, m);
+            }
         }
+        const uint32_t mxb = *reinterpret_cast<const uint32_t *>(&mx2);
+        const uint32_t key = max(ord_key16(mxb & 0xffffu), ord_key16(mxb >> 16));
+        sm.list.gmax[s][tid] = (uint16_t)key;
+        best = max(best, key);
+    }
+    // ---- the n_sel-th largest of the threads' maxima, bit by bit: the largest value that n_sel of them reach
+    uint32_t bound = 0u;
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            mx2 = __hmax2(__hmax2(__hmax2(as_bf162(v[u].x), as_bf162(v[u].y)), __hmax2(as_bf162(v[u].z), as_bf162(v[u].w))), mx2);
-    }
-    const uint32_t mxb = *reinterpret_cast<const uint32_t *>(&mx2);
-    const uint32_t best = max(ord_key16(mxb & 0xffffu), ord_key16(mxb >> 16));
-    sm.list.best[tid] = best;
+    for (int bit = 15; bit >= 0; --bit)
+        if (__syncthreads_count(best >= (bound | (1u << bit))) >= n_sel) bound |= 1u << bit;
+    // ---- the groups that reach the bound
+    for (int s = 0; s < slots; ++s)
+        if (sm.list.gmax[s][tid] >= bound) sm.list.hit[atomicAdd(&sh_hits, 1)] = (uint16_t)(s * TOPK_THREADS + tid);
     __syncthreads();
-    {
-        // the n_sel-th largest of the threads' values (ties broken by thread index: any of them will do as the bound)
-        // (compared as (value, thread) pairs in one word; the loads do not depend on the count: unrolled)
-        const uint32_t mine = (best << 10) | (uint32_t)(TOPK_THREADS - 1 - tid);
-        int rk = 0;
-#pragma unroll 8
-        for (int j = 0; j < TOPK_THREADS; ++j) rk += ((sm.list.best[j] << 10) | (uint32_t)(TOPK_THREADS - 1 - j)) > mine;
-        if (rk == min(n_sel, TOPK_THREADS) - 1) sh_bound = best;
-    }
-    __syncthreads();
-    const uint32_t bound = sh_bound;
-    // ---- pass 2: everything at or above the bound.  Compared as values, two at a time, against the bound's
-    //      value; a vector of eight with nothing to keep (nearly all of them) costs four compares and one branch.
+    // ---- their elements at or above the bound.  Compared as values, two at a time, against the bound's value.
     const uint32_t bbits = (bound & 0x8000u) ? (bound & 0x7fffu) : (~bound & 0xffffu);  // the key undone
     const __nv_bfloat162 bnd2 = as_bf162(bbits | (bbits << 16));
-    for (int i0 = tid; i0 < nvec; i0 += 8 * TOPK_THREADS) {  // eight loads in flight per thread
-        uint4 vv[8];
+    const int n_vec = sh_hits * 4 * per;
+    for (int h = tid; h < n_vec; h += TOPK_THREADS) {
+        const int g = sm.list.hit[h / (4 * per)], q = h % (4 * per);
+        const int i = ((g / TOPK_THREADS) * per * 4 + q) * TOPK_THREADS + g % TOPK_THREADS;
+        if (i >= nvec) continue;
+        const uint4 v = ld_nc_v4(p + i);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int iu = i0 + u * TOPK_THREADS;
-            vv[u] = iu < nvec ? ld_nc_v4(p + iu) : make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = i0 + u * TOPK_THREADS;
-            if (i >= nvec) continue;  // (a -inf filler would pass a bound of -inf)
-            const uint32_t w[4] = {vv[u].x, vv[u].y, vv[u].z, vv[u].w};
-            uint32_t m[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) m[j] = __hge2_mask(as_bf162(w[j]), bnd2);
-            if ((m[0] | m[1] | m[2] | m[3]) == 0u) continue;
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                if ((m[t >> 1] >> (16 * (t & 1))) & 0xffffu) {
-                    const uint32_t key = ord_key16((t & 1) ? (w[t >> 1] >> 16) : (w[t >> 1] & 0xffffu));
-                    const int pos = atomicAdd(&sh_n, 1);
-                    if (pos < TOPK_LIST_CAP)
-                        sm.list.ent[pos] = ((unsigned long long)key << 32) | (uint32_t)(0x7fffffff - (i * 8 + t));
-                }
+        for (int t = 0; t < 8; ++t) {
+            const uint32_t m = __hge2_mask(as_bf162(w[t >> 1]), bnd2);
+            if ((m >> (16 * (t & 1))) & 0xffffu) {
+                const uint32_t key = ord_key16((t & 1) ? (w[t >> 1] >> 16) : (w[t >> 1] & 0xffffu));
+                const int pos = atomicAdd(&sh_n, 1);
+                if (pos < TOPK_LIST_CAP)
+                    sm.list.ent[pos] = ((unsigned long long)key << 32) | (uint32_t)(0x7fffffff - (i * 8 + t));
             }
         }
     }
@@ -369,7 +367,9 @@ struct FeedbackSmall {
 
 // q, p on S, the coefficient of every support row, the scalar outputs.  All threads fetch the ids and the target
 // logits at them (two rounds of independent loads); one warp does the rest from shared memory.  Ends with a barrier.
-__device__ void feedback_small(const FeedbackArgs &a, int r, FeedbackSmall &s) {
+// ready(): called by thread 0 as soon as the support (s.id, s.n) is known, ahead of the coefficients.
+template <class Ready>
+__device__ void feedback_small(const FeedbackArgs &a, int r, FeedbackSmall &s, Ready ready) {
     using namespace fb;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k = a.k, kS = a.kS;
@@ -396,19 +396,6 @@ __device__ void feedback_small(const FeedbackArgs &a, int r, FeedbackSmall &s) {
     }
     __syncthreads();
     if (warp == 0) {
-        // ---- q on the candidates
-        float mx = -INFINITY;
-        for (int j = lane; j < k; j += 32) mx = fmaxf(mx, cl[j]);
-        mx = warp_max(mx);
-        float qs = 0.f;
-        for (int j = lane; j < k; j += 32) {
-            const float w = __expf((cl[j] - mx) * a.inv_T);
-            s.q[j] = w;
-            qs += w;
-        }
-        qs = warp_sum(qs);
-        __syncwarp();
-        for (int j = lane; j < k; j += 32) s.q[j] /= qs;
         // ---- S = C u Top_kS u {y*}, duplicates removed (first occurrence kept; the candidates come first)
         if (lane == 0) s.n = 0;
         __syncwarp();
@@ -428,6 +415,20 @@ __device__ void feedback_small(const FeedbackArgs &a, int r, FeedbackSmall &s) {
             if (lane == 0) s.n = base + __popc(bal);
             __syncwarp();
         }
+        if (lane == 0) ready();
+        // ---- q on the candidates
+        float mx = -INFINITY;
+        for (int j = lane; j < k; j += 32) mx = fmaxf(mx, cl[j]);
+        mx = warp_max(mx);
+        float qs = 0.f;
+        for (int j = lane; j < k; j += 32) {
+            const float w = __expf((cl[j] - mx) * a.inv_T);
+            s.q[j] = w;
+            qs += w;
+        }
+        qs = warp_sum(qs);
+        __syncwarp();
+        for (int j = lane; j < k; j += 32) s.q[j] /= qs;
         const int n = s.n;
         for (int i = lane; i < n_raw; i += 32) {  // repeated tokens: the place of their first occurrence
             const int f = s.first[i];
@@ -496,7 +497,9 @@ __global__ void __launch_bounds__(fb::FB_THREADS) feedback_kernel(FeedbackArgs a
     __shared__ float red[FB_THREADS / 32];
     const int r = blockIdx.x, tid = threadIdx.x;
     const int d = a.d;
-    feedback_small(a, r, sm);
+    pdl_wait();
+    pdl_launch_dependents();
+    feedback_small(a, r, sm, [] {});
     const int *s_id = sm.id;
     const float *s_adist = sm.adist, *s_acov = sm.acov;
     const int s_n = sm.n;
@@ -555,28 +558,30 @@ __global__ void __launch_bounds__(fb::FB_THREADS) feedback_kernel(FeedbackArgs a
     }
 }
 
-// Hidden sizes that are a multiple of eight.  The support rows of W come through shared memory in batches of rps
-// rows, three batches deep, as bulk copies of whole rows issued by one thread and counted on an mbarrier per stage
-// (asynchronous copies issued by all threads cost more instructions in address arithmetic than the sums they feed).
-// A row is nvec 8-column vectors.  When a row is shorter than the CTA (NV = 1), the threads form groups of nvec,
-// group g takes rows g, g + groups, ... of every batch, and the groups' partial sums are added through shared
-// memory at the end; otherwise the CTA has ceil(nvec / NV) threads (rounded up to whole warps) and thread t owns
-// the vectors t, t + blockDim, ... (NV of them) of every row.
+// Hidden sizes that are a multiple of eight.  The support rows of W come through shared memory in batches of
+// rows_per_stage rows, three batches deep, as bulk copies of whole rows issued by one thread and counted on an mbarrier
+// per stage (asynchronous copies issued by all threads cost more instructions in address arithmetic than the sums they
+// feed); the first three batches are asked for as soon as the support is known, ahead of its coefficients.  A row is nvec
+// 8-column vectors; the CTA has ceil(nvec / NV) threads (rounded up to whole warps) and thread t owns the vectors t,
+// t + blockDim, ... (NV of them) of every row.  A record's CTA spends half its time in serial steps (the small quantities,
+// the reductions), so what counts is how many records an SM has at once: thin CTAs, and stages sized so that a whole
+// wave's share of the records fits (fbv_rows).  512 records, d 3584: 46 us with four CTAs of 224 threads per SM, 73 with three of 512
+// (which is 1.15 waves of them).
 constexpr int FBV_THREADS = 512;
 constexpr int FBV_STAGES = 3;
 
-// Row groups of the vector kernel: as many as fit the CTA, at most one per row of a batch.
-__host__ __device__ inline int fbv_groups(int d, int rows_per_stage) {
-    const int nvec = d >> 3;
-    if (nvec >= FBV_THREADS) return 1;
-    const int g = FBV_THREADS / nvec;
-    return g < rows_per_stage ? g : rows_per_stage;
+__host__ __device__ inline int fbv_nv(int d) { return d <= 2048 ? 1 : d <= 16 * FBV_THREADS ? 2 : 3; }
+// Threads of the vector kernel's CTA for hidden size d.
+__host__ __device__ inline int fbv_threads(int d) {
+    const int t = (((d >> 3) + fbv_nv(d) - 1) / fbv_nv(d) + 31) / 32 * 32;
+    return t < 128 ? 128 : t;
 }
-// Threads of the vector kernel's CTA for hidden size d with NV vectors per thread.
-__host__ __device__ inline int fbv_threads(int d, int NV) {
-    const int nvec = d >> 3;
-    if (NV == 1) return FBV_THREADS;
-    return ((nvec + NV - 1) / NV + 31) / 32 * 32;
+// Rows of W per batch: the shared memory of an SM, less the static part, shared by the CTAs it gets of a wave of R records.
+static int fbv_rows(int R, int d, int n_sm) {
+    const int most = std::max(1, 65536 / (fbv_threads(d) * (fbv_nv(d) == 1 ? 40 : 64)));  // (by registers)
+    const int per_sm = std::min(most, std::max(1, (R + n_sm - 1) / n_sm));
+    const int bytes = std::min(216 * 1024 / per_sm - 6 * 1024, 100 * 1024) / FBV_STAGES;
+    return std::max(1, std::min(8, bytes / (d * 2)));
 }
 
 __device__ __forceinline__ void fbv_bulk_row(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
@@ -586,13 +591,13 @@ __device__ __forceinline__ void fbv_bulk_row(uint32_t dst, const void *src, uint
 }
 
 template <int NV>
-__global__ void __launch_bounds__(FBV_THREADS, NV == 1 ? 3 : (NV == 2 ? 2 : 1)) feedback_vec_kernel(FeedbackArgs a) {
+__global__ void __launch_bounds__(NV == 1 ? 256 : FBV_THREADS, NV == 1 ? 6 : (NV == 2 ? 2 : 1)) feedback_vec_kernel(FeedbackArgs a) {
     using namespace fb;
     __shared__ FeedbackSmall sm;
-    __shared__ float red[FBV_THREADS / 32];
+    __shared__ float2 red[FBV_THREADS / 32];
     __shared__ __align__(8) unsigned long long full[FBV_STAGES];
     __shared__ volatile int abort_flag;
-    extern __shared__ __align__(16) unsigned char fb_stage[];  // [3][rows_per_stage][d] bf16; then the groups' partial sums
+    extern __shared__ __align__(16) unsigned char fb_stage[];  // [3][rows_per_stage][d] bf16
     const int r = blockIdx.x, tid = threadIdx.x, tpb = blockDim.x;
     const int d = a.d, nvec = d >> 3;
     if (tid == 0) {
@@ -600,45 +605,47 @@ __global__ void __launch_bounds__(FBV_THREADS, NV == 1 ? 3 : (NV == 2 ? 2 : 1)) 
         abort_flag = 0;
         fence_mbar_init();
     }
-    feedback_small(a, r, sm);  // (ends with a barrier)
+    const int rps = a.rows_per_stage;
+    const uint32_t row_bytes = (uint32_t)d * 2u;
+    const size_t stage_bytes = (size_t)rps * row_bytes;
+    auto issue = [&](int batch) {  // one thread
+        const int s = batch % FBV_STAGES;
+        const int rows = min(rps, sm.n - batch * rps);
+        const uint32_t bar = smem_u32(&full[s]);
+        mbar_arrive_expect_tx(bar, (uint32_t)rows * row_bytes);
+        const uint32_t dst = smem_u32(fb_stage + (size_t)s * stage_bytes);
+        for (int q = 0; q < rows; ++q)
+            fbv_bulk_row(dst + (uint32_t)q * row_bytes, a.W + (size_t)sm.id[batch * rps + q] * d, row_bytes, bar);
+    };
+    pdl_wait();
+    pdl_launch_dependents();
+    float4 *mr = reinterpret_cast<float4 *>(a.m + (size_t)a.rec_mem[r] * d);
+    for (int c = tid; c * 32 < d; c += tpb)  // (the memory row, wanted at the end)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const float *>(mr) + c * 32));
+    feedback_small(a, r, sm, [&] {
+        for (int b = 0; b < FBV_STAGES && b * rps < sm.n; ++b) issue(b);
+    });  // (ends with a barrier)
     const int n = sm.n;
     const float dd = sm.dd, dc = sm.dc, sev = sm.w;
-    const int *sh_id = sm.id;
     const float *sh_ad = sm.adist, *sh_ac = sm.acov;
     float rd[NV][8], rc[NV][8];
 #pragma unroll
     for (int c = 0; c < NV; ++c)
 #pragma unroll
         for (int t = 0; t < 8; ++t) rd[c][t] = rc[c][t] = 0.f;
-    const int rps = a.rows_per_stage;
-    const uint32_t row_bytes = (uint32_t)d * 2u;
-    const size_t stage_bytes = (size_t)rps * row_bytes;
     const int nb = (n + rps - 1) / rps;
-    const int groups = NV == 1 ? fbv_groups(d, rps) : 1;
-    const int grp = NV == 1 ? tid / nvec : 0, vi0 = NV == 1 ? tid - grp * nvec : tid;
-    auto issue = [&](int batch) {  // one thread
-        const int s = batch % FBV_STAGES;
-        const int rows = min(rps, n - batch * rps);
-        const uint32_t bar = smem_u32(&full[s]);
-        mbar_arrive_expect_tx(bar, (uint32_t)rows * row_bytes);
-        const uint32_t dst = smem_u32(fb_stage + (size_t)s * stage_bytes);
-        for (int q = 0; q < rows; ++q)
-            fbv_bulk_row(dst + (uint32_t)q * row_bytes, a.W + (size_t)sh_id[batch * rps + q] * d, row_bytes, bar);
-    };
-    if (tid == 0)
-        for (int b = 0; b < FBV_STAGES && b < nb; ++b) issue(b);
     bool ok = true;
     for (int b = 0; b < nb; ++b) {
         ok = mbar_wait(smem_u32(&full[b % FBV_STAGES]), (uint32_t)(b / FBV_STAGES) & 1u, &abort_flag);
-        if (ok && grp < groups) {
+        if (ok) {
             const unsigned char *src = fb_stage + (size_t)(b % FBV_STAGES) * stage_bytes;
             const int rows = min(rps, n - b * rps);
-            for (int q = grp; q < rows; q += groups) {
+            for (int q = 0; q < rows; ++q) {
                 const int i = b * rps + q;
                 const float ad = sh_ad[i], ac = sh_ac[i];
 #pragma unroll
                 for (int c = 0; c < NV; ++c) {
-                    const int vi = vi0 + c * tpb;
+                    const int vi = tid + c * tpb;
                     if (vi < nvec) {
                         const uint4 v = *reinterpret_cast<const uint4 *>(src + ((size_t)q * nvec + vi) * 16);
                         const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
@@ -673,28 +680,7 @@ __global__ void __launch_bounds__(FBV_THREADS, NV == 1 ? 3 : (NV == 2 ? 2 : 1)) 
         }
         return;
     }
-    if (NV == 1 && groups > 1) {
-        // add the groups' partial sums: group g > 0 leaves its 16 numbers, group 0 collects
-        float *part = reinterpret_cast<float *>(fb_stage);  // [groups - 1][16][nvec]; the stages are free now
-        if (grp > 0 && grp < groups) {
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                part[((size_t)(grp - 1) * 16 + t) * nvec + vi0] = rd[0][t];
-                part[((size_t)(grp - 1) * 16 + 8 + t) * nvec + vi0] = rc[0][t];
-                rd[0][t] = rc[0][t] = 0.f;
-            }
-        }
-        __syncthreads();
-        if (grp == 0) {
-            for (int g = 1; g < groups; ++g)
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    rd[0][t] += part[((size_t)(g - 1) * 16 + t) * nvec + vi0];
-                    rc[0][t] += part[((size_t)(g - 1) * 16 + 8 + t) * nvec + vi0];
-                }
-        }
-    }
-    // (from here on only the threads with vectors of their own hold anything but zeros)
+    // (only the threads with vectors of their own hold anything but zeros)
     float sd = 0.f, scv = 0.f;
 #pragma unroll
     for (int c = 0; c < NV; ++c)
@@ -703,8 +689,7 @@ __global__ void __launch_bounds__(FBV_THREADS, NV == 1 ? 3 : (NV == 2 ? 2 : 1)) 
             sd += rd[c][t] * rd[c][t];
             scv += rc[c][t] * rc[c][t];
         }
-    sd = block_sum_rt(sd, red);
-    scv = block_sum_rt(scv, red);
+    block_sum_rt(sd, scv, red);
     const float fd = dd / (sqrtf(sd / d) + a.eps), fc = dc / (sqrtf(scv / d) + a.eps);
     float sg = 0.f;
 #pragma unroll
@@ -714,18 +699,17 @@ __global__ void __launch_bounds__(FBV_THREADS, NV == 1 ? 3 : (NV == 2 ? 2 : 1)) 
             rd[c][t] = fd * rd[c][t] + fc * rc[c][t];  // g
             sg += rd[c][t] * rd[c][t];
         }
-    sg = block_sum_rt(sg, red);
+    float none = 0.f;
+    block_sum_rt(sg, none, red);
     const float fe = (dd + dc) / (sqrtf(sg / d) + a.eps);
     const float rho = a.rho[r];
     const bool keep = !a.weighted || sev >= a.severity_min;
     const float gain = (1.f - rho) * (a.weighted ? sev : 1.f);
-    float4 *mr = reinterpret_cast<float4 *>(a.m + (size_t)a.rec_mem[r] * d);
     float4 *er = a.e_out ? reinterpret_cast<float4 *>(a.e_out + (size_t)r * d) : nullptr;
-    const bool owner = NV > 1 || grp == 0;
 #pragma unroll
     for (int c = 0; c < NV; ++c) {
-        const int vi = vi0 + c * tpb;
-        if (owner && vi < nvec) {
+        const int vi = tid + c * tpb;
+        if (vi < nvec) {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const float4 e = make_float4(fe * rd[c][4 * h], fe * rd[c][4 * h + 1], fe * rd[c][4 * h + 2], fe * rd[c][4 * h + 3]);
@@ -787,9 +771,8 @@ extern "C" int specroll_reflex_feedback_ex(const specroll_feedback_desc *d, cons
         return SPECROLL_EWORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     int32_t *top_id = static_cast<int32_t *>(workspace);
-    feedback_topk_kernel<<<d->R, fb::TOPK_THREADS, 0, st>>>(static_cast<const uint16_t *>(logits), rec_row, d->V,
-                                                            d->k_support, top_id);
-    SR_LAUNCH_CHECK();
+    SR_CUDA_TRY(launch_dependent(true, feedback_topk_kernel, dim3((unsigned)d->R), dim3(fb::TOPK_THREADS), 0, st,
+                                 static_cast<const uint16_t *>(logits), rec_row, d->V, d->k_support, top_id));
     FeedbackArgs a;
     a.logits = static_cast<const uint16_t *>(logits);
     a.rec_row = rec_row;
@@ -820,30 +803,19 @@ extern "C" int specroll_reflex_feedback_ex(const specroll_feedback_desc *d, cons
     // (m and e_out rows start at multiples of d floats: 16-byte aligned when d % 8 == 0 and the bases are)
     // (bulk copies of W rows: 16-byte aligned rows)
     const bool vec = (d->d % 8) == 0 && aligned16(m) && (!e_out || aligned16(e_out)) && aligned16(W);
-    // batches of at most 20 KB of W rows, three deep: three CTAs fit an SM
-    a.rows_per_stage = std::max(1, std::min(8, 20480 / (d->d * 2)));
-    const size_t fb_smem =
-        std::max((size_t)FBV_STAGES * a.rows_per_stage * d->d * 2,
-                 (size_t)(fbv_groups(d->d, a.rows_per_stage) - 1) * 16 * (size_t)(d->d >> 3) * sizeof(float));
     if (vec) {
-        const void *kern = d->d <= 8 * FBV_THREADS    ? reinterpret_cast<const void *>(feedback_vec_kernel<1>)
-                           : d->d <= 16 * FBV_THREADS ? reinterpret_cast<const void *>(feedback_vec_kernel<2>)
-                                                      : reinterpret_cast<const void *>(feedback_vec_kernel<3>);
-        const int rc_ = device_setup(kern, 112 * 1024, nullptr);
+        auto *const kern = fbv_nv(d->d) == 1 ? feedback_vec_kernel<1> : fbv_nv(d->d) == 2 ? feedback_vec_kernel<2> : feedback_vec_kernel<3>;
+        int n_sm = 0;
+        const int rc_ = device_setup(reinterpret_cast<const void *>(kern), 112 * 1024, &n_sm);
         if (rc_ != SPECROLL_OK) return rc_;
+        a.rows_per_stage = fbv_rows(d->R, d->d, n_sm);
+        SR_CUDA_TRY(launch_dependent(true, kern, dim3((unsigned)d->R), dim3((unsigned)fbv_threads(d->d)),
+                                     (size_t)FBV_STAGES * a.rows_per_stage * d->d * 2, st, a));
+        return SPECROLL_OK;
     }
-    if (vec && d->d <= 8 * FBV_THREADS)
-        feedback_vec_kernel<1><<<d->R, fbv_threads(d->d, 1), fb_smem, st>>>(a);
-    else if (vec && d->d <= 16 * FBV_THREADS)
-        feedback_vec_kernel<2><<<d->R, fbv_threads(d->d, 2), fb_smem, st>>>(a);
-    else if (vec)
-        feedback_vec_kernel<3><<<d->R, fbv_threads(d->d, 3), fb_smem, st>>>(a);
-    else if (d->d <= 8 * fb::FB_THREADS)
-        feedback_kernel<8><<<d->R, fb::FB_THREADS, 0, st>>>(a);
-    else if (d->d <= 24 * fb::FB_THREADS)
-        feedback_kernel<24><<<d->R, fb::FB_THREADS, 0, st>>>(a);
-    else
-        feedback_kernel<48><<<d->R, fb::FB_THREADS, 0, st>>>(a);
-    SR_LAUNCH_CHECK();
+    auto *const kern = d->d <= 8 * fb::FB_THREADS    ? feedback_kernel<8>
+                       : d->d <= 24 * fb::FB_THREADS ? feedback_kernel<24>
+                                                     : feedback_kernel<48>;
+    SR_CUDA_TRY(launch_dependent(true, kern, dim3((unsigned)d->R), dim3(fb::FB_THREADS), 0, st, a));
     return SPECROLL_OK;
 }

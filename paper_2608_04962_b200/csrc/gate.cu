@@ -5,54 +5,126 @@
 // Small, latency-bound kernels: a few thousand records and slots per call.
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace specroll {
 
 namespace gt {
 constexpr int SK_THREADS = 256;
+constexpr int SK_WARPS = SK_THREADS / 32;
 constexpr int MAX_RANK = 32;
+constexpr int SK_CLUSTER = 4;   // CTAs that share the columns of their records
+constexpr int SK_SMEM = 208 * 1024;
+constexpr int GATE_THREADS = 128;
+constexpr int GATE_BATCH = 4 * GATE_THREADS;
 }  // namespace gt
 
-// One block per record: y = Pi x (rank dot products of length d), then y / ||y||.  A warp takes the ranks warp,
-// warp + 8, ... (four at most) together, so x is read once per warp; with d % 4 == 0 and 16-byte aligned rows the
-// loads are 128-bit and independent of the running sums, several in flight per lane.  (A record's x and Pi's rows
-// are a few hundred KB fetched by one CTA: what bounds the kernel is how many bytes it keeps in flight.)
-__global__ void __launch_bounds__(gt::SK_THREADS) sketch_kernel(int d, int rank, const float *__restrict__ X,
+// Sums of 2^L values per lane over the warp: every step halves what a lane carries.  Returns the sum of value (lane >> (5 - L)).
+template <int L>
+__device__ __forceinline__ float warp_sum_many(float (&x)[1 << L], int lane) {
+#pragma unroll
+    for (int s = 0; s < L; ++s) {
+        const int o = 16 >> s, h = (1 << L) >> (s + 1);
+        const bool up = lane & o;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const float give = up ? x[q] : x[q + h], keep = up ? x[q + h] : x[q];
+            x[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    float r = x[0];
+#pragma unroll
+    for (int o = 16 >> L; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    return r;
+}
+
+// y = Pi x (rank dot products of length d), then y / ||y||, for VPW records per warp; d % 4 == 0 and 16-byte aligned rows.
+// Pi is a few hundred KB that every record meets: with a CTA per record the kernel was bound by bringing it from L2 once
+// per record (512 records, d 3584, rank 24: 17-22 us).  A cluster of four CTAs takes 8 VPW records, each CTA a quarter of
+// the columns: it asks for its part of Pi and of the records in one go (asynchronous copies, `cols` columns of four at a
+// time), so there is one memory latency and not one per step of a loop; the partial dot products meet in distributed
+// shared memory.
+template <int VPW>
+__global__ void __launch_bounds__(gt::SK_THREADS) sketch_kernel(int R, int d4, int rank, int cols, const float4 *__restrict__ X,
                                                                  const int32_t *__restrict__ rows,
-                                                                 const float *__restrict__ Pi, float *__restrict__ sketch,
-                                                                 int vec) {
+                                                                 const float4 *__restrict__ Pi, float *__restrict__ sketch) {
+    using namespace gt;
+    __shared__ float part[SK_WARPS * VPW][MAX_RANK];
+    extern __shared__ __align__(16) float4 sh_cols[];  // [rank + SK_WARPS * VPW][cols]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cta = (int)cluster_ctarank();
+    const int r0 = (blockIdx.x / SK_CLUSTER) * SK_WARPS * VPW;
+    const int per = (d4 + SK_CLUSTER - 1) / SK_CLUSTER, c0 = min(d4, cta * per), c1 = min(d4, c0 + per);
+    for (int e = threadIdx.x; e < SK_WARPS * VPW * MAX_RANK; e += SK_THREADS) part[e / MAX_RANK][e % MAX_RANK] = 0.f;
+    pdl_wait();
+    pdl_launch_dependents();
+    for (int cb = c0; cb < c1; cb += cols) {
+        const int n = min(cols, c1 - cb);
+        __syncthreads();  // (part cleared; the columns before have been read)
+        for (int i = warp; i < rank + SK_WARPS * VPW; i += SK_WARPS) {
+            const int r = min(r0 + i - rank, R - 1);  // (beyond the last record: its copy, not written)
+            const float4 *src = (i < rank ? Pi + (size_t)i * d4 : X + (size_t)(rows ? rows[r] : r) * d4) + cb;
+            for (int c = lane; c < n; c += 32) cp_async16(smem_u32(sh_cols + (size_t)i * cols + c), src + c, true);
+        }
+        cp_async_commit();
+        cp_async_wait<0>();
+        __syncthreads();
+        const float4 *x = sh_cols + (size_t)(rank + warp * VPW) * cols;
+        for (int i0 = 0; i0 < rank; i0 += 8) {  // eight ranks at a time: independent sums
+            float acc[VPW * 8];
+#pragma unroll
+            for (int q = 0; q < VPW * 8; ++q) acc[q] = 0.f;
+            for (int c = lane; c < n; c += 32) {
+                float4 xv[VPW];
+#pragma unroll
+                for (int v = 0; v < VPW; ++v) xv[v] = x[v * cols + c];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const float4 pv = sh_cols[(size_t)min(i0 + q, rank - 1) * cols + c];
+#pragma unroll
+                    for (int v = 0; v < VPW; ++v)
+                        acc[v * 8 + q] = fmaf(pv.x, xv[v].x, fmaf(pv.y, xv[v].y, fmaf(pv.z, xv[v].z, fmaf(pv.w, xv[v].w, acc[v * 8 + q]))));
+                }
+            }
+            constexpr int L = VPW == 2 ? 4 : 3;
+            const float t = warp_sum_many<L>(acc, lane);
+            const int e = lane >> (5 - L);
+            if ((lane & ((1 << (5 - L)) - 1)) == 0) part[warp * VPW + e / 8][i0 + e % 8] += t;  // (a warp's own rows)
+        }
+    }
+    cluster_sync_all();
+    // records in turn over the cluster's warps
+    for (int j = cta * SK_WARPS + warp; j < SK_WARPS * VPW && r0 + j < R; j += SK_CLUSTER * SK_WARPS) {
+        float v = 0.f;
+        if (lane < rank)
+#pragma unroll
+            for (int k = 0; k < SK_CLUSTER; ++k) v += __uint_as_float(ld_dsmem_u32(&part[j][lane], k));
+        const float nrm = sqrtf(warp_sum(v * v));
+        if (lane < rank) sketch[(size_t)(r0 + j) * rank + lane] = nrm > 0.f ? v / nrm : 0.f;
+    }
+    cluster_sync_all();  // (a CTA's partial products stay until all have read them)
+}
+
+// The same for any d and alignment: a CTA per record, a warp takes the ranks warp, warp + 8, ... (four at most).
+__global__ void __launch_bounds__(gt::SK_THREADS) sketch_any_kernel(int d, int rank, const float *__restrict__ X,
+                                                                     const int32_t *__restrict__ rows,
+                                                                     const float *__restrict__ Pi, float *__restrict__ sketch) {
     __shared__ float y[gt::MAX_RANK];
-    constexpr int NW = gt::SK_THREADS / 32, RPW = gt::MAX_RANK / NW;
+    constexpr int NW = gt::SK_WARPS, RPW = gt::MAX_RANK / NW;
     const int r = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_wait();
+    pdl_launch_dependents();
     const float *x = X + (size_t)(rows ? rows[r] : r) * d;
     float acc[RPW];
 #pragma unroll
     for (int q = 0; q < RPW; ++q) acc[q] = 0.f;
-    if (vec) {
-        const float4 *x4 = reinterpret_cast<const float4 *>(x);
-        const float4 *p4 = reinterpret_cast<const float4 *>(Pi);
-        const int d4 = d >> 2;
-#pragma unroll 2
-        for (int c = lane; c < d4; c += 32) {
-            const float4 xv = x4[c];
+    for (int c = lane; c < d; c += 32) {
+        const float xv = x[c];
 #pragma unroll
-            for (int q = 0; q < RPW; ++q) {
-                const int i = warp + q * NW;
-                if (i < rank) {
-                    const float4 pv = p4[(size_t)i * d4 + c];
-                    acc[q] = fmaf(pv.x, xv.x, fmaf(pv.y, xv.y, fmaf(pv.z, xv.z, fmaf(pv.w, xv.w, acc[q]))));
-                }
-            }
-        }
-    } else {
-        for (int c = lane; c < d; c += 32) {
-            const float xv = x[c];
-#pragma unroll
-            for (int q = 0; q < RPW; ++q) {
-                const int i = warp + q * NW;
-                if (i < rank) acc[q] = fmaf(Pi[(size_t)i * d + c], xv, acc[q]);
-            }
+        for (int q = 0; q < RPW; ++q) {
+            const int i = warp + q * NW;
+            if (i < rank) acc[q] = fmaf(Pi[(size_t)i * d + c], xv, acc[q]);
         }
     }
 #pragma unroll
@@ -85,6 +157,8 @@ struct GateArgs {
 // Realised alignment of every record: a warp per record.
 __global__ void __launch_bounds__(256) align_kernel(GateArgs g) {
     const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    pdl_wait();
+    pdl_launch_dependents();
     if (r >= g.R) return;
     if (g.keep && !g.keep[r]) {
         if (lane == 0 && g.a) g.a[r] = __int_as_float(0x7fc00000);
@@ -96,46 +170,28 @@ __global__ void __launch_bounds__(256) align_kernel(GateArgs g) {
     if (lane == 0) g.a[r] = (ns > 0.f && nx > 0.f) ? dot / (ns * nx) : 0.f;
 }
 
-// A warp per slot: its records, in order, go into the running moments (lane 0 does the recurrences; the lanes
-// look for the slot's records 32 at a time); then the score and the gate, with the RMS of the memory row.
-__global__ void __launch_bounds__(256) gate_kernel(GateArgs g, const float *__restrict__ a) {
-    const int j = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (j >= g.S) return;
+// A CTA per slot: its records, in order, go into the running moments; then the score and the gate, with the RMS of the
+// memory row.  Bound by latency: all threads look for the slot's records (512 at a time) and have the memory row's loads
+// in flight meanwhile (a warp per slot took 14 us for 512 slots and records of d 3584).
+__global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g, const float *__restrict__ a) {
+    using namespace gt;
+    __shared__ int hit[GATE_BATCH];
+    __shared__ float val[GATE_BATCH];
+    __shared__ int n_hit;
+    __shared__ float red[GATE_THREADS / 32];
+    const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    pdl_wait();
+    pdl_launch_dependents();
+    if (tid == 0) n_hit = 0;
     int n = g.n[j], nfb = g.n_fb[j];
     float mean = g.mean[j], M2 = g.M2[j];
-    // the records in batches of 256: a lane's eight loads of a batch are independent of the recurrences
-    for (int r0 = 0; r0 < g.R; r0 += 256) {
-        unsigned mine = 0u;
-        float av[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int r = r0 + q * 32 + lane;
-            const bool mq = r < g.R && g.slot[r] == j && (!g.keep || g.keep[r]);
-            mine |= (mq ? 1u : 0u) << q;
-            av[q] = r < g.R ? a[r] : 0.f;
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            unsigned bal = __ballot_sync(0xffffffffu, (mine >> q) & 1u);
-            while (bal) {
-                const int src = __ffs(bal) - 1;
-                bal &= bal - 1;
-                const float v = __shfl_sync(0xffffffffu, av[q], src);
-                n += 1;
-                const float delta = v - mean;
-                mean += delta / (float)n;
-                M2 += delta * (v - mean);
-                nfb += 1;
-            }
-        }
-    }
     float ss = 0.f;
     const float *mr = g.m + (size_t)j * g.d;
     if ((g.d % 4) == 0 && (reinterpret_cast<uintptr_t>(g.m) & 15u) == 0) {
         const float4 *m4 = reinterpret_cast<const float4 *>(mr);
         float s4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-        for (int c = lane; c < (g.d >> 2); c += 32) {
+#pragma unroll 8
+        for (int c = tid; c < (g.d >> 2); c += GATE_THREADS) {
             const float4 v = m4[c];
             s4[0] = fmaf(v.x, v.x, s4[0]);
             s4[1] = fmaf(v.y, v.y, s4[1]);
@@ -144,10 +200,49 @@ __global__ void __launch_bounds__(256) gate_kernel(GateArgs g, const float *__re
         }
         ss = (s4[0] + s4[1]) + (s4[2] + s4[3]);
     } else {
-        for (int c = lane; c < g.d; c += 32) ss = fmaf(mr[c], mr[c], ss);
+        for (int c = tid; c < g.d; c += GATE_THREADS) ss = fmaf(mr[c], mr[c], ss);
+    }
+    __syncthreads();
+    for (int r0 = 0; r0 < g.R; r0 += GATE_BATCH) {
+        int sl[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = r0 + q * GATE_THREADS + tid;
+            sl[q] = r < g.R ? g.slot[r] : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = r0 + q * GATE_THREADS + tid;
+            if (sl[q] == j && r < g.R && (!g.keep || g.keep[r])) hit[atomicAdd(&n_hit, 1)] = r;
+        }
+        __syncthreads();
+        const int nh = n_hit;
+        if (nh == 0) continue;
+        // in record order
+        for (int e = tid; e < nh; e += GATE_THREADS) {
+            const int r = hit[e];
+            int rk = 0;
+            for (int f = 0; f < nh; ++f) rk += hit[f] < r;
+            val[rk] = a[r];
+        }
+        __syncthreads();
+        if (tid == 0) {
+            n_hit = 0;
+            for (int e = 0; e < nh; ++e) {
+                n += 1;
+                const float delta = val[e] - mean;
+                mean += delta / (float)n;
+                M2 += delta * (val[e] - mean);
+                nfb += 1;
+            }
+        }
+        __syncthreads();
     }
     ss = warp_sum(ss);
-    if (lane == 0) {
+    if (lane == 0) red[tid >> 5] = ss;
+    __syncthreads();
+    if (tid == 0) {
+        ss = (red[0] + red[1]) + (red[2] + red[3]);
         g.n[j] = n;
         g.n_fb[j] = nfb;
         g.mean[j] = mean;
@@ -171,9 +266,20 @@ extern "C" int specroll_reflex_sketch(int32_t R, int32_t d, int32_t rank, const 
     if (R < 0 || d < 1 || rank < 1 || rank > gt::MAX_RANK) return SPECROLL_EINVAL;
     if (R == 0) return SPECROLL_OK;
     if (!X || !Pi || !sketch) return SPECROLL_EINVAL;
-    const int vec = (d % 4) == 0 && aligned16(X) && aligned16(Pi);
-    sketch_kernel<<<R, gt::SK_THREADS, 0, static_cast<cudaStream_t>(cuda_stream)>>>(d, rank, X, rows, Pi, sketch, vec);
-    SR_LAUNCH_CHECK();
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    if ((d % 4) == 0 && aligned16(X) && aligned16(Pi)) {
+        // two records per warp halve the reads of Pi; with few records, one, for more CTAs
+        const int vpw = R > 296 ? 2 : 1, per = gt::SK_WARPS * vpw, cols_all = (d / 4 + gt::SK_CLUSTER - 1) / gt::SK_CLUSTER;
+        const int cols = std::min(cols_all, gt::SK_SMEM / 16 / (rank + per));
+        auto *const kern = vpw == 2 ? sketch_kernel<2> : sketch_kernel<1>;
+        const int rc = device_setup(reinterpret_cast<const void *>(kern), gt::SK_SMEM, nullptr);
+        if (rc != SPECROLL_OK) return rc;
+        SR_CUDA_TRY(launch_clusters(true, gt::SK_CLUSTER, kern, dim3((unsigned)((R + per - 1) / per * gt::SK_CLUSTER)),
+                                    dim3(gt::SK_THREADS), (size_t)(rank + per) * cols * 16, st, R, d / 4, rank, cols,
+                                    reinterpret_cast<const float4 *>(X), rows, reinterpret_cast<const float4 *>(Pi), sketch));
+        return SPECROLL_OK;
+    }
+    SR_CUDA_TRY(launch_dependent(true, sketch_any_kernel, dim3((unsigned)R), dim3(gt::SK_THREADS), 0, st, d, rank, X, rows, Pi, sketch));
     return SPECROLL_OK;
 }
 
@@ -216,11 +322,7 @@ extern "C" int specroll_reflex_gate(const specroll_gate_desc *d, const float *s,
     g.H = d->H;
     g.z_delta = d->z_delta;
     g.mem_eps = d->mem_eps;
-    if (d->R > 0) {
-        align_kernel<<<(d->R + 7) / 8, 256, 0, st>>>(g);
-        SR_LAUNCH_CHECK();
-    }
-    gate_kernel<<<(d->S + 7) / 8, 256, 0, st>>>(g, a);
-    SR_LAUNCH_CHECK();
+    if (d->R > 0) SR_CUDA_TRY(launch_dependent(true, align_kernel, dim3((unsigned)(d->R + 7) / 8), dim3(256), 0, st, g));
+    SR_CUDA_TRY(launch_dependent(true, gate_kernel, dim3((unsigned)d->S), dim3(gt::GATE_THREADS), 0, st, g, (const float *)a));
     return SPECROLL_OK;
 }

@@ -14,16 +14,20 @@ struct CommitLayers {
 };
 
 // grid = (B, K + 1, layers): block (b, i, l) copies tree row path_node[b, i] of layer l's K and V to cache
-// position kv_len[b] + i of that layer's pool.
+// position kv_len[b] + i of that layer's pool.  kv_len_out (nullable; not where the lengths are updated in place, since other
+// blocks read them): the new lengths.
 __global__ void __launch_bounds__(128)
 commit_path_kernel(const __grid_constant__ CommitLayers lay, const int32_t *__restrict__ path_node,
                    const int32_t *__restrict__ n_acc, long long n_pages,
                    const int32_t *__restrict__ page_table, const int32_t *__restrict__ page_indptr,
-                   const int32_t *__restrict__ kv_len, int N, int K, int row_vec, int32_t *__restrict__ status) {
+                   const int32_t *__restrict__ kv_len, int N, int K, int row_vec, int32_t *__restrict__ status, int32_t *__restrict__ kv_len_out) {
+    pdl_wait();
+    pdl_launch_dependents();
     const int b = blockIdx.x, i = blockIdx.y;
     const uint4 *__restrict__ Kt = lay.Kt[blockIdx.z], *__restrict__ Vt = lay.Vt[blockIdx.z];
     uint4 *__restrict__ Kp = lay.Kp[blockIdx.z], *__restrict__ Vp = lay.Vp[blockIdx.z];
     const int na = n_acc[b];
+    if (kv_len_out && i == 0 && blockIdx.z == 0 && threadIdx.x == 0) kv_len_out[b] = kv_len[b] + ((na < 0 || na > K) ? 0 : na + 1);
     if (i > na || na < 0 || na > K) return;
     const int node = path_node[(size_t)b * (K + 1) + i];
     const long long pos = (long long)kv_len[b] + i;
@@ -44,8 +48,10 @@ commit_path_kernel(const __grid_constant__ CommitLayers lay, const int32_t *__re
     }
 }
 
-__global__ void commit_len_kernel(const int32_t *__restrict__ kv_len, const int32_t *__restrict__ n_acc, int B, int K,
-                                  int32_t *__restrict__ kv_len_out) {
+__global__ void commit_len_kernel(const int32_t *kv_len, const int32_t *__restrict__ n_acc, int B, int K,
+                                  int32_t *kv_len_out) {
+    pdl_wait();
+    pdl_launch_dependents();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
     const int na = n_acc[b];
@@ -56,6 +62,8 @@ __global__ void commit_len_kernel(const int32_t *__restrict__ kv_len, const int3
 __global__ void __launch_bounds__(128)
 gather_hidden_kernel(const uint4 *__restrict__ hidden, const int32_t *__restrict__ term_node, int N, int row_vec,
                      uint4 *__restrict__ h_next) {
+    pdl_wait();
+    pdl_launch_dependents();
     const int b = blockIdx.x;
     int node = term_node[b];
     if (node < 0 || node >= N) node = 0;
@@ -83,6 +91,7 @@ static int commit_layers(int32_t B, int32_t N, int32_t K, int32_t Hkv, int32_t D
     }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int row_vec = Hkv * D / 8;  // 16-byte vectors per token row
+    const bool apart = kv_len_out && (kv_len_out >= kv_len + B || kv_len_out + B <= kv_len);
     for (int l0 = 0; l0 < n_layers; l0 += COMMIT_MAX_LAYERS) {
         const int nl = n_layers - l0 < COMMIT_MAX_LAYERS ? n_layers - l0 : COMMIT_MAX_LAYERS;
         CommitLayers lay;
@@ -92,15 +101,14 @@ static int commit_layers(int32_t B, int32_t N, int32_t K, int32_t Hkv, int32_t D
             lay.Kp[l] = static_cast<uint4 *>(Kp[l0 + l]);
             lay.Vp[l] = static_cast<uint4 *>(Vp[l0 + l]);
         }
-        commit_path_kernel<<<dim3((unsigned)B, (unsigned)(K + 1), (unsigned)nl), 128, 0, st>>>(
-            lay, path_node, n_acc, (long long)n_pages, page_table, page_indptr, kv_len, N, K, row_vec, status);
-        SR_LAUNCH_CHECK();
+        SR_CUDA_TRY(launch_dependent(true, commit_path_kernel, dim3((unsigned)B, (unsigned)(K + 1), (unsigned)nl), dim3(128), 0, st, lay,
+                                     path_node, n_acc, (long long)n_pages, page_table, page_indptr, kv_len, N, K, row_vec, status,
+                                     apart && l0 == 0 ? kv_len_out : nullptr));
     }
-    if (kv_len_out) {
-        // after the copies in stream order, so that the lengths may be updated in place
-        commit_len_kernel<<<(B + 255) / 256, 256, 0, st>>>(kv_len, n_acc, B, K, kv_len_out);
-        SR_LAUNCH_CHECK();
-    }
+    // in place: after the copies in stream order
+    if (kv_len_out && !apart)
+        SR_CUDA_TRY(launch_dependent(true, commit_len_kernel, dim3((unsigned)(B + 255) / 256), dim3(256), 0, st, kv_len, n_acc, B, K,
+                                     kv_len_out));
     return SPECROLL_OK;
 }
 
@@ -129,8 +137,7 @@ extern "C" int specroll_gather_hidden(int32_t B, int32_t N, int32_t d, const voi
     if (B == 0) return SPECROLL_OK;  // (an empty batch has empty arrays: their pointers may be NULL)
     if (!hidden || !term_node || !h_next) return SPECROLL_EINVAL;
     if (!aligned16(hidden) || !aligned16(h_next)) return SPECROLL_EALIGN;
-    gather_hidden_kernel<<<(unsigned)B, 128, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-        static_cast<const uint4 *>(hidden), term_node, N, d / 8, static_cast<uint4 *>(h_next));
-    SR_LAUNCH_CHECK();
+    SR_CUDA_TRY(launch_dependent(true, gather_hidden_kernel, dim3((unsigned)B), dim3(128), 0, static_cast<cudaStream_t>(cuda_stream),
+                                 static_cast<const uint4 *>(hidden), term_node, N, d / 8, static_cast<uint4 *>(h_next)));
     return SPECROLL_OK;
 }

@@ -112,3 +112,25 @@ def test_thousands_of_equal_maxima_take_the_exact_fallback():
     want[rec_mem] = o["m"]
     np.testing.assert_allclose(host(dm), want, rtol=1e-3, atol=1e-4 * np.abs(want).max())
 
+
+
+@pytest.mark.parametrize("R,V,d,kS", [(2, 264208, 64, 48), (3, 16384, 2048, 16), (3, 16392, 2056, 16), (2, 1024, 8192, 8),
+                                      (2, 1024, 8200, 8), (640, 1032, 512, 8), (300, 64, 1536, 48)])
+def test_sizes_at_the_ends_of_the_kernels_ranges(R, V, d, kS):
+    """Rows of more rounds than the top-k kernel has slots, whole and ragged rounds; hidden sizes at which the vectors per
+    thread change; more records than a wave of CTAs; a support of three quarters of the vocabulary."""
+    k, rows = 4, R + 1
+    W, logits, rec_row, cand_id, cand_logit, y, m, rec_mem, rho = _case(70 + R, R, V, d, k, rows)
+    o = ref.reflex_feedback(logits[rec_row], W, cand_id, cand_logit, y, m[rec_mem], rho, kS)
+    lf = I.bf16_bits_to_f32(logits).astype(np.float64)
+    row_max = lf.max(-1)
+    row_sum = np.exp(lf - row_max[:, None]).sum(-1)
+    dm = dev(m.copy())
+    g = S.reflex_feedback(dev_bf16(logits), dev(rec_row), dev(row_max.astype(np.float32)), dev(row_sum.astype(np.float32)),
+                          dev(cand_id), dev(cand_logit), dev(y), dev_bf16(W), dev(rho), dev(rec_mem), dm, kS)
+    torch.cuda.synchronize()
+    np.testing.assert_allclose(host(g["d_dist"]), o["d_dist"], rtol=2e-4, atol=1e-6)
+    np.testing.assert_allclose(host(g["d_cov"]), o["d_cov"], rtol=2e-4, atol=1e-6)
+    want = m.astype(np.float64).copy()
+    want[rec_mem] = o["m"]
+    np.testing.assert_allclose(host(dm), want, rtol=1e-3, atol=1e-4 * np.abs(want).max())

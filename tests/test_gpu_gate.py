@@ -116,3 +116,12 @@ def test_gate(R, S_, rank, d, use_keep):
         assert host(out["alpha"])[2] == 0.0  # an empty memory row never opens the gate
     if R >= 500 and S_ > 10:
         assert (o["alpha"] > 0).any() and (o["alpha"] == 0).any()
+
+
+@pytest.mark.parametrize("R,d,rank", [(9, 12288, 32), (297, 4, 3), (313, 12284, 9), (8, 36, 8)])
+def test_sketches_at_the_ends_of_the_ranges(R, d, rank):
+    """More columns than a CTA's shared memory takes at once, CTAs of the cluster without columns, ragged records and ranks."""
+    g = I.rng(31 + R)
+    Pi = g.standard_normal((rank, d)).astype(np.float32)
+    X = g.standard_normal((R, d)).astype(np.float32)
+    np.testing.assert_allclose(host(S.reflex_sketch(dev(X), dev(Pi))), ref.reflex_sketch(X, Pi), rtol=0, atol=2e-5)
