@@ -356,7 +356,7 @@ struct FeedbackSmall {
     float p[fb::MAX_S];      // target mass exp((l - M)/T) / row_sum of the support tokens
     float adist[fb::MAX_S];  // coefficient of W_v in r_dist
     float acov[fb::MAX_S];   // coefficient of W_v in r_cov
-    float q[SPECROLL_MAX_TOPK];
+    float cl[SPECROLL_MAX_TOPK];  // the candidates' proposal logits
     int raw_id[fb::MAX_S];   // C, Top_kS, y* as they come (with duplicates)
     float raw_p[fb::MAX_S];
     int first[fb::MAX_S];    // raw index of the first occurrence of the same token (-1: not a token of the vocabulary)
@@ -377,9 +377,9 @@ __device__ void feedback_small(const FeedbackArgs &a, int r, FeedbackSmall &s, R
     const uint16_t *lg = a.logits + row * a.V;
     const float M = a.row_max[row], Ssum = a.row_sum[row];
     const int32_t *cid = a.cand_id + (size_t)r * k;
-    const float *cl = a.cand_logit + (size_t)r * k;
     const int32_t *top = a.top_id + (size_t)r * kS;
     const int n_raw = k + kS + 1;
+    for (int j = tid; j < k; j += blockDim.x) s.cl[j] = a.cand_logit[(size_t)r * k + j];
     for (int i = tid; i < n_raw; i += blockDim.x) {
         const int v = i < k ? cid[i] : (i < k + kS ? top[i - k] : a.y_star[r]);
         s.raw_id[i] = v;
@@ -387,90 +387,86 @@ __device__ void feedback_small(const FeedbackArgs &a, int r, FeedbackSmall &s, R
         s.first[i] = (v >= 0 && v < a.V) ? i : -1;
     }
     __syncthreads();
-    // the first occurrence of every token in the concatenation: all pairs (i, j < i), spread over the CTA (matches
-    // are rare: a candidate that is also among the target's largest, y* among either)
-    for (int pp = tid; pp < n_raw * 64; pp += blockDim.x) {
-        const int i = pp >> 6;
-        for (int j = pp & 63; j < i; j += 64)
-            if (s.raw_id[j] == s.raw_id[i] && s.first[i] >= 0) atomicMin(&s.first[i], j);
+    // the first occurrence of every token in the concatenation: a thread per entry, against all before it
+    for (int i = tid; i < n_raw; i += blockDim.x) {
+        const int v = s.raw_id[i];
+        int f = i;
+#pragma unroll 8
+        for (int j = 0; j < n_raw; ++j)
+            if (s.raw_id[j] == v) f = min(f, j);
+        if (s.first[i] >= 0) s.first[i] = f;
     }
     __syncthreads();
+    // One warp for the rest: a chain of reductions over a few dozen numbers, the independent ones side by side (one after
+    // the other, with the sums kept in shared memory, it was a third of the record's time).
     if (warp == 0) {
         // ---- S = C u Top_kS u {y*}, duplicates removed (first occurrence kept; the candidates come first)
-        if (lane == 0) s.n = 0;
-        __syncwarp();
+        int n = 0;
         for (int i0 = 0; i0 < n_raw; i0 += 32) {
             const int i = i0 + lane;
-            const int v = i < n_raw ? s.raw_id[i] : -1;
             const bool fresh = i < n_raw && s.first[i] == i;
             const unsigned bal = __ballot_sync(0xffffffffu, fresh);
-            const int base = s.n;
             if (fresh) {
-                const int pos = base + __popc(bal & ((1u << lane) - 1u));
-                s.id[pos] = v;
+                const int pos = n + __popc(bal & ((1u << lane) - 1u));
+                s.id[pos] = s.raw_id[i];
                 s.p[pos] = s.raw_p[i];
+                s.acov[pos] = 0.f;
                 s.where[i] = pos;
             }
-            __syncwarp();
-            if (lane == 0) s.n = base + __popc(bal);
-            __syncwarp();
+            n += __popc(bal);
         }
+        if (lane == 0) s.n = n;
+        __syncwarp();
         if (lane == 0) ready();
-        // ---- q on the candidates
+        // ---- q on the candidates; masses p(S), p(C), p(C*)
         float mx = -INFINITY;
-        for (int j = lane; j < k; j += 32) mx = fmaxf(mx, cl[j]);
+        for (int j = lane; j < k; j += 32) mx = fmaxf(mx, s.cl[j]);
         mx = warp_max(mx);
-        float qs = 0.f;
+        float qs = 0.f, pS = 0.f, pC = 0.f, pCs = 0.f;
         for (int j = lane; j < k; j += 32) {
-            const float w = __expf((cl[j] - mx) * a.inv_T);
-            s.q[j] = w;
-            qs += w;
+            qs += __expf((s.cl[j] - mx) * a.inv_T);
+            pC += s.p[j];  // the first k support entries are the candidates
+            pCs += s.raw_p[k + j];  // C* = the first k of Top_kS
         }
-        qs = warp_sum(qs);
-        __syncwarp();
-        for (int j = lane; j < k; j += 32) s.q[j] /= qs;
-        const int n = s.n;
-        for (int i = lane; i < n_raw; i += 32) {  // repeated tokens: the place of their first occurrence
-            const int f = s.first[i];
-            if (f != i) s.where[i] = f < 0 ? -1 : s.where[f];
-        }
-        __syncwarp();
-        // ---- masses: p(S), p(C), p(C*); TV on C
-        float pS = 0.f;
         for (int i = lane; i < n; i += 32) pS += s.p[i];
-        pS = warp_sum(pS);
-        float pC = 0.f;
-        for (int j = lane; j < k; j += 32) pC += s.p[j];  // the first k support entries are the candidates
-        pC = warp_sum(pC);
-        float tvs = 0.f;
-        for (int j = lane; j < k; j += 32) tvs += fabsf(s.p[j] / pC - s.q[j]);
-        tvs = 0.5f * warp_sum(tvs);
-        // C* = the first k of Top_kS; O = C* \ C
-        float pCs = 0.f, cov_b = 0.f;
-        for (int i = lane; i < n; i += 32) s.acov[i] = 0.f;
-        __syncwarp();
-        for (int t = lane; t < k; t += 32) {
-            const float pv = s.raw_p[k + t];
-            pCs += pv;
-            const int f = s.first[k + t];
-            const bool inC = f >= 0 && f < k;  // (first seen among the candidates, which come first)
-            if (!inC) {
-                // an omitted target-important token: +p_S(y) on its own row, -p_S(y) on the weakest candidate's
-                const int pos = s.where[k + t];
-                if (pos >= k) s.acov[pos] = pv / pS;
-                cov_b += pv / pS;
-            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            qs += __shfl_xor_sync(0xffffffffu, qs, o);
+            pS += __shfl_xor_sync(0xffffffffu, pS, o);
+            pC += __shfl_xor_sync(0xffffffffu, pC, o);
+            pCs += __shfl_xor_sync(0xffffffffu, pCs, o);
         }
-        pCs = warp_sum(pCs);
-        cov_b = warp_sum(cov_b);
-        __syncwarp();
-        float tvS = 0.f;  // TV(p_S, q_S)
+        // ---- the coefficients; TV on C, TV(p_S, q_S)
+        float tvs = 0.f, cov_b = 0.f, tvS = 0.f;
         for (int i = lane; i < n; i += 32) {
-            const float ad = s.p[i] / pS - (i < k ? s.q[i] : 0.f);
+            float q = 0.f;
+            if (i < k) {
+                q = __expf((s.cl[i] - mx) * a.inv_T) / qs;
+                tvs += fabsf(s.p[i] / pC - q);
+            }
+            const float ad = s.p[i] / pS - q;
             s.adist[i] = ad;
             tvS += fabsf(ad);
         }
-        tvS = 0.5f * warp_sum(tvS);
+        for (int t = lane; t < k; t += 32) {
+            const int f = s.first[k + t];
+            if (!(f >= 0 && f < k)) {  // O = C* \ C (the candidates come first)
+                // an omitted target-important token: +p_S(y) on its own row, -p_S(y) on the weakest candidate's
+                const float c = s.raw_p[k + t] / pS;
+                const int pos = f < 0 ? -1 : s.where[f];
+                if (pos >= k) s.acov[pos] = c;
+                cov_b += c;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            tvs += __shfl_xor_sync(0xffffffffu, tvs, o);
+            cov_b += __shfl_xor_sync(0xffffffffu, cov_b, o);
+            tvS += __shfl_xor_sync(0xffffffffu, tvS, o);
+        }
+        tvs *= 0.5f;
+        tvS *= 0.5f;
+        __syncwarp();
         if (lane == 0) {
             // severity of the observation: w = clip(0.3 TV(p_S, q_S) + 0.7 p_out, 0, 1), p_out = 1 - p(C)
             const float w = fminf(1.f, fmaxf(0.f, 0.3f * tvS + 0.7f * (1.f - pC)));
