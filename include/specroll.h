@@ -377,6 +377,16 @@ int specroll_target_head_stats(int32_t R, int32_t d, int32_t V, float temperatur
                                float *row_sum, void *want_logit, void *workspace,
                                size_t workspace_bytes, void *cuda_stream);
 
+/* The same, and every row's maximum (so far in the tile's range) and sum of exp((l - maximum)/T) of every tile of 128
+ * tokens: tile_mass, pairs of fp32 [ceil(V / 128)][R], specroll_target_head_tile_mass_bytes bytes, 8-byte aligned,
+ * nullable. */
+size_t specroll_target_head_tile_mass_bytes(int32_t R, int32_t V);
+
+int specroll_target_head_stats_tiles(int32_t R, int32_t d, int32_t V, float temperature, const void *H,
+                                     const void *W, const int32_t *want_id, int32_t kw, float *row_max,
+                                     float *row_sum, void *want_logit, void *tile_mass, void *workspace,
+                                     size_t workspace_bytes, void *cuda_stream);
+
 int specroll_target_head_rows(int32_t R, int32_t d, int32_t V, const void *H, const void *W,
                               void *logits, int32_t *status, void *cuda_stream);
 
@@ -436,6 +446,10 @@ int specroll_verify(const specroll_verify_desc *desc, const void *logits,
  *                                term_kind, min_margin (nullable) and leaves the residual in the workspace;
  *   specroll_verify_terminal_rows  the step's last token from term_logits[B, V] bf16, the full logits row of
  *                                every sequence's terminal node, with the same workspace.
+ *   specroll_verify_hidden  walk and last token in one launch, from the wanted logits and the tile masses of
+ *                                specroll_target_head_stats_tiles: the logits of the one tile of 128 tokens that holds the
+ *                                drawn token are made from hidden[B*N, d] and W[V, d] (fp32 sums rounded to bf16; their
+ *                                order differs from the projection's).  No workspace; d % 8 == 0.
  * The workspace has specroll_verify_workspace_bytes(desc) bytes; desc.flags must be 0. */
 int specroll_verify_want_ids(const specroll_verify_desc *desc, const int32_t *parent_host,
                              const int32_t *cand_id, int32_t *want_id, void *cuda_stream);
@@ -447,6 +461,14 @@ int specroll_verify_walk_sparse(const specroll_verify_desc *desc, const void *ca
                                 int32_t *path_node, int32_t *out_tok, int32_t *term_node,
                                 int32_t *term_kind, float *min_margin, void *workspace,
                                 size_t workspace_bytes, void *cuda_stream);
+
+int specroll_verify_hidden(const specroll_verify_desc *desc, int32_t d, const void *hidden, const void *W,
+                           const void *cand_target, const void *tile_mass, const float *row_max,
+                           const float *row_sum, const int32_t *parent_host, const int32_t *tree_tok,
+                           const uint8_t *tree_cand, const int32_t *cand_id, const float *cand_logit,
+                           const float *u_acc, const float *u_fin, int32_t *n_acc, int32_t *path_node,
+                           int32_t *out_tok, int32_t *term_node, int32_t *term_kind, float *min_margin,
+                           void *cuda_stream);
 
 int specroll_verify_terminal_rows(const specroll_verify_desc *desc, const void *term_logits,
                                   const float *row_max, const int32_t *n_acc, const int32_t *term_node,

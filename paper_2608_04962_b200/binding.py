@@ -33,7 +33,8 @@ EXPORTS = ("specroll_version", "specroll_strerror", "specroll_node_budget", "spe
            "specroll_reflex_feedback_workspace_bytes", "specroll_reflex_feedback", "specroll_reflex_feedback_ex",
            "specroll_reflex_sketch", "specroll_reflex_gate",
            "specroll_target_head_stats_workspace_bytes", "specroll_target_head_stats", "specroll_target_head_rows",
-           "specroll_verify_want_ids", "specroll_verify_walk_sparse", "specroll_verify_terminal_rows")
+           "specroll_verify_want_ids", "specroll_verify_walk_sparse", "specroll_verify_terminal_rows",
+           "specroll_target_head_tile_mass_bytes", "specroll_target_head_stats_tiles", "specroll_verify_hidden")
 
 
 PROPOSE_LEGACY_MMA = 1
@@ -296,9 +297,9 @@ def verify(logits, parent, tree_tok, tree_cand, cand_id, cand_logit, u_acc, u_fi
 
 def verify_fused(hidden, W, parent, tree_tok, tree_cand, cand_id, cand_logit, u_acc, u_fin, temperature=1.0):
     """Exact verification from the target's final hidden states, without the logits tensor: the projection with
-    fused row statistics over all (sequence, node) rows (specroll_target_head_stats), the walk on the target logits
-    of the candidate tokens (specroll_verify_walk_sparse), then the one row per sequence that the terminal draw
-    needs (specroll_gather_hidden, specroll_target_head_rows, specroll_verify_terminal_rows).
+    fused row statistics and tile masses over all (sequence, node) rows (specroll_target_head_stats_tiles), then the walk
+    on the target logits of the candidate tokens and the terminal draw from the one vocabulary tile that holds its
+    token (specroll_verify_hidden).
     hidden [B, N, d] bf16, W [V, d] bf16; the other arguments as for ``verify``.  Returns the same dict."""
     return _n().verify_fused(hidden, W, parent, tree_tok, tree_cand, cand_id, cand_logit, u_acc, u_fin, temperature)
 

@@ -100,6 +100,9 @@ void register_check_reader(CheckReader fn);
 static inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// Tokens per vocabulary tile of the target projection's table of tile masses.
+constexpr int HEAD_TILE = 128;
+
 // Tree topology, validated on the host and handed to kernels by value (200 bytes).
 struct Topo {
     int32_t N;

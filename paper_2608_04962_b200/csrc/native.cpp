@@ -52,7 +52,8 @@ constexpr at::ScalarType BF16 = at::kBFloat16, F32 = at::kFloat, I32 = at::kInt,
     X(specroll_verify_nucleus) X(specroll_reflex_feedback_workspace_bytes) X(specroll_reflex_feedback_ex)            \
     X(specroll_reflex_sketch) X(specroll_reflex_gate) X(specroll_target_head_stats_workspace_bytes)                  \
     X(specroll_target_head_stats) X(specroll_target_head_rows) X(specroll_verify_want_ids)                           \
-    X(specroll_verify_walk_sparse) X(specroll_verify_terminal_rows)
+    X(specroll_target_head_tile_mass_bytes)                                                                          \
+    X(specroll_target_head_stats_tiles) X(specroll_verify_hidden)
 struct Entries {
 #define X(name) decltype(&::name) name;
     SPECROLL_ENTRIES(X)
@@ -495,18 +496,16 @@ PyObject *verify_fused(PyObject *const *a) {
     if (need_ws == 0) fail("target_head_stats: invalid shape");
     const at::Tensor ws_head = alloc_bytes(need_ws, hidden);
     const void *ph = dev(hidden, BF16, "H"), *pw = dev(W, BF16, "W");
-    CALL(specroll_target_head_stats, (int32_t)(B * N), (int32_t)d, (int32_t)v.V, T, ph, pw, (const int32_t *)ptr(want), (int32_t)v.k,
-         (float *)ptr(row_max), (float *)ptr(row_sum), ptr(want_logit), ptr(ws_head), bytes_of(ws_head));
+    const at::Tensor tiles = alloc_bytes(lib.specroll_target_head_tile_mass_bytes((int32_t)(B * N), (int32_t)v.V), hidden);
+    CALL(specroll_target_head_stats_tiles, (int32_t)(B * N), (int32_t)d, (int32_t)v.V, T, ph, pw, (const int32_t *)ptr(want), (int32_t)v.k,
+         (float *)ptr(row_max), (float *)ptr(row_sum), ptr(want_logit), ptr(tiles), ptr(ws_head), bytes_of(ws_head));
     Out out(nullptr);
     const VerifyOut o(out, v, hidden, false);
     out.put("row_max", row_max);
     out.put("row_sum", row_sum);
-    const at::Tensor ws = alloc_bytes(lib.specroll_verify_workspace_bytes(&D), hidden);
-    CALL(specroll_verify_walk_sparse, &D, ptr(want_logit), (const float *)ptr(row_max), (const float *)ptr(row_sum), parent.data(), v.tree_tok,
-         v.tree_cand, v.cand_id, v.cand_logit, v.u_acc, o.n_acc, o.path_node, o.out_tok, o.term_node, o.term_kind, o.min_margin, ptr(ws), bytes_of(ws));
-    const at::Tensor term = THPVariable_Unpack(PyDict_GetItemString(out.peek(), "term_node"));
-    const at::Tensor rows = target_head_rows_t(gather_hidden_t(hidden, &term, nullptr), W, nullptr);
-    CALL(specroll_verify_terminal_rows, &D, ptr(rows), (const float *)ptr(row_max), o.n_acc, o.term_node, v.u_fin, o.out_tok, ptr(ws), bytes_of(ws));
+    CALL(specroll_verify_hidden, &D, (int32_t)d, ph, pw, ptr(want_logit), ptr(tiles), (const float *)ptr(row_max), (const float *)ptr(row_sum),
+         parent.data(), v.tree_tok, v.tree_cand, v.cand_id, v.cand_logit, v.u_acc, v.u_fin, o.n_acc, o.path_node, o.out_tok, o.term_node,
+         o.term_kind, o.min_margin);
     return out.release();
 }
 

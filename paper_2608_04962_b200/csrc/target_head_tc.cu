@@ -12,7 +12,8 @@
 // handed to the verification.  Same pipeline as the proposal's projection: persistent warp-specialised CTAs, TMA
 // producer, one MMA-issuing thread (tcgen05, M=128, N=256, K=16, two accumulator buffers in TMEM), four epilogue
 // warps with one thread per row.  A CTA owns a block of 128 rows and a contiguous range of vocabulary tiles; the
-// per-(row, range) partial statistics are merged by a small kernel.
+// per-(row, range) partial statistics are merged by a small kernel.  On request the epilogue also leaves every row's
+// maximum and sum of every 128 tokens, 8 bytes each, from which the terminal draw finds the tile that holds its token.
 #include "tc05.cuh"
 
 namespace specroll {
@@ -33,8 +34,9 @@ target_head_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                       int d, int n_mblocks, int n_groups, int tiles_per_group, float c_log2,
                       const int32_t *__restrict__ want_id, int kw, float *__restrict__ pm, float *__restrict__ ps,
                       uint16_t *__restrict__ want_logit, uint16_t *__restrict__ logits_out,
-                      int32_t *__restrict__ status) {
+                      int32_t *__restrict__ status, float2 *__restrict__ tile_mass) {
     using namespace thtc;
+    pdl_launch_dependents();  // (the merge is set up under this kernel's end)
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // 1024-byte alignment for the 128-byte swizzle atoms
@@ -159,6 +161,7 @@ target_head_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         const int row = lg * 32 + lane;
         const bool row_ok = m0 + row < M;
         float m_run = -INFINITY, s_run = 0.f;  // online maximum (of the logits) and sum of exp((l - m) / T)
+        float s_tile = 0.f;                    // the part of the HEAD_TILE tokens at hand, still to be added to it
         int32_t want[KW_MAX];
 #pragma unroll
         for (int q = 0; q < KW_MAX; ++q) want[q] = (!STORE && row_ok && q < kw) ? want_id[(size_t)(m0 + row) * kw + q] : -1;
@@ -206,7 +209,9 @@ target_head_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                     for (int i = 0; i < 32; ++i)
                         if (i < nv) cm = fmaxf(cm, __uint_as_float(r[i]));
                     if (cm > m_run) {
-                        s_run *= ex2_approx((m_run - cm) * c_log2);  // (0 * 2^-inf = 0 on the first chunk)
+                        const float f = ex2_approx((m_run - cm) * c_log2);  // (0 * 2^-inf = 0 on the first chunk)
+                        s_run *= f;
+                        s_tile *= f;
                         m_run = cm;
                     }
                     const float nm = -m_run * c_log2;
@@ -218,7 +223,7 @@ target_head_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                         s0 += (i < nv) ? e0 : 0.f;
                         s1 += (i + 1 < nv) ? e1 : 0.f;
                     }
-                    s_run += s0 + s1;
+                    s_tile += s0 + s1;
                     // the row's wanted tokens that fall into these 32 columns (rare)
 #pragma unroll
                     for (int q = 0; q < KW_MAX; ++q) {
@@ -230,6 +235,11 @@ target_head_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                                 if ((uint32_t)i == off) val = r[i];
                             want_logit[(size_t)(m0 + row) * kw + q] = (uint16_t)(val >> 16);
                         }
+                    }
+                    if ((c + 32) % HEAD_TILE == 0 || c + 32 >= ncol) {
+                        if (tile_mass && row_ok) tile_mass[(size_t)((n0 + c) / HEAD_TILE) * M + m0 + row] = make_float2(m_run, s_tile);
+                        s_run += s_tile;
+                        s_tile = 0.f;
                     }
                 }
             }
@@ -255,6 +265,8 @@ target_head_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 // row_max = max over the ranges, row_sum = sum of the ranges' sums brought to that maximum
 __global__ void target_head_merge_kernel(const float *__restrict__ pm, const float *__restrict__ ps, int M, int n_groups,
                                          float c_log2, float *__restrict__ row_max, float *__restrict__ row_sum) {
+    pdl_wait();
+    pdl_launch_dependents();  // (what follows reads the projection's other results ahead of its own wait)
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= M) return;
     float m = -INFINITY;
@@ -317,14 +329,27 @@ extern "C" size_t specroll_target_head_stats_workspace_bytes(int32_t R, int32_t 
     return p.total;
 }
 
+extern "C" size_t specroll_target_head_tile_mass_bytes(int32_t R, int32_t V) {
+    if (R < 0 || V < 8 || (V % 8)) return 0;
+    return (size_t)((V + HEAD_TILE - 1) / HEAD_TILE) * R * sizeof(float2);
+}
+
 extern "C" int specroll_target_head_stats(int32_t R, int32_t d, int32_t V, float temperature, const void *H, const void *W,
                                           const int32_t *want_id, int32_t kw, float *row_max, float *row_sum,
                                           void *want_logit, void *workspace, size_t workspace_bytes, void *cuda_stream) {
+    return specroll_target_head_stats_tiles(R, d, V, temperature, H, W, want_id, kw, row_max, row_sum, want_logit, nullptr, workspace,
+                                            workspace_bytes, cuda_stream);
+}
+
+extern "C" int specroll_target_head_stats_tiles(int32_t R, int32_t d, int32_t V, float temperature, const void *H, const void *W,
+                                                const int32_t *want_id, int32_t kw, float *row_max, float *row_sum,
+                                                void *want_logit, void *tile_mass, void *workspace, size_t workspace_bytes,
+                                                void *cuda_stream) {
     using namespace thtc;
     if (!head_shape_ok(R, d, V) || !(temperature > 0.f) || kw < 0 || kw > KW_MAX) return SPECROLL_EINVAL;
     if (R == 0) return SPECROLL_OK;
     if (!H || !W || !row_max || !row_sum || (kw > 0 && (!want_id || !want_logit))) return SPECROLL_EINVAL;
-    if (!aligned16(H) || !aligned16(W)) return SPECROLL_EALIGN;
+    if (!aligned16(H) || !aligned16(W) || (reinterpret_cast<uintptr_t>(tile_mass) & 7u)) return SPECROLL_EALIGN;
     HeadPlan p;
     plan_head(R, V, &p);
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < p.total) return SPECROLL_EWORKSPACE;
@@ -342,10 +367,10 @@ extern "C" int specroll_target_head_stats(int32_t R, int32_t d, int32_t V, float
     const float c_log2 = 1.4426950408889634f / temperature;
     target_head_tc_kernel<false><<<p.n_mblocks * p.n_groups, THREADS, SMEM_BYTES, st>>>(
         tmA, tmB, R, V, d, p.n_mblocks, p.n_groups, p.tiles_per_group, c_log2, want_id, kw, pm, ps,
-        static_cast<uint16_t *>(want_logit), nullptr, status);
+        static_cast<uint16_t *>(want_logit), nullptr, status, static_cast<float2 *>(tile_mass));
     SR_LAUNCH_CHECK();
-    target_head_merge_kernel<<<(R + 255) / 256, 256, 0, st>>>(pm, ps, R, p.n_groups, c_log2, row_max, row_sum);
-    SR_LAUNCH_CHECK();
+    SR_CUDA_TRY(launch_dependent(true, target_head_merge_kernel, dim3((unsigned)(R + 63) / 64), dim3(64), 0, st, (const float *)pm,
+                                 (const float *)ps, R, p.n_groups, c_log2, row_max, row_sum));
     return SPECROLL_OK;
 }
 
@@ -368,7 +393,7 @@ extern "C" int specroll_target_head_rows(int32_t R, int32_t d, int32_t V, const 
     if ((rc = device_setup(reinterpret_cast<const void *>(target_head_tc_kernel<true>), SMEM_BYTES, nullptr)) != SPECROLL_OK) return rc;
     target_head_tc_kernel<true><<<p.n_mblocks * p.n_groups, THREADS, SMEM_BYTES, st>>>(
         tmA, tmB, R, V, d, p.n_mblocks, p.n_groups, p.tiles_per_group, 0.f, nullptr, 0, nullptr, nullptr, nullptr,
-        static_cast<uint16_t *>(logits), status);
+        static_cast<uint16_t *>(logits), status, nullptr);
     SR_LAUNCH_CHECK();
     return SPECROLL_OK;
 }

@@ -11,9 +11,9 @@
 //                       for the rest of the vocabulary, all in fp64; the terminal draw is an
 //                       inverse CDF over the vocabulary in token order with fp64 segment sums, the
 //                       walk's <= k residual entries overriding the plain softmax mass.
-// The other forms (statistics only of visited rows, nucleus targets, logits that were never
-// stored) use walk_kernel / walk_cta_kernel (one warp / one CTA per sequence) and
-// terminal_kernel (one CTA per sequence).
+// Logits that were never stored: the same kernel with the projection's numbers (wanted logits, tile masses) in
+// place of the rows.  The other forms (statistics only of visited rows, nucleus targets, the steps one by one) use
+// walk_kernel / walk_cta_kernel and terminal_kernel.
 #include <math.h>
 
 #include <mutex>
@@ -834,7 +834,7 @@ __device__ __forceinline__ void walk_buf_fetch(const WalkArgs &a, const Topo &to
         const int u = e / k, j = e - u * k;
         if (topo.n_child[u] > 0) {  // (a node with children is at depth < K)
             const int t = SR_CHECKED(a.cand_id[((size_t)b * K + topo.depth[u]) * k + j], a.V, b);
-            w.pre[e] = a.logits[((size_t)b * N + u) * a.V + t];
+            w.pre[e] = a.logits ? a.logits[((size_t)b * N + u) * a.V + t] : a.cand_target[(size_t)b * N * k + e];
         }
     }
     // the proposal weights of every head's candidates, relative to the head's largest logit
@@ -1479,12 +1479,13 @@ nucleus_rows_kernel(const uint16_t *__restrict__ logits, int V, int N, NodeList 
 //       of every slice of every row, so that this step reads a table and one slice, was tried: the table costs the
 //       statistics kernel as much as it saves here.)
 constexpr int WT_THREADS = TERM_THREADS;
+constexpr int WT_SMEM_LIMIT = 160 * 1024;
 constexpr int WT_WARPS = WT_THREADS / 32;
 
 struct WtLayout {
     size_t stage, ovm, first, mm, slices, p, total;
 };
-__host__ __device__ inline WtLayout wt_layout(int N, int K, int k, int V, int S) {
+__host__ __device__ inline WtLayout wt_layout(int N, int K, int k, size_t draw_bytes) {
     WtLayout L;
     auto up = [](size_t x) { return (x + 15) / 16 * 16; };
     size_t o = 0;
@@ -1497,23 +1498,164 @@ __host__ __device__ inline WtLayout wt_layout(int N, int K, int k, int V, int S)
     L.mm = o;
     o += up((size_t)N * sizeof(float));
     L.slices = o;
-    o += up(draw_smem_bytes(V, S));
+    o += up(draw_bytes);
     L.p = o;
     o += up((size_t)N * k * sizeof(double));
     L.total = o;
     return L;
 }
 
+// The terminal draw without the logits row: the masses of the row's vocabulary tiles are known (mass, per tile and row:
+// maximum and sum), and the logits of the one tile that holds the target are made here, from the row's hidden state and 128
+// rows of W (a few hundred KB to a MB; the storing projection, with all of W, took 178 us for 32 sequences of the 7B
+// shape).  fp32 sums rounded to bf16, as the projection's; the order of a sum's terms differs from the tensor pipe's, so a
+// token's mass may be that of the neighbouring bf16 value and the draw turn where its target lies that close to a bound.
+struct TileArgs {
+    const __nv_bfloat16 *H, *W;  // [B * N, d], [V, d]
+    const float2 *mass;          // [tiles][B * N]
+    int32_t d, rows;
+};
+__host__ __device__ inline size_t tile_smem_bytes(int V, int d) {
+    return ((size_t)(V + HEAD_TILE - 1) / HEAD_TILE + HEAD_TILE) * sizeof(double) + 16 + (size_t)d * 2;
+}
+
+// By all threads of the n_cta CTAs of a cluster, which share the tile's tokens; smem: tile_smem_bytes, at the same offset in
+// every CTA.  bits(j): the bf16 logit of the residual's token j.
+template <class Bits>
+__device__ void draw_tile(const TileArgs &t, size_t row, int V, float M, float c, int n_cta, int rank, int nov, const int32_t *ovid,
+                          const double *ovm, Bits bits, unsigned char *smem, float u, int32_t *dst) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n_tiles = (V + HEAD_TILE - 1) / HEAD_TILE;
+    double *mt = reinterpret_cast<double *>(smem);  // masses of the tiles, then of the tile's tokens
+    double *tok = mt + n_tiles;
+    uint4 *h = reinterpret_cast<uint4 *>(smem + (((size_t)n_tiles + HEAD_TILE) * sizeof(double) + 15) / 16 * 16);
+    __shared__ double seg[TERM_WARPS], sh_base[2];
+    __shared__ int sh_tile, sh_last;
+    for (int i = tid; i < n_tiles; i += TERM_THREADS) {
+        const float2 e = t.mass[(size_t)i * t.rows + row];
+        mt[i] = e.x == NEG_INF ? 0.0 : (double)e.y * (double)ex2_approx((e.x - M) * c);
+    }
+    const int d8 = t.d >> 3;
+    for (int i = tid; i < d8; i += TERM_THREADS) h[i] = reinterpret_cast<const uint4 *>(t.H + row * t.d)[i];
+    __syncthreads();
+    if (tid == 0)
+        for (int j = 0; j < nov; ++j) {
+            double &m = mt[ovid[j] / HEAD_TILE];
+            m = fmax(m + ovm[j] - (double)mass1(bits(j), M, c, 0u), 0.0);  // (a tile whose mass was all in replaced tokens, after rounding)
+        }
+    __syncthreads();
+    // a run of tiles per warp, then the tile within the run; every CTA for itself
+    const int per = (n_tiles + TERM_WARPS - 1) / TERM_WARPS;
+    {
+        double x = 0.0;
+        for (int i = warp * per + lane; i < min(n_tiles, (warp + 1) * per); i += 32) x += mt[i];
+        x = warp_sum(x);
+        if (lane == 0) seg[warp] = x;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const double v = lane < TERM_WARPS ? seg[lane] : 0.0;
+        double incl = warp_incl_scan(v, lane);
+        const double target = (double)u * __shfl_sync(0xffffffffu, incl, 31);
+        unsigned hit = __ballot_sync(0xffffffffu, incl > target), pos = __ballot_sync(0xffffffffu, v > 0.0);
+        bool last = hit == 0u;  // (rounding: the last token with mass)
+        const int w = hit ? __ffs(hit) - 1 : pos ? 31 - __clz(pos) : 0;
+        double base = __shfl_sync(0xffffffffu, incl - v, w);
+        int at = -1, at_pos = min(w * per, n_tiles - 1);
+        double base_pos = base;
+        for (int i0 = w * per; i0 < min(n_tiles, (w + 1) * per) && at < 0; i0 += 32) {
+            const double x = i0 + lane < min(n_tiles, (w + 1) * per) ? mt[i0 + lane] : 0.0;
+            incl = warp_incl_scan(x, lane);
+            hit = last ? 0u : __ballot_sync(0xffffffffu, base + incl > target);
+            pos = __ballot_sync(0xffffffffu, x > 0.0);
+            if (pos) {
+                at_pos = i0 + 31 - __clz(pos);
+                base_pos = base + __shfl_sync(0xffffffffu, incl - x, 31 - __clz(pos));
+            }
+            if (hit) {
+                at = i0 + __ffs(hit) - 1;
+                base += __shfl_sync(0xffffffffu, incl - x, __ffs(hit) - 1);
+            } else {
+                base += __shfl_sync(0xffffffffu, incl, 31);
+            }
+        }
+        if (at < 0) {
+            at = at_pos;
+            base = base_pos;
+            last = true;
+        }
+        if (lane == 0) {
+            sh_tile = at;
+            sh_last = last ? 1 : 0;
+            sh_base[0] = base;
+            sh_base[1] = target;
+        }
+    }
+    __syncthreads();
+    // the tile's logits: a warp per pair of tokens, the pairs spread over the cluster's warps
+    const int v0 = sh_tile * HEAD_TILE, n_tok = min(HEAD_TILE, V - v0);
+    for (int q = (rank * TERM_WARPS + warp) * 2; q < HEAD_TILE; q += n_cta * TERM_WARPS * 2) {
+        float acc[2] = {0.f, 0.f};
+        const uint4 *w0 = reinterpret_cast<const uint4 *>(t.W + (size_t)min(v0 + q, V - 1) * t.d);
+        const uint4 *w1 = reinterpret_cast<const uint4 *>(t.W + (size_t)min(v0 + q + 1, V - 1) * t.d);
+#pragma unroll 4
+        for (int i = lane; i < d8; i += 32) {
+            const uint4 x[2] = {ld_nc_v4(w0 + i), ld_nc_v4(w1 + i)};
+            const uint4 y = h[i];
+            const uint32_t yw[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const uint32_t xw[4] = {x[e].x, x[e].y, x[e].z, x[e].w};
+#pragma unroll
+                for (int z = 0; z < 4; ++z) {
+                    acc[e] = fmaf(__uint_as_float(xw[z] << 16), __uint_as_float(yw[z] << 16), acc[e]);
+                    acc[e] = fmaf(__uint_as_float(xw[z] & 0xffff0000u), __uint_as_float(yw[z] & 0xffff0000u), acc[e]);
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float l = warp_sum(acc[e]);
+            if (lane == 0) tok[q + e] = q + e < n_tok ? (double)mass1(__bfloat16_as_ushort(__float2bfloat16_rn(l)), M, c, 0u) : 0.0;
+        }
+    }
+    if (n_cta > 1) {
+        cluster_sync_all();
+        if (rank == 0)
+            for (int q = tid; q < HEAD_TILE; q += TERM_THREADS) {
+                const int r = (q / 2 / TERM_WARPS) % n_cta;
+                if (r > 0) tok[q] = ld_dsmem_f64(tok + q, r);
+            }
+        cluster_sync_all();  // the other CTAs may leave
+        if (rank != 0) return;
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    double ms[8], lsum = 0.0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) ms[e] = lane * 8 < HEAD_TILE ? tok[lane * 8 + e] : 0.0;
+    for (int j = 0; j < nov; ++j) {
+        const int off = lane * 8 < HEAD_TILE ? ovid[j] - v0 - lane * 8 : -1;
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (e == off) ms[e] = ovm[j];
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) lsum += ms[e];
+    term_pick_token(v0 / 8 + lane, ms, lsum, sh_base[0], sh_base[1], sh_last != 0, (v0 + n_tok) / 8, dst, lane);
+}
+
+// TILES: the target's numbers come from the projection (a.cand_target, tile.mass) and not from stored logits.
+template <bool TILES>
 __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, Topo topo, const float *__restrict__ u_fin, float c,
-                                                               int S, const float2 *__restrict__ run_tab) {
+                                                               int S, const float2 *__restrict__ run_tab, TileArgs tile) {
     __shared__ WalkSmem sh[WT_WARPS];
     extern __shared__ __align__(16) unsigned char sh_dyn[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = S > 1 ? (int)cluster_ctarank() : 0;
     const int b = blockIdx.x / S;
     const int N = a.N, K = a.K, k = a.k;
-    const WtLayout L = wt_layout(N, K, k, a.V, S);
-    auto up = [](size_t x) { return (x + 15) / 16 * 16; };
+    const WtLayout L = wt_layout(N, K, k, TILES ? tile_smem_bytes(a.V, tile.d) : draw_smem_bytes(a.V, S));
     const WalkBuf buf = walk_buf(sh_dyn + L.stage, N, K, k);
     float *rmax = buf.rmax, *rsum = buf.rsum;
     const int32_t *ttok = buf.ttok, *cid = buf.cid;
@@ -1524,7 +1666,8 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     double *slices = reinterpret_cast<double *>(sh_dyn + L.slices);
     double *wp = reinterpret_cast<double *>(sh_dyn + L.p);
     const double inv_T = 1.0 / a.T;
-    // (1) inputs of this call, none of them written by the kernel before this one
+    // (1) inputs of this call, none of them written by the kernel before this one (the statistics, or the projection's merge,
+    // which itself waits for the projection before it lets this kernel start)
     walk_buf_fetch(a, topo, b, buf);
     pdl_wait();  // the row statistics are complete from here on
     for (int n = tid; n < N; n += WT_THREADS) {
@@ -1607,6 +1750,11 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     const int32_t *ovid = cid + (resid ? topo.depth[u] : 0) * k;
     const double *ovm_u = ovm + u * k;
     const float M = rmax[u];
+    if constexpr (TILES) {
+        draw_tile(tile, (size_t)b * N + u, a.V, M, c, S, rank, nov, ovid, ovm_u, [&](int j) { return pre[u * k + j]; },
+                  sh_dyn + L.slices, u_fin[b], a.out_tok + (size_t)b * (K + 1) + nacc);
+        return;
+    }
     const uint16_t *lg = a.logits + ((size_t)b * N + u) * a.V;
     const int nvec = a.V >> 3;
     // With the statistics kernel's table of the row's eight runs (run_tab; then S = 1): the run that holds the target
@@ -1806,14 +1954,13 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
         return SPECROLL_OK;
     }
     // plain verification: the walk and the terminal draw in one launch, overlapping the statistics kernel's tail
-    constexpr int WT_SMEM_LIMIT = 160 * 1024;
     const int S = use_runs ? 1 : walk_term_split(d->B);
-    const WtLayout L = wt_layout(d->N, d->K, d->k, d->V, S);
+    const WtLayout L = wt_layout(d->N, d->K, d->k, draw_smem_bytes(d->V, S));
     if (L.total > (size_t)WT_SMEM_LIMIT) return SPECROLL_ELIMIT;
-    const int rc_ = device_setup(reinterpret_cast<const void *>(walk_term_kernel), WT_SMEM_LIMIT, nullptr);
+    const int rc_ = device_setup(reinterpret_cast<const void *>(walk_term_kernel<false>), WT_SMEM_LIMIT, nullptr);
     if (rc_ != SPECROLL_OK) return rc_;
-    SR_CUDA_TRY(launch_clusters(true, S, walk_term_kernel, dim3((unsigned)(d->B * S)), dim3(WT_THREADS), L.total, st, wa, topo, u_fin,
-                                c, S, (const float2 *)run_tab));
+    SR_CUDA_TRY(launch_clusters(true, S, walk_term_kernel<false>, dim3((unsigned)(d->B * S)), dim3(WT_THREADS), L.total, st, wa, topo,
+                                u_fin, c, S, (const float2 *)run_tab, TileArgs{}));
     return SPECROLL_OK;
 }
 
@@ -1895,6 +2042,58 @@ extern "C" int specroll_verify_walk_sparse(const specroll_verify_desc *d, const 
     wa.T = (double)d->temperature;
     walk_kernel<<<(d->B + WALK_WARPS - 1) / WALK_WARPS, WALK_WARPS * 32, 0, st>>>(wa, topo);
     SR_LAUNCH_CHECK();
+    return SPECROLL_OK;
+}
+
+extern "C" int specroll_verify_hidden(const specroll_verify_desc *d, int32_t dim, const void *hidden, const void *W,
+                                      const void *cand_target, const void *tile_mass, const float *row_max, const float *row_sum,
+                                      const int32_t *parent_host, const int32_t *tree_tok, const uint8_t *tree_cand,
+                                      const int32_t *cand_id, const float *cand_logit, const float *u_acc, const float *u_fin,
+                                      int32_t *n_acc, int32_t *path_node, int32_t *out_tok, int32_t *term_node, int32_t *term_kind,
+                                      float *min_margin, void *cuda_stream) {
+    if (check_verify_desc(d) != SPECROLL_OK || d->flags != 0 || dim < 8 || (dim % 8)) return SPECROLL_EINVAL;
+    Topo topo;
+    if (build_topo(parent_host, d->N, d->K, d->k, &topo, nullptr) != SPECROLL_OK) return SPECROLL_EINVAL;
+    if (d->B == 0) return SPECROLL_OK;  // (an empty batch has empty arrays: their pointers may be NULL)
+    if (!hidden || !W || !cand_target || !tile_mass || !row_max || !row_sum || !tree_tok || !tree_cand || !cand_id || !cand_logit ||
+        !u_acc || !u_fin || !n_acc || !path_node || !out_tok || !term_node || !term_kind)
+        return SPECROLL_EINVAL;
+    if (!aligned16(hidden) || !aligned16(W) || (reinterpret_cast<uintptr_t>(tile_mass) & 7u)) return SPECROLL_EALIGN;
+    WalkArgs wa;
+    wa.logits = nullptr;
+    wa.cand_target = static_cast<const uint16_t *>(cand_target);
+    wa.tree_tok = tree_tok;
+    wa.tree_cand = tree_cand;
+    wa.cand_id = cand_id;
+    wa.cand_logit = cand_logit;
+    wa.u_acc = u_acc;
+    wa.row_max = row_max;
+    wa.row_sum = row_sum;
+    wa.n_acc = n_acc;
+    wa.path_node = path_node;
+    wa.out_tok = out_tok;
+    wa.term_node = term_node;
+    wa.term_kind = term_kind;
+    wa.min_margin = min_margin;
+    wa.ws_nov = nullptr;
+    wa.ws_ovid = nullptr;
+    wa.ws_ovm = nullptr;
+    wa.B = d->B;
+    wa.N = d->N;
+    wa.K = d->K;
+    wa.k = d->k;
+    wa.V = d->V;
+    wa.T = (double)d->temperature;
+    const TileArgs tile{static_cast<const __nv_bfloat16 *>(hidden), static_cast<const __nv_bfloat16 *>(W),
+                        static_cast<const float2 *>(tile_mass), dim, d->B * d->N};
+    const int S = walk_term_split(d->B);
+    const WtLayout L = wt_layout(d->N, d->K, d->k, tile_smem_bytes(d->V, dim));
+    if (L.total > (size_t)WT_SMEM_LIMIT) return SPECROLL_ELIMIT;
+    const int rc = device_setup(reinterpret_cast<const void *>(walk_term_kernel<true>), WT_SMEM_LIMIT, nullptr);
+    if (rc != SPECROLL_OK) return rc;
+    SR_CUDA_TRY(launch_clusters(true, S, walk_term_kernel<true>, dim3((unsigned)(d->B * S)), dim3(WT_THREADS), L.total,
+                                static_cast<cudaStream_t>(cuda_stream), wa, topo, u_fin, (float)(1.4426950408889634 / (double)d->temperature),
+                                S, (const float2 *)nullptr, tile));
     return SPECROLL_OK;
 }
 

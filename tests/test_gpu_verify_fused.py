@@ -63,3 +63,10 @@ def test_fused_path_equals_the_path_through_stored_logits(name, B, V, d, T):
                     temperature=T)
     agree = (f["n_acc"] == oo["n_acc"]) & (f["out_tok"] == oo["out_tok"]).all(1)
     assert agree.mean() >= 0.9
+
+
+@pytest.mark.parametrize("name,B,V,d,T", [("tiny", 300, 264, 64, 1.0), ("tiny", 100, 4360, 192, 1.3), ("qwen1.5b", 60, 256, 128, 0.7),
+                                          ("qwen7b", 3, 40, 4096, 1.0)])
+def test_last_token_from_one_tile(name, B, V, d, T):
+    """One to eight CTAs per sequence; vocabularies below, at and above one tile, with a ragged last one."""
+    test_fused_path_equals_the_path_through_stored_logits(name, B, V, d, T)
