@@ -1469,7 +1469,7 @@ nucleus_rows_kernel(const uint16_t *__restrict__ logits, int V, int N, NodeList 
 //       kernel in the stream, which this kernel is launched to overlap with (programmatic dependent launch).
 //   (2) Which nodes the walk reaches depends on its decisions, but what happens AT a node does not: its children
 //       are tried in slot order until one is accepted, each against the residual left by the rejections before it.
-//       So every node with children is examined on its own, one warp per node, all at once: the first accepted
+//       So every node with children is examined on its own, all at once: the first accepted
 //       child (or none, and then the residual), and the smallest margin on the way.  The walk itself is then a
 //       chain of at most K + 1 look-ups.  Every CTA of a cluster does (1) and (2) for itself: same inputs, same
 //       arithmetic, same result, nothing to exchange.
@@ -1482,8 +1482,144 @@ constexpr int WT_THREADS = TERM_THREADS;
 constexpr int WT_SMEM_LIMIT = 160 * 1024;
 constexpr int WT_WARPS = WT_THREADS / 32;
 
+// The children of every node, grouped by parent in slot order, and what a slot's test needs of the proposal (k <= 32): known
+// before the row statistics are.
+struct WalkSlots {
+    double *q;       // [N, k] the slot's proposal on the candidates: e_j / s over those the earlier siblings left, 0 on the others
+    double *u;       // [N]    the acceptance uniform
+    int32_t *node;   // [N]    the child
+    int32_t *jc;     // [N]    its own candidate
+    int32_t *start;  // [N]    first slot of a parent's children
+};
+__host__ __device__ inline size_t walk_slots_bytes(int N, int k) {
+    auto up = [](size_t x) { return (x + 15) / 16 * 16; };
+    return k > 32 ? 0 : up((size_t)N * k * sizeof(double)) + up((size_t)N * sizeof(double)) + 3 * up((size_t)N * sizeof(int32_t));
+}
+__device__ __forceinline__ WalkSlots walk_slots(unsigned char *p, int N, int k) {
+    auto take = [&](size_t x) {
+        unsigned char *q = p;
+        p += (x + 15) / 16 * 16;
+        return q;
+    };
+    WalkSlots w;
+    w.q = reinterpret_cast<double *>(take((size_t)N * k * sizeof(double)));
+    w.u = reinterpret_cast<double *>(take((size_t)N * sizeof(double)));
+    w.node = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
+    w.jc = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
+    w.start = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
+    return w;
+}
+// By all threads of a CTA, from a filled WalkBuf (a barrier before and after is the caller's).  *odd: set where a slot's weights
+// underflow (such trees go through walk_node).
+__device__ __forceinline__ void walk_slots_fill(const WalkBuf &buf, const Topo &topo, int N, int k, int where, const WalkSlots &w,
+                                                int *odd) {
+    // a thread per (child, candidate): the sums over the candidates are formed by each for itself, in the order walk_node has
+    for (int e = threadIdx.x; e < (N - 1) * k; e += blockDim.x) {
+        const int c = 1 + e / k, j = e - (c - 1) * k, u = buf.parent[c];
+        int at = 0, first = 0;
+        unsigned taken = 0u;
+        for (int n = 1; n < N; ++n) {
+            const int pn = buf.parent[n];
+            at += pn < u || (pn == u && n < c);
+            first += pn < u;
+            if (pn == u && n < c) taken |= 1u << SR_CHECKED((int)buf.tcand[n], k, where);
+        }
+        const double *eh = buf.e + topo.depth[u] * k;
+        double s = 0.0;
+        for (int i = 0; i < k; ++i)
+            if (!((taken >> i) & 1u)) s += eh[i];
+        if (!(s > 0.0 && s < INFINITY)) *odd = 1;
+        w.q[at * k + j] = ((taken >> j) & 1u) ? 0.0 : eh[j] * (1.0 / s);
+        if (j == 0) {
+            w.node[at] = c;
+            w.jc[at] = SR_CHECKED((int)buf.tcand[c], k, where);
+            w.u[at] = (double)buf.uacc[c];
+            w.start[u] = first;
+        }
+    }
+}
+
+// Every node with children on its own, kp lanes (the power of two that holds k <= 32 candidates, and so all children) per node,
+// several nodes per warp: the arithmetic of walk_node with the slots' proposals ready.  first[u]: accepted child or -1,
+// mm[u]: smallest margin, ovm[u, j]: the residual's masses where all children were rejected.  (A warp per node took 9 k
+// cycles, two rounds of them where more than sixteen nodes have children: 10 us of the 66 us of 16 sequences x 48 nodes.)
+__device__ __forceinline__ void walk_nodes(const Topo &topo, int N, int k, const double *p, const float *rsum, const WalkSlots &w,
+                                           int32_t *first, float *mm, double *ovm) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int kp = 1;
+    while (kp < k) kp <<= 1;
+    const int per_warp = 32 / kp, grp = lane / kp, j = lane & (kp - 1);
+    int n_par = 0;
+    for (int u = 0; u < N; ++u) n_par += topo.n_child[u] > 0;
+    // as few nodes per warp as give every node a place in one round
+    const int share = min(per_warp, (n_par + TERM_WARPS - 1) / TERM_WARPS);
+    for (int i0 = warp * share; i0 < n_par; i0 += TERM_WARPS * share) {
+        int u = -1;
+        if (grp < share && i0 + grp < n_par) {
+            int idx = 0;
+            for (int n = 0; n < N; ++n)
+                if (topo.n_child[n] > 0 && idx++ == i0 + grp) u = n;
+        }
+        const int m = u >= 0 ? topo.n_child[u] : 0, st = u >= 0 ? w.start[u] : 0;
+        int most = m;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+        double rho = u >= 0 && j < k ? p[u * k + j] : 0.0;
+        double pc = rho;
+        for (int o = kp >> 1; o > 0; o >>= 1) pc += __shfl_xor_sync(0xffffffffu, pc, o);
+        const double p_off = pc < 1.0 ? 1.0 - pc : 0.0;
+        double Zc = 1.0, my_rho = 0.0, my_Zc = 1.0;
+#pragma unroll 2
+        for (int i = 0; i < most; ++i) {
+            const bool on = i < m;
+            const double q = on && j < k ? w.q[(st + i) * k + j] : 0.0;
+            const double rho_jc = __shfl_sync(0xffffffffu, rho, on ? w.jc[st + i] : 0, kp);
+            if (j == i) {
+                my_rho = rho_jc;
+                my_Zc = Zc;
+            }
+            const double t0 = rho - Zc * q, t = t0 > 0.0 ? t0 : 0.0;
+            double Zn = t;
+            for (int o = kp >> 1; o > 0; o >>= 1) Zn += __shfl_xor_sync(0xffffffffu, Zn, o);
+            Zn += p_off;
+            if (on && Zn > 1e-300 * Zc) {
+                rho = t;
+                Zc = Zn;
+            }
+        }
+        // every child's test at once, lane i of the group child i
+        bool acc = false;
+        float mg = INFINITY;
+        int c = -1;
+        if (j < m) {
+            c = w.node[st + j];
+            const double my_q = w.q[(st + j) * k + w.jc[st + j]], uu = w.u[st + j];
+            double ratio;
+            if (my_q > 0.0)
+                ratio = my_rho > 0.0 ? (my_rho / my_Zc) / my_q : 0.0;
+            else
+                ratio = my_rho > 0.0 ? INFINITY : 0.0;
+            acc = uu < (ratio < 1.0 ? ratio : 1.0);
+            mg = (float)fabs(uu - ratio);
+        }
+        const unsigned mask = kp == 32 ? 0xffffffffu : ((1u << kp) - 1u) << (grp * kp);
+        const unsigned hits = __ballot_sync(0xffffffffu, acc) & mask;
+        const int f = hits ? __ffs(hits) - 1 : -1;
+        if (f >= 0 && lane > f) mg = INFINITY;
+        for (int o = kp >> 1; o > 0; o >>= 1) mg = fminf(mg, __shfl_xor_sync(0xffffffffu, mg, o));
+        const int child = __shfl_sync(0xffffffffu, c, f >= 0 ? f : lane);
+        if (u >= 0) {
+            if (f < 0 && j < k) ovm[u * k + j] = rho * (double)rsum[u];  // (r = rho / Zc and sigma = 1 / Zc)
+            if (j == 0) {
+                first[u] = f < 0 ? -1 : child;
+                mm[u] = mg;
+            }
+        }
+    }
+}
+
 struct WtLayout {
-    size_t stage, ovm, first, mm, slices, p, total;
+    size_t stage, ovm, first, mm, slices, p, slots, total;
 };
 __host__ __device__ inline WtLayout wt_layout(int N, int K, int k, size_t draw_bytes) {
     WtLayout L;
@@ -1501,6 +1637,8 @@ __host__ __device__ inline WtLayout wt_layout(int N, int K, int k, size_t draw_b
     o += up(draw_bytes);
     L.p = o;
     o += up((size_t)N * k * sizeof(double));
+    L.slots = o;
+    o += up(walk_slots_bytes(N, k));
     L.total = o;
     return L;
 }
@@ -1668,7 +1806,12 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     const double inv_T = 1.0 / a.T;
     // (1) inputs of this call, none of them written by the kernel before this one (the statistics, or the projection's merge,
     // which itself waits for the projection before it lets this kernel start)
+    const WalkSlots slots = walk_slots(sh_dyn + L.slots, N, k);
+    __shared__ int sh_odd;
+    if (tid == 0) sh_odd = k > 32;
     walk_buf_fetch(a, topo, b, buf);
+    __syncthreads();
+    if (k <= 32) walk_slots_fill(buf, topo, N, k, b, slots, &sh_odd);
     pdl_wait();  // the row statistics are complete from here on
     for (int n = tid; n < N; n += WT_THREADS) {
         rmax[n] = a.row_max[(size_t)b * N + n];
@@ -1685,7 +1828,9 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     }
     __syncthreads();
     // (2) every node with children on its own
-    {
+    if (!sh_odd) {
+        walk_nodes(topo, N, k, wp, rsum, slots, first, mmin, ovm);
+    } else {
         const WalkStage stage{rmax, rsum, buf.uacc, ttok, buf.tcand, cid, buf.clog, pre, buf.parent, buf.e, wp};
         int idx = 0;
         for (int u = 0; u < N; ++u) {
