@@ -2,8 +2,9 @@
 // accept / resample walk, and the terminal (fallback or bonus) draw.
 //
 // Two launches per plain call:
-//   row_stats_kernel    one CTA per (sequence, node) row: streams the bf16 logits once with
-//                       128-bit loads and keeps an online (max, sum-exp) pair per thread.
+//   run_stats_kernel    streams the bf16 logits once with 128-bit loads, an online (max, sum-exp) pair
+//                       per thread, and leaves the pair of every eighth of every (sequence, node) row
+//                       (row_stats_kernel: one CTA per row, for the forms that read the rows' own pairs).
 //   walk_term_kernel    one CTA (or cluster) per sequence, launched to overlap the tail of the
 //                       statistics kernel: the walk, then the terminal draw.  The residual of the
 //                       walk differs from p only on the <= k candidates of the current node (the
@@ -73,51 +74,89 @@ __host__ __device__ inline int rs_run_of_vec(int nvec, int vi) {
     return (vi / 128) / gpw;
 }
 
-// run_tab (nullable): [rows][RS_WARPS] (m, s) of every warp's run, s = sum over the run of exp((l - m)/T): what the
-// warps hand to the final reduction anyway.  The terminal draw of a row then finds the eighth of the row that holds
-// its target from these and reads only that.
+// Maximum and sum of one warp's part of a run [v_lo, v_hi): groups of 128 vectors, every `step`-th from the `sub`-th on.
+__device__ __forceinline__ void run_stats(const uint4 *__restrict__ p, int nvec, int v_lo, int v_hi, int sub, int step, int lane,
+                                          float c, float &m, float &s) {
+    float nmc = 0.f;
+    m = NEG_INF;
+    s = 0.f;
+#pragma unroll 1
+    for (int i0 = v_lo + sub * 128 + lane; i0 - lane < v_hi; i0 += step * 128) {
+        if (i0 + 3 * 32 < nvec) {  // (for lane 31: the whole group is inside the row)
+            uint4 v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = ld_nc_v4(p + i0 + q * 32);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) online_update(v[q], c, m, nmc, s);
+        } else {
+            for (int q = 0; q < 4; ++q)
+                if (i0 + q * 32 < nvec) online_update(ld_nc_v4(p + i0 + q * 32), c, m, nmc, s);
+        }
+    }
+    const float mw = warp_max(m);
+    s = (m == NEG_INF) ? 0.f : s * ex2_approx((m - mw) * c);
+    s = warp_sum(s);
+    m = mw;
+}
+
+// run_tab: [rows][RS_WARPS] (m, s) of every run of every row, s = sum over the run of exp((l - m)/T).  The kernel that
+// walks adds a row's pairs up; the terminal draw finds the eighth of the row that holds its target from them and reads
+// only that.  A CTA takes the eight runs of a row; where there are fewer runs than resident warps, a run is shared by
+// wpr = 2, 4 or 8 warps of a CTA, and the runs are spread over more CTAs (a run of one warp is 19 dependent rounds of
+// loads: 20 rows of 151936 tokens 19 us, so 6).
 __global__ void __launch_bounds__(RS_THREADS, 8)
-row_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, float *__restrict__ row_max,
-                 float *__restrict__ row_sum, float2 *__restrict__ run_tab) {
+run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs, int wpr, float2 *__restrict__ run_tab) {
     // Set up under the tail of the kernel before, which may have written the logits.  The kernel launched behind this
     // one as its programmatic dependent reads the call's other inputs before it waits for the statistics: it may only
     // start once everything in front of this kernel is complete.
     pdl_wait();
     pdl_launch_dependents();
+    __shared__ float2 sh[RS_WARPS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, slot = warp / wpr, sub = warp - slot * wpr;
+    const int nvec = V >> 3;
+    const int r = wpr == 1 ? blockIdx.x * RS_WARPS + warp : slot * gridDim.x + blockIdx.x;
+    if (r < n_runs) {
+        int v_lo, v_hi;
+        rs_run(nvec, r % RS_WARPS, &v_lo, &v_hi);
+        float m, s;
+        run_stats(reinterpret_cast<const uint4 *>(logits + (size_t)(r / RS_WARPS) * V), nvec, v_lo, v_hi, sub, wpr, lane, c, m, s);
+        if (lane == 0) {
+            if (wpr == 1)
+                run_tab[r] = make_float2(m, s);
+            else
+                sh[warp] = make_float2(m, s);
+        }
+    }
+    if (wpr > 1) {
+        __syncthreads();
+        if (sub == 0 && r < n_runs && lane == 0) {
+            float mb = NEG_INF, sb = 0.f;
+            for (int w = 0; w < wpr; ++w) mb = fmaxf(mb, sh[warp + w].x);
+            for (int w = 0; w < wpr; ++w) sb += sh[warp + w].x == NEG_INF ? 0.f : sh[warp + w].y * ex2_approx((sh[warp + w].x - mb) * c);
+            run_tab[r] = make_float2(mb, sb);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(RS_THREADS, 8)
+row_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, float *__restrict__ row_max,
+                 float *__restrict__ row_sum) {
+    pdl_wait();  // (as in run_stats_kernel)
+    pdl_launch_dependents();
     const size_t row = blockIdx.x;
     const uint4 *p = reinterpret_cast<const uint4 *>(logits + row * (size_t)V);
     const int nvec = V >> 3;
-    float m = NEG_INF, nmc = 0.f, s = 0.f;
-    {
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        const int G = (nvec + 127) / 128, gpw = (G + RS_WARPS - 1) / RS_WARPS;
-        const int g_hi = min(G, (warp + 1) * gpw);
-#pragma unroll 1
-        for (int g = warp * gpw; g < g_hi; ++g) {
-            const int i0 = g * 128 + lane;
-            if (i0 + 3 * 32 < nvec) {  // (for lane 31: the whole group is inside the row)
-                uint4 v[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) v[q] = ld_nc_v4(p + i0 + q * 32);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) online_update(v[q], c, m, nmc, s);
-            } else {
-                for (int q = 0; q < 4; ++q)
-                    if (i0 + q * 32 < nvec) online_update(ld_nc_v4(p + i0 + q * 32), c, m, nmc, s);
-            }
-        }
-    }
-
-    // warp, then block reduction of (m, s)
-    float mw = warp_max(m);
-    s = (m == NEG_INF) ? 0.f : s * ex2_approx((m - mw) * c);
-    s = warp_sum(s);
-    __shared__ float sm_m[RS_THREADS / 32], sm_s[RS_THREADS / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int v_lo, v_hi;
+    rs_run(nvec, warp, &v_lo, &v_hi);
+    float m, s;
+    run_stats(p, nvec, v_lo, v_hi, 0, 1, lane, c, m, s);
+
+    // block reduction of (m, s)
+    __shared__ float sm_m[RS_THREADS / 32], sm_s[RS_THREADS / 32];
     if (lane == 0) {
-        sm_m[warp] = mw;
+        sm_m[warp] = m;
         sm_s[warp] = s;
-        if (run_tab) run_tab[row * RS_WARPS + warp] = make_float2(mw, s);
     }
     __syncthreads();
     if (warp == 0) {
@@ -1786,7 +1825,8 @@ __device__ void draw_tile(const TileArgs &t, size_t row, int V, float M, float c
 // TILES: the target's numbers come from the projection (a.cand_target, tile.mass) and not from stored logits.
 template <bool TILES>
 __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, Topo topo, const float *__restrict__ u_fin, float c,
-                                                               int S, const float2 *__restrict__ run_tab, TileArgs tile) {
+                                                               int S, const float2 *__restrict__ run_tab, float *__restrict__ row_max_w,
+                                                               float *__restrict__ row_sum_w, TileArgs tile) {
     __shared__ WalkSmem sh[WT_WARPS];
     extern __shared__ __align__(16) unsigned char sh_dyn[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1813,18 +1853,35 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     __syncthreads();
     if (k <= 32) walk_slots_fill(buf, topo, N, k, b, slots, &sh_odd);
     pdl_wait();  // the row statistics are complete from here on
-    for (int n = tid; n < N; n += WT_THREADS) {
-        rmax[n] = a.row_max[(size_t)b * N + n];
-        rsum[n] = a.row_sum[(size_t)b * N + n];
+    if (!TILES && run_tab) {
+        // a row's statistics from its eight runs, eight lanes per row (N <= 64: one round; the result as row_stats_kernel's)
+        static_assert(WT_THREADS / RS_WARPS >= SPECROLL_MAX_NODES, "all rows at once");
+        const int n = tid / RS_WARPS;
+        const float2 e = n < N ? run_tab[((size_t)b * N + n) * RS_WARPS + tid % RS_WARPS] : make_float2(NEG_INF, 0.f);
+        float m = e.x;
+#pragma unroll
+        for (int o = RS_WARPS / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        float s = e.x == NEG_INF ? 0.f : e.y * ex2_approx((e.x - m) * c);
+#pragma unroll
+        for (int o = RS_WARPS / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (n < N && tid % RS_WARPS == 0) {
+            rmax[n] = m;
+            rsum[n] = s;
+            row_max_w[(size_t)b * N + n] = m;
+            row_sum_w[(size_t)b * N + n] = s;
+        }
+    } else {
+        for (int n = tid; n < N; n += WT_THREADS) {
+            rmax[n] = a.row_max[(size_t)b * N + n];
+            rsum[n] = a.row_sum[(size_t)b * N + n];
+        }
     }
-    // the target probabilities of every walkable node's candidates (the statistics straight from global memory:
-    // one round trip for everything)
+    __syncthreads();
+    // the target probabilities of every walkable node's candidates
     for (int e = tid; e < N * k; e += WT_THREADS) {
         const int u = e / k;
-        if (topo.n_child[u] > 0) {
-            const double M = (double)a.row_max[(size_t)b * N + u], S = (double)a.row_sum[(size_t)b * N + u];
-            wp[e] = exp(((double)bf16_bits_to_float(pre[e]) - M) * inv_T) * (1.0 / S);
-        }
+        if (topo.n_child[u] > 0)
+            wp[e] = exp(((double)bf16_bits_to_float(pre[e]) - (double)rmax[u]) * inv_T) * (1.0 / (double)rsum[u]);
     }
     __syncthreads();
     // (2) every node with children on its own
@@ -2035,9 +2092,18 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     const float c = (float)(1.4426950408889634 / (double)d->temperature);
     const int rows = d->B * d->N;
     float2 *run_tab = use_runs ? reinterpret_cast<float2 *>(ws) : nullptr;  // (behind the hand-over area; no nucleus arrays in this form)
-    if (!lazy) {
+    if (use_runs) {
+        int n_sm = 0;
+        const int rc_ = device_setup(nullptr, 0, &n_sm);
+        if (rc_ != SPECROLL_OK) return rc_;
+        const int resident = 8 * n_sm, n_runs = rows * RS_WARPS;  // (eight CTAs per SM)
+        int wpr = 8;
+        while (wpr > 1 && (long long)n_runs * wpr > (long long)resident * RS_WARPS) wpr >>= 1;
+        SR_CUDA_TRY(launch_dependent(true, run_stats_kernel, dim3((unsigned)(wpr == 1 ? rows : n_runs < resident ? n_runs : resident)), dim3(RS_THREADS), 0,
+                                     st, static_cast<const uint16_t *>(logits), d->V, c, n_runs, wpr, run_tab));
+    } else if (!lazy) {
         SR_CUDA_TRY(launch_dependent(true, row_stats_kernel, dim3((unsigned)rows), dim3(RS_THREADS), 0, st,
-                                     static_cast<const uint16_t *>(logits), d->V, c, row_max, row_sum, run_tab));
+                                     static_cast<const uint16_t *>(logits), d->V, c, row_max, row_sum));
     }
 
     WalkArgs wa;
@@ -2105,7 +2171,7 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     const int rc_ = device_setup(reinterpret_cast<const void *>(walk_term_kernel<false>), WT_SMEM_LIMIT, nullptr);
     if (rc_ != SPECROLL_OK) return rc_;
     SR_CUDA_TRY(launch_clusters(true, S, walk_term_kernel<false>, dim3((unsigned)(d->B * S)), dim3(WT_THREADS), L.total, st, wa, topo,
-                                u_fin, c, S, (const float2 *)run_tab, TileArgs{}));
+                                u_fin, c, S, (const float2 *)run_tab, row_max, row_sum, TileArgs{}));
     return SPECROLL_OK;
 }
 
@@ -2238,7 +2304,7 @@ extern "C" int specroll_verify_hidden(const specroll_verify_desc *d, int32_t dim
     if (rc != SPECROLL_OK) return rc;
     SR_CUDA_TRY(launch_clusters(true, S, walk_term_kernel<true>, dim3((unsigned)(d->B * S)), dim3(WT_THREADS), L.total,
                                 static_cast<cudaStream_t>(cuda_stream), wa, topo, u_fin, (float)(1.4426950408889634 / (double)d->temperature),
-                                S, (const float2 *)nullptr, tile));
+                                S, (const float2 *)nullptr, (float *)nullptr, (float *)nullptr, tile));
     return SPECROLL_OK;
 }
 

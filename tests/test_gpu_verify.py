@@ -208,3 +208,18 @@ def test_lazy_row_statistics_give_the_same_walk(name, B, V, T):
     same = (g["n_acc"] == o["n_acc"]) & (g["out_tok"] == o["out_tok"]).all(1)
     assert (same | (o["min_margin"] < NEAR_TIE) | (o["fin_margin"] < 1e-6)).all()
 
+
+
+@pytest.mark.parametrize("B,N,k,V", [(1, 8, 4, 151936), (18, 8, 4, 4104), (19, 8, 3, 4096), (37, 8, 2, 1032), (38, 8, 4, 40008), (75, 8, 8, 8),
+                                     (150, 8, 5, 4104), (3, 64, 8, 8200), (40, 40, 16, 2056), (5, 64, 32, 4104)])
+def test_runs_shared_by_warps_and_nodes_by_lane_groups(B, N, k, V):
+    """Eight, four, two warps or one per run of a row (by the number of rows), vocabularies that leave runs ragged or empty,
+    and 1 to 32 lanes per node with up to two nodes' rounds per warp."""
+    w = I.scaled(I.WORKLOADS["qwen7b"], B=B, N=N, V=V, k=min(k, V))
+    parent = I.topology(w)
+    cid, cl = I.synthetic_candidates(w)
+    d = ref.tree_draw(parent, np.zeros(w.B, np.int32), cid, cl, I.uniforms24(3 + B, (w.B, w.N)))
+    lg = I.target_logits(w, parent, d["tree_tok"], boost=4.0)
+    u_acc, u_fin = I.verify_uniforms(w)
+    o, g = run_both(w, parent, lg, d["tree_tok"], d["tree_cand"], cid, cl, u_acc, u_fin)
+    check(w, o, g, lg)
