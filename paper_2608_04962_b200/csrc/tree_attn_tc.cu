@@ -1155,25 +1155,24 @@ static int launch_tc(const AttnArgs &a, const TopoMask &mask, long long T_kv, in
 // Sums the chunks of every split sequence (the plan uses this instead of merging inside the attention kernel
 // when some sequence has many chunks: there the last chunk's CTA would sit on a long chain of dependent loads).
 // grid = (chunks in work order, Hkv * n_rb, D / 8); only the blocks of a split sequence's first chunk work: 128 rows x
-// 2 halves of the chunks, two float4 columns each.  What bounds it is round trips to L2, not bytes: the chunks of a
-// half are taken eight at a time with all their loads in flight, and the halves meet in shared memory (one thread per
-// row for all chunks, four at a time: 7.5 us between the end of the attention kernel and the end of this one for
-// 19 chunks).
+// MERGE_PARTS parts of the chunks, two float4 columns each.  What bounds it is round trips to L2, not bytes: a part's chunks
+// are taken eight at a time with all their loads in flight, references included (weights relative to the largest so far),
+// and the parts meet in shared memory.  Up to 32 chunks are one round trip.
 // Launched as a programmatic dependent of the attention kernel: its blocks are in place (on SMs that the attention
 // leaves idle or has finished on) when the partials are complete; nothing is read before.
+constexpr int MERGE_PARTS = 4;
 template <int D>
-__global__ void __launch_bounds__(256) attn_merge_tc_kernel(AttnArgs a) {
+__global__ void __launch_bounds__(128 * MERGE_PARTS) attn_merge_tc_kernel(AttnArgs a) {
     constexpr int STEP = 8;
-    __shared__ float sh_m[2][128];
-    __shared__ float4 sh_acc[2][128];
-    __shared__ float sh_l[128];
+    __shared__ float2 sh_ml[MERGE_PARTS][128];
+    __shared__ float4 sh_acc[2][MERGE_PARTS][128];
     pdl_launch_dependents();
     pdl_wait();
     const int4 e0 = __ldg(reinterpret_cast<const int4 *>(a.unit_tab) + 2 * (size_t)blockIdx.x);
     const int b = e0.x, n_splits = e0.z, item0 = e0.w;
     if (e0.y != 0 || n_splits < 2) return;
     const int hkv = blockIdx.y / a.n_rb, rb = blockIdx.y % a.n_rb;
-    const int row = threadIdx.x & 127, half = threadIdx.x >> 7;
+    const int row = threadIdx.x & 127, part = threadIdx.x >> 7;
     const int gr = rb * a.rows_per_block + row;
     const bool ok = row < a.rows_per_block && gr < a.rows;
     const int c4 = blockIdx.z * 2;  // first of this block's float4 columns
@@ -1181,36 +1180,31 @@ __global__ void __launch_bounds__(256) attn_merge_tc_kernel(AttnArgs a) {
     const float2 *ml = reinterpret_cast<const float2 *>(a.part_ml) + ((size_t)item0 * a.Hkv + hkv) * a.rows_pad + (ok ? gr : 0);
     const float4 *po = reinterpret_cast<const float4 *>(a.part_o) + ((size_t)item0 * a.Hkv + hkv) * (size_t)(D / 4) * a.rows_pad +
                        (size_t)c4 * a.rows_pad + (ok ? gr : 0);
-    // this thread's chunks: half, half + 2, ...
-    const int n_mine = (n_splits - half + 1) / 2;
-    float Mx = -INFINITY;
-#pragma unroll 1
-    for (int i0 = 0; i0 < n_mine; i0 += STEP) {
-        float v[STEP];
-#pragma unroll
-        for (int i = 0; i < STEP; ++i) v[i] = i0 + i < n_mine ? __ldcg(&ml[(size_t)(half + 2 * (i0 + i)) * unit_ml].x) : -INFINITY;
-#pragma unroll
-        for (int i = 0; i < STEP; ++i) Mx = fmaxf(Mx, v[i]);
-    }
-    sh_m[half][row] = Mx;
-    __syncthreads();
-    Mx = fmaxf(sh_m[0][row], sh_m[1][row]);
-    float lsum = 0.f;
+    // this thread's chunks: part, part + MERGE_PARTS, ...; a batch's weights are relative to the largest reference so far
+    float Mx = -INFINITY, lsum = 0.f;
     float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
 #pragma unroll 1
-    for (int i0 = 0; i0 < n_mine; i0 += STEP) {
+    for (int i0 = part; i0 < n_splits; i0 += STEP * MERGE_PARTS) {
         float2 v[STEP];
         float4 x[STEP][2];
 #pragma unroll
         for (int i = 0; i < STEP; ++i) {
-            const size_t s = (size_t)(half + 2 * min(i0 + i, n_mine - 1));  // (a chunk beyond the last: weight zero below)
+            const size_t s = (size_t)min(i0 + i * MERGE_PARTS, n_splits - 1);  // (a chunk beyond the last: weight zero below)
             v[i] = __ldcg(&ml[s * unit_ml]);
 #pragma unroll
             for (int c = 0; c < 2; ++c) x[i][c] = __ldcg(po + s * unit_o + (size_t)c * a.rows_pad);
         }
+        float mx = Mx;
+#pragma unroll
+        for (int i = 0; i < STEP; ++i) mx = fmaxf(mx, v[i].x);  // (the copies of the last chunk change nothing)
+        const float f = Mx == -INFINITY ? 0.f : ex2_approx(Mx - mx);
+        Mx = mx;
+        lsum *= f;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) acc[c] = make_float4(acc[c].x * f, acc[c].y * f, acc[c].z * f, acc[c].w * f);
 #pragma unroll
         for (int i = 0; i < STEP; ++i) {
-            const float wgt = (i0 + i >= n_mine || v[i].x == -INFINITY) ? 0.f : ex2_approx(v[i].x - Mx);
+            const float wgt = (i0 + i * MERGE_PARTS >= n_splits || v[i].x == -INFINITY) ? 0.f : ex2_approx(v[i].x - Mx);
             lsum += wgt * v[i].y;
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -1221,22 +1215,29 @@ __global__ void __launch_bounds__(256) attn_merge_tc_kernel(AttnArgs a) {
             }
         }
     }
-    if (half == 1) {
-        sh_acc[0][row] = acc[0];
-        sh_acc[1][row] = acc[1];
-        sh_l[row] = lsum;
-    }
+    sh_ml[part][row] = make_float2(Mx, lsum);
+    sh_acc[0][part][row] = acc[0];
+    sh_acc[1][part][row] = acc[1];
     __syncthreads();
-    if (half == 1 || !ok) return;
+    if (part != 0 || !ok) return;
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        const float4 y = sh_acc[c][row];
-        acc[c].x += y.x;
-        acc[c].y += y.y;
-        acc[c].z += y.z;
-        acc[c].w += y.w;
+    for (int q = 1; q < MERGE_PARTS; ++q) Mx = fmaxf(Mx, sh_ml[q][row].x);
+    lsum = 0.f;
+    acc[0] = acc[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < MERGE_PARTS; ++q) {
+        const float2 e = sh_ml[q][row];
+        const float wgt = e.x == -INFINITY ? 0.f : ex2_approx(e.x - Mx);
+        lsum += wgt * e.y;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const float4 y = sh_acc[c][q][row];
+            acc[c].x += wgt * y.x;
+            acc[c].y += wgt * y.y;
+            acc[c].z += wgt * y.z;
+            acc[c].w += wgt * y.w;
+        }
     }
-    lsum += sh_l[row];
     const float inv = lsum > 0.f ? 1.0f / lsum : 0.f;
     const int n = gr / a.G, g = gr % a.G;
     uint4 q;
@@ -1250,7 +1251,7 @@ __global__ void __launch_bounds__(256) attn_merge_tc_kernel(AttnArgs a) {
 
 int launch_attn_merge_tc(const AttnArgs &a, int D, int items, cudaStream_t st) {
     const dim3 grid((unsigned)items, (unsigned)(a.Hkv * a.n_rb), (unsigned)(D / 8));
-    SR_CUDA_TRY(launch_dependent(!a.no_pdl, D == 128 ? attn_merge_tc_kernel<128> : attn_merge_tc_kernel<64>, grid, dim3(256), 0, st, a));
+    SR_CUDA_TRY(launch_dependent(!a.no_pdl, D == 128 ? attn_merge_tc_kernel<128> : attn_merge_tc_kernel<64>, grid, dim3(128 * MERGE_PARTS), 0, st, a));
     return SPECROLL_OK;
 }
 

@@ -138,38 +138,47 @@ run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs
     }
 }
 
+// The rows' own pairs; n_cta > 1: a cluster of n_cta CTAs per row (few rows), each with every n_cta-th group of every run.
 __global__ void __launch_bounds__(RS_THREADS, 8)
-row_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, float *__restrict__ row_max,
+row_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_cta, float *__restrict__ row_max,
                  float *__restrict__ row_sum) {
     pdl_wait();  // (as in run_stats_kernel)
     pdl_launch_dependents();
-    const size_t row = blockIdx.x;
-    const uint4 *p = reinterpret_cast<const uint4 *>(logits + row * (size_t)V);
+    __shared__ float2 sh[RS_WARPS];
+    const size_t row = blockIdx.x / n_cta;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = n_cta > 1 ? (int)cluster_ctarank() : 0;
     const int nvec = V >> 3;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int v_lo, v_hi;
     rs_run(nvec, warp, &v_lo, &v_hi);
     float m, s;
-    run_stats(p, nvec, v_lo, v_hi, 0, 1, lane, c, m, s);
-
-    // block reduction of (m, s)
-    __shared__ float sm_m[RS_THREADS / 32], sm_s[RS_THREADS / 32];
-    if (lane == 0) {
-        sm_m[warp] = m;
-        sm_s[warp] = s;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        float m2 = lane < RS_THREADS / 32 ? sm_m[lane] : NEG_INF;
-        float s2 = lane < RS_THREADS / 32 ? sm_s[lane] : 0.f;
-        float mb = warp_max(m2);
-        s2 = (m2 == NEG_INF) ? 0.f : s2 * ex2_approx((m2 - mb) * c);
-        s2 = warp_sum(s2);
+    run_stats(reinterpret_cast<const uint4 *>(logits + row * (size_t)V), nvec, v_lo, v_hi, rank, n_cta, lane, c, m, s);
+    if (lane == 0) sh[warp] = make_float2(m, s);
+    if (n_cta > 1)
+        cluster_sync_all();
+    else
+        __syncthreads();
+    if (rank == 0 && warp == 0) {
+        float mb = NEG_INF, sb = 0.f;
+        for (int w0 = 0; w0 < RS_WARPS * n_cta; w0 += 32) {
+            const int w = w0 + lane;
+            float2 e = make_float2(NEG_INF, 0.f);
+            if (w < RS_WARPS) {
+                e = sh[w];
+            } else if (w < RS_WARPS * n_cta) {
+                const double d = ld_dsmem_f64(sh + w % RS_WARPS, w / RS_WARPS);
+                e = make_float2(__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d)));
+            }
+            const float mn = fmaxf(mb, warp_max(e.x));
+            const float part = warp_sum(e.x == NEG_INF ? 0.f : e.y * ex2_approx((e.x - mn) * c));
+            sb = (mb == NEG_INF ? 0.f : sb * ex2_approx((mb - mn) * c)) + part;
+            mb = mn;
+        }
         if (lane == 0) {
             row_max[row] = mb;
-            row_sum[row] = s2;
+            row_sum[row] = sb;
         }
     }
+    if (n_cta > 1) cluster_sync_all();  // (a CTA's pairs stay until they have been read)
 }
 
 // ------------------------------------------------------------------------------ nucleus threshold
@@ -2092,18 +2101,21 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     const float c = (float)(1.4426950408889634 / (double)d->temperature);
     const int rows = d->B * d->N;
     float2 *run_tab = use_runs ? reinterpret_cast<float2 *>(ws) : nullptr;  // (behind the hand-over area; no nucleus arrays in this form)
+    int n_sm = 0;
+    const int rc_sm = device_setup(nullptr, 0, &n_sm);
+    if (rc_sm != SPECROLL_OK) return rc_sm;
+    const int resident = 8 * n_sm;  // CTAs of the statistics kernels
     if (use_runs) {
-        int n_sm = 0;
-        const int rc_ = device_setup(nullptr, 0, &n_sm);
-        if (rc_ != SPECROLL_OK) return rc_;
-        const int resident = 8 * n_sm, n_runs = rows * RS_WARPS;  // (eight CTAs per SM)
+        const int n_runs = rows * RS_WARPS;
         int wpr = 8;
         while (wpr > 1 && (long long)n_runs * wpr > (long long)resident * RS_WARPS) wpr >>= 1;
         SR_CUDA_TRY(launch_dependent(true, run_stats_kernel, dim3((unsigned)(wpr == 1 ? rows : n_runs < resident ? n_runs : resident)), dim3(RS_THREADS), 0,
                                      st, static_cast<const uint16_t *>(logits), d->V, c, n_runs, wpr, run_tab));
     } else if (!lazy) {
-        SR_CUDA_TRY(launch_dependent(true, row_stats_kernel, dim3((unsigned)rows), dim3(RS_THREADS), 0, st,
-                                     static_cast<const uint16_t *>(logits), d->V, c, row_max, row_sum));
+        int n_cta = 8;
+        while (n_cta > 1 && (long long)rows * n_cta > resident) n_cta >>= 1;
+        SR_CUDA_TRY(launch_clusters(true, n_cta, row_stats_kernel, dim3((unsigned)(rows * n_cta)), dim3(RS_THREADS), 0, st,
+                                    static_cast<const uint16_t *>(logits), d->V, c, n_cta, row_max, row_sum));
     }
 
     WalkArgs wa;
