@@ -183,6 +183,11 @@ __device__ __forceinline__ uint32_t ld_dsmem_u32(const void *own_smem_ptr, uint3
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
     return v;
 }
+__device__ __forceinline__ void st_dsmem_u32(const void *own_smem_ptr, uint32_t cta_rank, uint32_t v) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(own_smem_ptr)), "r"(cta_rank));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
+}
 __device__ __forceinline__ double ld_dsmem_f64(const void *own_smem_ptr, uint32_t cta_rank) {
     uint32_t remote;
     double v;

@@ -262,22 +262,31 @@ target_head_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     }
 }
 
-// row_max = max over the ranges, row_sum = sum of the ranges' sums brought to that maximum
-__global__ void target_head_merge_kernel(const float *__restrict__ pm, const float *__restrict__ ps, int M, int n_groups,
-                                         float c_log2, float *__restrict__ row_max, float *__restrict__ row_sum) {
+// row_max = max over the ranges, row_sum = sum of the ranges' sums brought to that maximum: a warp per row (a thread per row
+// took 12 us where the projection has 148 ranges)
+__global__ void __launch_bounds__(256) target_head_merge_kernel(const float *__restrict__ pm, const float *__restrict__ ps, int M,
+                                                                int n_groups, float c_log2, float *__restrict__ row_max,
+                                                                float *__restrict__ row_sum) {
     pdl_wait();
     pdl_launch_dependents();  // (what follows reads the projection's other results ahead of its own wait)
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (r >= M) return;
-    float m = -INFINITY;
-    for (int g = 0; g < n_groups; ++g) m = fmaxf(m, pm[(size_t)r * n_groups + g]);
-    float s = 0.f;
-    for (int g = 0; g < n_groups; ++g) {
-        const float mg = pm[(size_t)r * n_groups + g];
-        if (mg > -INFINITY) s += ps[(size_t)r * n_groups + g] * ex2_approx((mg - m) * c_log2);
+    float m = -INFINITY, s = 0.f;
+#pragma unroll 4
+    for (int g = lane; g < n_groups; g += 32) {
+        const float mg = pm[(size_t)r * n_groups + g], sg = ps[(size_t)r * n_groups + g];
+        if (mg > -INFINITY) {
+            const float mn = fmaxf(m, mg);
+            s = s * ex2_approx((m - mn) * c_log2) + sg * ex2_approx((mg - mn) * c_log2);
+            m = mn;
+        }
     }
-    row_max[r] = m;
-    row_sum[r] = s;
+    const float mw = warp_max(m);
+    s = warp_sum(m > -INFINITY ? s * ex2_approx((m - mw) * c_log2) : 0.f);
+    if (lane == 0) {
+        row_max[r] = mw;
+        row_sum[r] = s;
+    }
 }
 
 }  // namespace specroll
@@ -369,7 +378,7 @@ extern "C" int specroll_target_head_stats_tiles(int32_t R, int32_t d, int32_t V,
         tmA, tmB, R, V, d, p.n_mblocks, p.n_groups, p.tiles_per_group, c_log2, want_id, kw, pm, ps,
         static_cast<uint16_t *>(want_logit), nullptr, status, static_cast<float2 *>(tile_mass));
     SR_LAUNCH_CHECK();
-    SR_CUDA_TRY(launch_dependent(true, target_head_merge_kernel, dim3((unsigned)(R + 63) / 64), dim3(64), 0, st, (const float *)pm,
+    SR_CUDA_TRY(launch_dependent(true, target_head_merge_kernel, dim3((unsigned)(R + 7) / 8), dim3(256), 0, st, (const float *)pm,
                                  (const float *)ps, R, p.n_groups, c_log2, row_max, row_sum));
     return SPECROLL_OK;
 }

@@ -340,19 +340,17 @@ __device__ __forceinline__ int nucleus_place(uint32_t bits) {
 __device__ __forceinline__ uint32_t nucleus_value(int r) {  // (bf16 bits; the counter around zero: 0)
     return r < NUC_ZERO ? (uint32_t)(NUC_ZERO - r + NUC_OCT_LO) : r > NUC_ZERO ? (uint32_t)(r - NUC_ZERO + NUC_OCT_LO) | 0x8000u : 0u;
 }
-__device__ __forceinline__ uint32_t nucleus_count_at(const NucleusSmem *st, int r, int n_cta) {
+__device__ __forceinline__ uint32_t nucleus_count_at(const NucleusSmem *st, int r) {
     const int at = r <= NUC_ZERO ? NUC_ZERO - r : NUC_SIGN + r - NUC_ZERO;
-    uint32_t n = st->count[at] + (r == NUC_ZERO ? st->count[NUC_SIGN] : 0u);
-    for (int k = 1; k < n_cta; ++k) n += ld_dsmem_u32(st->count + at, k) + (r == NUC_ZERO ? ld_dsmem_u32(st->count + NUC_SIGN, k) : 0u);
-    return n;
+    return st->count[at] + (r == NUC_ZERO ? st->count[NUC_SIGN] : 0u);
 }
 
 // The first place of [r0, r1] at which the mass from r0 on reaches the target, by all threads of a CTA.  Result in
 // st->last (-1: not reached) and st->keep.
-__device__ void nucleus_scan(NucleusSmem *st, int r0, int r1, double target, float M, float c, int n_cta) {
+__device__ void nucleus_scan(NucleusSmem *st, int r0, int r1, double target, float M, float c) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     auto mass_at = [&](int r) {
-        const uint32_t n = nucleus_count_at(st, r, n_cta);
+        const uint32_t n = nucleus_count_at(st, r);
         return (float)n * ex2_approx(fmaf(bf16_bits_to_float(nucleus_value(r)), c, -M * c));  // (an empty counter's value is finite)
     };
     const int per = (r1 - r0 + NUC_THREADS) / NUC_THREADS;  // (<= 14)
@@ -443,20 +441,36 @@ __device__ void nucleus_row(const uint16_t *__restrict__ row_logits, int V, floa
         for (int q = 0; q < 3; ++q)
             if (i + q * step < nvec) count8(v[q]);
     }
+    const int r0 = nucleus_place(__float_as_uint(M) >> 16), r1 = nucleus_place(lo_bits);
     if (n_cta > 1) {
+        cluster_sync_all();
+        // The CTAs' counts into the first CTA's tables, the places spread over the cluster's threads: a counter is read and
+        // written by one thread, all its copies in flight together.  (The first CTA adding them up as it scanned, one
+        // round trip after the other, took 30 us.)
+        auto add_up = [&](uint32_t *at) {
+            uint32_t v[8], n = 0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = k < n_cta ? ld_dsmem_u32(at, k) : 0u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) n += v[k];
+            st_dsmem_u32(at, 0, n);
+        };
+        for (int r = r0 + rank * NUC_THREADS + tid; r <= r1; r += n_cta * NUC_THREADS) {
+            add_up(st->count + (r <= NUC_ZERO ? NUC_ZERO - r : NUC_SIGN + r - NUC_ZERO));
+            if (r == NUC_ZERO) add_up(st->count + NUC_SIGN);
+        }
         cluster_sync_all();
         if (rank != 0) return;
     } else {
         __syncthreads();
     }
-    const int r0 = nucleus_place(__float_as_uint(M) >> 16), r1 = nucleus_place(lo_bits);
-    nucleus_scan(st, r0, r1, (double)target, M, c, n_cta);
+    nucleus_scan(st, r0, r1, (double)target, M, c);
     const int last = st->last;
     // The counter around zero: it must not be the cut, and its values must not differ by more than their mass's rounding
     // if it lies above the cut.
     bool ok = last >= 0 && last != NUC_ZERO;
     if (ok && last > NUC_ZERO && r0 <= NUC_ZERO) {
-        const double m0 = (double)nucleus_count_at(st, NUC_ZERO, n_cta) * (double)ex2_approx(-M * c);
+        const double m0 = (double)nucleus_count_at(st, NUC_ZERO) * (double)ex2_approx(-M * c);
         ok = m0 * (double)(c * 0.6931472f) * 0x1p-13 <= 0x1p-24 * (double)S;
     }
     if (ok) {
