@@ -80,12 +80,21 @@ head_mlp_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    // The weights were there before the call (its first kernel starts when all work in front of it is complete): the first
+    // stages' tiles are loaded while the LayerNorm is still running, its outputs follow the wait.
+    const int w_row = hd * d + o0;  // rows of A viewed as [K * d, d]
+    if (threadIdx.x == 0)
+        for (int kb = 0; kb < min(STAGES, KB); ++kb) {
+            mbar_arrive_expect_tx(full_bar(kb), C::STAGE_BYTES);
+#pragma unroll
+            for (int bx = 0; bx < NBOX; ++bx)
+                tma_load_2d(base + kb * C::STAGE_BYTES + bx * W_BYTES, &tmW, (kb * NBOX + bx) * BK, w_row, full_bar(kb));
+        }
     pdl_wait();  // set up under the tail of the kernel before; its outputs are read from here on
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
-            const int w_row = hd * d + o0;                  // rows of A viewed as [K * d, d]
             const int x_row = (KX > 1 ? hd * B : 0) + b0;   // rows of xhat viewed as [KX * B, d]
             bool ok = true;
             int kb = 0;
@@ -96,10 +105,10 @@ head_mlp_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                     break;
                 }
                 const uint32_t sw = base + stage * C::STAGE_BYTES, sx = sw + NBOX * W_BYTES;
-                mbar_arrive_expect_tx(full_bar(stage), C::STAGE_BYTES);
+                if (kb >= STAGES) mbar_arrive_expect_tx(full_bar(stage), C::STAGE_BYTES);
 #pragma unroll
                 for (int bx = 0; bx < NBOX; ++bx) {
-                    tma_load_2d(sw + bx * W_BYTES, &tmW, (kb * NBOX + bx) * BK, w_row, full_bar(stage));
+                    if (kb >= STAGES) tma_load_2d(sw + bx * W_BYTES, &tmW, (kb * NBOX + bx) * BK, w_row, full_bar(stage));
                     tma_load_2d(sx + bx * C::X_BYTES, &tmX, (kb * NBOX + bx) * BK, x_row, full_bar(stage));
                 }
             }

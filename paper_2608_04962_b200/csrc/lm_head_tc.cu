@@ -116,6 +116,16 @@ lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    // The weights do not come from the kernels before this one in the call, which the first of them starts only when all
+    // work in front of the call is complete: the first stages' W tiles are loaded while the heads' outputs are still being made; Zt follows the
+    // wait.  (Asking L2 for the next 16 or 40 tiles as well made the call slower, 128 -> 133 / 148 us for two sequences.)
+    const int pre = min(STAGES, (t_hi - t_lo) * KB);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < pre; ++i) {
+            mbar_arrive_expect_tx(full_bar(i), STAGE_BYTES);
+            tma_load_2d(base + i * STAGE_BYTES + A_BYTES, &tmB, (i % KB) * BK, (t_lo + i / KB) * BN, full_bar(i));
+        }
+    }
     pdl_wait();  // set up under the tail of the kernel before; its outputs are read from here on
 
     if (warp == 0) {
@@ -134,9 +144,10 @@ lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                         break;
                     }
                     const uint32_t sa = base + stage * STAGE_BYTES, sb = sa + A_BYTES;
-                    mbar_arrive_expect_tx(full_bar(stage), STAGE_BYTES);
+                    const bool ahead = (tile - t_lo) * KB + kb < pre;  // (its W tile is on its way)
+                    if (!ahead) mbar_arrive_expect_tx(full_bar(stage), STAGE_BYTES);
                     tma_load_2d(sa, &tmA, kb * BK, m0, full_bar(stage));
-                    tma_load_2d(sb, &tmB, kb * BK, tile * BN, full_bar(stage));
+                    if (!ahead) tma_load_2d(sb, &tmB, kb * BK, tile * BN, full_bar(stage));
                     issued[stage] = (int)phase;
                     if (++stage == STAGES) {
                         stage = 0;

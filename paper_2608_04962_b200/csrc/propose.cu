@@ -28,12 +28,13 @@ constexpr int LN_THREADS = 256;
 __global__ void __launch_bounds__(LN_THREADS)
 layernorm_kernel(const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__restrict__ gamma,
                  const __nv_bfloat16 *__restrict__ beta, __nv_bfloat16 *__restrict__ xhat, int B, int d,
-                 int KX, float eps) {
+                 int KX, float eps, int32_t *__restrict__ status) {
     extern __shared__ float row[];  // d floats
     __shared__ float red[LN_THREADS / 32];
     pdl_launch_dependents();
     pdl_wait();
     const int b = blockIdx.x;
+    if (b == 0 && threadIdx.x == 0) *status = 0;  // (of the call; a kernel behind this one may set it)
     float s = 0.f;
     for (int i = threadIdx.x; i < d; i += LN_THREADS) {
         const float v = __bfloat162float(h[(size_t)b * d + i]);
@@ -676,7 +677,6 @@ extern "C" int specroll_propose(const specroll_propose_desc *d, const void *h, c
     const __nv_bfloat16 *hb = static_cast<const __nv_bfloat16 *>(h);
     const int B = d->B, K = d->K, dd = d->d, k = d->k, V = d->V;
     int32_t *status = reinterpret_cast<int32_t *>(ws + p.off_status);
-    SR_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int32_t), st));
     const bool pre_head = (d->flags & SPECROLL_REFLEX_PRE_HEAD) != 0;
     if (pre_head) {
         // the correction moves the hidden state itself (m [B, d], alpha [B]); everything after it reads the
@@ -692,7 +692,7 @@ extern "C" int specroll_propose(const specroll_propose_desc *d, const void *h, c
     // completion before it touches global memory.
     SR_CUDA_TRY(launch_dependent(pre_head, layernorm_kernel, dim3(B), dim3(LN_THREADS), dd * sizeof(float), st, hb,
                                  static_cast<const __nv_bfloat16 *>(ln_gamma), static_cast<const __nv_bfloat16 *>(ln_beta),
-                                 xhat, B, dd, p.KX, d->ln_eps));
+                                 xhat, B, dd, p.KX, d->ln_eps, status));
 
     if (!(d->flags & SPECROLL_PROPOSE_LEGACY_MMA)) {
         int rc = launch_head_mlp_tc(xhat, p.KX, A, bias, hb, z, B, K, dd, status, st);
