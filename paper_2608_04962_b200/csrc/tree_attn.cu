@@ -519,6 +519,7 @@ static long long estimate_makespan(const std::vector<int> &tiles, int ct, int co
 
 struct AttnPlan {
     int rows, n_rb, rows_per_block, rows_pad, chunk_tiles, items, tile_tokens, nodes_per_block, n_counters;
+    int max_splits;  // chunks of the longest sequence
     int merge_mode;  // tcgen05 path: 0 = split sequences are merged inside the attention kernel, 2 = by a kernel after it
     bool use_tc;
     size_t off_status, off_items, off_sorted, off_rank, off_tab, off_counters, off_po, off_pml, off_hand, total;
@@ -610,6 +611,7 @@ static int compute_attn_plan(const specroll_attn_desc *d, const int32_t *indptr_
     }
     p->items = items;
     if (max_tiles / p->chunk_tiles + 1 > 65535) return SPECROLL_EINVAL;
+    p->max_splits = (max_tiles + p->chunk_tiles - 1) / p->chunk_tiles;
     p->merge_mode = (p->use_tc && merge_by_kernel((long long)items * ctas_per_tile, (max_tiles + p->chunk_tiles - 1) / p->chunk_tiles)) ? 2 : 0;
     if (p->use_tc && items == d->B) p->merge_mode = 2;  // (nothing is split: nothing is merged anywhere)
     p->n_counters = 64 + d->B * d->Hkv * p->n_rb;  // [0]: work counter, [1]: CTAs that have left; [64 ...]: per (b, hkv, rb) arrivals
@@ -786,7 +788,7 @@ static int run_tree_attn(const specroll_attn_desc *d, const void *Q, const void 
     if (p.use_tc) {
         const int rc = launch_attn_tc(a, mask, d->D, T_kv, status, st);
         if (rc != SPECROLL_OK || p.merge_mode != 2 || p.items <= d->B) return rc;
-        return launch_attn_merge_tc(a, d->D, p.items, st);
+        return launch_attn_merge_tc(a, d->D, p.items, p.max_splits, st);
     }
     if (d->D == 128) return launch_attn<128>(a, mask, p, d->Hkv, n_out, st);
     return launch_attn<64>(a, mask, p, d->Hkv, n_out, st);

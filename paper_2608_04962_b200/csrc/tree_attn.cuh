@@ -38,7 +38,8 @@ constexpr int ATTN_HAND_CTAS = 256;  // CTAs the hand-over area is sized for (th
 
 // tcgen05 kernel (tree_attn_tc.cu).  T_kv = total cached tokens.  Launches the main kernel only.
 int launch_attn_tc(const AttnArgs &a, const TopoMask &mask, int D, long long T_kv, int32_t *status, cudaStream_t st);
-// Merges the chunks of split sequences after launch_attn_tc when a.merge_mode == 2.  items = chunks in the plan.
-int launch_attn_merge_tc(const AttnArgs &a, int D, int items, cudaStream_t st);
+// Merges the chunks of split sequences after launch_attn_tc when a.merge_mode == 2.  items = chunks in the plan, max_splits = those of
+// the longest sequence.
+int launch_attn_merge_tc(const AttnArgs &a, int D, int items, int max_splits, cudaStream_t st);
 
 }  // namespace specroll

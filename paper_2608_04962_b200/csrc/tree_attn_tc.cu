@@ -1157,20 +1157,24 @@ static int launch_tc(const AttnArgs &a, const TopoMask &mask, long long T_kv, in
 // grid = (chunks in work order, Hkv * n_rb, D / 8); only the blocks of a split sequence's first chunk work: 128 rows x
 // MERGE_PARTS parts of the chunks, two float4 columns each.  What bounds it is round trips to L2, not bytes: a part's chunks
 // are taken eight at a time with all their loads in flight, references included (weights relative to the largest so far),
-// and the parts meet in shared memory.  Up to 32 chunks are one round trip.
+// and the parts meet in shared memory.  One part per eight chunks of the longest sequence, up to four: one round trip up to
+// 32 chunks, and no idle threads where a launch has many blocks (16 sequences of few chunks each lost 5 % of the layer to
+// them).
 // Launched as a programmatic dependent of the attention kernel: its blocks are in place (on SMs that the attention
 // leaves idle or has finished on) when the partials are complete; nothing is read before.
-constexpr int MERGE_PARTS = 4;
-template <int D>
+template <int D, int MERGE_PARTS>
 __global__ void __launch_bounds__(128 * MERGE_PARTS) attn_merge_tc_kernel(AttnArgs a) {
     constexpr int STEP = 8;
     __shared__ float2 sh_ml[MERGE_PARTS][128];
     __shared__ float4 sh_acc[2][MERGE_PARTS][128];
     pdl_launch_dependents();
-    pdl_wait();
-    const int4 e0 = __ldg(reinterpret_cast<const int4 *>(a.unit_tab) + 2 * (size_t)blockIdx.x);
+    // The plan is complete when this block starts: the attention kernel lets it start only behind a wait for a plan that
+    // was being made.  Reading it ahead of the wait for the partials, all blocks but those of first chunks leave at once
+    // (19 of 20 blocks otherwise hold the places of the ones that work until the partials are there).
+    const int4 e0 = __ldcg(reinterpret_cast<const int4 *>(a.unit_tab) + 2 * (size_t)blockIdx.x);
     const int b = e0.x, n_splits = e0.z, item0 = e0.w;
     if (e0.y != 0 || n_splits < 2) return;
+    pdl_wait();
     const int hkv = blockIdx.y / a.n_rb, rb = blockIdx.y % a.n_rb;
     const int row = threadIdx.x & 127, part = threadIdx.x >> 7;
     const int gr = rb * a.rows_per_block + row;
@@ -1249,9 +1253,12 @@ __global__ void __launch_bounds__(128 * MERGE_PARTS) attn_merge_tc_kernel(AttnAr
     if (a.lse && c4 == 0) a.lse[((size_t)b * a.N + n) * a.Hq + hkv * a.G + g] = (Mx + log2f(lsum)) * 0.6931471805599453f;
 }
 
-int launch_attn_merge_tc(const AttnArgs &a, int D, int items, cudaStream_t st) {
+int launch_attn_merge_tc(const AttnArgs &a, int D, int items, int max_splits, cudaStream_t st) {
     const dim3 grid((unsigned)items, (unsigned)(a.Hkv * a.n_rb), (unsigned)(D / 8));
-    SR_CUDA_TRY(launch_dependent(!a.no_pdl, D == 128 ? attn_merge_tc_kernel<128> : attn_merge_tc_kernel<64>, grid, dim3(128 * MERGE_PARTS), 0, st, a));
+    const int parts = max_splits > 16 ? 4 : max_splits > 8 ? 2 : 1;
+    auto *const kern = D == 128 ? (parts == 4 ? attn_merge_tc_kernel<128, 4> : parts == 2 ? attn_merge_tc_kernel<128, 2> : attn_merge_tc_kernel<128, 1>)
+                                : (parts == 4 ? attn_merge_tc_kernel<64, 4> : parts == 2 ? attn_merge_tc_kernel<64, 2> : attn_merge_tc_kernel<64, 1>);
+    SR_CUDA_TRY(launch_dependent(!a.no_pdl, kern, grid, dim3(128 * parts), 0, st, a));
     return SPECROLL_OK;
 }
 
