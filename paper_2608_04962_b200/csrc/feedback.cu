@@ -580,12 +580,6 @@ static int fbv_rows(int R, int d, int n_sm) {
     return std::max(1, std::min(8, bytes / (d * 2)));
 }
 
-__device__ __forceinline__ void fbv_bulk_row(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-
 template <int NV>
 __global__ void __launch_bounds__(NV == 1 ? 256 : FBV_THREADS, NV == 1 ? 6 : (NV == 2 ? 2 : 1)) feedback_vec_kernel(FeedbackArgs a) {
     using namespace fb;
@@ -611,7 +605,7 @@ __global__ void __launch_bounds__(NV == 1 ? 256 : FBV_THREADS, NV == 1 ? 6 : (NV
         mbar_arrive_expect_tx(bar, (uint32_t)rows * row_bytes);
         const uint32_t dst = smem_u32(fb_stage + (size_t)s * stage_bytes);
         for (int q = 0; q < rows; ++q)
-            fbv_bulk_row(dst + (uint32_t)q * row_bytes, a.W + (size_t)sm.id[batch * rps + q] * d, row_bytes, bar);
+            bulk_load(dst + (uint32_t)q * row_bytes, a.W + (size_t)sm.id[batch * rps + q] * d, row_bytes, bar);
     };
     pdl_wait();
     pdl_launch_dependents();

@@ -373,7 +373,7 @@ extern "C" int specroll_target_head_stats_tiles(int32_t R, int32_t d, int32_t V,
     rc = make_tmap_2d_bf16(&tmB, W, (uint64_t)V, (uint64_t)d, (uint64_t)d, BN);
     if (rc != SPECROLL_OK) return rc;
     if ((rc = device_setup(reinterpret_cast<const void *>(target_head_tc_kernel<false>), SMEM_BYTES, nullptr)) != SPECROLL_OK) return rc;
-    const float c_log2 = 1.4426950408889634f / temperature;
+    const float c_log2 = (float)(1.4426950408889634 / (double)temperature);  // (the verification's)
     target_head_tc_kernel<false><<<p.n_mblocks * p.n_groups, THREADS, SMEM_BYTES, st>>>(
         tmA, tmB, R, V, d, p.n_mblocks, p.n_groups, p.tiles_per_group, c_log2, want_id, kw, pm, ps,
         static_cast<uint16_t *>(want_logit), nullptr, status, static_cast<float2 *>(tile_mass));

@@ -2,9 +2,8 @@
 // accept / resample walk, and the terminal (fallback or bonus) draw.
 //
 // Two launches per plain call:
-//   run_stats_kernel    streams the bf16 logits once with 128-bit loads, an online (max, sum-exp) pair
-//                       per thread, and leaves the pair of every eighth of every (sequence, node) row
-//                       (row_stats_kernel: one CTA per row, for the forms that read the rows' own pairs).
+//   row_stats_kernel    (few rows: run_stats_kernel) streams the bf16 logits once, an online (max, sum-exp)
+//                       pair per thread, and leaves the pair of every eighth of every (sequence, node) row.
 //   walk_term_kernel    one CTA (or cluster) per sequence, launched to overlap the tail of the
 //                       statistics kernel: the walk, then the terminal draw.  The residual of the
 //                       walk differs from p only on the <= k candidates of the current node (the
@@ -20,6 +19,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "tc05.cuh"
 
 namespace specroll {
 
@@ -55,6 +55,32 @@ __device__ __forceinline__ void online_update(const uint4 &v, float c, float &m,
 #pragma unroll
     for (int i = 0; i < 8; ++i) acc += ex2_approx(fmaf(x[i], c, nmc));
     s += acc;
+}
+
+// Four vectors in turn with the same result to the last bit, for a warp that has its scheduler to itself: the four sums of
+// exponentials are independent of one another once the maxima are known, and nothing branches.
+__device__ __forceinline__ void online_update4(const uint4 (&v)[4], float c, float &m, float &nmc, float &s) {
+    float f[4], acc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint32_t w[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+        float x[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            x[2 * i] = __uint_as_float(w[i] << 16);
+            x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+        }
+        const float vm = fmaxf(fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3])), fmaxf(fmaxf(x[4], x[5]), fmaxf(x[6], x[7])));
+        const bool up = vm > m;
+        f[q] = up ? ex2_approx((m - vm) * c) : 1.f;
+        nmc = up ? -vm * c : nmc;
+        m = up ? vm : m;
+        acc[q] = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[q] += ex2_approx(fmaf(x[i], c, nmc));
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s = __fadd_rn(__fmul_rn(s, f[q]), acc[q]);
 }
 
 // logits[rows, V] bf16; c = log2(e) / T.  row_max = max_v l_v, row_sum = sum_v exp((l_v - max)/T).
@@ -101,47 +127,107 @@ __device__ __forceinline__ void run_stats(const uint4 *__restrict__ p, int nvec,
 
 // run_tab: [rows][RS_WARPS] (m, s) of every run of every row, s = sum over the run of exp((l - m)/T).  The kernel that
 // walks adds a row's pairs up; the terminal draw finds the eighth of the row that holds its target from them and reads
-// only that.  A CTA takes the eight runs of a row; where there are fewer runs than resident warps, a run is shared by
-// wpr = 2, 4 or 8 warps of a CTA, and the runs are spread over more CTAs (a run of one warp is 19 dependent rounds of
-// loads: 20 rows of 151936 tokens 19 us, so 6).
-__global__ void __launch_bounds__(RS_THREADS, 8)
-run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs, int wpr, float2 *__restrict__ run_tab) {
+// only that.  This is the form for few rows: one warp per CTA, which takes the runs blockIdx, blockIdx + grid, ... through a
+// ring of bulk copies, 20 KB in flight per warp (with its loads in registers a warp has 2 KB, so a run is 19 dependent
+// rounds however empty the machine), ten CTAs per SM.  The terms of a lane's sum keep the order that the CTA-per-row form
+// (row_stats_kernel) gives them: the terminal draw follows the last bits of the runs' sums.
+constexpr int RUN_PIECE = 256, RUN_RING = 5;  // vectors per copy (two groups of 128), copies in flight
+__global__ void __launch_bounds__(32)
+run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs, float2 *__restrict__ run_tab) {
+    extern __shared__ __align__(128) uint4 ring[];  // [RUN_RING][RUN_PIECE]
+    __shared__ __align__(8) unsigned long long full[RUN_RING];
+    __shared__ volatile int abort_flag;
+    const int lane = threadIdx.x, nvec = V >> 3;
+    if (lane == 0) {
+        for (int s = 0; s < RUN_RING; ++s) mbar_init(smem_u32(&full[s]), 1);
+        abort_flag = 0;
+        fence_mbar_init();
+    }
+    __syncwarp();
     // Set up under the tail of the kernel before, which may have written the logits.  The kernel launched behind this
     // one as its programmatic dependent reads the call's other inputs before it waits for the statistics: it may only
     // start once everything in front of this kernel is complete.
     pdl_wait();
     pdl_launch_dependents();
-    __shared__ float2 sh[RS_WARPS];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, slot = warp / wpr, sub = warp - slot * wpr;
-    const int nvec = V >> 3;
-    const int r = wpr == 1 ? blockIdx.x * RS_WARPS + warp : slot * gridDim.x + blockIdx.x;
-    if (r < n_runs) {
-        int v_lo, v_hi;
-        rs_run(nvec, r % RS_WARPS, &v_lo, &v_hi);
-        float m, s;
-        run_stats(reinterpret_cast<const uint4 *>(logits + (size_t)(r / RS_WARPS) * V), nvec, v_lo, v_hi, sub, wpr, lane, c, m, s);
-        if (lane == 0) {
-            if (wpr == 1)
-                run_tab[r] = make_float2(m, s);
-            else
-                sh[warp] = make_float2(m, s);
+    // the copies ahead: run, and vector within it
+    int r_next = blockIdx.x, v_next = 0, v_end = 0;
+    uint32_t n_issued = 0, n_used = 0;
+    auto bounds = [&](int r, int *lo, int *hi) { rs_run(nvec, r % RS_WARPS, lo, hi); };
+    auto skip_empty = [&]() {  // (a run of a short row may be empty)
+        while (r_next < n_runs) {
+            bounds(r_next, &v_next, &v_end);
+            if (v_next < v_end) return;
+            r_next += gridDim.x;
         }
+    };
+    auto issue = [&]() {
+        if (r_next >= n_runs) return;
+        const int n = min(RUN_PIECE, v_end - v_next);
+        if (lane == 0) {
+            const uint32_t s = n_issued % RUN_RING, bar = smem_u32(&full[s]);
+            mbar_arrive_expect_tx(bar, (uint32_t)n * 16u);
+            bulk_load(smem_u32(ring + s * RUN_PIECE), reinterpret_cast<const uint4 *>(logits + (size_t)(r_next / RS_WARPS) * V) + v_next,
+                      (uint32_t)n * 16u, bar);
+        }
+        ++n_issued;
+        v_next += n;
+        if (v_next >= v_end) {
+            r_next += gridDim.x;
+            skip_empty();
+        }
+    };
+    skip_empty();
+    for (int s = 0; s < RUN_RING; ++s) issue();
+    bool ok = true;
+    for (int r = blockIdx.x; r < n_runs; r += gridDim.x) {
+        int v_lo, v_hi;
+        bounds(r, &v_lo, &v_hi);
+        float m = NEG_INF, nmc = 0.f, s = 0.f;
+        for (int v0 = v_lo; v0 < v_hi && ok; v0 += RUN_PIECE) {
+            const uint32_t slot = n_used % RUN_RING;
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&full[slot]), (n_used / RUN_RING) & 1u, &abort_flag));
+            if (!ok) break;
+            const uint4 *p = ring + slot * RUN_PIECE + lane;
+            const int n = v_hi - v0 - lane;
+#pragma unroll
+            for (int g = 0; g < RUN_PIECE / 128; ++g) {
+                uint4 v[4];
+                if (g * 128 + 128 <= v_hi - v0) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) v[q] = p[g * 128 + q * 32];
+                    online_update4(v, c, m, nmc, s);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (g * 128 + q * 32 < n) online_update(p[g * 128 + q * 32], c, m, nmc, s);
+                }
+            }
+            ++n_used;
+            __syncwarp();
+            if (lane == 0) fence_proxy_async();  // the piece has been read before the copy engine writes its place again
+            issue();
+        }
+        const float mw = warp_max(m);
+        s = (m == NEG_INF) ? 0.f : s * ex2_approx((m - mw) * c);
+        s = warp_sum(s);
+        // (a copy that does not arrive: cannot happen with readable logits; marked instead of left looking valid)
+        if (lane == 0) run_tab[r] = ok ? make_float2(mw, s) : make_float2(nanf(""), nanf(""));
+        if (!ok) break;
     }
-    if (wpr > 1) {
-        __syncthreads();
-        if (sub == 0 && r < n_runs && lane == 0) {
-            float mb = NEG_INF, sb = 0.f;
-            for (int w = 0; w < wpr; ++w) mb = fmaxf(mb, sh[warp + w].x);
-            for (int w = 0; w < wpr; ++w) sb += sh[warp + w].x == NEG_INF ? 0.f : sh[warp + w].y * ex2_approx((sh[warp + w].x - mb) * c);
-            run_tab[r] = make_float2(mb, sb);
+    if (!ok && lane == 0) {  // let the copies still in flight land before the CTA goes away
+        for (uint32_t i = n_used; i < n_issued; ++i) {
+            const unsigned long long t0 = globaltimer_ns();
+            while (!mbar_try_wait(smem_u32(&full[i % RUN_RING]), (i / RUN_RING) & 1u) && globaltimer_ns() - t0 < 100000000ull) {
+            }
         }
     }
 }
 
-// The rows' own pairs; n_cta > 1: a cluster of n_cta CTAs per row (few rows), each with every n_cta-th group of every run.
+// A CTA per row: the pairs of the row's runs to run_tab (not null; n_cta = 1), or the row's own pair; n_cta > 1: a cluster of
+// n_cta CTAs per row (few rows), each with every n_cta-th group of every run.
 __global__ void __launch_bounds__(RS_THREADS, 8)
 row_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_cta, float *__restrict__ row_max,
-                 float *__restrict__ row_sum) {
+                 float *__restrict__ row_sum, float2 *__restrict__ run_tab) {
     pdl_wait();  // (as in run_stats_kernel)
     pdl_launch_dependents();
     __shared__ float2 sh[RS_WARPS];
@@ -152,6 +238,10 @@ row_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_cta,
     rs_run(nvec, warp, &v_lo, &v_hi);
     float m, s;
     run_stats(reinterpret_cast<const uint4 *>(logits + row * (size_t)V), nvec, v_lo, v_hi, rank, n_cta, lane, c, m, s);
+    if (run_tab) {
+        if (lane == 0) run_tab[row * RS_WARPS + warp] = make_float2(m, s);
+        return;
+    }
     if (lane == 0) sh[warp] = make_float2(m, s);
     if (n_cta > 1)
         cluster_sync_all();
@@ -1733,7 +1823,8 @@ __device__ void draw_tile(const TileArgs &t, size_t row, int V, float M, float c
     __shared__ int sh_tile, sh_last;
     for (int i = tid; i < n_tiles; i += TERM_THREADS) {
         const float2 e = t.mass[(size_t)i * t.rows + row];
-        mt[i] = e.x == NEG_INF ? 0.0 : (double)e.y * (double)ex2_approx((e.x - M) * c);
+        // (the tokens' exponents were formed with -m c rounded, as those of the tile at hand below are with -M c)
+        mt[i] = e.x == NEG_INF ? 0.0 : (double)e.y * exp2((double)(e.x * c) - (double)(M * c));
     }
     const int d8 = t.d >> 3;
     for (int i = tid; i < d8; i += TERM_THREADS) h[i] = reinterpret_cast<const uint4 *>(t.H + row * t.d)[i];
@@ -2120,16 +2211,22 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     if (rc_sm != SPECROLL_OK) return rc_sm;
     const int resident = 8 * n_sm;  // CTAs of the statistics kernels
     if (use_runs) {
-        const int n_runs = rows * RS_WARPS;
-        int wpr = 8;
-        while (wpr > 1 && (long long)n_runs * wpr > (long long)resident * RS_WARPS) wpr >>= 1;
-        SR_CUDA_TRY(launch_dependent(true, run_stats_kernel, dim3((unsigned)(wpr == 1 ? rows : n_runs < resident ? n_runs : resident)), dim3(RS_THREADS), 0,
-                                     st, static_cast<const uint16_t *>(logits), d->V, c, n_runs, wpr, run_tab));
+        // Up to two rounds of ten one-warp CTAs per SM (370 rows) the form with the deep ring, every CTA the same number of runs
+        // (to one); with more rows there are warps enough, and one warp per CTA is short of issue slots (verification, V 152 k:
+        // 20 rows 31.5 -> 18.7 us, 256 rows 50 -> 38, 512 rows 54 against 57, 4096 rows 200 against 298).
+        const int n_runs = rows * RS_WARPS, most = 10 * n_sm, rounds = (n_runs + most - 1) / most;
+        if (rounds <= 2)
+            SR_CUDA_TRY(launch_dependent(true, run_stats_kernel, dim3((unsigned)((n_runs + rounds - 1) / rounds)), dim3(32),
+                                         RUN_RING * RUN_PIECE * sizeof(uint4), st, static_cast<const uint16_t *>(logits), d->V, c,
+                                         n_runs, run_tab));
+        else
+            SR_CUDA_TRY(launch_dependent(true, row_stats_kernel, dim3((unsigned)rows), dim3(RS_THREADS), 0, st,
+                                         static_cast<const uint16_t *>(logits), d->V, c, 1, (float *)nullptr, (float *)nullptr, run_tab));
     } else if (!lazy) {
         int n_cta = 8;
         while (n_cta > 1 && (long long)rows * n_cta > resident) n_cta >>= 1;
         SR_CUDA_TRY(launch_clusters(true, n_cta, row_stats_kernel, dim3((unsigned)(rows * n_cta)), dim3(RS_THREADS), 0, st,
-                                    static_cast<const uint16_t *>(logits), d->V, c, n_cta, row_max, row_sum));
+                                    static_cast<const uint16_t *>(logits), d->V, c, n_cta, row_max, row_sum, (float2 *)nullptr));
     }
 
     WalkArgs wa;

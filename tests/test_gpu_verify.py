@@ -210,11 +210,11 @@ def test_lazy_row_statistics_give_the_same_walk(name, B, V, T):
 
 
 
-@pytest.mark.parametrize("B,N,k,V", [(1, 8, 4, 151936), (18, 8, 4, 4104), (19, 8, 3, 4096), (37, 8, 2, 1032), (38, 8, 4, 40008), (75, 8, 8, 8),
+@pytest.mark.parametrize("B,N,k,V", [(1, 8, 4, 151936), (18, 8, 4, 4104), (19, 8, 3, 4096), (37, 8, 2, 1032), (38, 8, 4, 40008), (24, 8, 4, 151936), (75, 8, 8, 8),
                                      (150, 8, 5, 4104), (3, 64, 8, 8200), (40, 40, 16, 2056), (5, 64, 32, 4104)])
-def test_runs_shared_by_warps_and_nodes_by_lane_groups(B, N, k, V):
-    """Eight, four, two warps or one per run of a row (by the number of rows), vocabularies that leave runs ragged or empty,
-    and 1 to 32 lanes per node with up to two nodes' rounds per warp."""
+def test_runs_by_one_warp_each_and_nodes_by_lane_groups(B, N, k, V):
+    """One or two runs of a row per warp, or a CTA per row (by the number of rows), vocabularies that leave runs ragged or
+    empty, and 1 to 32 lanes per node with up to two nodes' rounds per warp."""
     w = I.scaled(I.WORKLOADS["qwen7b"], B=B, N=N, V=V, k=min(k, V))
     parent = I.topology(w)
     cid, cl = I.synthetic_candidates(w)
