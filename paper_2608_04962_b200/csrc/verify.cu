@@ -127,20 +127,26 @@ __device__ __forceinline__ void run_stats(const uint4 *__restrict__ p, int nvec,
 
 // run_tab: [rows][RS_WARPS] (m, s) of every run of every row, s = sum over the run of exp((l - m)/T).  The kernel that
 // walks adds a row's pairs up; the terminal draw finds the eighth of the row that holds its target from them and reads
-// only that.  This is the form for few rows: one warp per CTA, which takes the runs blockIdx, blockIdx + grid, ... through a
-// ring of bulk copies, 20 KB in flight per warp (with its loads in registers a warp has 2 KB, so a run is 19 dependent
-// rounds however empty the machine), ten CTAs per SM.  The terms of a lane's sum keep the order that the CTA-per-row form
+// only that.  This is the form for few rows: a warp takes a run, or a few in turn, through a ring of bulk copies of 2 KB
+// (with its loads in registers a warp has 2 KB in flight, so a run is 19 dependent rounds however empty the machine); the
+// ring is as deep as the CTAs of an SM leave room for.  The terms of a lane's sum keep the order that the CTA-per-row form
 // (row_stats_kernel) gives them: the terminal draw follows the last bits of the runs' sums.
-constexpr int RUN_PIECE = 256, RUN_RING = 5;  // vectors per copy (two groups of 128), copies in flight
-__global__ void __launch_bounds__(32)
-run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs, float2 *__restrict__ run_tab) {
-    extern __shared__ __align__(128) uint4 ring[];  // [RUN_RING][RUN_PIECE]
-    __shared__ __align__(8) unsigned long long full[RUN_RING];
-    __shared__ volatile int abort_flag;
-    const int lane = threadIdx.x, nvec = V >> 3;
+constexpr int RUN_PIECE = 128;                 // vectors per copy (a group)
+constexpr int RUN_RING_MIN = 3, RUN_RING_MAX = 10;  // copies in flight per warp
+constexpr int RUN_WARPS = 4, RUN_CTAS = 8;     // warps per CTA, CTAs per SM
+__global__ void __launch_bounds__(32 * RUN_WARPS, RUN_CTAS)
+run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs, int ring_n, float2 *__restrict__ run_tab) {
+    extern __shared__ __align__(128) uint4 ring_all[];  // [RUN_WARPS][ring_n][RUN_PIECE]
+    __shared__ __align__(8) unsigned long long full_all[RUN_WARPS][RUN_RING_MAX];
+    __shared__ volatile int abort_all[RUN_WARPS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nvec = V >> 3;
+    const int first = warp * gridDim.x + blockIdx.x, stride = RUN_WARPS * gridDim.x;
+    uint4 *ring = ring_all + (size_t)warp * ring_n * RUN_PIECE;
+    unsigned long long *full = full_all[warp];
+    volatile int *abort_flag = &abort_all[warp];
     if (lane == 0) {
-        for (int s = 0; s < RUN_RING; ++s) mbar_init(smem_u32(&full[s]), 1);
-        abort_flag = 0;
+        for (int s = 0; s < ring_n; ++s) mbar_init(smem_u32(&full[s]), 1);
+        *abort_flag = 0;
         fence_mbar_init();
     }
     __syncwarp();
@@ -150,44 +156,46 @@ run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs
     pdl_wait();
     pdl_launch_dependents();
     // the copies ahead: run, and vector within it
-    int r_next = blockIdx.x, v_next = 0, v_end = 0;
+    int r_next = first, v_next = 0, v_end = 0;
     uint32_t n_issued = 0, n_used = 0;
+    int s_in = 0, s_out = 0;    // slots of the next copy and of the next piece to use
+    uint32_t phase = 0;         // parity of s_out's round
     auto bounds = [&](int r, int *lo, int *hi) { rs_run(nvec, r % RS_WARPS, lo, hi); };
     auto skip_empty = [&]() {  // (a run of a short row may be empty)
         while (r_next < n_runs) {
             bounds(r_next, &v_next, &v_end);
             if (v_next < v_end) return;
-            r_next += gridDim.x;
+            r_next += stride;
         }
     };
     auto issue = [&]() {
         if (r_next >= n_runs) return;
         const int n = min(RUN_PIECE, v_end - v_next);
         if (lane == 0) {
-            const uint32_t s = n_issued % RUN_RING, bar = smem_u32(&full[s]);
+            const uint32_t bar = smem_u32(&full[s_in]);
             mbar_arrive_expect_tx(bar, (uint32_t)n * 16u);
-            bulk_load(smem_u32(ring + s * RUN_PIECE), reinterpret_cast<const uint4 *>(logits + (size_t)(r_next / RS_WARPS) * V) + v_next,
+            bulk_load(smem_u32(ring + s_in * RUN_PIECE), reinterpret_cast<const uint4 *>(logits + (size_t)(r_next / RS_WARPS) * V) + v_next,
                       (uint32_t)n * 16u, bar);
         }
         ++n_issued;
+        if (++s_in == ring_n) s_in = 0;
         v_next += n;
         if (v_next >= v_end) {
-            r_next += gridDim.x;
+            r_next += stride;
             skip_empty();
         }
     };
     skip_empty();
-    for (int s = 0; s < RUN_RING; ++s) issue();
+    for (int s = 0; s < ring_n; ++s) issue();
     bool ok = true;
-    for (int r = blockIdx.x; r < n_runs; r += gridDim.x) {
+    for (int r = first; r < n_runs; r += stride) {
         int v_lo, v_hi;
         bounds(r, &v_lo, &v_hi);
         float m = NEG_INF, nmc = 0.f, s = 0.f;
         for (int v0 = v_lo; v0 < v_hi && ok; v0 += RUN_PIECE) {
-            const uint32_t slot = n_used % RUN_RING;
-            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&full[slot]), (n_used / RUN_RING) & 1u, &abort_flag));
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s_out]), phase, abort_flag));
             if (!ok) break;
-            const uint4 *p = ring + slot * RUN_PIECE + lane;
+            const uint4 *p = ring + s_out * RUN_PIECE + lane;
             const int n = v_hi - v0 - lane;
 #pragma unroll
             for (int g = 0; g < RUN_PIECE / 128; ++g) {
@@ -203,6 +211,10 @@ run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs
                 }
             }
             ++n_used;
+            if (++s_out == ring_n) {
+                s_out = 0;
+                phase ^= 1u;
+            }
             __syncwarp();
             if (lane == 0) fence_proxy_async();  // the piece has been read before the copy engine writes its place again
             issue();
@@ -217,7 +229,7 @@ run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs
     if (!ok && lane == 0) {  // let the copies still in flight land before the CTA goes away
         for (uint32_t i = n_used; i < n_issued; ++i) {
             const unsigned long long t0 = globaltimer_ns();
-            while (!mbar_try_wait(smem_u32(&full[i % RUN_RING]), (i / RUN_RING) & 1u) && globaltimer_ns() - t0 < 100000000ull) {
+            while (!mbar_try_wait(smem_u32(&full[i % ring_n]), (i / ring_n) & 1u) && globaltimer_ns() - t0 < 100000000ull) {
             }
         }
     }
@@ -2211,17 +2223,24 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     if (rc_sm != SPECROLL_OK) return rc_sm;
     const int resident = 8 * n_sm;  // CTAs of the statistics kernels
     if (use_runs) {
-        // Up to two rounds of ten one-warp CTAs per SM (370 rows) the form with the deep ring, every CTA the same number of runs
-        // (to one); with more rows there are warps enough, and one warp per CTA is short of issue slots (verification, V 152 k:
-        // 20 rows 31.5 -> 18.7 us, 256 rows 50 -> 38, 512 rows 54 against 57, 4096 rows 200 against 298).
-        const int n_runs = rows * RS_WARPS, most = 10 * n_sm, rounds = (n_runs + most - 1) / most;
-        if (rounds <= 2)
-            SR_CUDA_TRY(launch_dependent(true, run_stats_kernel, dim3((unsigned)((n_runs + rounds - 1) / rounds)), dim3(32),
-                                         RUN_RING * RUN_PIECE * sizeof(uint4), st, static_cast<const uint16_t *>(logits), d->V, c,
-                                         n_runs, run_tab));
-        else
+        // Up to 44 runs per SM (814 rows) the form with the rings; with more rows there are warps enough, and the ring's
+        // bookkeeping costs issue slots (verification, V 152 k: 20 rows 29 -> 19 us, 256 rows 48 -> 34, 512 rows 54 -> 47,
+        // 768 rows 63.5 -> 60.5, 1024 rows 70 -> 72.6, 4096 rows 198 -> 234).
+        const int n_runs = rows * RS_WARPS, most = RUN_WARPS * RUN_CTAS * n_sm, rounds = (n_runs + most - 1) / most;
+        if (n_runs <= 44 * n_sm) {
+            // every warp the same number of runs (to one), and a CTA for each while there is room
+            const int warps = (n_runs + rounds - 1) / rounds, grid = warps <= RUN_CTAS * n_sm ? warps : RUN_CTAS * n_sm;
+            const int per_sm = (grid + n_sm - 1) / n_sm, piece_bytes = RUN_WARPS * RUN_PIECE * (int)sizeof(uint4);
+            int ring_n = 200 * 1024 / per_sm / piece_bytes;
+            ring_n = ring_n < RUN_RING_MIN ? RUN_RING_MIN : ring_n > RUN_RING_MAX ? RUN_RING_MAX : ring_n;
+            const int rc_ = device_setup(reinterpret_cast<const void *>(run_stats_kernel), RUN_RING_MAX * piece_bytes, nullptr);
+            if (rc_ != SPECROLL_OK) return rc_;
+            SR_CUDA_TRY(launch_dependent(true, run_stats_kernel, dim3((unsigned)grid), dim3(32 * RUN_WARPS), (size_t)ring_n * piece_bytes,
+                                         st, static_cast<const uint16_t *>(logits), d->V, c, n_runs, ring_n, run_tab));
+        } else {
             SR_CUDA_TRY(launch_dependent(true, row_stats_kernel, dim3((unsigned)rows), dim3(RS_THREADS), 0, st,
                                          static_cast<const uint16_t *>(logits), d->V, c, 1, (float *)nullptr, (float *)nullptr, run_tab));
+        }
     } else if (!lazy) {
         int n_cta = 8;
         while (n_cta > 1 && (long long)rows * n_cta > resident) n_cta >>= 1;

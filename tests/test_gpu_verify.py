@@ -210,7 +210,7 @@ def test_lazy_row_statistics_give_the_same_walk(name, B, V, T):
 
 
 
-@pytest.mark.parametrize("B,N,k,V", [(1, 8, 4, 151936), (18, 8, 4, 4104), (19, 8, 3, 4096), (37, 8, 2, 1032), (38, 8, 4, 40008), (24, 8, 4, 151936), (75, 8, 8, 8),
+@pytest.mark.parametrize("B,N,k,V", [(1, 8, 4, 151936), (18, 8, 4, 4104), (19, 8, 3, 4096), (37, 8, 2, 1032), (38, 8, 4, 40008), (24, 8, 4, 151936), (100, 8, 4, 8200), (102, 8, 4, 8200), (75, 8, 8, 8),
                                      (150, 8, 5, 4104), (3, 64, 8, 8200), (40, 40, 16, 2056), (5, 64, 32, 4104)])
 def test_runs_by_one_warp_each_and_nodes_by_lane_groups(B, N, k, V):
     """One or two runs of a row per warp, or a CTA per row (by the number of rows), vocabularies that leave runs ragged or
