@@ -1012,6 +1012,118 @@ __device__ __forceinline__ void walk_buf_fetch(const WalkArgs &a, const Topo &to
     }
 }
 
+// The children of every node, grouped by parent in slot order, and what a slot's test needs of the proposal (k <= 32): known
+// before the row statistics are.
+struct WalkSlots {
+    double *q;       // [N, k] the slot's proposal on the candidates: e_j / s over those the earlier siblings left, 0 on the others
+    double *u;       // [N]    the acceptance uniform
+    int32_t *node;   // [N]    the child
+    int32_t *jc;     // [N]    its own candidate
+    int32_t *start;  // [N]    first slot of a parent's children
+};
+__host__ __device__ inline size_t walk_slots_bytes(int N, int k) {
+    auto up = [](size_t x) { return (x + 15) / 16 * 16; };
+    return k > 32 ? 0 : up((size_t)N * k * sizeof(double)) + up((size_t)N * sizeof(double)) + 3 * up((size_t)N * sizeof(int32_t));
+}
+__device__ __forceinline__ WalkSlots walk_slots(unsigned char *p, int N, int k) {
+    auto take = [&](size_t x) {
+        unsigned char *q = p;
+        p += (x + 15) / 16 * 16;
+        return q;
+    };
+    WalkSlots w;
+    w.q = reinterpret_cast<double *>(take((size_t)N * k * sizeof(double)));
+    w.u = reinterpret_cast<double *>(take((size_t)N * sizeof(double)));
+    w.node = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
+    w.jc = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
+    w.start = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
+    return w;
+}
+// By all threads of a CTA, from a filled WalkBuf (a barrier before and after is the caller's).  *odd: set where a slot's weights
+// underflow (such trees go through walk_node).
+__device__ __forceinline__ void walk_slots_fill(const WalkBuf &buf, const Topo &topo, int N, int k, int where, const WalkSlots &w,
+                                                int *odd) {
+    // a thread per (child, candidate): the sums over the candidates are formed by each for itself, in the order walk_node has
+    for (int e = threadIdx.x; e < (N - 1) * k; e += blockDim.x) {
+        const int c = 1 + e / k, j = e - (c - 1) * k, u = buf.parent[c];
+        int at = 0, first = 0;
+        unsigned taken = 0u;
+        for (int n = 1; n < N; ++n) {
+            const int pn = buf.parent[n];
+            at += pn < u || (pn == u && n < c);
+            first += pn < u;
+            if (pn == u && n < c) taken |= 1u << SR_CHECKED((int)buf.tcand[n], k, where);
+        }
+        const double *eh = buf.e + topo.depth[u] * k;
+        double s = 0.0;
+        for (int i = 0; i < k; ++i)
+            if (!((taken >> i) & 1u)) s += eh[i];
+        if (!(s > 0.0 && s < INFINITY)) *odd = 1;
+        w.q[at * k + j] = ((taken >> j) & 1u) ? 0.0 : eh[j] * (1.0 / s);
+        if (j == 0) {
+            w.node[at] = c;
+            w.jc[at] = SR_CHECKED((int)buf.tcand[c], k, where);
+            w.u[at] = (double)buf.uacc[c];
+            w.start[u] = first;
+        }
+    }
+}
+
+// One node by kp lanes (the power of two that holds k <= 32 candidates, and so all children; several nodes per warp, u < 0: a
+// group without one): the arithmetic of walk_node with the slots' proposals ready.  rho: lane j's candidate's target
+// probability, at the end its residual, not normalised.  Returns the accepted child or -1; mg: the smallest margin.
+__device__ __forceinline__ int walk_group(const Topo &topo, int u, int k, int kp, double &rho, const WalkSlots &w, float &mg) {
+    const int lane = threadIdx.x & 31, grp = lane / kp, j = lane & (kp - 1);
+    const int m = u >= 0 ? topo.n_child[u] : 0, st = u >= 0 ? w.start[u] : 0;
+    int most = m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+    double pc = rho;
+    for (int o = kp >> 1; o > 0; o >>= 1) pc += __shfl_xor_sync(0xffffffffu, pc, o);
+    const double p_off = pc < 1.0 ? 1.0 - pc : 0.0;
+    double Zc = 1.0, my_rho = 0.0, my_Zc = 1.0;
+#pragma unroll 2
+    for (int i = 0; i < most; ++i) {
+        const bool on = i < m;
+        const double q = on && j < k ? w.q[(st + i) * k + j] : 0.0;
+        const double rho_jc = __shfl_sync(0xffffffffu, rho, on ? w.jc[st + i] : 0, kp);
+        if (j == i) {
+            my_rho = rho_jc;
+            my_Zc = Zc;
+        }
+        const double t0 = rho - Zc * q, t = t0 > 0.0 ? t0 : 0.0;
+        double Zn = t;
+        for (int o = kp >> 1; o > 0; o >>= 1) Zn += __shfl_xor_sync(0xffffffffu, Zn, o);
+        Zn += p_off;
+        if (on && Zn > 1e-300 * Zc) {
+            rho = t;
+            Zc = Zn;
+        }
+    }
+    // every child's test at once, lane i of the group child i
+    bool acc = false;
+    int c = -1;
+    mg = INFINITY;
+    if (j < m) {
+        c = w.node[st + j];
+        const double my_q = w.q[(st + j) * k + w.jc[st + j]], uu = w.u[st + j];
+        double ratio;
+        if (my_q > 0.0)
+            ratio = my_rho > 0.0 ? (my_rho / my_Zc) / my_q : 0.0;
+        else
+            ratio = my_rho > 0.0 ? INFINITY : 0.0;
+        acc = uu < (ratio < 1.0 ? ratio : 1.0);
+        mg = (float)fabs(uu - ratio);
+    }
+    const unsigned mask = kp == 32 ? 0xffffffffu : ((1u << kp) - 1u) << (grp * kp);
+    const unsigned hits = __ballot_sync(0xffffffffu, acc) & mask;
+    const int f = hits ? __ffs(hits) - 1 : -1;
+    if (f >= 0 && lane > f) mg = INFINITY;
+    for (int o = kp >> 1; o > 0; o >>= 1) mg = fminf(mg, __shfl_xor_sync(0xffffffffu, mg, o));
+    const int child = __shfl_sync(0xffffffffu, c, f >= 0 ? f : lane);
+    return f < 0 ? -1 : child;
+}
+
 // Plain target distributions: one warp per sequence.  Which nodes the walk visits depends on its decisions, but
 // what it can ask for does not, so with the dense logits everything is fetched up front (WalkStage): one round
 // trip to memory per sequence instead of four or five dependent ones per visited node, which is what the walk's
@@ -1455,14 +1567,15 @@ __global__ void __launch_bounds__(TERM_THREADS) terminal_kernel(TermArgs a) {
 // A sequence's rows come one after the other and each waits for memory and shared-memory atomics, so a sequence gets a
 // cluster of n_cta CTAs that share the passes over a row (walk_cta_split); the cluster's first CTA does the nodes.
 struct WalkCtaLayout {
-    size_t stage, total;  // in front of the stage: the threshold search, whose place the draw's slice masses take
+    size_t stage, slots, total;  // in front of the stage: the threshold search, whose place the draw's slice masses take
 };
 __host__ __device__ inline WalkCtaLayout walk_cta_layout(int N, int K, int k, int V, int n_cta, bool nuc) {
     WalkCtaLayout L;
     L.stage = draw_smem_bytes(V, n_cta);
     if (nuc && L.stage < sizeof(NucleusSmem)) L.stage = sizeof(NucleusSmem);
     L.stage = (L.stage + 15) / 16 * 16;
-    L.total = L.stage + walk_buf_bytes(N, K, k);
+    L.slots = L.stage + (walk_buf_bytes(N, K, k) + 15) / 16 * 16;
+    L.total = L.slots + walk_slots_bytes(N, k);
     return L;
 }
 
@@ -1481,13 +1594,24 @@ walk_cta_kernel(WalkArgs a, Topo topo, float c, float top_p, float *__restrict__
     __shared__ double sh_ovm[SPECROLL_MAX_TOPK];
     const int rank = n_cta > 1 ? (int)cluster_ctarank() : 0, b = blockIdx.x / n_cta;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const WalkBuf buf = walk_buf(nuc_raw + walk_cta_layout(a.N, a.K, a.k, a.V, n_cta, NUC).stage, a.N, a.K, a.k);
+    __shared__ int sh_odd;            // the slots' weights underflow, or k > 32: walk_node
+    const WalkCtaLayout L = walk_cta_layout(a.N, a.K, a.k, a.V, n_cta, NUC);
+    const WalkBuf buf = walk_buf(nuc_raw + L.stage, a.N, a.K, a.k);
+    const WalkSlots slots = walk_slots(nuc_raw + L.slots, a.N, a.k);
+    const double inv_T = 1.0 / a.T;
+    int kp = 1;
+    while (kp < a.k) kp <<= 1;
     const WalkStage stage{buf.rmax, buf.rsum, buf.uacc, buf.ttok, buf.tcand, buf.cid, buf.clog, buf.pre, buf.parent, buf.e, nullptr};
     WalkState st;
     // Set up under the tail of the kernel before.  Where that is this call's own (statistics, thresholds), which itself
     // started when everything in front of the call was complete, the call's inputs are staged ahead of the wait.
     if (LAZY) pdl_wait();
-    if (rank == 0) walk_buf_fetch(a, topo, b, buf);
+    if (threadIdx.x == 0) sh_odd = a.k > 32;
+    if (rank == 0) {
+        walk_buf_fetch(a, topo, b, buf);
+        __syncthreads();
+        if (a.k <= 32) walk_slots_fill(buf, topo, a.N, a.k, b, slots, &sh_odd);
+    }
     if (!LAZY) {
         pdl_wait();
         if (rank == 0)
@@ -1535,14 +1659,31 @@ walk_cta_kernel(WalkArgs a, Topo topo, float c, float top_p, float *__restrict__
                 if (topo.n_child[u] == 0) {
                     st.kind = (u != 0) ? 1 : 0;
                     st.have_residual = false;
+                } else if (!sh_odd) {
+                    const bool mine = lane < a.k;  // (the first group of lanes has the node)
+                    double rho = 0.0;
+                    if (mine) {
+                        const uint32_t bits = buf.pre[u * a.k + lane];
+                        if (ord_key(bits) >= thr) rho = exp(((double)bf16_bits_to_float((uint16_t)bits) - (double)M) * inv_T) * (1.0 / (double)norm);
+                    }
+                    float mg;
+                    next = __shfl_sync(0xffffffffu, walk_group(topo, lane < kp ? u : -1, a.k, kp, rho, slots, mg), 0);
+                    st.mm = fminf(st.mm, __shfl_sync(0xffffffffu, mg, 0));
+                    if (next >= 0) {
+                        if (lane == 0) {
+                            a.out_tok[(size_t)b * (a.K + 1) + st.nacc] = buf.ttok[next];
+                            a.path_node[(size_t)b * (a.K + 1) + st.nacc + 1] = next;
+                        }
+                        ++st.nacc;
+                    } else {
+                        st.have_residual = true;
+                        if (mine) sh_ovm[lane] = rho * (double)norm;  // (r = rho / Zc and sigma = 1 / Zc)
+                    }
                 } else {
                     next = walk_node(a, topo, b, u, (double)M, (double)norm, thr, lane, &sm, &st, &stage);
-                    if (next < 0) {
-                        st.kind = 0;
-                        st.have_residual = true;
-                    }
+                    if (next < 0) st.have_residual = true;
                 }
-                if (next < 0 && st.have_residual) {
+                if (next < 0 && st.have_residual && sh_odd) {
                     const double f = (double)norm / __shfl_sync(0xffffffffu, st.sigma, 0);  // (one division; the entries may be zero)
                     for (int j = lane; j < a.k; j += 32) sh_ovm[j] = sm.r[j] * f;
                 }
@@ -1646,66 +1787,8 @@ constexpr int WT_THREADS = TERM_THREADS;
 constexpr int WT_SMEM_LIMIT = 160 * 1024;
 constexpr int WT_WARPS = WT_THREADS / 32;
 
-// The children of every node, grouped by parent in slot order, and what a slot's test needs of the proposal (k <= 32): known
-// before the row statistics are.
-struct WalkSlots {
-    double *q;       // [N, k] the slot's proposal on the candidates: e_j / s over those the earlier siblings left, 0 on the others
-    double *u;       // [N]    the acceptance uniform
-    int32_t *node;   // [N]    the child
-    int32_t *jc;     // [N]    its own candidate
-    int32_t *start;  // [N]    first slot of a parent's children
-};
-__host__ __device__ inline size_t walk_slots_bytes(int N, int k) {
-    auto up = [](size_t x) { return (x + 15) / 16 * 16; };
-    return k > 32 ? 0 : up((size_t)N * k * sizeof(double)) + up((size_t)N * sizeof(double)) + 3 * up((size_t)N * sizeof(int32_t));
-}
-__device__ __forceinline__ WalkSlots walk_slots(unsigned char *p, int N, int k) {
-    auto take = [&](size_t x) {
-        unsigned char *q = p;
-        p += (x + 15) / 16 * 16;
-        return q;
-    };
-    WalkSlots w;
-    w.q = reinterpret_cast<double *>(take((size_t)N * k * sizeof(double)));
-    w.u = reinterpret_cast<double *>(take((size_t)N * sizeof(double)));
-    w.node = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
-    w.jc = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
-    w.start = reinterpret_cast<int32_t *>(take((size_t)N * sizeof(int32_t)));
-    return w;
-}
-// By all threads of a CTA, from a filled WalkBuf (a barrier before and after is the caller's).  *odd: set where a slot's weights
-// underflow (such trees go through walk_node).
-__device__ __forceinline__ void walk_slots_fill(const WalkBuf &buf, const Topo &topo, int N, int k, int where, const WalkSlots &w,
-                                                int *odd) {
-    // a thread per (child, candidate): the sums over the candidates are formed by each for itself, in the order walk_node has
-    for (int e = threadIdx.x; e < (N - 1) * k; e += blockDim.x) {
-        const int c = 1 + e / k, j = e - (c - 1) * k, u = buf.parent[c];
-        int at = 0, first = 0;
-        unsigned taken = 0u;
-        for (int n = 1; n < N; ++n) {
-            const int pn = buf.parent[n];
-            at += pn < u || (pn == u && n < c);
-            first += pn < u;
-            if (pn == u && n < c) taken |= 1u << SR_CHECKED((int)buf.tcand[n], k, where);
-        }
-        const double *eh = buf.e + topo.depth[u] * k;
-        double s = 0.0;
-        for (int i = 0; i < k; ++i)
-            if (!((taken >> i) & 1u)) s += eh[i];
-        if (!(s > 0.0 && s < INFINITY)) *odd = 1;
-        w.q[at * k + j] = ((taken >> j) & 1u) ? 0.0 : eh[j] * (1.0 / s);
-        if (j == 0) {
-            w.node[at] = c;
-            w.jc[at] = SR_CHECKED((int)buf.tcand[c], k, where);
-            w.u[at] = (double)buf.uacc[c];
-            w.start[u] = first;
-        }
-    }
-}
-
-// Every node with children on its own, kp lanes (the power of two that holds k <= 32 candidates, and so all children) per node,
-// several nodes per warp: the arithmetic of walk_node with the slots' proposals ready.  first[u]: accepted child or -1,
-// mm[u]: smallest margin, ovm[u, j]: the residual's masses where all children were rejected.  (A warp per node took 9 k
+// Every node with children on its own.  first[u]: accepted child or -1, mm[u]: smallest margin, ovm[u, j]: the residual's
+// masses where all children were rejected.  (A warp per node took 9 k
 // cycles, two rounds of them where more than sixteen nodes have children: 10 us of the 66 us of 16 sequences x 48 nodes.)
 __device__ __forceinline__ void walk_nodes(const Topo &topo, int N, int k, const double *p, const float *rsum, const WalkSlots &w,
                                            int32_t *first, float *mm, double *ovm) {
@@ -1724,58 +1807,13 @@ __device__ __forceinline__ void walk_nodes(const Topo &topo, int N, int k, const
             for (int n = 0; n < N; ++n)
                 if (topo.n_child[n] > 0 && idx++ == i0 + grp) u = n;
         }
-        const int m = u >= 0 ? topo.n_child[u] : 0, st = u >= 0 ? w.start[u] : 0;
-        int most = m;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
         double rho = u >= 0 && j < k ? p[u * k + j] : 0.0;
-        double pc = rho;
-        for (int o = kp >> 1; o > 0; o >>= 1) pc += __shfl_xor_sync(0xffffffffu, pc, o);
-        const double p_off = pc < 1.0 ? 1.0 - pc : 0.0;
-        double Zc = 1.0, my_rho = 0.0, my_Zc = 1.0;
-#pragma unroll 2
-        for (int i = 0; i < most; ++i) {
-            const bool on = i < m;
-            const double q = on && j < k ? w.q[(st + i) * k + j] : 0.0;
-            const double rho_jc = __shfl_sync(0xffffffffu, rho, on ? w.jc[st + i] : 0, kp);
-            if (j == i) {
-                my_rho = rho_jc;
-                my_Zc = Zc;
-            }
-            const double t0 = rho - Zc * q, t = t0 > 0.0 ? t0 : 0.0;
-            double Zn = t;
-            for (int o = kp >> 1; o > 0; o >>= 1) Zn += __shfl_xor_sync(0xffffffffu, Zn, o);
-            Zn += p_off;
-            if (on && Zn > 1e-300 * Zc) {
-                rho = t;
-                Zc = Zn;
-            }
-        }
-        // every child's test at once, lane i of the group child i
-        bool acc = false;
-        float mg = INFINITY;
-        int c = -1;
-        if (j < m) {
-            c = w.node[st + j];
-            const double my_q = w.q[(st + j) * k + w.jc[st + j]], uu = w.u[st + j];
-            double ratio;
-            if (my_q > 0.0)
-                ratio = my_rho > 0.0 ? (my_rho / my_Zc) / my_q : 0.0;
-            else
-                ratio = my_rho > 0.0 ? INFINITY : 0.0;
-            acc = uu < (ratio < 1.0 ? ratio : 1.0);
-            mg = (float)fabs(uu - ratio);
-        }
-        const unsigned mask = kp == 32 ? 0xffffffffu : ((1u << kp) - 1u) << (grp * kp);
-        const unsigned hits = __ballot_sync(0xffffffffu, acc) & mask;
-        const int f = hits ? __ffs(hits) - 1 : -1;
-        if (f >= 0 && lane > f) mg = INFINITY;
-        for (int o = kp >> 1; o > 0; o >>= 1) mg = fminf(mg, __shfl_xor_sync(0xffffffffu, mg, o));
-        const int child = __shfl_sync(0xffffffffu, c, f >= 0 ? f : lane);
+        float mg;
+        const int child = walk_group(topo, u, k, kp, rho, w, mg);
         if (u >= 0) {
-            if (f < 0 && j < k) ovm[u * k + j] = rho * (double)rsum[u];  // (r = rho / Zc and sigma = 1 / Zc)
+            if (child < 0 && j < k) ovm[u * k + j] = rho * (double)rsum[u];  // (r = rho / Zc and sigma = 1 / Zc)
             if (j == 0) {
-                first[u] = f < 0 ? -1 : child;
+                first[u] = child;
                 mm[u] = mg;
             }
         }
