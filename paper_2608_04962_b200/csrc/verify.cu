@@ -100,14 +100,13 @@ __host__ __device__ inline int rs_run_of_vec(int nvec, int vi) {
     return (vi / 128) / gpw;
 }
 
-// Maximum and sum of one warp's part of a run [v_lo, v_hi): groups of 128 vectors, every `step`-th from the `sub`-th on.
-__device__ __forceinline__ void run_stats(const uint4 *__restrict__ p, int nvec, int v_lo, int v_hi, int sub, int step, int lane,
-                                          float c, float &m, float &s) {
+// Maximum and sum of a run [v_lo, v_hi) by one warp, in groups of 128 vectors.
+__device__ __forceinline__ void run_stats(const uint4 *__restrict__ p, int nvec, int v_lo, int v_hi, int lane, float c, float &m, float &s) {
     float nmc = 0.f;
     m = NEG_INF;
     s = 0.f;
 #pragma unroll 1
-    for (int i0 = v_lo + sub * 128 + lane; i0 - lane < v_hi; i0 += step * 128) {
+    for (int i0 = v_lo + lane; i0 - lane < v_hi; i0 += 128) {
         if (i0 + 3 * 32 < nvec) {  // (for lane 31: the whole group is inside the row)
             uint4 v[4];
 #pragma unroll
@@ -125,6 +124,17 @@ __device__ __forceinline__ void run_stats(const uint4 *__restrict__ p, int nvec,
     m = mw;
 }
 
+// A row's own pair from its runs' pairs, by warp 0 of a CTA.
+__device__ __forceinline__ void row_from_runs(const float2 *sh, int lane, float c, float *row_max, float *row_sum) {
+    const float2 e = lane < RS_WARPS ? sh[lane] : make_float2(NEG_INF, 0.f);
+    const float mb = warp_max(e.x);
+    const float s = warp_sum(e.x == NEG_INF ? 0.f : e.y * ex2_approx((e.x - mb) * c));
+    if (lane == 0) {
+        *row_max = mb;
+        *row_sum = s;
+    }
+}
+
 // run_tab: [rows][RS_WARPS] (m, s) of every run of every row, s = sum over the run of exp((l - m)/T).  The kernel that
 // walks adds a row's pairs up; the terminal draw finds the eighth of the row that holds its target from them and reads
 // only that.  This is the form for few rows: a warp takes a run, or a few in turn, through a ring of bulk copies of 2 KB
@@ -134,13 +144,18 @@ __device__ __forceinline__ void run_stats(const uint4 *__restrict__ p, int nvec,
 constexpr int RUN_PIECE = 128;                 // vectors per copy (a group)
 constexpr int RUN_RING_MIN = 3, RUN_RING_MAX = 10;  // copies in flight per warp
 constexpr int RUN_WARPS = 4, RUN_CTAS = 8;     // warps per CTA, CTAs per SM
-__global__ void __launch_bounds__(32 * RUN_WARPS, RUN_CTAS)
-run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs, int ring_n, float2 *__restrict__ run_tab) {
-    extern __shared__ __align__(128) uint4 ring_all[];  // [RUN_WARPS][ring_n][RUN_PIECE]
-    __shared__ __align__(8) unsigned long long full_all[RUN_WARPS][RUN_RING_MAX];
-    __shared__ volatile int abort_all[RUN_WARPS];
+// ROWS: a CTA of eight warps takes the eight runs of row blockIdx and leaves the row's own pair (up to four rows per SM).
+template <bool ROWS>
+__global__ void __launch_bounds__(32 * (ROWS ? RS_WARPS : RUN_WARPS), ROWS ? 4 : RUN_CTAS)
+run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs, int ring_n, float2 *__restrict__ run_tab,
+                 float *__restrict__ row_max, float *__restrict__ row_sum) {
+    constexpr int WARPS = ROWS ? RS_WARPS : RUN_WARPS;
+    extern __shared__ __align__(128) uint4 ring_all[];  // [WARPS][ring_n][RUN_PIECE]
+    __shared__ __align__(8) unsigned long long full_all[WARPS][RUN_RING_MAX];
+    __shared__ volatile int abort_all[WARPS];
+    __shared__ float2 sh[RS_WARPS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nvec = V >> 3;
-    const int first = warp * gridDim.x + blockIdx.x, stride = RUN_WARPS * gridDim.x;
+    const int first = ROWS ? blockIdx.x * RS_WARPS + warp : warp * gridDim.x + blockIdx.x, stride = ROWS ? n_runs : RUN_WARPS * gridDim.x;
     uint4 *ring = ring_all + (size_t)warp * ring_n * RUN_PIECE;
     unsigned long long *full = full_all[warp];
     volatile int *abort_flag = &abort_all[warp];
@@ -223,7 +238,13 @@ run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs
         s = (m == NEG_INF) ? 0.f : s * ex2_approx((m - mw) * c);
         s = warp_sum(s);
         // (a copy that does not arrive: cannot happen with readable logits; marked instead of left looking valid)
-        if (lane == 0) run_tab[r] = ok ? make_float2(mw, s) : make_float2(nanf(""), nanf(""));
+        const float2 e = ok ? make_float2(mw, s) : make_float2(nanf(""), nanf(""));
+        if (lane == 0) {
+            if (ROWS)
+                sh[warp] = e;
+            else
+                run_tab[r] = e;
+        }
         if (!ok) break;
     }
     if (!ok && lane == 0) {  // let the copies still in flight land before the CTA goes away
@@ -233,54 +254,33 @@ run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs
             }
         }
     }
+    if (ROWS) {
+        __syncthreads();
+        if (warp == 0) row_from_runs(sh, lane, c, row_max + blockIdx.x, row_sum + blockIdx.x);
+    }
 }
 
-// A CTA per row: the pairs of the row's runs to run_tab (not null; n_cta = 1), or the row's own pair; n_cta > 1: a cluster of
-// n_cta CTAs per row (few rows), each with every n_cta-th group of every run.
+// A CTA per row: the pairs of the row's runs to run_tab, or (run_tab null) the row's own pair.
 __global__ void __launch_bounds__(RS_THREADS, 8)
-row_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_cta, float *__restrict__ row_max,
-                 float *__restrict__ row_sum, float2 *__restrict__ run_tab) {
+row_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, float *__restrict__ row_max, float *__restrict__ row_sum,
+                 float2 *__restrict__ run_tab) {
     pdl_wait();  // (as in run_stats_kernel)
     pdl_launch_dependents();
     __shared__ float2 sh[RS_WARPS];
-    const size_t row = blockIdx.x / n_cta;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = n_cta > 1 ? (int)cluster_ctarank() : 0;
+    const size_t row = blockIdx.x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nvec = V >> 3;
     int v_lo, v_hi;
     rs_run(nvec, warp, &v_lo, &v_hi);
     float m, s;
-    run_stats(reinterpret_cast<const uint4 *>(logits + row * (size_t)V), nvec, v_lo, v_hi, rank, n_cta, lane, c, m, s);
+    run_stats(reinterpret_cast<const uint4 *>(logits + row * (size_t)V), nvec, v_lo, v_hi, lane, c, m, s);
     if (run_tab) {
         if (lane == 0) run_tab[row * RS_WARPS + warp] = make_float2(m, s);
         return;
     }
     if (lane == 0) sh[warp] = make_float2(m, s);
-    if (n_cta > 1)
-        cluster_sync_all();
-    else
-        __syncthreads();
-    if (rank == 0 && warp == 0) {
-        float mb = NEG_INF, sb = 0.f;
-        for (int w0 = 0; w0 < RS_WARPS * n_cta; w0 += 32) {
-            const int w = w0 + lane;
-            float2 e = make_float2(NEG_INF, 0.f);
-            if (w < RS_WARPS) {
-                e = sh[w];
-            } else if (w < RS_WARPS * n_cta) {
-                const double d = ld_dsmem_f64(sh + w % RS_WARPS, w / RS_WARPS);
-                e = make_float2(__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d)));
-            }
-            const float mn = fmaxf(mb, warp_max(e.x));
-            const float part = warp_sum(e.x == NEG_INF ? 0.f : e.y * ex2_approx((e.x - mn) * c));
-            sb = (mb == NEG_INF ? 0.f : sb * ex2_approx((mb - mn) * c)) + part;
-            mb = mn;
-        }
-        if (lane == 0) {
-            row_max[row] = mb;
-            row_sum[row] = sb;
-        }
-    }
-    if (n_cta > 1) cluster_sync_all();  // (a CTA's pairs stay until they have been read)
+    __syncthreads();
+    if (warp == 0) row_from_runs(sh, lane, c, row_max + row, row_sum + row);
 }
 
 // ------------------------------------------------------------------------------ nucleus threshold
@@ -300,16 +300,14 @@ constexpr int NUC_THREADS = 512;
 // token is kept iff ord_key(logit) >= key), st->keep = sum of the kept exp((l - M)/T).
 //
 // A token's mass depends on its 16 bits alone, so one pass COUNTS the tokens of every bf16 value in shared memory and
-// the cut is found by a scan over the values, largest first, with the masses count * exp((l - M)/T): exact key, exact
-// integer counts, no order of additions.  Two tables (the signs), one counter per value from 2^-13 up to 2^15 in
-// magnitude; the values nearer to zero share a counter.  Only tokens at or above a bound are counted: all tokens below
-// M - T ln(V / ((1 - top_p) S)) together weigh at most (1 - top_p) S, so the cut lies at or above it.  Peaked rows then
-// count a few tokens.  What the pass waits for is the count: a warp's shared-memory atomic takes five to six cycles of the
-// SM whether twelve or twenty-four of its lanes count (with the integer instructions of the addresses
-// about 15 k cycles for a row of 152 k tokens; loads a round ahead do not help, nor does a closer bound from a sample).  Where a counter does not tell the values apart, or the counted mass
-// stays below the target by rounding, the radix search over the whole row gives the same result in four passes
-// (nucleus_row_radix).  Verification of 256 sequences x 16 nodes, V 151936: 588 us with a search of two passes and lists
-// per row, 327 us with this one.
+// the cut is found from the counts alone, values in falling order (nucleus_cut).  Only tokens at or above a bound are
+// counted: all tokens below M - T ln(V / ((1 - top_p) S)) together weigh at most (1 - top_p) S, so the cut lies at or above it,
+// and peaked rows count a few tokens.  What the pass waits for is the count: a warp's shared-memory atomic takes five to six
+// cycles of the SM whether twelve or twenty-four of its lanes count (with the integer instructions of the addresses about
+// 15 k cycles for a row of 152 k tokens; loads a round ahead do not help, nor does a closer bound from a sample).  Where a
+// counter does not tell the values apart, or the counted mass stays below the target by rounding, the radix search over the
+// whole row gives the same result in four passes (nucleus_row_radix).  Verification of 256 sequences x 16 nodes, V 151936:
+// 590 us with a search of two passes over the tokens per row, 325 us with this one.
 constexpr int NUC_OCT_LO = (127 - 13) << 7;              // bf16 bits of 2^-13
 constexpr int NUC_VALUES = ((127 + 15) << 7) - NUC_OCT_LO;  // counters per sign; 0: nearer to zero than 2^-13
 constexpr int NUC_SIGN = 8192;                           // the negative values' table, 2^15 bytes behind the other: the sign bit of a
@@ -322,8 +320,11 @@ struct NucleusSmem {
         float bins[16][NUC_THREADS];
     };
     float wsum[NUC_THREADS / 32][16];
-    double wtot[NUC_THREADS / 32];
-    int last;      // place of the last counter at which nucleus_scan's target was reached, -1: nowhere
+    unsigned long long wtot[NUC_THREADS / 32];
+    unsigned long long upto, inside;  // fixed-point mass up to and including the place of the cut; of its bin down to there
+    int last;      // place at which the fixed-point mass from the top reaches the target, -1: nowhere
+    uint32_t k_min, k_max;            // the bin's keys
+    float digit[16];
     int sel;       // bin selected by the last level
     float above, keep;
     uint32_t prefix;
@@ -447,54 +448,172 @@ __device__ __forceinline__ uint32_t nucleus_count_at(const NucleusSmem *st, int 
     return st->count[at] + (r == NUC_ZERO ? st->count[NUC_SIGN] : 0u);
 }
 
-// The first place of [r0, r1] at which the mass from r0 on reaches the target, by all threads of a CTA.  Result in
-// st->last (-1: not reached) and st->keep.
-__device__ void nucleus_scan(NucleusSmem *st, int r0, int r1, double target, float M, float c) {
+// The cut, from the counts of the places [r0, r1], by all threads of a CTA; false: it is not resolved by the counts.
+//   1  The place at which the mass from the top reaches the target, masses as 32-bit fixed point (the row's largest element is
+//      2^32), exact integer sums.  It names a bin of the distance below the maximum, 1/8 unit of log2 wide.
+//   2  Within the bin the cut is found digit by digit over the 16-bit key, in fp32 from the mass above the bin on.
+// (The steps of a search that adds up the tokens themselves, first in bins and then by digits: the cut follows the rounding
+// of its sums where a cumulative mass lies within 1e-7 of the target, so the arithmetic is the same.)
+__device__ bool nucleus_cut(NucleusSmem *st, int r0, int r1, float M, float c, float target) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    auto mass_at = [&](int r) {
+    const float Mc = M * c;
+    auto dist = [&](uint32_t bits) { return Mc - __uint_as_float(bits << 16) * c; };
+    auto bin = [&](float e) { return (int)(__float_as_uint(e * 8.0f + 12582912.0f) - 0x4B400000u); };  // (rounded to nearest)
+    auto fixed_at = [&](int r) {
         const uint32_t n = nucleus_count_at(st, r);
-        return (float)n * ex2_approx(fmaf(bf16_bits_to_float(nucleus_value(r)), c, -M * c));  // (an empty counter's value is finite)
+        if (n == 0u) return 0ull;
+        const float e = dist(nucleus_value(r));
+        return bin(e) < 256 ? (unsigned long long)n * __float2uint_rn(ex2_approx(-e) * 4294967296.0f) : 0ull;
     };
+    auto scan_u64 = [&](unsigned long long v) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long x = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += x;
+        }
+        return v;
+    };
+    const unsigned long long tgt = (unsigned long long)((double)target * 4294967296.0);
     const int per = (r1 - r0 + NUC_THREADS) / NUC_THREADS;  // (<= 14)
     const int my0 = r0 + tid * per, my1 = min(r1 + 1, my0 + per);
-    float part = 0.f;
-    for (int r = my0; r < my1; ++r) part += mass_at(r);
-    double incl = (double)part;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double x = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += x;
-    }
+    unsigned long long part = 0ull;
+    for (int r = my0; r < my1; ++r) part += fixed_at(r);
+    const unsigned long long incl = scan_u64(part);
     if (lane == 31) st->wtot[warp] = incl;
-    if (tid == 0) st->last = -1;
+    if (tid == 0) {
+        st->last = -1;
+        st->inside = 0ull;
+        st->k_min = 0xffffu;
+        st->k_max = 0u;
+    }
     __syncthreads();
-    // (a thread's end is formed as its successor's beginning, so that one thread at most holds the target)
-    double before = 0.0;
+    unsigned long long before = 0ull;
     for (int w = 0; w < warp; ++w) before += st->wtot[w];
-    const double up = __shfl_up_sync(0xffffffffu, incl, 1);
-    const double excl = lane ? before + up : before, end = before + incl;
-    const unsigned mine = __ballot_sync(0xffffffffu, excl < target && end >= target);
+    const unsigned long long end = before + incl, excl = end - part;
+    const unsigned mine = __ballot_sync(0xffffffffu, excl < tgt && end >= tgt);
     if (mine) {  // the counters of that thread, one per lane
         const int L = __ffs(mine) - 1;
-        const double e0 = __shfl_sync(0xffffffffu, excl, L);
+        const unsigned long long e0 = __shfl_sync(0xffffffffu, excl, L);
         const int f = __shfl_sync(0xffffffffu, my0, L), n = __shfl_sync(0xffffffffu, my1, L) - f;
-        const float m = lane < n ? mass_at(f + lane) : 0.f;
-        double cum = (double)m;
-#pragma unroll
-        for (int o = 1; o < 16; o <<= 1) {
-            const double x = __shfl_up_sync(0xffffffffu, cum, o);
-            if (lane >= o) cum += x;
-        }
-        cum += e0;
-        const unsigned hit = __ballot_sync(0xffffffffu, lane < n && cum >= target);
-        const unsigned pos = __ballot_sync(0xffffffffu, m > 0.f);
-        const int at = hit ? __ffs(hit) - 1 : 31 - __clz(pos);  // (no hit: rounding; the thread's mass is positive)
-        if (lane == at) {
-            st->last = f + at;
-            st->keep = (float)cum;
+        const unsigned long long cum = e0 + scan_u64(lane < n ? fixed_at(f + lane) : 0ull);
+        const unsigned hit = __ballot_sync(0xffffffffu, lane < n && cum >= tgt);
+        if (hit && lane == __ffs(hit) - 1) {
+            st->last = f + lane;
+            st->upto = cum;
         }
     }
     __syncthreads();
+    const int last = st->last;
+    if (last < 0) return false;
+    const int jb = bin(dist(nucleus_value(last)));
+    // this thread's places of the bin, [b0, b1) (the bins do not fall from place to place); sums over a warp go to shared memory
+    // as one addition (near zero a bin has thousands of places, and additions to one word wait for one another)
+    int b0 = my0, b1 = my0;
+    {
+        unsigned long long in = 0ull;
+        uint32_t lo = 0xffffu, hi = 0u;
+        for (int r = my0; r < my1; ++r) {
+            const int b = bin(dist(nucleus_value(r)));
+            if (b < jb) b0 = b1 = r + 1;
+            if (b != jb) continue;
+            b1 = r + 1;
+            if (nucleus_count_at(st, r) == 0u) continue;
+            if (r <= last) in += fixed_at(r);
+            const uint32_t key = ord_key(nucleus_value(r));
+            lo = min(lo, key);
+            hi = max(hi, key);
+        }
+        if (__any_sync(0xffffffffu, b1 > b0)) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) in += __shfl_xor_sync(0xffffffffu, in, o);
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if (lane == 0) {
+                atomicAdd(&st->inside, in);
+                atomicMin(&st->k_min, lo);
+                atomicMax(&st->k_max, hi);
+            }
+        }
+    }
+    __syncthreads();
+    const uint32_t k_min = st->k_min, k_max = st->k_max;
+    float cum = (float)((double)(st->upto - st->inside) * (1.0 / 4294967296.0));
+    float keep = cum;
+    uint32_t prefix = 0u;
+    for (int level = 0; level < 4; ++level) {
+        const int shift = 12 - 4 * level;
+        // (one digit for all of the bin: nothing to decide, except the last one's sum)
+        if (level < 3 && ((k_min ^ k_max) >> shift) == 0u) {
+            prefix = k_min >> shift;
+            continue;
+        }
+        __syncthreads();
+        if (tid < 16) st->digit[tid] = 0.f;
+        __syncthreads();
+        if (__any_sync(0xffffffffu, b1 > b0)) {
+            // a thread's places follow one another: a sum per digit, added when the digit changes or, where the warp has one
+            // digit, once for the warp
+            int dg = -1;
+            float sum = 0.f;
+            bool several = false;
+            for (int r = b0; r < b1; ++r) {
+                const uint32_t n = nucleus_count_at(st, r), bits = nucleus_value(r), key = ord_key(bits);
+                if (n == 0u || (level > 0 && (key >> (shift + 4)) != prefix)) continue;
+                const int d1 = (int)((key >> shift) & 15u);
+                if (d1 != dg && dg >= 0) {
+                    atomicAdd(&st->digit[dg], sum);
+                    sum = 0.f;
+                    several = true;
+                }
+                dg = d1;
+                sum += (float)n * ex2_approx((bf16_bits_to_float(bits) - M) * c);
+            }
+            const int top = __reduce_max_sync(0xffffffffu, dg);
+            if (__all_sync(0xffffffffu, !several && (dg == top || dg < 0))) {
+                sum = warp_sum(sum);
+                if (lane == 0 && top >= 0) atomicAdd(&st->digit[top], sum);
+            } else if (dg >= 0) {
+                atomicAdd(&st->digit[dg], sum);
+            }
+        }
+        __syncthreads();
+        // every thread for itself: digits from the largest on
+        float d[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) d[j] = st->digit[15 - j];
+        int sel = -1, lastd = 0;
+        float run = cum, tsel = 0.f;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            if (d[j] > 0.f) lastd = j;
+            if (sel < 0) {
+                if (run + d[j] >= target) {
+                    sel = j;
+                    tsel = d[j];
+                } else {
+                    run += d[j];
+                }
+            }
+        }
+        if (sel < 0) {  // (rounding kept the total below the target: the last digit with mass)
+            sel = lastd;
+            run = cum;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                if (j < lastd) run += d[j];
+                if (j == lastd) tsel = d[j];
+            }
+        }
+        cum = run;
+        keep = cum + tsel;
+        prefix = (prefix << 4) | (uint32_t)(15 - sel);
+    }
+    if (prefix == 0x8000u) return false;  // (the counter around zero: several values)
+    if (tid == 0) {
+        st->prefix = prefix;
+        st->keep = keep;
+    }
+    return true;
 }
 
 // n_cta > 1: the CTAs of a cluster share the pass, and its first CTA, which alone gets the result, adds their counts;
@@ -566,18 +685,13 @@ __device__ void nucleus_row(const uint16_t *__restrict__ row_logits, int V, floa
     } else {
         __syncthreads();
     }
-    nucleus_scan(st, r0, r1, (double)target, M, c);
-    const int last = st->last;
-    // The counter around zero: it must not be the cut, and its values must not differ by more than their mass's rounding
-    // if it lies above the cut.
-    bool ok = last >= 0 && last != NUC_ZERO;
-    if (ok && last > NUC_ZERO && r0 <= NUC_ZERO) {
+    bool ok = nucleus_cut(st, r0, r1, M, c, target);  // (the same for all threads)
+    // The counter around zero, if it lies above the cut: its values must not differ by more than their mass's rounding.
+    if (ok && r0 <= NUC_ZERO && st->last > NUC_ZERO) {
         const double m0 = (double)nucleus_count_at(st, NUC_ZERO) * (double)ex2_approx(-M * c);
-        ok = m0 * (double)(c * 0.6931472f) * 0x1p-13 <= 0x1p-24 * (double)S;
+        ok = m0 * (double)(c * 0.6931472f) * 0x1p-13 <= 0x1p-25 * (double)S;
     }
-    if (ok) {
-        if (tid == 0) st->prefix = ord_key(nucleus_value(last));
-    } else {
+    if (!ok) {
         __syncthreads();  // (all have read the counts)
         nucleus_row_radix(p, nvec, c, M, target, st);
     }
@@ -2259,7 +2373,6 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     int n_sm = 0;
     const int rc_sm = device_setup(nullptr, 0, &n_sm);
     if (rc_sm != SPECROLL_OK) return rc_sm;
-    const int resident = 8 * n_sm;  // CTAs of the statistics kernels
     if (use_runs) {
         // Up to 44 runs per SM (814 rows) the form with the rings; with more rows there are warps enough, and the ring's
         // bookkeeping costs issue slots (verification, V 152 k: 20 rows 29 -> 19 us, 256 rows 48 -> 34, 512 rows 54 -> 47,
@@ -2271,19 +2384,30 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
             const int per_sm = (grid + n_sm - 1) / n_sm, piece_bytes = RUN_WARPS * RUN_PIECE * (int)sizeof(uint4);
             int ring_n = 200 * 1024 / per_sm / piece_bytes;
             ring_n = ring_n < RUN_RING_MIN ? RUN_RING_MIN : ring_n > RUN_RING_MAX ? RUN_RING_MAX : ring_n;
-            const int rc_ = device_setup(reinterpret_cast<const void *>(run_stats_kernel), RUN_RING_MAX * piece_bytes, nullptr);
+            const int rc_ = device_setup(reinterpret_cast<const void *>(run_stats_kernel<false>), RUN_RING_MAX * piece_bytes, nullptr);
             if (rc_ != SPECROLL_OK) return rc_;
-            SR_CUDA_TRY(launch_dependent(true, run_stats_kernel, dim3((unsigned)grid), dim3(32 * RUN_WARPS), (size_t)ring_n * piece_bytes,
-                                         st, static_cast<const uint16_t *>(logits), d->V, c, n_runs, ring_n, run_tab));
+            SR_CUDA_TRY(launch_dependent(true, run_stats_kernel<false>, dim3((unsigned)grid), dim3(32 * RUN_WARPS),
+                                         (size_t)ring_n * piece_bytes, st, static_cast<const uint16_t *>(logits), d->V, c, n_runs, ring_n,
+                                         run_tab, (float *)nullptr, (float *)nullptr));
         } else {
             SR_CUDA_TRY(launch_dependent(true, row_stats_kernel, dim3((unsigned)rows), dim3(RS_THREADS), 0, st,
-                                         static_cast<const uint16_t *>(logits), d->V, c, 1, (float *)nullptr, (float *)nullptr, run_tab));
+                                         static_cast<const uint16_t *>(logits), d->V, c, (float *)nullptr, (float *)nullptr, run_tab));
         }
     } else if (!lazy) {
-        int n_cta = 8;
-        while (n_cta > 1 && (long long)rows * n_cta > resident) n_cta >>= 1;
-        SR_CUDA_TRY(launch_clusters(true, n_cta, row_stats_kernel, dim3((unsigned)(rows * n_cta)), dim3(RS_THREADS), 0, st,
-                                    static_cast<const uint16_t *>(logits), d->V, c, n_cta, row_max, row_sum, (float2 *)nullptr));
+        // up to four rows per SM by the form with the rings (20 rows of 152 k tokens 19 -> 8 us), more by a CTA per row
+        const int per_sm = (rows + n_sm - 1) / n_sm, piece_bytes = RS_WARPS * RUN_PIECE * (int)sizeof(uint4);
+        if (per_sm <= 4) {
+            int ring_n = 200 * 1024 / per_sm / piece_bytes;
+            if (ring_n > RUN_RING_MAX) ring_n = RUN_RING_MAX;
+            const int rc_ = device_setup(reinterpret_cast<const void *>(run_stats_kernel<true>), RUN_RING_MAX * piece_bytes, nullptr);
+            if (rc_ != SPECROLL_OK) return rc_;
+            SR_CUDA_TRY(launch_dependent(true, run_stats_kernel<true>, dim3((unsigned)rows), dim3(RS_THREADS), (size_t)ring_n * piece_bytes,
+                                         st, static_cast<const uint16_t *>(logits), d->V, c, rows * RS_WARPS, ring_n, (float2 *)nullptr,
+                                         row_max, row_sum));
+        } else {
+            SR_CUDA_TRY(launch_dependent(true, row_stats_kernel, dim3((unsigned)rows), dim3(RS_THREADS), 0, st,
+                                         static_cast<const uint16_t *>(logits), d->V, c, row_max, row_sum, (float2 *)nullptr));
+        }
     }
 
     WalkArgs wa;
