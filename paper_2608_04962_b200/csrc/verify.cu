@@ -307,7 +307,7 @@ constexpr int NUC_THREADS = 512;
 // 15 k cycles for a row of 152 k tokens; loads a round ahead do not help, nor does a closer bound from a sample).  Where a
 // counter does not tell the values apart, or the counted mass stays below the target by rounding, the radix search over the
 // whole row gives the same result in four passes (nucleus_row_radix).  Verification of 256 sequences x 16 nodes, V 151936:
-// 590 us with a search of two passes over the tokens per row, 325 us with this one.
+// 590 us with a search of two passes over the tokens per row, 350 us with this one.
 constexpr int NUC_OCT_LO = (127 - 13) << 7;              // bf16 bits of 2^-13
 constexpr int NUC_VALUES = ((127 + 15) << 7) - NUC_OCT_LO;  // counters per sign; 0: nearer to zero than 2^-13
 constexpr int NUC_SIGN = 8192;                           // the negative values' table, 2^15 bytes behind the other: the sign bit of a
@@ -324,6 +324,7 @@ struct NucleusSmem {
     unsigned long long upto, inside;  // fixed-point mass up to and including the place of the cut; of its bin down to there
     int last;      // place at which the fixed-point mass from the top reaches the target, -1: nowhere
     uint32_t k_min, k_max;            // the bin's keys
+    int p_min, p_max;                 // its places
     float digit[16];
     int sel;       // bin selected by the last level
     float above, keep;
@@ -485,6 +486,8 @@ __device__ bool nucleus_cut(NucleusSmem *st, int r0, int r1, float M, float c, f
         st->inside = 0ull;
         st->k_min = 0xffffu;
         st->k_max = 0u;
+        st->p_min = 0x7fffffff;
+        st->p_max = -1;
     }
     __syncthreads();
     unsigned long long before = 0ull;
@@ -533,6 +536,10 @@ __device__ bool nucleus_cut(NucleusSmem *st, int r0, int r1, float M, float c, f
                 atomicMin(&st->k_min, lo);
                 atomicMax(&st->k_max, hi);
             }
+            if (b1 > b0) {
+                atomicMin(&st->p_min, b0);
+                atomicMax(&st->p_max, b1 - 1);
+            }
         }
     }
     __syncthreads();
@@ -540,6 +547,47 @@ __device__ bool nucleus_cut(NucleusSmem *st, int r0, int r1, float M, float c, f
     float cum = (float)((double)(st->upto - st->inside) * (1.0 / 4294967296.0));
     float keep = cum;
     uint32_t prefix = 0u;
+    // Usually the bin has a few dozen places: their masses side by side in shared memory, and one thread takes the digits'
+    // sums in falling order, about a thousand cycles (with a barrier and an addition in shared memory per digit and thread
+    // the digits took 12 k).
+    const int p0 = st->p_min, np = st->p_max - p0 + 1;
+    float *const f = &st->wsum[0][0];
+    if (np <= (NUC_THREADS / 32) * 16 && (p0 > NUC_ZERO || p0 + np <= NUC_ZERO)) {  // (all of one sign)
+        for (int r = b0; r < b1; ++r)
+            f[r - p0] = (float)nucleus_count_at(st, r) * ex2_approx((bf16_bits_to_float(nucleus_value(r)) - M) * c);
+        __syncthreads();
+        if (tid == 0) {
+            const uint32_t key0 = ord_key(nucleus_value(p0));  // (the keys fall by one from place to place)
+            int lo = 0, hi = np;
+            for (int shift = 12; shift >= 0; shift -= 4) {
+                if (shift > 0 && ((k_min ^ k_max) >> shift) == 0u) continue;
+                float run = cum, before = cum, tsel = 0.f;
+                int s_lo = lo, s_hi = hi;
+                for (int i = lo; i < hi;) {
+                    const int j = min(hi, i + (int)((key0 - i) & ((1u << shift) - 1u)) + 1);
+                    float sum = 0.f;
+#pragma unroll 8
+                    for (int q = i; q < j; ++q) sum += f[q];
+                    if (sum > 0.f) {
+                        s_lo = i;
+                        s_hi = j;
+                        tsel = sum;
+                        before = run;
+                        if (run + sum >= target) break;
+                        run += sum;
+                    }
+                    i = j;
+                }
+                cum = before;  // (none reached the target by rounding: the last digit with mass)
+                keep = cum + tsel;
+                lo = s_lo;
+                hi = s_hi;
+            }
+            st->prefix = key0 - lo;
+            st->keep = keep;
+        }
+        return true;
+    }
     for (int level = 0; level < 4; ++level) {
         const int shift = 12 - 4 * level;
         // (one digit for all of the bin: nothing to decide, except the last one's sum)
