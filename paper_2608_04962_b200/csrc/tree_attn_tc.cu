@@ -132,7 +132,10 @@ __device__ __forceinline__ unsigned short bf16_bits_rn(float x) {
 __device__ __forceinline__ float bf16_bits_to_float(unsigned short b) { return __uint_as_float((uint32_t)b << 16); }
 }  // namespace attc
 
-template <int D, bool TEAMS>
+// ONE: every CTA has one unit at most (few sequences): the second Q buffer is free for the hand-over area, and nothing is
+// counted - the merge, if any, is a kernel of its own - so the CTA leaves without a round trip to memory.  (A template flag:
+// asked at run time it cost the shapes with many units 1-4 %.)
+template <int D, bool TEAMS, bool ONE>
 __global__ void __launch_bounds__(attc::Cfg<D, TEAMS>::THREADS, 1)
 tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKt,
@@ -156,9 +159,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     volatile int *tickets = reinterpret_cast<volatile int *>(extra + 8);
     unsigned char *xch_base = extra + 16;
     volatile UnitDesc *ring = reinterpret_cast<volatile UnitDesc *>(extra + 16 + C::XCH_BYTES);  // 2 slots of 64 bytes
-    // Every CTA has one unit at most (few sequences): the second Q buffer is free for the hand-over area, and nothing
-    // is counted - the merge, if any, is a kernel of its own - so the CTA leaves without a round trip to memory.
-    const bool one_wave = a.total_work <= (int)gridDim.x && a.merge_mode != 0;
+    constexpr bool one_wave = ONE;
     // [l of team 0 | l of team 1 | m of team 0 | m of team 1][128 rows]
     float *hand = a.hand + (size_t)blockIdx.x * C::HAND_FLOATS;
     volatile float *hand_s = reinterpret_cast<volatile float *>(aligned + C::Q_BYTES);
@@ -1131,9 +1132,11 @@ static int launch_tc(const AttnArgs &a, const TopoMask &mask, long long T_kv, in
     if ((rc = make_tmap_3d_bf16(&tmKt, a.Kt, D, a.Hkv, tree_rows, 1, attc::BN)) != SPECROLL_OK) return rc;
     if ((rc = make_tmap_3d_bf16(&tmVt, a.Vt, D, a.Hkv, tree_rows, 1, attc::BN)) != SPECROLL_OK) return rc;
     int n_sm = 0;
-    if ((rc = device_setup(reinterpret_cast<const void *>(tree_attn_tc_kernel<D, TEAMS>), C::SMEM, &n_sm)) != SPECROLL_OK) return rc;
+    if ((rc = device_setup(nullptr, 0, &n_sm)) != SPECROLL_OK) return rc;
     const int ctas = n_sm < ATTN_HAND_CTAS ? n_sm : ATTN_HAND_CTAS;  // every CTA has a hand-over area of its own
     const unsigned grid = (unsigned)(a.total_work < ctas ? a.total_work : ctas);
+    auto *const kern = a.total_work <= (int)grid && a.merge_mode != 0 ? tree_attn_tc_kernel<D, TEAMS, true> : tree_attn_tc_kernel<D, TEAMS, false>;
+    if ((rc = device_setup(reinterpret_cast<const void *>(kern), C::SMEM, nullptr)) != SPECROLL_OK) return rc;
     // Programmatic stream serialization: the CTAs may be set up (barriers, tensor memory, zeroed Q buffers) while
     // the kernel before this one in the stream is still running its last CTAs; the kernel itself waits for
     // that kernel's completion before it reads anything (griddepcontrol.wait).
@@ -1147,7 +1150,7 @@ static int launch_tc(const AttnArgs &a, const TopoMask &mask, long long T_kv, in
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = a.no_pdl ? 0 : 1;
-    SR_CUDA_TRY(cudaLaunchKernelEx(&cfg, tree_attn_tc_kernel<D, TEAMS>, tmQ, tmK, tmV, tmKt, tmVt, a, mask, status));
+    SR_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, tmQ, tmK, tmV, tmKt, tmVt, a, mask, status));
     SR_LAUNCH_CHECK();
     return SPECROLL_OK;
 }
