@@ -778,7 +778,9 @@ static int run_tree_attn(const specroll_attn_desc *d, const void *Q, const void 
     a.early_cache = ((d->flags & SPECROLL_ATTN_CACHE_SETTLED) && (d->flags & SPECROLL_ATTN_REUSE_PLAN)) ? 1 : 0;
     if (!(p.use_tc && (d->flags & SPECROLL_ATTN_REUSE_PLAN))) {
         // (the tcgen05 kernel leaves its scheduling counters cleared, so a kept plan can be run again as is)
-        SR_CUDA_TRY(launch_dependent(true, attn_prep_kernel, dim3(1), dim3(PREP_THREADS), 0, st, kv_indptr_dev,
+        // (set up under the end of the kernel before only where the call is a chain of latencies: a layer of many units takes
+        // hundreds of microseconds)
+        SR_CUDA_TRY(launch_dependent(p.items * d->Hkv * p.n_rb <= PLAN_SMS, attn_prep_kernel, dim3(1), dim3(PREP_THREADS), 0, st, kv_indptr_dev,
                                      paged ? kv_len_dev : nullptr, page_indptr_dev, d->B, p.chunk_tiles, p.tile_tokens,
                                      reinterpret_cast<int32_t *>(ws + p.off_items), p.use_tc ? sorted_start : nullptr,
                                      seq_at_rank, p.use_tc ? unit_tab : nullptr, status, counters, p.n_counters));
