@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g, cons
         }
         __syncthreads();
         const int nh = n_hit;
+        __syncthreads();  // (all have read it before the next records are counted)
         if (nh == 0) continue;
         // in record order
         for (int e = tid; e < nh; e += GATE_THREADS) {

@@ -125,3 +125,32 @@ def test_sketches_at_the_ends_of_the_ranges(R, d, rank):
     Pi = g.standard_normal((rank, d)).astype(np.float32)
     X = g.standard_normal((R, d)).astype(np.float32)
     np.testing.assert_allclose(host(S.reflex_sketch(dev(X), dev(Pi))), ref.reflex_sketch(X, Pi), rtol=0, atol=2e-5)
+
+
+@pytest.mark.parametrize("R,S_,kind", [(1500, 1500, "own"), (1500, 1500, "shuffled"), (1100, 700, "last"), (1025, 3, "last")])
+def test_slots_whose_records_lie_in_later_batches(R, S_, kind):
+    """A slot's records are looked for 512 at a time: slots without a record in the first batch or the first two, and slots
+    without any.  Bounds as in test_gate."""
+    g = I.rng(300 + R + S_)
+    rank, d = 24, 64
+    s = g.standard_normal((R, rank)).astype(np.float32)
+    xi = (0.7 * s + g.standard_normal((R, rank))).astype(np.float32)
+    slot = np.arange(R) % S_
+    if kind == "shuffled":
+        slot = g.permutation(slot)
+    elif kind == "last":  # slot 0 has all records but the last of them
+        slot = np.where(np.arange(R) < 1024, 0, 1 + np.arange(R) % (S_ - 1))
+    slot = slot.astype(np.int32)
+    m = g.standard_normal((S_, d)).astype(np.float32)
+    n0 = g.integers(0, 5, size=S_).astype(np.int32)
+    mean0 = (0.2 * g.standard_normal(S_)).astype(np.float32)
+    M20 = (0.1 * g.random(S_) * np.maximum(n0 - 1, 0)).astype(np.float32)
+    horizon, need = np.zeros(S_, np.int32), np.array([2], np.int32)
+    lo, hi = np.array([0.01], np.float32), np.array([0.025], np.float32)
+    o = ref.reflex_gate(s, xi, slot, None, n0, mean0, M20, n0, m, horizon, need, need, lo, hi, z_delta=0.6)
+    dn, dmean, dM2, dnfb = dev(n0.copy()), dev(mean0.copy()), dev(M20.copy()), dev(n0.copy())
+    S.reflex_gate(dev(s), dev(xi), dev(slot), None, dn, dmean, dM2, dnfb, dev(m), dev(horizon), dev(need), dev(need), dev(lo),
+                  dev(hi), z_delta=0.6)
+    assert np.array_equal(host(dn), o["n"]) and np.array_equal(host(dnfb), o["n_fb"])
+    np.testing.assert_allclose(host(dmean), o["mean"], rtol=0, atol=2e-5)
+    np.testing.assert_allclose(host(dM2), o["M2"], rtol=2e-4, atol=2e-5)
