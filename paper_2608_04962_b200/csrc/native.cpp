@@ -201,16 +201,18 @@ class Out {
 
 void *stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-// The C call itself runs without the interpreter lock, as a ctypes call does.
-#define CALL(name, ...)                  \
-    do {                                 \
-        void *st_ = stream();            \
-        int rc_;                         \
-        Py_BEGIN_ALLOW_THREADS           \
-        rc_ = lib.name(__VA_ARGS__, st_); \
-        Py_END_ALLOW_THREADS             \
-        check(rc_, #name);               \
-    } while (0)
+// The C call itself runs without the interpreter lock, as a ctypes call does.  Its arguments are evaluated before the lock is
+// given up (they may raise, or turn Python objects into numbers), and it is taken back however the call ends.
+struct Unlocked {
+    PyThreadState *state = PyEval_SaveThread();
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+template <class F, class... Args>
+int call_unlocked(F *entry, Args... args) {
+    Unlocked u;
+    return entry(args...);
+}
+#define CALL(name, ...) check(call_unlocked(lib.name, __VA_ARGS__, stream()), #name)
 
 // ------------------------------------------------------------------------------ proposal
 
