@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(256) target_head_merge_kernel(const float *__r
                                                                 int n_groups, float c_log2, float *__restrict__ row_max,
                                                                 float *__restrict__ row_sum) {
     pdl_wait();
-    pdl_launch_dependents();  // (what follows reads the projection's other results ahead of its own wait)
+    pdl_launch_dependents();
     const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (r >= M) return;
     float m = -INFINITY, s = 0.f;

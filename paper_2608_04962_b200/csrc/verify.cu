@@ -2170,8 +2170,9 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     double *slices = reinterpret_cast<double *>(sh_dyn + L.slices);
     double *wp = reinterpret_cast<double *>(sh_dyn + L.p);
     const double inv_T = 1.0 / a.T;
-    // (1) inputs of this call, none of them written by the kernel before this one (the statistics, or the projection's merge,
-    // which itself waits for the projection before it lets this kernel start)
+    // (1) inputs of this call, none of them written by the kernel before this one where that is the call's own (the
+    // statistics).  TILES: whatever the caller has put in front of the call may still be writing them.
+    if (TILES) pdl_wait();
     const WalkSlots slots = walk_slots(sh_dyn + L.slots, N, k);
     __shared__ int sh_odd;
     if (tid == 0) sh_odd = k > 32;
