@@ -448,8 +448,9 @@ int specroll_verify(const specroll_verify_desc *desc, const void *logits,
  *                                every sequence's terminal node, with the same workspace.
  *   specroll_verify_hidden  walk and last token in one launch, from the wanted logits and the tile masses of
  *                                specroll_target_head_stats_tiles: the logits of the one tile of 128 tokens that holds the
- *                                drawn token are made from hidden[B*N, d] and W[V, d] (fp32 sums rounded to bf16; their
- *                                order differs from the projection's).  No workspace; d % 8 == 0.
+ *                                drawn token are made again from hidden[B*N, d] and W[V, d], the projection's own to the
+ *                                bit.  No workspace; d % 8 == 0; a bounded wait that runs out leaves -1 in the place of
+ *                                the sequence's last token.
  * The workspace has specroll_verify_workspace_bytes(desc) bytes; desc.flags must be 0. */
 int specroll_verify_want_ids(const specroll_verify_desc *desc, const int32_t *parent_host,
                              const int32_t *cand_id, int32_t *want_id, void *cuda_stream);

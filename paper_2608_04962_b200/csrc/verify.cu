@@ -16,6 +16,7 @@
 // walk_kernel / walk_cta_kernel and terminal_kernel.
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -1948,6 +1949,8 @@ nucleus_rows_kernel(const uint16_t *__restrict__ logits, int V, int N, NodeList 
 constexpr int WT_THREADS = TERM_THREADS;
 constexpr int WT_SMEM_LIMIT = 160 * 1024;
 constexpr int WT_WARPS = WT_THREADS / 32;
+constexpr int WT_STATIC_SMEM = WT_WARPS * (int)sizeof(WalkSmem) + 2048;       // (at most)
+constexpr int TILE_SMEM_LIMIT = 227 * 1024 - WT_STATIC_SMEM;                  // dynamic, of the form without stored logits
 
 // Every node with children on its own.  first[u]: accepted child or -1, mm[u]: smallest margin, ovm[u, j]: the residual's
 // masses where all children were rejected.  (A warp per node took 9 k
@@ -2010,52 +2013,70 @@ __host__ __device__ inline WtLayout wt_layout(int N, int K, int k, size_t draw_b
 // The terminal draw without the logits row: the masses of the row's vocabulary tiles are known (mass, per tile and row:
 // maximum and sum), and the logits of the one tile that holds the target are made here, from the row's hidden state and 128
 // rows of W (a few hundred KB to a MB; the storing projection, with all of W, took 178 us for 32 sequences of the 7B
-// shape).  fp32 sums rounded to bf16, as the projection's; the order of a sum's terms differs from the tensor pipe's, so a
-// token's mass may be that of the neighbouring bf16 value and the draw turn where its target lies that close to a bound.
+// shape).  They are the projection's own logits to the bit: the same tensor operations over the same slices of the
+// contraction, with the tokens as M and the hidden row as the first of N = 16.  (Sums of another order, in fp32 by all threads,
+// rounded to the neighbouring bf16 value now and then, and the draw turned or the difference fell to the tile's last token.)
+// Bound by the latency of the ring's loads, one CTA per sequence.
+namespace dt {
+constexpr int ROWS = 16, BK = 64, UMMA_K = 16, MAX_STAGES = 8, MIN_STAGES = 2;
+constexpr int W_BYTES = HEAD_TILE * BK * 2, H_BYTES = ROWS * BK * 2, STAGE_BYTES = W_BYTES + H_BYTES;
+constexpr int TMEM_COLS = 32;
+}  // namespace dt
 struct TileArgs {
-    const __nv_bfloat16 *H, *W;  // [B * N, d], [V, d]
-    const float2 *mass;          // [tiles][B * N]
-    int32_t d, rows;
+    CUtensorMap H, W;    // [B * N, d] in boxes of dt::ROWS rows, [V, d] in boxes of HEAD_TILE
+    const float2 *mass;  // [tiles][B * N]
+    int32_t d, rows, stages;
 };
-__host__ __device__ inline size_t tile_smem_bytes(int V, int d) {
-    return ((size_t)(V + HEAD_TILE - 1) / HEAD_TILE + HEAD_TILE) * sizeof(double) + 16 + (size_t)d * 2;
-}
 
-// By all threads of the n_cta CTAs of a cluster, which share the tile's tokens; smem: tile_smem_bytes, at the same offset in
-// every CTA.  bits(j): the bf16 logit of the residual's token j.
+// By all threads of a CTA.  tok: HEAD_TILE doubles; ring: 1024-byte aligned, t.stages * dt::STAGE_BYTES.  bits(j): the bf16 logit of
+// the residual's token j.  *dst is -1 where a bounded wait ran out.
 template <class Bits>
-__device__ void draw_tile(const TileArgs &t, size_t row, int V, float M, float c, int n_cta, int rank, int nov, const int32_t *ovid,
-                          const double *ovm, Bits bits, unsigned char *smem, float u, int32_t *dst) {
+__device__ void draw_tile(const TileArgs &t, size_t row, int V, float M, float c, int nov, const int32_t *ovid, const double *ovm,
+                          Bits bits, double *tok, uint32_t ring, float u, int32_t *dst) {
+    using namespace dt;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n_tiles = (V + HEAD_TILE - 1) / HEAD_TILE;
-    double *mt = reinterpret_cast<double *>(smem);  // masses of the tiles, then of the tile's tokens
-    double *tok = mt + n_tiles;
-    uint4 *h = reinterpret_cast<uint4 *>(smem + (((size_t)n_tiles + HEAD_TILE) * sizeof(double) + 15) / 16 * 16);
     __shared__ double seg[TERM_WARPS], sh_base[2];
     __shared__ int sh_tile, sh_last;
-    for (int i = tid; i < n_tiles; i += TERM_THREADS) {
+    __shared__ __align__(8) unsigned long long bars[2 * MAX_STAGES + 1];
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int abort_flag;
+    auto full_bar = [&](int s) { return smem_u32(&bars[s]); };
+    auto empty_bar = [&](int s) { return smem_u32(&bars[MAX_STAGES + s]); };
+    const uint32_t done_bar = smem_u32(&bars[2 * MAX_STAGES]);
+    if (tid == 0) {
+        for (int s = 0; s < t.stages; ++s) {
+            mbar_init(full_bar(s), 1);
+            mbar_init(empty_bar(s), 1);
+        }
+        mbar_init(done_bar, 1);
+        abort_flag = 0;
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(smem_u32(&tmem_slot), TMEM_COLS);
+        tmem_relinquish();
+    }
+    auto tile_mass = [&](int i) {
         const float2 e = t.mass[(size_t)i * t.rows + row];
         // (the tokens' exponents were formed with -m c rounded, as those of the tile at hand below are with -M c)
-        mt[i] = e.x == NEG_INF ? 0.0 : (double)e.y * exp2((double)(e.x * c) - (double)(M * c));
-    }
-    const int d8 = t.d >> 3;
-    for (int i = tid; i < d8; i += TERM_THREADS) h[i] = reinterpret_cast<const uint4 *>(t.H + row * t.d)[i];
-    __syncthreads();
-    if (tid == 0)
-        for (int j = 0; j < nov; ++j) {
-            double &m = mt[ovid[j] / HEAD_TILE];
-            m = fmax(m + ovm[j] - (double)mass1(bits(j), M, c, 0u), 0.0);  // (a tile whose mass was all in replaced tokens, after rounding)
-        }
-    __syncthreads();
-    // a run of tiles per warp, then the tile within the run; every CTA for itself
+        double m = e.x == NEG_INF ? 0.0 : (double)e.y * exp2((double)(e.x * c) - (double)(M * c));
+        for (int j = 0; j < nov; ++j)
+            if (ovid[j] / HEAD_TILE == i) m += ovm[j] - (double)mass1(bits(j), M, c, 0u);
+        return fmax(m, 0.0);  // (a tile whose mass was all in replaced tokens, after rounding)
+    };
+    // a run of tiles per warp, then the tile within the run
     const int per = (n_tiles + TERM_WARPS - 1) / TERM_WARPS;
     {
         double x = 0.0;
-        for (int i = warp * per + lane; i < min(n_tiles, (warp + 1) * per); i += 32) x += mt[i];
+        for (int i = warp * per + lane; i < min(n_tiles, (warp + 1) * per); i += 32) x += tile_mass(i);
         x = warp_sum(x);
         if (lane == 0) seg[warp] = x;
     }
+    tc_fence_before();
     __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
     if (warp == 0) {
         const double v = lane < TERM_WARPS ? seg[lane] : 0.0;
         double incl = warp_incl_scan(v, lane);
@@ -2067,7 +2088,7 @@ __device__ void draw_tile(const TileArgs &t, size_t row, int V, float M, float c
         int at = -1, at_pos = min(w * per, n_tiles - 1);
         double base_pos = base;
         for (int i0 = w * per; i0 < min(n_tiles, (w + 1) * per) && at < 0; i0 += 32) {
-            const double x = i0 + lane < min(n_tiles, (w + 1) * per) ? mt[i0 + lane] : 0.0;
+            const double x = i0 + lane < min(n_tiles, (w + 1) * per) ? tile_mass(i0 + lane) : 0.0;
             incl = warp_incl_scan(x, lane);
             hit = last ? 0u : __ballot_sync(0xffffffffu, base + incl > target);
             pos = __ballot_sync(0xffffffffu, x > 0.0);
@@ -2095,45 +2116,66 @@ __device__ void draw_tile(const TileArgs &t, size_t row, int V, float M, float c
         }
     }
     __syncthreads();
-    // the tile's logits: a warp per pair of tokens, the pairs spread over the cluster's warps
-    const int v0 = sh_tile * HEAD_TILE, n_tok = min(HEAD_TILE, V - v0);
-    for (int q = (rank * TERM_WARPS + warp) * 2; q < HEAD_TILE; q += n_cta * TERM_WARPS * 2) {
-        float acc[2] = {0.f, 0.f};
-        const uint4 *w0 = reinterpret_cast<const uint4 *>(t.W + (size_t)min(v0 + q, V - 1) * t.d);
-        const uint4 *w1 = reinterpret_cast<const uint4 *>(t.W + (size_t)min(v0 + q + 1, V - 1) * t.d);
-#pragma unroll 4
-        for (int i = lane; i < d8; i += 32) {
-            const uint4 x[2] = {ld_nc_v4(w0 + i), ld_nc_v4(w1 + i)};
-            const uint4 y = h[i];
-            const uint32_t yw[4] = {y.x, y.y, y.z, y.w};
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const uint32_t xw[4] = {x[e].x, x[e].y, x[e].z, x[e].w};
-#pragma unroll
-                for (int z = 0; z < 4; ++z) {
-                    acc[e] = fmaf(__uint_as_float(xw[z] << 16), __uint_as_float(yw[z] << 16), acc[e]);
-                    acc[e] = fmaf(__uint_as_float(xw[z] & 0xffff0000u), __uint_as_float(yw[z] & 0xffff0000u), acc[e]);
+    // the tile's logits: D[token, 0] = W[token, :] . hidden row
+    const int v0 = sh_tile * HEAD_TILE, n_tok = min(HEAD_TILE, V - v0), KB = (t.d + BK - 1) / BK;
+    if (warp == 0) {
+        if (lane == 0) {
+            int kb = 0;
+            for (; kb < KB; ++kb) {
+                const int s = kb % t.stages;
+                if (!mbar_wait(empty_bar(s), ((uint32_t)(kb / t.stages) & 1u) ^ 1u, &abort_flag)) break;
+                const uint32_t sw = ring + s * STAGE_BYTES;
+                mbar_arrive_expect_tx(full_bar(s), STAGE_BYTES);
+                tma_load_2d(sw, &t.W, kb * BK, v0, full_bar(s));
+                tma_load_2d(sw + W_BYTES, &t.H, kb * BK, (int)row, full_bar(s));
+            }
+            if (kb < KB)  // aborting: let the copies already in flight land before the CTA goes away
+                for (int q = max(0, kb - t.stages); q < kb; ++q) {
+                    const unsigned long long t0 = globaltimer_ns();
+                    while (!mbar_try_wait(full_bar(q % t.stages), (uint32_t)(q / t.stages) & 1u) && globaltimer_ns() - t0 < 100000000ull) {
+                    }
                 }
-            }
         }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = idesc_bf16(HEAD_TILE, ROWS, false, false);
+            bool ok = true;
+            for (int kb = 0; kb < KB && ok; ++kb) {
+                const int s = kb % t.stages;
+                ok = mbar_wait(full_bar(s), (uint32_t)(kb / t.stages) & 1u, &abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t sw = ring + s * STAGE_BYTES;
+                const uint64_t adesc = smem_desc_sw128(sw, 1024, 0), bdesc = smem_desc_sw128(sw + W_BYTES, 1024, 0);
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const float l = warp_sum(acc[e]);
-            if (lane == 0) tok[q + e] = q + e < n_tok ? (double)mass1(__bfloat16_as_ushort(__float2bfloat16_rn(l)), M, c, 0u) : 0.0;
+                for (int kk = 0; kk < BK / UMMA_K; ++kk) umma_ss(tmem, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+                umma_commit(empty_bar(s));
+            }
+            if (ok) umma_commit(done_bar);
+        }
+    } else if (warp < 6) {
+        const int at = (warp & 3) * 32;  // the TMEM lanes this warp may read
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(done_bar, 0u, &abort_flag));
+        tc_fence_after();
+        if (ok) {
+            uint32_t r[32];
+            tmem_ld32(tmem + ((uint32_t)at << 16), r);
+            tmem_ld_wait();
+            tok[at + lane] = at + lane < n_tok ? (double)mass1(__bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(r[0]))), M, c, 0u) : 0.0;
         }
     }
-    if (n_cta > 1) {
-        cluster_sync_all();
-        if (rank == 0)
-            for (int q = tid; q < HEAD_TILE; q += TERM_THREADS) {
-                const int r = (q / 2 / TERM_WARPS) % n_cta;
-                if (r > 0) tok[q] = ld_dsmem_f64(tok + q, r);
-            }
-        cluster_sync_all();  // the other CTAs may leave
-        if (rank != 0) return;
-    }
+    tc_fence_before();
     __syncthreads();
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        tmem_dealloc(tmem, TMEM_COLS);
+    }
     if (warp != 0) return;
+    if (abort_flag) {
+        if (lane == 0) *dst = -1;
+        return;
+    }
     double ms[8], lsum = 0.0;
 #pragma unroll
     for (int e = 0; e < 8; ++e) ms[e] = lane * 8 < HEAD_TILE ? tok[lane * 8 + e] : 0.0;
@@ -2152,14 +2194,14 @@ __device__ void draw_tile(const TileArgs &t, size_t row, int V, float M, float c
 template <bool TILES>
 __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, Topo topo, const float *__restrict__ u_fin, float c,
                                                                int S, const float2 *__restrict__ run_tab, float *__restrict__ row_max_w,
-                                                               float *__restrict__ row_sum_w, TileArgs tile) {
+                                                               float *__restrict__ row_sum_w, const __grid_constant__ TileArgs tile) {
     __shared__ WalkSmem sh[WT_WARPS];
     extern __shared__ __align__(16) unsigned char sh_dyn[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = S > 1 ? (int)cluster_ctarank() : 0;
     const int b = blockIdx.x / S;
     const int N = a.N, K = a.K, k = a.k;
-    const WtLayout L = wt_layout(N, K, k, TILES ? tile_smem_bytes(a.V, tile.d) : draw_smem_bytes(a.V, S));
+    const WtLayout L = wt_layout(N, K, k, TILES ? HEAD_TILE * sizeof(double) : draw_smem_bytes(a.V, S));
     const WalkBuf buf = walk_buf(sh_dyn + L.stage, N, K, k);
     float *rmax = buf.rmax, *rsum = buf.rsum;
     const int32_t *ttok = buf.ttok, *cid = buf.cid;
@@ -2280,8 +2322,8 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     const double *ovm_u = ovm + u * k;
     const float M = rmax[u];
     if constexpr (TILES) {
-        draw_tile(tile, (size_t)b * N + u, a.V, M, c, S, rank, nov, ovid, ovm_u, [&](int j) { return pre[u * k + j]; },
-                  sh_dyn + L.slices, u_fin[b], a.out_tok + (size_t)b * (K + 1) + nacc);
+        draw_tile(tile, (size_t)b * N + u, a.V, M, c, nov, ovid, ovm_u, [&](int j) { return pre[u * k + j]; }, slices,
+                  (smem_u32(sh_dyn + L.total) + 1023u) & ~1023u, u_fin[b], a.out_tok + (size_t)b * (K + 1) + nacc);
         return;
     }
     const uint16_t *lg = a.logits + ((size_t)b * N + u) * a.V;
@@ -2648,16 +2690,24 @@ extern "C" int specroll_verify_hidden(const specroll_verify_desc *d, int32_t dim
     wa.k = d->k;
     wa.V = d->V;
     wa.T = (double)d->temperature;
-    const TileArgs tile{static_cast<const __nv_bfloat16 *>(hidden), static_cast<const __nv_bfloat16 *>(W),
-                        static_cast<const float2 *>(tile_mass), dim, d->B * d->N};
-    const int S = walk_term_split(d->B);
-    const WtLayout L = wt_layout(d->N, d->K, d->k, tile_smem_bytes(d->V, dim));
-    if (L.total > (size_t)WT_SMEM_LIMIT) return SPECROLL_ELIMIT;
-    const int rc = device_setup(reinterpret_cast<const void *>(walk_term_kernel<true>), WT_SMEM_LIMIT, nullptr);
+    const WtLayout L = wt_layout(d->N, d->K, d->k, HEAD_TILE * sizeof(double));
+    int n_sm = 0;
+    int rc = device_setup(reinterpret_cast<const void *>(walk_term_kernel<true>), TILE_SMEM_LIMIT, &n_sm);
     if (rc != SPECROLL_OK) return rc;
-    SR_CUDA_TRY(launch_clusters(true, S, walk_term_kernel<true>, dim3((unsigned)(d->B * S)), dim3(WT_THREADS), L.total,
-                                static_cast<cudaStream_t>(cuda_stream), wa, topo, u_fin, (float)(1.4426950408889634 / (double)d->temperature),
-                                S, (const float2 *)nullptr, (float *)nullptr, (float *)nullptr, tile));
+    // a ring as deep as fits beside the walk, with room for a second CTA on an SM where there are more sequences than SMs
+    TileArgs tile;
+    const int room = (d->B > n_sm ? TILE_SMEM_LIMIT / 2 - WT_STATIC_SMEM / 2 - 1024 : TILE_SMEM_LIMIT) - (int)L.total - 1024;
+    tile.stages = std::max(dt::MIN_STAGES, std::min(dt::MAX_STAGES, room / dt::STAGE_BYTES));
+    const size_t smem = L.total + 1024 + (size_t)tile.stages * dt::STAGE_BYTES;
+    if (smem > (size_t)TILE_SMEM_LIMIT) return SPECROLL_ELIMIT;
+    tile.mass = static_cast<const float2 *>(tile_mass);
+    tile.d = dim;
+    tile.rows = d->B * d->N;
+    if ((rc = make_tmap_2d_bf16(&tile.H, hidden, (uint64_t)tile.rows, (uint64_t)dim, (uint64_t)dim, dt::ROWS)) != SPECROLL_OK) return rc;
+    if ((rc = make_tmap_2d_bf16(&tile.W, W, (uint64_t)d->V, (uint64_t)dim, (uint64_t)dim, HEAD_TILE)) != SPECROLL_OK) return rc;
+    SR_CUDA_TRY(launch_dependent(true, walk_term_kernel<true>, dim3((unsigned)d->B), dim3(WT_THREADS), smem,
+                                 static_cast<cudaStream_t>(cuda_stream), wa, topo, u_fin, (float)(1.4426950408889634 / (double)d->temperature),
+                                 1, (const float2 *)nullptr, (float *)nullptr, (float *)nullptr, tile));
     return SPECROLL_OK;
 }
 

@@ -70,3 +70,25 @@ def test_fused_path_equals_the_path_through_stored_logits(name, B, V, d, T):
 def test_last_token_from_one_tile(name, B, V, d, T):
     """One to eight CTAs per sequence; vocabularies below, at and above one tile, with a ragged last one."""
     test_fused_path_equals_the_path_through_stored_logits(name, B, V, d, T)
+
+
+@pytest.mark.parametrize("name,B,V,d,T", [("tiny", 300, 4104, 512, 1.0), ("qwen7b", 20, 40008, 64, 0.7), ("tiny", 150, 264, 4096, 1.3),
+                                          ("tiny", 2, 8, 128, 1.0)])
+def test_last_token_follows_the_projections_own_logits(name, B, V, d, T):
+    """Two large products that cancel, one at either end of the contraction: a logit then follows the order of its sum by many
+    bf16 steps, and a last token drawn from logits of another order is often another token.  Compared with the oracle on the
+    stored logits of the same projection; excluded are draws within 3e-6 of a bound (the tiles' masses are fp32 sums of
+    exponentials with a relative error of 1e-6) and walks within 1e-4 of a uniform."""
+    w, parent, H, W, _, cid, cl, dr, u_acc, u_fin = _case(name, B, V, d, T, 190 + B)
+    big, a = I.f32_to_bf16_bits(np.float32([8192.0, -1.0])), I.f32_to_bf16_bits(I.rng(3).standard_normal(V).astype(np.float32))
+    H[:, :, 0] = H[:, :, -1] = big[0]
+    W[:, 0], W[:, -1] = a, a ^ np.uint16(0x8000)
+    dH, dW = dev_bf16(H), dev_bf16(W)
+    args = (parent, dev(dr["tree_tok"]), dev(dr["tree_cand"]), dev(cid), dev(cl), dev(u_acc), dev(u_fin))
+    f = {k: host(v) for k, v in S.verify_fused(dH, dW, *args, temperature=T).items()}
+    logits = S.bf16_bits(S.target_head_rows(dH.reshape(B * w.N, d), dW)).reshape(B, w.N, V)
+    o = ref.verify(logits, parent, dr["tree_tok"], dr["tree_cand"], cid, cl, u_acc, u_fin, temperature=T)
+    sure = (o["min_margin"] >= 1e-4) & (o["fin_margin"] >= 3e-6)
+    assert sure.mean() >= 0.8
+    for key in ("n_acc", "path_node", "out_tok", "term_node", "term_kind"):
+        assert np.array_equal(f[key][sure], o[key][sure]), key
