@@ -66,7 +66,8 @@ int specroll_check_status(int32_t *detail, int32_t reset);
  * that the path on which a kernel gives up can be tested without a fault or a hang.  what == 1: the next
  * specroll_propose leaves out one barrier arrival in its projection kernel (nothing asynchronous is abandoned);
  * the waiting warps give up after the debug build's 20 ms limit, the kernel returns, and
- * specroll_workspace_status reports SPECROLL_ETIMEOUT.  Returns SPECROLL_OK, SPECROLL_EINVAL for an unknown
+ * specroll_workspace_status reports SPECROLL_ETIMEOUT.  what == 2: the next specroll_verify of few rows leaves out one copy
+ * of its statistics kernel; row_sum of the rows that the waiting warp had still to do is NaN.  Returns SPECROLL_OK, SPECROLL_EINVAL for an unknown
  * `what`, -1 in a normal build (where nothing of this exists). */
 int specroll_check_inject(int32_t what);
 

@@ -58,6 +58,7 @@ void register_check_reader(CheckReader fn) {
 }
 
 int lm_head_arm_dropped_signal();  // lm_head_tc.cu
+int run_stats_arm_dropped_copy();  // verify.cu
 
 int build_topo(const int32_t *parent_host, int N, int K, int k, Topo *t, TopoMask *m) {
     if (!parent_host || N < 1 || N > SPECROLL_MAX_NODES || parent_host[0] != -1) return SPECROLL_EINVAL;
@@ -131,6 +132,7 @@ int specroll_check_status(int32_t *detail, int32_t reset) {
 
 int specroll_check_inject(int32_t what) {
     if (what == 1) return specroll::lm_head_arm_dropped_signal();
+    if (what == 2) return specroll::run_stats_arm_dropped_copy();
     return SPECROLL_EINVAL;
 }
 

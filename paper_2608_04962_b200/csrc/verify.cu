@@ -146,6 +146,17 @@ constexpr int RUN_PIECE = 128;                 // vectors per copy (a group)
 constexpr int RUN_RING_MIN = 3, RUN_RING_MAX = 10;  // copies in flight per warp
 constexpr int RUN_WARPS = 4, RUN_CTAS = 8;     // warps per CTA, CTAs per SM
 // ROWS: a CTA of eight warps takes the eight runs of row blockIdx and leaves the row's own pair (up to four rows per SM).
+#ifdef SPECROLL_CHECK
+// Debug build only: when armed (specroll_check_inject(2)), the first warp of CTA 0 leaves out its first copy, once.  Its wait runs
+// into the time limit; the copies behind it land before the CTA goes away.
+static __device__ int g_drop_one_copy;
+int run_stats_arm_dropped_copy() {
+    const int one = 1;
+    return cudaMemcpyToSymbol(g_drop_one_copy, &one, sizeof(one)) == cudaSuccess ? SPECROLL_OK : SPECROLL_ECUDA;
+}
+#else
+int run_stats_arm_dropped_copy() { return -1; }
+#endif
 template <bool ROWS>
 __global__ void __launch_bounds__(32 * (ROWS ? RS_WARPS : RUN_WARPS), ROWS ? 4 : RUN_CTAS)
 run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs, int ring_n, float2 *__restrict__ run_tab,
@@ -190,7 +201,11 @@ run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs
         if (lane == 0) {
             const uint32_t bar = smem_u32(&full[s_in]);
             mbar_arrive_expect_tx(bar, (uint32_t)n * 16u);
-            bulk_load(smem_u32(ring + s_in * RUN_PIECE), reinterpret_cast<const uint4 *>(logits + (size_t)(r_next / RS_WARPS) * V) + v_next,
+            bool copy = true;
+#ifdef SPECROLL_CHECK
+            if (blockIdx.x == 0 && warp == 0 && n_issued == 0 && atomicExch(&g_drop_one_copy, 0) == 1) copy = false;
+#endif
+            if (copy) bulk_load(smem_u32(ring + s_in * RUN_PIECE), reinterpret_cast<const uint4 *>(logits + (size_t)(r_next / RS_WARPS) * V) + v_next,
                       (uint32_t)n * 16u, bar);
         }
         ++n_issued;
@@ -238,7 +253,8 @@ run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs
         const float mw = warp_max(m);
         s = (m == NEG_INF) ? 0.f : s * ex2_approx((m - mw) * c);
         s = warp_sum(s);
-        // (a copy that does not arrive: cannot happen with readable logits; marked instead of left looking valid)
+        // (a copy that does not arrive: cannot happen with readable logits; this run and those after it are marked instead of
+        // left looking valid)
         const float2 e = ok ? make_float2(mw, s) : make_float2(nanf(""), nanf(""));
         if (lane == 0) {
             if (ROWS)
@@ -246,7 +262,6 @@ run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs
             else
                 run_tab[r] = e;
         }
-        if (!ok) break;
     }
     if (!ok && lane == 0) {  // let the copies still in flight land before the CTA goes away
         for (uint32_t i = n_used; i < n_issued; ++i) {

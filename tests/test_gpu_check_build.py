@@ -71,6 +71,22 @@ g2 = S.propose(*pargs, k=w.k, clip_c=w.clip_c, workspace=ws)
 torch.cuda.synchronize()
 assert S.workspace_status(ws) == 0
 assert np.array_equal(host(g2["cand_id"]), o["cand_id"]) and np.array_equal(host(g2["tree_tok"]), o["tree_tok"])
+# ---- a copy of the row statistics that does not arrive: the warp's run at hand and its run of the second round are marked,
+#      whatever the workspace held from the call before
+wb = I.scaled(w, B=100)
+par = I.topology(wb)
+cid, cl = I.synthetic_candidates(wb)
+t = ref.tree_draw(par, np.zeros(wb.B, np.int32), cid, cl, I.uniforms24(3, (wb.B, wb.N)))
+ua, uf = I.verify_uniforms(wb)
+vargs = (dev_bf16(I.target_logits(wb, par, t["tree_tok"])), par, dev(t["tree_tok"]), dev(t["tree_cand"]), dev(cid), dev(cl),
+         dev(ua), dev(uf))
+ws = torch.zeros(S.verify_workspace_bytes(wb.B, wb.N, wb.K, wb.k, wb.V), dtype=torch.uint8, device="cuda")
+good = host(S.verify(*vargs, workspace=ws)["row_sum"]).reshape(-1)
+assert S.lib().specroll_check_inject(C.c_int32(2)) == 0
+bad = host(S.verify(*vargs, workspace=ws)["row_sum"]).reshape(-1)
+lost = np.flatnonzero(np.isnan(bad))
+assert lost[0] == 0 and len(lost) >= 2 and np.array_equal(np.delete(bad, lost), np.delete(good, lost)), lost
+assert np.array_equal(host(S.verify(*vargs, workspace=ws)["row_sum"]).reshape(-1), good)
 print("check build ok")
 """
 
