@@ -142,6 +142,31 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// The same maximum by one integer reduction (a float's bits, with the magnitude turned where it is negative, are ordered).
+__device__ __forceinline__ float warp_max_redux(float v) {
+    const int b = __float_as_int(v), o = __reduce_max_sync(0xffffffffu, b ^ ((b >> 31) & 0x7fffffff));
+    return __int_as_float(o ^ ((o >> 31) & 0x7fffffff));
+}
+// Sums of 2^L values per lane over the warp: every step halves what a lane carries.  Returns the sum of value
+// (lane >> (5 - L)), formed by the additions of warp_sum.
+template <int L>
+__device__ __forceinline__ float warp_sum_many(float (&x)[1 << L], int lane) {
+#pragma unroll
+    for (int s = 0; s < L; ++s) {
+        const int o = 16 >> s, h = (1 << L) >> (s + 1);
+        const bool up = lane & o;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const float give = up ? x[q] : x[q + h], keep = up ? x[q + h] : x[q];
+            x[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    float r = x[0];
+#pragma unroll
+    for (int o = 16 >> L; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    return r;
+}
+
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

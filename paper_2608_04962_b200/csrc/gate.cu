@@ -21,25 +21,6 @@ constexpr int GATE_THREADS = 128;
 constexpr int GATE_BATCH = 4 * GATE_THREADS;
 }  // namespace gt
 
-// Sums of 2^L values per lane over the warp: every step halves what a lane carries.  Returns the sum of value (lane >> (5 - L)).
-template <int L>
-__device__ __forceinline__ float warp_sum_many(float (&x)[1 << L], int lane) {
-#pragma unroll
-    for (int s = 0; s < L; ++s) {
-        const int o = 16 >> s, h = (1 << L) >> (s + 1);
-        const bool up = lane & o;
-#pragma unroll
-        for (int q = 0; q < h; ++q) {
-            const float give = up ? x[q] : x[q + h], keep = up ? x[q + h] : x[q];
-            x[q] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-        }
-    }
-    float r = x[0];
-#pragma unroll
-    for (int o = 16 >> L; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-    return r;
-}
-
 // y = Pi x (rank dot products of length d), then y / ||y||, for VPW records per warp; d % 4 == 0 and 16-byte aligned rows.
 // Pi is a few hundred KB that every record meets: with a CTA per record the kernel was bound by bringing it from L2 once
 // per record (512 records, d 3584, rank 24: 17-22 us).  A cluster of four CTAs takes 8 VPW records, each CTA a quarter of

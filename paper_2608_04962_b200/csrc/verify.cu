@@ -1378,50 +1378,126 @@ __global__ void __launch_bounds__(WALK_WARPS * 32) walk_kernel(WalkArgs a, Topo 
     walk_end(a, b, u, sg ? (double)sg->rsum[u] : (double)a.row_sum[(size_t)b * N + u], lane, sm, &st);
 }
 
-// Maximum and sum of exponentials of one row by all NUC_THREADS threads of n_cta CTAs (a cluster; 1: a CTA alone), same
-// arithmetic as row_stats_kernel; every thread returns with the result.  sm_ms: NUC_THREADS / 32 pairs, at the same offset
-// in every CTA (the caller has a cluster barrier between two rows).
+// Maximum and sum of exponentials of one row by all NUC_THREADS threads of n_cta CTAs (a cluster; 1: a CTA alone); every
+// thread returns with the result.  The row is cut into interleaved parts, a number that follows its length, and the parts
+// are shared by the CTAs; a part's pairs (one per warp) and their sum are formed in one order however many CTAs there are, so
+// that the result does not follow the batch size to the last bit (the thresholds and draws behind it would).  sm_ms:
+// ROW_PARTS * NUC_THREADS / 32 pairs, at the same offset in every CTA (the caller has a cluster barrier between two rows).
+constexpr int ROW_PARTS = 8;  // at most; the largest cluster
+// The P parts from part0 on of n_parts: pairs of this warp to sm_ms[q * W + warp].  Vector j * NUC_THREADS + thread of the row
+// belongs to part j % n_parts.  A thread takes up to R of a part's vectors together, which is what keeps R loads in flight: their
+// maximum first, then the exponentials, which nothing rescales on the way.  The sums over the warp are formed for all parts
+// at once, with the additions of warp_sum.  MORE: a part has more than R vectors per thread.  (Lazy verification, V 151936: 4
+// sequences 37.4 -> 35.4 us, 256 sequences 105.5 -> 104.5 against sums in the order of the CTAs at hand; 256 of V 32000 38.4 ->
+// 40.5, 200 of V 129000 93 -> 98.  A running pair per part, rescaled vector by vector and reduced part by part: 125 us for 105.5.)
+template <int P, int R, bool MORE = false>
+__device__ __forceinline__ void row_parts(const uint4 *__restrict__ p, int nvec, int part0, int n_parts, float c, float2 *sm_ms) {
+    constexpr int W = NUC_THREADS / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, step = NUC_THREADS * n_parts;
+    auto as2 = [](uint32_t w) { return *reinterpret_cast<const __nv_bfloat162 *>(&w); };
+    float m[P], s[P];
+#pragma unroll
+    for (int q = 0; q < P; ++q) {
+        m[q] = NEG_INF;
+        s[q] = 0.f;
+#pragma unroll 1
+        for (int i = (part0 + q) * NUC_THREADS + threadIdx.x; !MORE || i < nvec; i += R * step) {
+            uint4 v[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = ld_nc_v4(p + min(i + r * step, nvec - 1));
+            __nv_bfloat162 m2 = as2(0xff80ff80u);  // (-inf, -inf)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const __nv_bfloat162 x = __hmax2(__hmax2(as2(v[r].x), as2(v[r].y)), __hmax2(as2(v[r].z), as2(v[r].w)));
+                if (i + r * step < nvec) m2 = __hmax2(m2, x);
+            }
+            const float mc = fmaxf(__low2float(m2), __high2float(m2));
+            if (mc > m[q]) {
+                s[q] *= ex2_approx((m[q] - mc) * c);  // (0 * 2^-inf = 0 at first)
+                m[q] = mc;
+            }
+            const float nmc = m[q] == NEG_INF ? 0.f : -m[q] * c;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (i + r * step >= nvec) break;
+                const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
+                float acc = 0.f;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    acc += ex2_approx(fmaf(__uint_as_float(w[t] << 16), c, nmc));
+                    acc += ex2_approx(fmaf(__uint_as_float(w[t] & 0xffff0000u), c, nmc));
+                }
+                s[q] += acc;
+            }
+            if (!MORE) break;
+        }
+    }
+    float mw[P];
+#pragma unroll
+    for (int q = 0; q < P; ++q) {
+        mw[q] = warp_max_redux(m[q]);
+        s[q] = m[q] == NEG_INF ? 0.f : s[q] * ex2_approx((m[q] - mw[q]) * c);
+    }
+    constexpr int L = P == 8 ? 3 : P == 4 ? 2 : P == 2 ? 1 : 0;
+    const float sum = warp_sum_many<L>(s, lane);  // (of part lane >> (5 - L))
+    float mine = mw[0];
+#pragma unroll
+    for (int q = 1; q < P; ++q)
+        if (lane >> (5 - L) == q) mine = mw[q];
+    if ((lane & ((1 << (5 - L)) - 1)) == 0) sm_ms[(lane >> (5 - L)) * W + warp] = make_float2(mine, sum);
+}
 __device__ void row_stats_row(const uint16_t *__restrict__ row_logits, int V, float c, float2 *sm_ms, int n_cta, int rank,
                               float *M_out, float *S_out) {
+    constexpr int W = NUC_THREADS / 32;
     const uint4 *p = reinterpret_cast<const uint4 *>(row_logits);
-    const int nvec = V >> 3, step = NUC_THREADS * n_cta;
-    float m = NEG_INF, nmc = 0.f, s = 0.f;
-    int i = rank * NUC_THREADS + threadIdx.x;
-    for (; i + 3 * step < nvec; i += 4 * step) {
-        uint4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = ld_nc_v4(p + i + u * step);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) online_update(v[u], c, m, nmc, s);
-    }
-    for (; i < nvec; i += step) online_update(ld_nc_v4(p + i), c, m, nmc, s);
-    const float mw = warp_max(m);
-    s = (m == NEG_INF) ? 0.f : s * ex2_approx((m - mw) * c);
-    s = warp_sum(s);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nvec = V >> 3, lane = threadIdx.x & 31;
+    // so many parts that a thread has two to four vectors of each (more where the row has more than eight times that)
+    const int lg = nvec > 8192 ? 3 : nvec > 4096 ? 2 : nvec > 2048 ? 1 : 0, n_parts = 1 << lg;
+    const int P = n_parts > n_cta ? n_parts / n_cta : 1;  // per CTA; CTAs beyond the parts have none
     __syncthreads();
-    if (lane == 0) sm_ms[warp] = make_float2(mw, s);
+    if (nvec > 5 * ROW_PARTS * NUC_THREADS) {
+        if (P == 8) row_parts<8, 5, true>(p, nvec, 0, 8, c, sm_ms);
+        else if (P == 4) row_parts<4, 5, true>(p, nvec, rank * 4, 8, c, sm_ms);
+        else if (P == 2) row_parts<2, 5, true>(p, nvec, rank * 2, 8, c, sm_ms);
+        else row_parts<1, 5, true>(p, nvec, rank, 8, c, sm_ms);
+    } else if (nvec > 4 * ROW_PARTS * NUC_THREADS) {
+        if (P == 8) row_parts<8, 5>(p, nvec, 0, 8, c, sm_ms);
+        else if (P == 4) row_parts<4, 5>(p, nvec, rank * 4, 8, c, sm_ms);
+        else if (P == 2) row_parts<2, 5>(p, nvec, rank * 2, 8, c, sm_ms);
+        else row_parts<1, 5>(p, nvec, rank, 8, c, sm_ms);
+    } else {
+        if (P == 8) row_parts<8, 4>(p, nvec, 0, 8, c, sm_ms);
+        else if (P == 4) row_parts<4, 4>(p, nvec, rank * 4, n_parts, c, sm_ms);
+        else if (P == 2) row_parts<2, 4>(p, nvec, rank * 2, n_parts, c, sm_ms);
+        else if (rank < n_parts) row_parts<1, 4>(p, nvec, rank, n_parts, c, sm_ms);
+    }
     if (n_cta > 1)
         cluster_sync_all();
     else
         __syncthreads();
-    constexpr int W = NUC_THREADS / 32;
-    auto at = [&](int w) {
-        if (n_cta == 1) return sm_ms[w];
-        const double d = ld_dsmem_f64(sm_ms + w % W, w / W);
-        return make_float2(__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d)));
-    };
-    // (every warp for itself, a lane per pair)
+    // every warp for itself: pair j of the row by lane j % 32, four pairs per lane
+    float2 e[ROW_PARTS * W / 32];
     float mb = NEG_INF, sb = 0.f;
-    for (int w0 = 0; w0 < W * n_cta; w0 += 32) {
-        const float2 e = w0 + lane < W * n_cta ? at(w0 + lane) : make_float2(NEG_INF, 0.f);
-        const float mn = fmaxf(mb, warp_max(e.x));
-        const float part = warp_sum(e.x == NEG_INF ? 0.f : e.y * ex2_approx((e.x - mn) * c));
-        sb = (mb == NEG_INF ? 0.f : sb * ex2_approx((mb - mn) * c)) + part;
-        mb = mn;
+#pragma unroll
+    for (int j = 0; j < ROW_PARTS * W / 32; ++j) {
+        const int w = j * 32 + lane, part = w / W;
+        e[j] = make_float2(NEG_INF, 0.f);
+        if (part < n_parts) {
+            const int r = part / P, at = w - r * P * W;
+            if (n_cta == 1) {
+                e[j] = sm_ms[at];
+            } else {
+                const double d = ld_dsmem_f64(sm_ms + at, r);
+                e[j] = make_float2(__int_as_float(__double2loint(d)), __int_as_float(__double2hiint(d)));
+            }
+        }
+        mb = fmaxf(mb, e[j].x);
     }
+    mb = warp_max_redux(mb);
+#pragma unroll
+    for (int j = 0; j < ROW_PARTS * W / 32; ++j) sb += e[j].x == NEG_INF ? 0.f : e[j].y * ex2_approx((e[j].x - mb) * c);
     *M_out = mb;
-    *S_out = sb;
+    *S_out = warp_sum(sb);
 }
 
 // ------------------------------------------------------------------------------ terminal draw
@@ -1623,7 +1699,8 @@ __device__ void term_pick(const uint4 *__restrict__ p, const double *seg_slices,
 }
 
 // The vectors [v_base, v_base + nvec_r) of a row are cut into one segment per warp of the draw's n_cta CTAs (a cluster;
-// 1: a CTA alone), each walked in slices of 32 vectors (one per lane).  Pass 1 (all warps, independent loads) leaves the
+// 1: a CTA alone), each walked in slices of 32 vectors (one per lane); the slices, whose masses are fp32 sums, are the same
+// ones however many CTAs there are.  Pass 1 (all warps, independent loads) leaves the
 // fp64 mass of every slice in shared memory, those of the cluster's other CTAs are read by its first CTA; the residual
 // entries (nov tokens ovid, masses ovm) then replace the plain mass of their tokens; two scans pick the segment and the
 // slice that hold the target, and only that slice is read again to find the token.
@@ -1647,8 +1724,7 @@ __device__ void draw_row(const uint16_t *__restrict__ lg, int v_base, int nvec_r
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint4 *p = reinterpret_cast<const uint4 *>(lg);
     const int G = n_cta * TERM_WARPS;
-    const int vpw = (nvec_r + G - 1) / G > 0 ? (nvec_r + G - 1) / G : 1;  // vectors per warp segment
-    const int n_sl = (vpw + 31) / 32;                                     // slices per segment
+    const int n_sl = draw_slices(nvec_r, n_cta), vpw = n_sl * 32;  // slices and vectors per warp segment
     double *seg = slices + (size_t)G * n_sl;
     {
         const int g = rank * TERM_WARPS + warp;
@@ -1766,7 +1842,7 @@ walk_cta_kernel(WalkArgs a, Topo topo, float c, float top_p, float *__restrict__
     extern __shared__ __align__(16) unsigned char nuc_raw[];
     NucleusSmem &nuc = *reinterpret_cast<NucleusSmem *>(nuc_raw);  // (NUC only)
     __shared__ WalkSmem sm;
-    __shared__ float2 sm_ms[NUC_THREADS / 32];
+    __shared__ float2 sm_ms[ROW_PARTS * NUC_THREADS / 32];
     __shared__ int sh_next[2];        // the next node, or -1 when the walk is over; rows in turn (one barrier per row)
     __shared__ uint32_t sh_last[4];   // of the last node, for the draw: threshold key, residual entries, accepted tokens
     __shared__ double sh_ovm[SPECROLL_MAX_TOPK];

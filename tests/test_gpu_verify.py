@@ -223,3 +223,35 @@ def test_runs_by_one_warp_each_and_nodes_by_lane_groups(B, N, k, V):
     u_acc, u_fin = I.verify_uniforms(w)
     o, g = run_both(w, parent, lg, d["tree_tok"], d["tree_cand"], cid, cl, u_acc, u_fin)
     check(w, o, g, lg)
+
+
+@pytest.mark.parametrize("top_p,V", [(1.0, 40008), (0.95, 40008), (1.0, 151936), (0.95, 8200), (1.0, 32776), (1.0, 8),
+                                     (1.0, 200008)])
+def test_lazy_row_statistics_do_not_follow_the_batch_size(top_p, V):
+    """Few sequences share their rows among the CTAs of a cluster; the same sequences in a batch of any size give the same
+    bits and tokens."""
+    w = I.scaled(I.WORKLOADS["qwen1.5b"], B=300, N=8 if V < 100000 else 2, V=V, k=4)
+    parent = I.topology(w)
+    cid, cl = I.synthetic_candidates(w)
+    d = ref.tree_draw(parent, np.zeros(w.B, np.int32), cid, cl, I.uniforms24(11, (w.B, w.N)))
+    lg = dev_bf16(I.target_logits(w, parent, d["tree_tok"], boost=3.0))
+    u_acc, u_fin = I.verify_uniforms(w)
+    args = [lg] + [dev(a) for a in (d["tree_tok"], d["tree_cand"], cid, cl, u_acc, u_fin)]
+
+    def run(n):
+        out = {k: torch.zeros(s, dtype=t, device="cuda") for k, s, t in (
+            ("n_acc", (n,), torch.int32), ("path_node", (n, w.K + 1), torch.int32), ("out_tok", (n, w.K + 1), torch.int32),
+            ("term_node", (n,), torch.int32), ("term_kind", (n,), torch.int32), ("row_max", (n, w.N), torch.float32),
+            ("row_sum", (n, w.N), torch.float32), ("min_margin", (n,), torch.float32))}
+        a = [t[:n].contiguous() for t in args]
+        if top_p < 1.0:
+            S.verify_nucleus(a[0], parent, *a[1:], top_p, out=out, flags=S.VERIFY_LAZY_STATS)
+        else:
+            S.verify(a[0], parent, *a[1:], out=out, flags=S.VERIFY_LAZY_STATS)
+        return out
+
+    whole = run(300)
+    for n in (3, 37, 70, 148):
+        part = run(n)
+        for k in part:
+            assert torch.equal(part[k], whole[k][:n]), (n, k)
