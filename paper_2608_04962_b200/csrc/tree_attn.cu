@@ -772,7 +772,6 @@ static int run_tree_attn(const specroll_attn_desc *d, const void *Q, const void 
     a.total_work = p.items * d->Hkv * p.n_rb;
     a.merge_mode = p.merge_mode;
     a.nodes_per_block = p.nodes_per_block;
-    a.plan_fresh = 0;
     a.no_pdl = (d->flags & SPECROLL_ATTN_NO_PDL) ? 1 : 0;
     // early cache loads need a plan that is not being made by the kernel just before the attention kernel
     a.early_cache = ((d->flags & SPECROLL_ATTN_CACHE_SETTLED) && (d->flags & SPECROLL_ATTN_REUSE_PLAN)) ? 1 : 0;
@@ -784,7 +783,6 @@ static int run_tree_attn(const specroll_attn_desc *d, const void *Q, const void 
                                      paged ? kv_len_dev : nullptr, page_indptr_dev, d->B, p.chunk_tiles, p.tile_tokens,
                                      reinterpret_cast<int32_t *>(ws + p.off_items), p.use_tc ? sorted_start : nullptr,
                                      seq_at_rank, p.use_tc ? unit_tab : nullptr, status, counters, p.n_counters));
-        a.plan_fresh = 1;
     }
     const size_t n_out = (size_t)d->B * d->N * d->Hq;
     if (p.use_tc) {

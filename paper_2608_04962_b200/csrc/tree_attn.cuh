@@ -28,7 +28,6 @@ struct AttnArgs {
     // sequence's first slot in this table instead of its first token
     const int32_t *page_table;
     int early_cache;              // plan, cache and page table were complete before the preceding kernel was launched
-    int32_t plan_fresh;           // the preceding kernel is the plan kernel of this call
     float *hand;                  // [ATTN_HAND_CTAS][4][128] per-CTA hand-over area between two groups of warps of the tcgen05 kernel
     int32_t merge_mode;           // chunks of a split sequence are merged 0: by the CTA that finishes last; 2: by a later kernel
     int32_t no_pdl;               // launch the attention kernel as an ordinary kernel, not as a programmatic dependent

@@ -221,15 +221,16 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     // Launched as a programmatic dependent of the kernel before it in the stream, this CTA may have done all
     // of the above while that kernel was still finishing.  From here on it reads what earlier kernels wrote
     // (the plan, the counters the launch before cleared, Q and the tree's K/V), so it waits for them to be
-    // complete.  The kernel after this one may be set up as early as its CTAs find room - except behind a plan that
-    // is only being made: that kernel may read the plan before it waits, so this one waits for the plan first.
+    // complete.  Only then may the kernel after this one be set up: that one may read the plan, or a cache that the kernel in
+    // front of this one was writing, ahead of its own wait.
     // Exception: when the caller has said that the plan and the cache were complete before that kernel was
     // even launched, the loading thread fetches its first cache tiles right away and waits just before it
     // needs Q (below).
     const bool early = a.early_cache != 0;
-    if (a.plan_fresh) asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (!(early && warp == 0)) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!(early && warp == 0)) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
 
     // Sums the partials of all chunks of one (sequence, kv head, row block) for columns [col0, col0 + ncols) of one row;
     // run by the threads that own the row block, after the tickets showed that every chunk has been written.
@@ -1171,8 +1172,7 @@ __global__ void __launch_bounds__(128 * MERGE_PARTS) attn_merge_tc_kernel(AttnAr
     __shared__ float2 sh_ml[MERGE_PARTS][128];
     __shared__ float4 sh_acc[2][MERGE_PARTS][128];
     pdl_launch_dependents();
-    // The plan is complete when this block starts: the attention kernel lets it start only behind a wait for a plan that
-    // was being made.  Reading it ahead of the wait for the partials, all blocks but those of first chunks leave at once
+    // The plan is complete when this block starts: the attention kernel lets it start only behind its own wait.  Reading it ahead of the wait for the partials, all blocks but those of first chunks leave at once
     // (19 of 20 blocks otherwise hold the places of the ones that work until the partials are there).
     const int4 e0 = __ldcg(reinterpret_cast<const int4 *>(a.unit_tab) + 2 * (size_t)blockIdx.x);
     const int b = e0.x, n_splits = e0.z, item0 = e0.w;

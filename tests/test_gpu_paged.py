@@ -176,3 +176,38 @@ def test_bad_arguments():
     with pytest.raises(S.SpecrollError):
         S.tree_attn_paged(dev_bf16(x["Q"]), dev_bf16(Kp[:, :64]), dev_bf16(Vp[:, :64]), dev(pt), dev(pi), dev(kl), kl,
                           dev_bf16(x["Kt"]), dev_bf16(x["Vt"]), x["parent"])
+
+
+def test_settled_cache_written_two_kernels_ago():
+    """commit into layer B's pool, attention of layer A, attention of layer B that may fetch its cache while A's is finishing:
+    B's cache was written before the kernel in front was launched, and has to be complete by then."""
+    w = I.scaled(I.WORKLOADS["qwen1.5b"], B=8, N=16, K=4)
+    x = _inputs(w, [700, 64, 1500, 333, 129, 2900, 256, 77])
+    Kp, Vp, pt, pi, kl = I.paged_cache(x["Kc"], x["Vc"], x["kv_indptr"], spare_tokens=0, seed=21)
+    path = np.tile(np.arange(w.K + 1, dtype=np.int32), (w.B, 1))
+    n_acc, first = np.full(w.B, w.K, np.int32), np.zeros(w.B, np.int32)  # (over the first tokens of every sequence)
+    Q, Kt, Vt = (dev_bf16(x[n]) for n in ("Q", "Kt", "Vt"))
+    A, pool = (dev_bf16(Kp), dev_bf16(Vp)), (dev_bf16(Kp), dev_bf16(Vp))
+    others = [torch.zeros_like(pool[0]) for _ in range(24)]
+    pt, pi, dkl, path, n_acc, first = dev(pt), dev(pi), dev(kl), dev(path), dev(n_acc), dev(first)
+    ws = S.alloc(S.tree_attn_paged_workspace_bytes(w.B, w.N, w.Hq, w.Hkv, w.D, kl), dtype=torch.uint8, device="cuda")
+
+    def attn(c, flags):
+        return S.tree_attn_paged(Q, c[0], c[1], pt, pi, dkl, kl, Kt, Vt, x["parent"], workspace=ws, flags=flags)
+
+    def commit(K, V):
+        S.commit_path_layers([Kt] * len(K), [Vt] * len(K), path, n_acc, K, V, pt, pi, first)
+
+    commit([pool[0]], [pool[1]])
+    want_a, want_b = attn(A, 0), attn(pool, 0)
+    torch.cuda.synchronize()
+    for _ in range(20):
+        for p, src in zip(pool, (Kp, Vp)):
+            p.copy_(dev_bf16(src))
+        torch.cuda.synchronize()
+        commit(others[:12] + [pool[0]], others[12:] + [pool[1]])
+        got_a = attn(A, S.ATTN_REUSE_PLAN | S.ATTN_CACHE_SETTLED)
+        got_b = attn(pool, S.ATTN_REUSE_PLAN | S.ATTN_CACHE_SETTLED)
+        torch.cuda.synchronize()
+        assert torch.equal(got_a, want_a) and torch.equal(got_b, want_b)
+    assert S.workspace_status(ws) == 0
