@@ -261,7 +261,7 @@ def tree_attn_paged(Q, Kp, Vp, page_table, page_indptr, kv_len_dev, kv_len_host,
 
 def commit_path(Kt, Vt, path_node, n_acc, Kp, Vp, page_table, page_indptr, kv_len, kv_len_out=None, status=None):
     """specroll_commit_path: appends the committed path's tree rows to one layer's paged cache (in place)."""
-    commit_path_layers([Kt], [Vt], path_node, n_acc, [Kp], [Vp], page_table, page_indptr, kv_len, kv_len_out, status)
+    _n().commit_path(Kt, Vt, path_node, n_acc, Kp, Vp, page_table, page_indptr, kv_len, kv_len_out, status)
 
 
 def commit_path_layers(Kt, Vt, path_node, n_acc, Kp, Vp, page_table, page_indptr, kv_len, kv_len_out=None,

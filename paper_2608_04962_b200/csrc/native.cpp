@@ -46,7 +46,7 @@ constexpr at::ScalarType BF16 = at::kBFloat16, F32 = at::kFloat, I32 = at::kInt,
 #define SPECROLL_ENTRIES(X)                                                                                          \
     X(specroll_strerror) X(specroll_propose_workspace_bytes) X(specroll_propose) X(specroll_tree_draw)               \
     X(specroll_tree_attn_workspace_bytes) X(specroll_tree_attn) X(specroll_tree_attn_paged_workspace_bytes)          \
-    X(specroll_tree_attn_paged) X(specroll_commit_path_layers) X(specroll_gather_hidden)                             \
+    X(specroll_tree_attn_paged) X(specroll_commit_path) X(specroll_commit_path_layers) X(specroll_gather_hidden)                             \
     X(specroll_verify_workspace_bytes) X(specroll_verify) X(specroll_verify_static)                                  \
     X(specroll_verify_nucleus_workspace_bytes)                                                                       \
     X(specroll_verify_nucleus) X(specroll_reflex_feedback_workspace_bytes) X(specroll_reflex_feedback_ex)            \
@@ -75,12 +75,17 @@ const at::Tensor &need(PyObject *o, const char *name, int dim) {
     if (!t || t->dim() != dim) fail("%s must be a tensor of %d dimensions", name, dim);
     return *t;
 }
+const at::Tensor &need(PyObject *o, const char *name) {  // (of any shape)
+    const at::Tensor *t = tensor(o, name);
+    if (!t) fail("%s must be a CUDA tensor", name);
+    return *t;
+}
 void *dev(const at::Tensor *t, at::ScalarType dtype, const char *name) {
     if (!t) return nullptr;
     if (!t->is_cuda()) fail("%s must be a CUDA tensor", name);
     if (t->scalar_type() != dtype) fail("%s must have dtype %s, got %s", name, c10::toString(dtype), c10::toString(t->scalar_type()));
     if (!t->is_contiguous()) fail("%s must be contiguous", name);
-    return const_cast<void *>(t->const_data_ptr());
+    return t->mutable_data_ptr();  // (as Tensor.data_ptr(): a lazily cloned tensor gets storage of its own)
 }
 void *dev(const at::Tensor &t, at::ScalarType dtype, const char *name) { return dev(&t, dtype, name); }
 void *dev(PyObject *o, at::ScalarType dtype, const char *name) { return dev(tensor(o, name), dtype, name); }
@@ -137,6 +142,18 @@ class HostI32 {
     PyObject *made_ = nullptr;
 };
 
+// A reference held for the length of a call.
+struct Ref {
+    PyObject *o;
+    explicit Ref(PyObject *o_) : o(o_) {
+        if (!o) throw Raised();
+    }
+    Ref(Ref &&r) noexcept : o(std::exchange(r.o, nullptr)) {}
+    ~Ref() { Py_XDECREF(o); }
+    Ref(const Ref &) = delete;
+    Ref &operator=(const Ref &) = delete;
+};
+
 // ---- results
 at::Tensor alloc(std::initializer_list<int64_t> size, at::ScalarType dtype, const at::Tensor &like) {
     if (!g_alloc) return at::empty(at::IntArrayRef(size), at::TensorOptions().dtype(dtype).device(like.device()));
@@ -161,21 +178,24 @@ at::Tensor workspace(PyObject *o, size_t n, const at::Tensor &like) {
     const at::Tensor *t = tensor(o, "workspace");
     return t ? *t : alloc_bytes(n, like);
 }
-void *ptr(const at::Tensor &t) { return const_cast<void *>(t.const_data_ptr()); }
+void *ptr(const at::Tensor &t) { return t.mutable_data_ptr(); }
 size_t bytes_of(const at::Tensor &t) { return (size_t)t.numel(); }
 
-// A dict of outputs: the caller's (borrowed), or a new one that new tensors go into.
+// The outputs by name: the caller's mapping, or a new dict that new tensors go into.
 class Out {
   public:
     explicit Out(PyObject *given) : given_(given && given != Py_None ? given : nullptr) {
-        if (given_ && !PyDict_Check(given_)) fail("out must be a dict");
         dict_ = given_ ? Py_NewRef(given_) : PyDict_New();
         if (!dict_) throw Raised();
     }
     ~Out() { Py_XDECREF(dict_); }
     void *get(const char *name, std::initializer_list<int64_t> size, at::ScalarType dtype, const at::Tensor &like, bool optional = false) {
         if (!given_) return put(name, alloc(size, dtype, like));
-        PyObject *o = PyDict_GetItemString(dict_, name);
+        if (!PyDict_CheckExact(given_)) {
+            const Ref o(optional ? PyObject_CallMethod(given_, "get", "s", name) : PyMapping_GetItemString(given_, name));
+            return dev(o.o, dtype, name);
+        }
+        PyObject *o = PyDict_GetItemString(given_, name);
         if (!o) {
             if (optional) return nullptr;
             PyErr_SetString(PyExc_KeyError, name);
@@ -276,7 +296,7 @@ PyObject *tree_attn(PyObject *const *a) {
     const at::Tensor &Q = need(a[0], "Q", 4), &Kc = need(a[1], "Kc", 3), &Vc = need(a[2], "Vc", 3), &Kt = need(a[5], "Kt", 4), &Vt = need(a[6], "Vt", 4);
     HostI32 ip(a[4], "kv_indptr_host"), parent(a[7], "parent");
     const int64_t B = Q.size(0), N = Q.size(1), Hq = Q.size(2), D = Q.size(3), Hkv = Kt.size(2);
-    if (ip.size() != B + 1 || !shape(Kt, {B, N, Hkv, D}) || !shape(Vt, {B, N, Hkv, D}) || parent.size() != N)
+    if (ip.size() != B + 1 || !shape(Kt, {B, N, Hkv, D}) || !shape(Vt, {B, N, Hkv, D}) || parent.size() < N)
         fail("tree_attn: inconsistent shapes");
     if (!shape(Kc, {ip.last(), Hkv, D}) || Vc.sizes() != Kc.sizes()) fail("tree_attn: cache shape does not match kv_indptr");
     const specroll_attn_desc desc = {(int32_t)B, (int32_t)N, (int32_t)Hq, (int32_t)Hkv, (int32_t)D, attn_scale(a[8], D), (int32_t)integer(a[13])};
@@ -295,14 +315,14 @@ PyObject *tree_attn(PyObject *const *a) {
 
 PyObject *tree_attn_paged(PyObject *const *a) {
     const at::Tensor &Q = need(a[0], "Q", 4), &Kp = need(a[1], "Kp", 4), &Vp = need(a[2], "Vp", 4), &Kt = need(a[7], "Kt", 4), &Vt = need(a[8], "Vt", 4);
-    const at::Tensor &pi = need(a[4], "page_indptr", 1), &kl = need(a[5], "kv_len_dev", 1);
+    const at::Tensor &pi = need(a[4], "page_indptr"), &kl = need(a[5], "kv_len_dev");
     HostI32 len(a[6], "kv_len_host"), parent(a[9], "parent");
     const int64_t B = Q.size(0), N = Q.size(1), Hq = Q.size(2), D = Q.size(3), Hkv = Kt.size(2);
-    if (len.size() != B || !shape(Kt, {B, N, Hkv, D}) || !shape(Vt, {B, N, Hkv, D}) || parent.size() != N)
+    if (len.size() != B || !shape(Kt, {B, N, Hkv, D}) || !shape(Vt, {B, N, Hkv, D}) || parent.size() < N)
         fail("tree_attn_paged: inconsistent shapes");
     if (!shape(Kp, {Kp.size(0), SPECROLL_PAGE_TOKENS, Hkv, D}) || Vp.sizes() != Kp.sizes())
         fail("tree_attn_paged: page pool must be [n_pages, 128, Hkv, D]");
-    if (pi.size(0) != B + 1 || kl.size(0) != B) fail("tree_attn_paged: page_indptr / kv_len_dev sizes");
+    if (pi.numel() != B + 1 || kl.numel() != B) fail("tree_attn_paged: page_indptr / kv_len_dev sizes");
     const specroll_attn_desc desc = {(int32_t)B, (int32_t)N, (int32_t)Hq, (int32_t)Hkv, (int32_t)D, attn_scale(a[10], D), (int32_t)integer(a[15])};
     const at::Tensor O = a[13] != Py_None ? *tensor(a[13], "O") : alloc({B, N, Hq, D}, BF16, Q);
     at::Tensor lse;
@@ -319,30 +339,45 @@ PyObject *tree_attn_paged(PyObject *const *a) {
 
 // ------------------------------------------------------------------------------ between two rounds
 
+PyObject *commit_path(PyObject *const *a) {
+    // Kt, Vt, path_node, n_acc, Kp, Vp, page_table, page_indptr, kv_len, kv_len_out, status
+    const at::Tensor &Kt = need(a[0], "Kt", 4), &path = need(a[2], "path_node"), &Kp = need(a[4], "Kp");
+    const int64_t B = Kt.size(0), N = Kt.size(1), Hkv = Kt.size(2), D = Kt.size(3), K = path.size(1) - 1, n_pages = Kp.size(0);
+    const void *pkt = dev(Kt, BF16, "Kt"), *pvt = dev(a[1], BF16, "Vt");
+    void *pk = dev(Kp, BF16, "Kp"), *pv = dev(a[5], BF16, "Vp");
+    const auto *pp = (const int32_t *)dev(path, I32, "path_node"), *pn = (const int32_t *)dev(a[3], I32, "n_acc");
+    const auto *pt = (const int32_t *)dev(a[6], I32, "page_table"), *pi = (const int32_t *)dev(a[7], I32, "page_indptr"), *pl = (const int32_t *)dev(a[8], I32, "kv_len");
+    auto *po = (int32_t *)dev(a[9], I32, "kv_len_out"), *ps = (int32_t *)dev(a[10], I32, "status");
+    CALL(specroll_commit_path, (int32_t)B, (int32_t)N, (int32_t)K, (int32_t)Hkv, (int32_t)D, pkt, pvt, pp, pn, pk, pv, n_pages, pt, pi, pl, po, ps);
+    return Py_NewRef(Py_None);
+}
+
 PyObject *commit_path_layers(PyObject *const *a) {
-    // the four lists of tensors, one per layer
+    // four sequences of tensors, one per layer (lists, tuples, or a tensor whose first dimension is the layer)
     static const char *const names[4] = {"Kt", "Vt", "Kp", "Vp"};
     PyObject *const src[4] = {a[0], a[1], a[4], a[5]};
+    std::vector<Ref> seqs;  // (hold the items of a sequence that makes them on the way)
     std::vector<void *> ptrs[4];
     const at::Tensor *first[4] = {};
     Py_ssize_t n = -1;
     for (int i = 0; i < 4; ++i) {
-        PyObject *seq = PySequence_Fast(src[i], "commit_path_layers: one tensor per layer in each list");
-        if (!seq) throw Raised();
-        const Py_ssize_t len = PySequence_Fast_GET_SIZE(seq);
-        Py_DECREF(seq);  // (the caller's list or tuple keeps its items alive)
+        const Py_ssize_t len = PyObject_Size(src[i]);
+        if (len < 0) throw Raised();
         if (n < 0) n = len;
-        if (len != n || n == 0 || !(PyList_Check(src[i]) || PyTuple_Check(src[i]))) fail("commit_path_layers: one tensor per layer in each list");
+        if (len != n || n == 0) fail("commit_path_layers: one tensor per layer in each list");
+        seqs.emplace_back(PySequence_Fast(src[i], "commit_path_layers: one tensor per layer in each list"));
+        if (PySequence_Fast_GET_SIZE(seqs.back().o) != n) fail("commit_path_layers: one tensor per layer in each list");
         ptrs[i].reserve((size_t)n);
         for (Py_ssize_t l = 0; l < n; ++l) {
-            const at::Tensor &t = need(PySequence_Fast_GET_ITEM(src[i], l), names[i], 4);
+            PyObject *o = PySequence_Fast_GET_ITEM(seqs.back().o, l);
+            const at::Tensor &t = i < 2 ? need(o, names[i], 4) : need(o, names[i]);
             if (l == 0) first[i] = &t;
             if (i < 2 && t.sizes() != first[0]->sizes()) fail("commit_path_layers: tree K/V shapes differ between layers");
             if (i >= 2 && t.sizes() != first[2]->sizes()) fail("commit_path_layers: page pools differ between layers");
             ptrs[i].push_back(dev(t, BF16, names[i]));
         }
     }
-    const at::Tensor &path = need(a[2], "path_node", 2);
+    const at::Tensor &path = need(a[2], "path_node");
     const int64_t B = first[0]->size(0), N = first[0]->size(1), Hkv = first[0]->size(2), D = first[0]->size(3), K = path.size(1) - 1;
     const auto *pp = (const int32_t *)dev(path, I32, "path_node"), *pn = (const int32_t *)dev(a[3], I32, "n_acc");
     const auto *pt = (const int32_t *)dev(a[6], I32, "page_table"), *pi = (const int32_t *)dev(a[7], I32, "page_indptr"), *pl = (const int32_t *)dev(a[8], I32, "kv_len");
@@ -373,12 +408,16 @@ struct VerifyArgs {
     const int32_t *tree_tok, *cand_id;
     const uint8_t *tree_cand;
     const float *cand_logit, *u_acc, *u_fin;
-    VerifyArgs(const char *what, int64_t B_, int64_t N_, int64_t V_, const HostI32 &parent, PyObject *const *a) : B(B_), N(N_), V(V_) {
+    VerifyArgs(const char *what, int64_t B_, int64_t N_, int64_t V_, const HostI32 &parent, PyObject *const *a, bool flat = false)
+        : B(B_), N(N_), V(V_) {
         // a: tree_tok, tree_cand, cand_id, cand_logit, u_acc, u_fin
-        const at::Tensor &tok = need(a[0], "tree_tok", 2), &id = need(a[2], "cand_id", 3), &ua = need(a[4], "u_acc", 2);
+        const at::Tensor &tok = need(a[0], "tree_tok"), &id = need(a[2], "cand_id", 3), &ua = need(a[4], "u_acc");
         K = id.size(1);
         k = id.size(2);
-        if (parent.size() != N || !shape(tok, {B, N}) || !shape(ua, {B, N})) fail("%s: inconsistent shapes", what);
+        // flat: the arrays of any shape that holds enough (verification from hidden states)
+        if (flat ? parent.size() < N || tok.numel() < B * N || ua.numel() < B * N
+                 : parent.size() != N || !shape(tok, {B, N}) || !shape(ua, {B, N}))
+            fail("%s: inconsistent shapes", what);
         tree_tok = (const int32_t *)dev(tok, I32, "tree_tok");
         tree_cand = (const uint8_t *)dev(a[1], U8, "tree_cand");
         cand_id = (const int32_t *)dev(id, I32, "cand_id");
@@ -487,7 +526,7 @@ PyObject *verify_fused(PyObject *const *a) {
     HostI32 parent(a[2], "parent");
     const at::Tensor &hidden = need(a[0], "hidden", 3), &W = need(a[1], "W", 2);
     const int64_t B = hidden.size(0), N = hidden.size(1), d = hidden.size(2);
-    const VerifyArgs v("verify_fused", B, N, W.size(0), parent, a + 3);
+    const VerifyArgs v("verify_fused", B, N, W.size(0), parent, a + 3, true);
     const float T = number(a[9]);
     const specroll_verify_desc D = {(int32_t)B, (int32_t)N, (int32_t)v.K, (int32_t)v.k, (int32_t)v.V, T, 0};
     const at::Tensor want = alloc({B * N, v.k}, I32, hidden);
@@ -555,7 +594,7 @@ PyObject *reflex_sketch(PyObject *const *a) {  // X, Pi, rows
 
 PyObject *reflex_gate(PyObject *const *a) {
     // s, xi, slot, keep, n, mean, M2, n_fb, m, horizon, n_align_min, n_fb_min, alpha_lo, alpha_hi, z_delta, mem_eps
-    const at::Tensor &s = need(a[0], "s", 2), &m = need(a[8], "m", 2), &am = need(a[10], "n_align_min", 1);
+    const at::Tensor &s = need(a[0], "s", 2), &m = need(a[8], "m", 2), &am = need(a[10], "n_align_min");
     const int64_t R = s.size(0), S = m.size(0);
     const specroll_gate_desc D = {(int32_t)R, (int32_t)S, (int32_t)m.size(1), (int32_t)s.size(1), (int32_t)am.size(0), number(a[14]), number(a[15]), 0};
     Out out(nullptr);
@@ -620,6 +659,7 @@ PyMethodDef methods[] = {METHOD(attach, 3),
                          METHOD(tree_draw, 6),
                          METHOD(tree_attn, 14),
                          METHOD(tree_attn_paged, 16),
+                         METHOD(commit_path, 11),
                          METHOD(commit_path_layers, 11),
                          METHOD(gather_hidden, 3),
                          METHOD(verify, 12),
