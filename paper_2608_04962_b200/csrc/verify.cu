@@ -30,7 +30,8 @@ constexpr int RS_THREADS = 256;
 constexpr int WALK_WARPS = 4;
 constexpr int TERM_THREADS = 512;  // two CTAs per SM
 constexpr int TERM_WARPS = TERM_THREADS / 32;
-constexpr int TERM_SMEM_LIMIT = 200 * 1024;  // slice masses of the terminal draw
+constexpr int TERM_SMEM_LIMIT = 200 * 1024;  // slice masses of the terminal draw by one CTA
+constexpr int WALK_CTA_SMEM = 220 * 1024;    // the same, by a cluster or alone, and the staged walk
 constexpr float NEG_INF = -INFINITY;
 
 // ------------------------------------------------------------------------------ row statistics
@@ -1822,6 +1823,7 @@ __global__ void __launch_bounds__(TERM_THREADS) terminal_kernel(TermArgs a) {
 // cluster of n_cta CTAs that share the passes over a row (walk_cta_split); the cluster's first CTA does the nodes.
 struct WalkCtaLayout {
     size_t stage, slots, total;  // in front of the stage: the threshold search, whose place the draw's slice masses take
+    bool grouped;                // a node by one group of lanes, with its slots' proposals (k <= 32, and where they fit: V < 5 M)
 };
 __host__ __device__ inline WalkCtaLayout walk_cta_layout(int N, int K, int k, int V, int n_cta, bool nuc) {
     WalkCtaLayout L;
@@ -1829,7 +1831,8 @@ __host__ __device__ inline WalkCtaLayout walk_cta_layout(int N, int K, int k, in
     if (nuc && L.stage < sizeof(NucleusSmem)) L.stage = sizeof(NucleusSmem);
     L.stage = (L.stage + 15) / 16 * 16;
     L.slots = L.stage + (walk_buf_bytes(N, K, k) + 15) / 16 * 16;
-    L.total = L.slots + walk_slots_bytes(N, k);
+    L.grouped = k <= 32 && L.slots + walk_slots_bytes(N, k) <= (size_t)TERM_SMEM_LIMIT;
+    L.total = L.slots + (L.grouped ? walk_slots_bytes(N, k) : 0);
     return L;
 }
 
@@ -1848,7 +1851,7 @@ walk_cta_kernel(WalkArgs a, Topo topo, float c, float top_p, float *__restrict__
     __shared__ double sh_ovm[SPECROLL_MAX_TOPK];
     const int rank = n_cta > 1 ? (int)cluster_ctarank() : 0, b = blockIdx.x / n_cta;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __shared__ int sh_odd;            // the slots' weights underflow, or k > 32: walk_node
+    __shared__ int sh_odd;            // not grouped, or the slots' weights underflow: walk_node
     const WalkCtaLayout L = walk_cta_layout(a.N, a.K, a.k, a.V, n_cta, NUC);
     const WalkBuf buf = walk_buf(nuc_raw + L.stage, a.N, a.K, a.k);
     const WalkSlots slots = walk_slots(nuc_raw + L.slots, a.N, a.k);
@@ -1860,11 +1863,11 @@ walk_cta_kernel(WalkArgs a, Topo topo, float c, float top_p, float *__restrict__
     // Set up under the tail of the kernel before.  Where that is this call's own (statistics, thresholds), which itself
     // started when everything in front of the call was complete, the call's inputs are staged ahead of the wait.
     if (LAZY) pdl_wait();
-    if (threadIdx.x == 0) sh_odd = a.k > 32;
+    if (threadIdx.x == 0) sh_odd = !L.grouped;
     if (rank == 0) {
         walk_buf_fetch(a, topo, b, buf);
         __syncthreads();
-        if (a.k <= 32) walk_slots_fill(buf, topo, a.N, a.k, b, slots, &sh_odd);
+        if (L.grouped) walk_slots_fill(buf, topo, a.N, a.k, b, slots, &sh_odd);
     }
     if (!LAZY) {
         pdl_wait();
@@ -2078,6 +2081,7 @@ __device__ __forceinline__ void walk_nodes(const Topo &topo, int N, int k, const
 
 struct WtLayout {
     size_t stage, ovm, first, mm, slices, p, slots, total;
+    bool grouped;  // (as WalkCtaLayout's; V < 3 M)
 };
 __host__ __device__ inline WtLayout wt_layout(int N, int K, int k, size_t draw_bytes) {
     WtLayout L;
@@ -2096,7 +2100,8 @@ __host__ __device__ inline WtLayout wt_layout(int N, int K, int k, size_t draw_b
     L.p = o;
     o += up((size_t)N * k * sizeof(double));
     L.slots = o;
-    o += up(walk_slots_bytes(N, k));
+    L.grouped = k <= 32 && o + walk_slots_bytes(N, k) <= (size_t)WT_SMEM_LIMIT;
+    if (L.grouped) o += up(walk_slots_bytes(N, k));
     L.total = o;
     return L;
 }
@@ -2308,10 +2313,10 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     if (TILES) pdl_wait();
     const WalkSlots slots = walk_slots(sh_dyn + L.slots, N, k);
     __shared__ int sh_odd;
-    if (tid == 0) sh_odd = k > 32;
+    if (tid == 0) sh_odd = !L.grouped;
     walk_buf_fetch(a, topo, b, buf);
     __syncthreads();
-    if (k <= 32) walk_slots_fill(buf, topo, N, k, b, slots, &sh_odd);
+    if (L.grouped) walk_slots_fill(buf, topo, N, k, b, slots, &sh_odd);
     pdl_wait();  // the row statistics are complete from here on
     if (!TILES && run_tab) {
         // a row's statistics from its eight runs, eight lanes per row (N <= 64: one round; the result as row_stats_kernel's)
@@ -2464,12 +2469,14 @@ static int walk_term_split(int B) {
     return S;
 }
 
+// Vocabularies whose slice masses one CTA can hold.
+static bool draw_fits(int V) { return (size_t)TERM_WARPS * draw_slices(V >> 3, 1) * sizeof(double) <= (size_t)TERM_SMEM_LIMIT; }
+
 static int launch_terminal(const TermArgs &ta, cudaStream_t st) {
-    const size_t smem = draw_smem_bytes(ta.V, 1);
-    if (smem > (size_t)TERM_SMEM_LIMIT) return SPECROLL_ELIMIT;
-    const int rc = device_setup(reinterpret_cast<const void *>(terminal_kernel), TERM_SMEM_LIMIT, nullptr);
+    if (!draw_fits(ta.V)) return SPECROLL_ELIMIT;
+    const int rc = device_setup(reinterpret_cast<const void *>(terminal_kernel), WALK_CTA_SMEM, nullptr);
     if (rc != SPECROLL_OK) return rc;
-    terminal_kernel<<<ta.B, TERM_THREADS, smem, st>>>(ta);
+    terminal_kernel<<<ta.B, TERM_THREADS, draw_smem_bytes(ta.V, 1), st>>>(ta);
     SR_LAUNCH_CHECK();
     return SPECROLL_OK;
 }
@@ -2620,9 +2627,9 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     if (truncate || lazy) {
         const int n_cta = walk_cta_split(d->B);
         const size_t smem = walk_cta_layout(d->N, d->K, d->k, d->V, n_cta, truncate).total;
-        if (smem > (size_t)TERM_SMEM_LIMIT) return SPECROLL_ELIMIT;
+        if (!draw_fits(d->V) || smem > (size_t)WALK_CTA_SMEM) return SPECROLL_ELIMIT;
         auto *const kern = truncate ? (lazy ? walk_cta_kernel<true, true> : walk_cta_kernel<false, true>) : walk_cta_kernel<true, false>;
-        int rc_ = device_setup(reinterpret_cast<const void *>(kern), TERM_SMEM_LIMIT, nullptr);
+        int rc_ = device_setup(reinterpret_cast<const void *>(kern), WALK_CTA_SMEM, nullptr);
         if (rc_ != SPECROLL_OK) return rc_;
         bool ahead = false;
         if (truncate && !lazy) {

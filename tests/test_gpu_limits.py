@@ -81,3 +81,28 @@ def test_empty_batch_is_accepted_and_launches_nothing_wrong():
                  z((0, K, k), torch.int32), z((0, K, k), torch.float32), z((0, N), torch.float32), z((0,), torch.float32))
     torch.cuda.synchronize()
     assert v["n_acc"].shape == (0,) and v["out_tok"].shape == (0, K + 1)
+
+
+@pytest.mark.parametrize("N,k,V,lazy,top_p", [(64, 32, 3400000, False, 1.0), (8, 4, 6553600, True, 1.0), (8, 4, 6553600, False, 0.9)])
+def test_the_largest_vocabularies_that_a_draw_takes(N, k, V, lazy, top_p):
+    """Slice masses that leave no room in shared memory for a whole tree's slot proposals: the walk node by node."""
+    w = I.scaled(I.WORKLOADS["qwen1.5b"], B=1, N=N, K=5 if k > 4 else 3, k=k, V=V)
+    parent = I.topology(w)
+    g = I.rng(9)
+    cid = (np.arange(w.K * k, dtype=np.int64).reshape(1, w.K, k) * (V // (w.K * k + 1)) + 7).astype(np.int32)
+    cl = -np.sort(-g.standard_normal((1, w.K, k)).astype(np.float32), axis=-1)
+    d = ref.tree_draw(parent, np.zeros(1, np.int32), cid, cl, I.uniforms24(3, (1, N)))
+    x = torch.randn((1, N, V), generator=torch.Generator(device="cuda").manual_seed(2), device="cuda", dtype=torch.bfloat16)
+    depth = I.node_depths(parent)
+    for u in range(N):  # mass on the candidates, so that something is accepted
+        x[0, u, torch.from_numpy(cid[0, min(depth[u], w.K - 1)]).cuda().long()] = 14.0
+    u_acc, u_fin = I.uniforms24(4, (1, N)), I.uniforms24(5, (1,))
+    args = (x, parent, dev(d["tree_tok"]), dev(d["tree_cand"]), dev(cid), dev(cl), dev(u_acc), dev(u_fin))
+    flags = S.VERIFY_LAZY_STATS if lazy else 0
+    got = S.verify_nucleus(*args, top_p, flags=flags) if top_p < 1.0 else S.verify(*args, flags=flags)
+    o = ref.verify(S.bf16_bits(x), parent, d["tree_tok"], d["tree_cand"], cid, cl, u_acc, u_fin, top_p=top_p)
+    assert o["min_margin"][0] > 1e-4
+    for key in ("n_acc", "path_node", "term_node", "term_kind"):
+        assert np.array_equal(host(got[key]), o[key]), key
+    if o["fin_margin"][0] > 1e-6:
+        assert np.array_equal(host(got["out_tok"]), o["out_tok"])
