@@ -12,8 +12,8 @@
 //                       inverse CDF over the vocabulary in token order with fp64 segment sums, the
 //                       walk's <= k residual entries overriding the plain softmax mass.
 // Logits that were never stored: the same kernel with the projection's numbers (wanted logits, tile masses) in
-// place of the rows.  The other forms (statistics only of visited rows, nucleus targets, the steps one by one) use
-// walk_kernel / walk_cta_kernel and terminal_kernel.
+// place of the rows.  Statistics only of visited rows, and nucleus targets: walk_cta_kernel, walk and draw too.  The steps
+// one by one, for logits that were never stored: walk_kernel and terminal_kernel.
 #include <math.h>
 
 #include <algorithm>
@@ -809,8 +809,8 @@ struct WalkSmem {
     int32_t jc[32];
 };
 
-// Everything the walk of one sequence can read, staged in shared memory in one round of independent loads (the
-// plain walk; the other forms read global memory node by node): per node the row's statistics, the acceptance
+// Everything the walk of one sequence can read, staged in shared memory in one round of independent loads (the walk on
+// its own reads global memory node by node): per node the row's statistics, the acceptance
 // uniform, the drawn token and its slot; per head the candidate ids and proposal logits; per walkable node the
 // target logits at its head's candidates.
 struct WalkStage {
@@ -844,7 +844,7 @@ __device__ __forceinline__ void walk_begin(const WalkArgs &a, int b, int lane, W
 // One node u (which has children), by one warp: the target's probabilities on the candidates of u's head -
 // S is the normaliser and thr the nucleus threshold key (0: none) of u's row - then u's children in slot order.
 // Returns the accepted child, or -1 when every child was rejected (the residual is then in sm->r, st->sigma).
-// sg (nullable): the sequence's inputs staged in shared memory.
+// sg (nullable: a.cand_target and the other arrays are read): the sequence's inputs staged in shared memory.
 // emit = false: nothing is written to the results and the count of accepted tokens stays (the node is examined
 // on its own, before it is known whether the walk reaches it).
 __device__ int walk_node_seq(const WalkArgs &a, const Topo &topo, int b, int u, double M, double S, uint32_t thr,
@@ -854,8 +854,7 @@ __device__ int walk_node_seq(const WalkArgs &a, const Topo &topo, int b, int u, 
     int32_t *id = sm->id;
     const int k = a.k, N = a.N, K = a.K;
     const int hd = topo.depth[u];
-    const uint16_t *lg = a.logits ? a.logits + ((size_t)b * N + u) * a.V : nullptr;
-    const uint16_t *ct = a.cand_target ? a.cand_target + ((size_t)b * N + u) * k : nullptr;
+    const uint16_t *ct = sg ? sg->pre + u * k : a.cand_target + ((size_t)b * N + u) * k;
     // Quotients whose numerator can be exactly zero (the largest logit minus itself, a taken candidate's weight, a
     // residual entry clamped to zero) are formed as products with a reciprocal: a double division with a zero
     // numerator leaves the division's fast path, and one lane on the slow path holds up the whole warp at every slot.
@@ -864,7 +863,7 @@ __device__ int walk_node_seq(const WalkArgs &a, const Topo &topo, int b, int u, 
         const int t = sg ? sg->cid[hd * k + j] : SR_CHECKED(a.cand_id[((size_t)b * K + hd) * k + j], a.V, b);
         id[j] = t;
         cl[j] = sg ? sg->clog[hd * k + j] : a.cand_logit[((size_t)b * K + hd) * k + j];
-        const uint32_t bits = sg ? sg->pre[u * k + j] : (lg ? lg[t] : ct[j]);
+        const uint32_t bits = ct[j];
         const double l = (double)bf16_bits_to_float((uint16_t)bits);
         r[j] = ord_key(bits) >= thr ? exp((l - M) * inv_T) * inv_S : 0.0;  // r = p_u on the candidates
     }
@@ -986,13 +985,7 @@ __device__ int walk_node(const WalkArgs &a, const Topo &topo, int b, int u, doub
         if (have) {
             const int tok = sg ? sg->cid[hd * k + j] : SR_CHECKED(a.cand_id[((size_t)b * K + hd) * k + j], a.V, b);
             clj = sg ? sg->clog[hd * k + j] : a.cand_logit[((size_t)b * K + hd) * k + j];
-            uint32_t bits;
-            if (sg)
-                bits = sg->pre[u * k + j];
-            else if (a.logits)
-                bits = a.logits[((size_t)b * N + u) * a.V + tok];
-            else
-                bits = a.cand_target[((size_t)b * N + u) * k + j];
+            const uint32_t bits = sg ? sg->pre[u * k + j] : a.cand_target[((size_t)b * N + u) * k + j];
             const double l = (double)bf16_bits_to_float((uint16_t)bits);
             rho = ord_key(bits) >= thr ? exp((l - M) * inv_T) * inv_S : 0.0;
             if (lane < k) sm->id[j] = tok;
@@ -1303,60 +1296,14 @@ __device__ __forceinline__ int walk_group(const Topo &topo, int u, int k, int kp
     return f < 0 ? -1 : child;
 }
 
-// Plain target distributions: one warp per sequence.  Which nodes the walk visits depends on its decisions, but
-// what it can ask for does not, so with the dense logits everything is fetched up front (WalkStage): one round
-// trip to memory per sequence instead of four or five dependent ones per visited node, which is what the walk's
-// time consisted of.  Dynamic shared memory: WALK_WARPS * walk_stage_bytes.
+// The walk alone, one warp per sequence, on the target logits of the nodes' candidates (a.cand_target): read node by node.
 __global__ void __launch_bounds__(WALK_WARPS * 32) walk_kernel(WalkArgs a, Topo topo) {
     __shared__ WalkSmem sh[WALK_WARPS];
-    extern __shared__ __align__(16) unsigned char sh_stage[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.x * WALK_WARPS + warp;
     if (b >= a.B) return;
     WalkSmem *sm = &sh[warp];
-    const int N = a.N, K = a.K, k = a.k;
-    WalkStage stage;
-    const WalkStage *sg = nullptr;
-    if (a.logits) {
-        auto up = [](size_t x) { return (x + 15) / 16 * 16; };
-        unsigned char *p = sh_stage + (size_t)warp * walk_stage_bytes(N, K, k);
-        float *rmax = reinterpret_cast<float *>(p);
-        p += up((size_t)N * 4);
-        float *rsum = reinterpret_cast<float *>(p);
-        p += up((size_t)N * 4);
-        float *uacc = reinterpret_cast<float *>(p);
-        p += up((size_t)N * 4);
-        int32_t *ttok = reinterpret_cast<int32_t *>(p);
-        p += up((size_t)N * 4);
-        uint8_t *tcand = reinterpret_cast<uint8_t *>(p);
-        p += up((size_t)N);
-        int32_t *cid = reinterpret_cast<int32_t *>(p);
-        p += up((size_t)K * k * 4);
-        float *clog = reinterpret_cast<float *>(p);
-        p += up((size_t)K * k * 4);
-        uint16_t *pre = reinterpret_cast<uint16_t *>(p);
-        for (int n = lane; n < N; n += 32) {
-            rmax[n] = a.row_max[(size_t)b * N + n];
-            rsum[n] = a.row_sum[(size_t)b * N + n];
-            uacc[n] = a.u_acc[(size_t)b * N + n];
-            ttok[n] = a.tree_tok[(size_t)b * N + n];
-            tcand[n] = a.tree_cand[(size_t)b * N + n];
-        }
-        for (int e = lane; e < K * k; e += 32) {
-            cid[e] = SR_CHECKED(a.cand_id[(size_t)b * K * k + e], a.V, b);
-            clog[e] = a.cand_logit[(size_t)b * K * k + e];
-        }
-        for (int e = lane; e < N * k; e += 32) {
-            const int u = e / k, j = e - u * k;
-            if (topo.n_child[u] > 0) {  // (a node with children is at depth < K)
-                const int t = SR_CHECKED(a.cand_id[((size_t)b * K + topo.depth[u]) * k + j], a.V, b);
-                pre[e] = a.logits[((size_t)b * N + u) * a.V + t];
-            }
-        }
-        __syncwarp();
-        stage = WalkStage{rmax, rsum, uacc, ttok, tcand, cid, clog, pre, nullptr, nullptr, nullptr};
-        sg = &stage;
-    }
+    const float *row_max = a.row_max + (size_t)b * a.N, *row_sum = a.row_sum + (size_t)b * a.N;
     WalkState st;
     walk_begin(a, b, lane, &st);
     int u = 0;
@@ -1366,9 +1313,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32) walk_kernel(WalkArgs a, Topo 
             st.have_residual = false;
             break;
         }
-        const double M = sg ? (double)sg->rmax[u] : (double)a.row_max[(size_t)b * N + u];
-        const double S = sg ? (double)sg->rsum[u] : (double)a.row_sum[(size_t)b * N + u];
-        const int acc = walk_node(a, topo, b, u, M, S, 0u, lane, sm, &st, sg);
+        const int acc = walk_node(a, topo, b, u, (double)row_max[u], (double)row_sum[u], 0u, lane, sm, &st);
         if (acc < 0) {
             st.kind = 0;
             st.have_residual = true;
@@ -1376,7 +1321,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32) walk_kernel(WalkArgs a, Topo 
         }
         u = acc;
     }
-    walk_end(a, b, u, sg ? (double)sg->rsum[u] : (double)a.row_sum[(size_t)b * N + u], lane, sm, &st);
+    walk_end(a, b, u, (double)row_sum[u], lane, sm, &st);
 }
 
 // Maximum and sum of exponentials of one row by all NUC_THREADS threads of n_cta CTAs (a cluster; 1: a CTA alone); every
@@ -2544,15 +2489,9 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < need)
         return SPECROLL_EWORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    const size_t B = (size_t)d->B, k = (size_t)d->k;
-    char *ws = static_cast<char *>(workspace);
-    double *ws_ovm = reinterpret_cast<double *>(ws);
-    ws += align_up(B * k * sizeof(double), 256);
-    int32_t *ws_ovid = reinterpret_cast<int32_t *>(ws);
-    ws += align_up(B * k * sizeof(int32_t), 256);
-    int32_t *ws_nov = reinterpret_cast<int32_t *>(ws);
-    ws += align_up(B * sizeof(int32_t), 256) + 256;
-    const size_t n_rows = B * (size_t)d->N;
+    // (the workspace begins with the hand-over area of the walk on its own, which these kernels do not need)
+    char *ws = static_cast<char *>(workspace) + verify_ws_base(d);
+    const size_t n_rows = (size_t)d->B * d->N;
     uint32_t *thr_key = truncate ? reinterpret_cast<uint32_t *>(ws) : nullptr;
     float *keep_sum = truncate ? reinterpret_cast<float *>(ws + align_up(n_rows * sizeof(uint32_t), 256)) : nullptr;
 
@@ -2615,9 +2554,9 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     wa.term_node = term_node;
     wa.term_kind = term_kind;
     wa.min_margin = min_margin;
-    wa.ws_nov = ws_nov;
-    wa.ws_ovid = ws_ovid;
-    wa.ws_ovm = ws_ovm;
+    wa.ws_nov = nullptr;
+    wa.ws_ovid = nullptr;
+    wa.ws_ovm = nullptr;
     wa.B = d->B;
     wa.N = d->N;
     wa.K = d->K;

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import ref
 from paper_2608_04962_b200 import binding as S
 from paper_2608_04962_b200 import inputs as I
 from tests.test_gpu_verify_fused import _case
@@ -91,3 +92,28 @@ def test_inputs_written_by_the_kernel_in_front_of_the_walk():
             assert torch.equal(got[k], want[k]), (i, k)
     x.u_acc.zero_()
     assert not torch.equal(x.hidden()["n_acc"], want["n_acc"])
+
+
+@pytest.mark.parametrize("name,B,V,d,T", [("tiny", 41, 1032, 128, 1.0), ("qwen7b", 6, 8200, 256, 0.7), ("qwen1.5b", 3, 151936, 64, 1.3)])
+def test_the_steps_of_a_verification_from_hidden_states_one_by_one(name, B, V, d, T):
+    """Walk on the wanted logits, the last nodes' rows by the storing projection, the draw from them; against the oracle on
+    the stored logits of the same projection.  Bounds: those of the verification on stored logits."""
+    x = Hidden(name, B, V, d, T, 60 + B)
+    x.project(tiles=False)
+    w, o = x.w, verify_outputs(x.w)
+    S.lib().specroll_verify_workspace_bytes.restype = C.c_size_t
+    ws = empty(S.lib().specroll_verify_workspace_bytes(C.byref(x.desc)), dtype=torch.uint8)
+    call("specroll_verify_walk_sparse", x.desc, x.want_logit, x.rmax, x.rsum, x.parent, x.tok, x.tcand, x.cid, x.cl, x.u_acc,
+         *o.values(), ws, C.c_size_t(ws.numel()))
+    last = S.target_head_rows(S.gather_hidden(x.H, o["term_node"]), x.W)
+    call("specroll_verify_terminal_rows", x.desc, last, x.rmax, o["n_acc"], o["term_node"], x.u_fin, o["out_tok"], ws,
+         C.c_size_t(ws.numel()))
+    logits = S.bf16_bits(S.target_head_rows(x.H.view(B * w.N, d), x.W)).reshape(B, w.N, V)
+    want = ref.verify(logits, x.parent, host(x.tok), host(x.tcand), host(x.cid), host(x.cl), host(x.u_acc), host(x.u_fin),
+                      temperature=T)
+    sure = want["min_margin"] >= 1e-4
+    assert sure.mean() >= 0.8
+    for key in ("n_acc", "path_node", "term_node", "term_kind"):
+        assert np.array_equal(host(o[key])[sure], want[key][sure]), key
+    sure &= want["fin_margin"] >= 1e-6
+    assert np.array_equal(host(o["out_tok"])[sure], want["out_tok"][sure])
