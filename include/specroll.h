@@ -248,7 +248,8 @@ int specroll_commit_path(int32_t B, int32_t N, int32_t K, int32_t Hkv, int32_t D
 
 /* The same for all layers of a model in one launch per 64 layers: Kt, Vt, Kp, Vp are HOST arrays of
  * n_layers device pointers (read during the call, not retained); every layer shares the page table,
- * the lengths and n_pages.  kv_len_out is written once, after the last layer's copies. */
+ * the lengths and n_pages.  kv_len_out is written once: beside the first layers' copies, or after the last ones where it
+ * overlaps kv_len. */
 int specroll_commit_path_layers(int32_t B, int32_t N, int32_t K, int32_t Hkv, int32_t D,
                                 int32_t n_layers, const void *const *Kt, const void *const *Vt,
                                 const int32_t *path_node, const int32_t *n_acc, void *const *Kp,
@@ -486,7 +487,8 @@ int specroll_verify_terminal_rows(const specroll_verify_desc *desc, const void *
  * terminal draw then use the truncated distributions, so the emitted tokens are exact samples of them.
  * row_max / row_sum are still those of the plain softmax.  Optional outputs (device, nullable):
  * nucleus_thr[B,N] fp32 = logit of the smallest kept token, nucleus_sum[B,N] fp32 = sum of
- * exp((l - row_max)/T) over the kept tokens.  Workspace: specroll_verify_nucleus_workspace_bytes. */
+ * exp((l - row_max)/T) over the kept tokens, written for the nodes that the walk visits (and, where the batch is small, for
+ * every node with children).  Workspace: specroll_verify_nucleus_workspace_bytes. */
 size_t specroll_verify_nucleus_workspace_bytes(const specroll_verify_desc *desc);
 
 int specroll_verify_nucleus(const specroll_verify_desc *desc, float top_p, const void *logits,

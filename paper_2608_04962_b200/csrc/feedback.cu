@@ -232,7 +232,7 @@ __device__ void topk_radix(TopkRadixSmem &sm, int &sh_above, int &sh_prefix, int
 // of the row (there are at least kS elements at or above it).  The groups that reach it, about kS of several thousand,
 // are read again, a thread per vector, and their elements at or above the bound ranked by (key desc, id asc): the rank
 // is the place in the result.  More elements than the list holds (a row with thousands of equal large values): the radix
-// search.  Bound by the one stream of the rows.  512 rows of 152064 tokens: 27 us (5.8 TB/s); reading the row twice and
+// search.  Bound by the one stream of the rows.  512 rows of 152064 tokens: 32 us (4.9 TB/s); reading the row twice and
 // ranking the 512 maxima against one another, as before, 76 us.
 __global__ void __launch_bounds__(fb::TOPK_THREADS, 4)
 feedback_topk_kernel(const uint16_t *__restrict__ logits, const int32_t *__restrict__ rec_row, int V, int kS,

@@ -1934,6 +1934,12 @@ static int walk_cta_split(int B) {
 // them the walk visits is not known yet, but a row's threshold depends on the row alone, and one pass of all
 // of them over the machine costs less than the visited ones one after the other inside a sequence's walk.  (A
 // sequence that ends at a leaf still needs that leaf's threshold for its last token: the walk kernel finds it.)
+// A whole verification, us, walk alone -> thresholds ahead; rows = sequences x nodes with children:
+//   V 151936, 8 such nodes:  32 rows 86 -> 73, 128: 99 -> 86, 256: 135 -> 127, 512: 155 -> 169, 768: 206 -> 240, 2048: 367 -> 475
+//   V 152064, 22 such nodes: 88 rows 103 -> 90, 352: 140 -> 150, 704: 187 -> 225, 1408: 251 -> 354
+//   V 32000, 8 such nodes:   32 rows 59 -> 53, 256: 67 -> 61, 512: 75 -> 78, 768: 85 -> 88, 2048: 105 -> 152
+// The times cross near 300 rows, two per SM.  The line stays at five because up to there a call also leaves the thresholds and
+// kept sums of the nodes with children that its walks do not visit.
 #ifndef NUC_AHEAD_ROWS_PER_SM
 #define NUC_AHEAD_ROWS_PER_SM 5
 #endif
@@ -2503,8 +2509,12 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     if (rc_sm != SPECROLL_OK) return rc_sm;
     if (use_runs) {
         // Up to 44 runs per SM (814 rows) the form with the rings; with more rows there are warps enough, and the ring's
-        // bookkeeping costs issue slots (verification, V 152 k: 20 rows 29 -> 19 us, 256 rows 48 -> 34, 512 rows 54 -> 47,
-        // 768 rows 63.5 -> 60.5, 1024 rows 70 -> 72.6, 4096 rows 198 -> 234).
+        // bookkeeping costs issue slots.  A whole verification, us, CTA per row -> rings:
+        //   V 151936: 512 rows 47.2 -> 45.1, 768: 61.3 -> 61.0, 896: 66.6 -> 65.9, 1024: 68.0 -> 71.9, 1536: 95.6 -> 101.3
+        //   V 64000:  512 rows 26.8 -> 25.9, 768: 34.0 -> 34.2, 896: 36.1 -> 36.9, 1024: 37.5 -> 39.5, 1536: 47.3 -> 51.6
+        //   V 32000:  512 rows 21.3 -> 19.7, 768: 24.0 -> 23.1, 1024: 26.9 -> 26.0, 1536: 31.8 -> 37.2
+        //   V 8000:   512 rows 18.8 -> 16.2, 1024: 20.3 -> 17.8, 1536: 21.6 -> 19.5
+        // (20 rows of 152 k tokens from HBM 29 -> 19, 4096 rows 198 -> 234.)
         const int n_runs = rows * RS_WARPS, most = RUN_WARPS * RUN_CTAS * n_sm, rounds = (n_runs + most - 1) / most;
         if (n_runs <= 44 * n_sm) {
             // every warp the same number of runs (to one), and a CTA for each while there is room

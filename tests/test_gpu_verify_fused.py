@@ -1,5 +1,5 @@
-"""GPU: verification from hidden states (fused projection statistics, sparse walk, terminal rows) against the
-verification on stored logits and against the CPU oracle."""
+"""GPU: verification from hidden states (projection with fused statistics and tile masses, then the walk and the last token from
+one vocabulary tile) against the verification on stored logits and against the CPU oracle."""
 import numpy as np
 import pytest
 import torch
