@@ -31,7 +31,7 @@ constexpr int WALK_WARPS = 4;
 constexpr int TERM_THREADS = 512;  // two CTAs per SM
 constexpr int TERM_WARPS = TERM_THREADS / 32;
 constexpr int TERM_SMEM_LIMIT = 200 * 1024;  // slice masses of the terminal draw by one CTA
-constexpr int WALK_CTA_SMEM = 220 * 1024;    // the same, by a cluster or alone, and the staged walk
+constexpr int WALK_CTA_SMEM = 220 * 1024;    // the same and the staged walk
 constexpr float NEG_INF = -INFINITY;
 
 // ------------------------------------------------------------------------------ row statistics
@@ -1644,24 +1644,22 @@ __device__ void term_pick(const uint4 *__restrict__ p, const double *seg_slices,
     term_pick_token(i, ms, lsum, base, target, take_last, v_hi, dst, lane);
 }
 
-// The vectors [v_base, v_base + nvec_r) of a row are cut into one segment per warp of the draw's n_cta CTAs (a cluster;
-// 1: a CTA alone), each walked in slices of 32 vectors (one per lane); the slices, whose masses are fp32 sums, are the same
-// ones however many CTAs there are.  Pass 1 (all warps, independent loads) leaves the
-// fp64 mass of every slice in shared memory, those of the cluster's other CTAs are read by its first CTA; the residual
-// entries (nov tokens ovid, masses ovm) then replace the plain mass of their tokens; two scans pick the segment and the
-// slice that hold the target, and only that slice is read again to find the token.
+// The vectors [v_base, v_base + nvec_r) of a row are cut into one segment per warp of a CTA, each walked in slices of 32
+// vectors (one per lane); the n_cta CTAs of a cluster (1: a CTA alone) share the slices of every segment.  Pass 1 (all warps,
+// independent loads) leaves the mass of every slice in shared memory, those of the cluster's other CTAs are read by its first
+// CTA; the residual entries (nov tokens ovid, masses ovm) then replace the plain mass of their tokens; two scans pick the segment
+// and the slice that hold the target, and only that slice is read again to find the token.  Segments, slices and the order of all
+// sums are the same however many CTAs there are: the draw from a flat tail follows their last bits.
 //   thr       nucleus threshold key of the row, 0 for none
 //   bits(j)   the bf16 logit of token ovid[j]
 //   base      the mass before v_base; target < 0: u times the total
 // By all TERM_THREADS threads of every CTA; slices: draw_smem_bytes, at the same offset in every CTA.  Bound by latency
 // (a few hundred KB per sequence), which is why the loads of a round are issued together.
-__host__ __device__ inline int draw_slices(int nvec, int n_cta) {
-    const int vpw = (nvec + TERM_WARPS * n_cta - 1) / (TERM_WARPS * n_cta);
+__host__ __device__ inline int draw_slices(int nvec) {
+    const int vpw = (nvec + TERM_WARPS - 1) / TERM_WARPS;
     return ((vpw > 0 ? vpw : 1) + 31) / 32;
 }
-__host__ __device__ inline size_t draw_smem_bytes(int V, int n_cta) {
-    return (size_t)TERM_WARPS * n_cta * (draw_slices(V >> 3, n_cta) + 1) * sizeof(double);
-}
+__host__ __device__ inline size_t draw_smem_bytes(int V) { return (size_t)TERM_WARPS * (draw_slices(V >> 3) + 1) * sizeof(double); }
 
 template <class Bits>
 __device__ void draw_row(const uint16_t *__restrict__ lg, int v_base, int nvec_r, float M, float c, uint32_t thr, int n_cta, int rank,
@@ -1669,23 +1667,23 @@ __device__ void draw_row(const uint16_t *__restrict__ lg, int v_base, int nvec_r
                          float u, int32_t *dst) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint4 *p = reinterpret_cast<const uint4 *>(lg);
-    const int G = n_cta * TERM_WARPS;
-    const int n_sl = draw_slices(nvec_r, n_cta), vpw = n_sl * 32;  // slices and vectors per warp segment
+    constexpr int G = TERM_WARPS;
+    const int vpw = (nvec_r + G - 1) / G > 0 ? (nvec_r + G - 1) / G : 1;  // vectors per segment
+    const int n_sl = draw_slices(nvec_r);                                 // slices per segment
+    const int per = (n_sl + n_cta - 1) / n_cta;                           // of them per CTA
     double *seg = slices + (size_t)G * n_sl;
     {
-        const int g = rank * TERM_WARPS + warp;
-        const int v_lo = v_base + min(nvec_r, g * vpw), v_hi = v_base + min(nvec_r, g * vpw + vpw);
-        term_slice_masses(p, v_lo, v_hi, n_sl, M, c, thr, lane, slices + (size_t)g * n_sl);
+        const int v_lo = v_base + min(nvec_r, warp * vpw), v_hi = v_base + min(nvec_r, warp * vpw + vpw);
+        const int s0 = min(n_sl, rank * per), s1 = min(n_sl, s0 + per);
+        term_slice_masses(p, v_lo + s0 * 32, v_hi, s1 - s0, M, c, thr, lane, slices + (size_t)warp * n_sl + s0);
     }
     if (n_cta > 1) {
         cluster_sync_all();  // every CTA's slice masses are in its shared memory
-        if (rank == 0) {
-            const int per = TERM_WARPS * n_sl;
-            for (int e = tid; e < (n_cta - 1) * per; e += TERM_THREADS) {
-                const int r = 1 + e / per;
-                slices[per + e] = ld_dsmem_f64(slices + per + e, r);
+        if (rank == 0)
+            for (int e = tid; e < G * n_sl; e += TERM_THREADS) {
+                const int r = e % n_sl / per;
+                if (r > 0) slices[e] = ld_dsmem_f64(slices + e, r);
             }
-        }
         cluster_sync_all();  // the other CTAs may leave
         if (rank != 0) return;
     }
@@ -1699,32 +1697,20 @@ __device__ void draw_row(const uint16_t *__restrict__ lg, int v_base, int nvec_r
         }
     }
     __syncthreads();
-    for (int g = warp; g < G; g += TERM_WARPS) {
+    {
         double acc = 0.0;
-        for (int sl = lane; sl < n_sl; sl += 32) acc += slices[g * n_sl + sl];
+        for (int sl = lane; sl < n_sl; sl += 32) acc += slices[warp * n_sl + sl];
         acc = warp_sum(acc);
-        if (lane == 0) seg[g] = acc;
+        if (lane == 0) seg[warp] = acc;
     }
     __syncthreads();
     if (warp != 0) return;
-    if (target < 0.0) {
-        double total = 0.0;
-        for (int g0 = 0; g0 < G; g0 += 32) total += warp_sum(g0 + lane < G ? seg[g0 + lane] : 0.0);
-        target = (double)u * total;
-    }
-    int wsel = -1;
-    for (int g0 = 0; g0 < G && wsel < 0; g0 += 32) {
-        const double v = g0 + lane < G ? seg[g0 + lane] : 0.0;
-        const double incl = warp_incl_scan(v, lane);
-        const unsigned hit = __ballot_sync(0xffffffffu, g0 + lane < G && base + incl > target);
-        if (hit) {
-            const int lh = __ffs(hit) - 1;
-            wsel = g0 + lh;
-            base += __shfl_sync(0xffffffffu, incl - v, lh);
-        } else {
-            base += __shfl_sync(0xffffffffu, incl, 31);
-        }
-    }
+    const double v = lane < G ? seg[lane] : 0.0;
+    if (target < 0.0) target = (double)u * warp_sum(v);
+    const double incl = warp_incl_scan(v, lane);
+    const unsigned hit = __ballot_sync(0xffffffffu, lane < G && base + incl > target);
+    const int wsel = hit ? __ffs(hit) - 1 : -1;
+    if (hit) base += __shfl_sync(0xffffffffu, incl - v, wsel);
     if (wsel < 0) {
         // the target reached the end of the masses through rounding: take the last token with positive mass (from the
         // end of the vectors the draw worked on, downwards)
@@ -1770,9 +1756,9 @@ struct WalkCtaLayout {
     size_t stage, slots, total;  // in front of the stage: the threshold search, whose place the draw's slice masses take
     bool grouped;                // a node by one group of lanes, with its slots' proposals (k <= 32, and where they fit: V < 5 M)
 };
-__host__ __device__ inline WalkCtaLayout walk_cta_layout(int N, int K, int k, int V, int n_cta, bool nuc) {
+__host__ __device__ inline WalkCtaLayout walk_cta_layout(int N, int K, int k, int V, bool nuc) {
     WalkCtaLayout L;
-    L.stage = draw_smem_bytes(V, n_cta);
+    L.stage = draw_smem_bytes(V);
     if (nuc && L.stage < sizeof(NucleusSmem)) L.stage = sizeof(NucleusSmem);
     L.stage = (L.stage + 15) / 16 * 16;
     L.slots = L.stage + (walk_buf_bytes(N, K, k) + 15) / 16 * 16;
@@ -1797,7 +1783,7 @@ walk_cta_kernel(WalkArgs a, Topo topo, float c, float top_p, float *__restrict__
     const int rank = n_cta > 1 ? (int)cluster_ctarank() : 0, b = blockIdx.x / n_cta;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __shared__ int sh_odd;            // not grouped, or the slots' weights underflow: walk_node
-    const WalkCtaLayout L = walk_cta_layout(a.N, a.K, a.k, a.V, n_cta, NUC);
+    const WalkCtaLayout L = walk_cta_layout(a.N, a.K, a.k, a.V, NUC);
     const WalkBuf buf = walk_buf(nuc_raw + L.stage, a.N, a.K, a.k);
     const WalkSlots slots = walk_slots(nuc_raw + L.slots, a.N, a.k);
     const double inv_T = 1.0 / a.T;
@@ -1986,8 +1972,8 @@ nucleus_rows_kernel(const uint16_t *__restrict__ logits, int V, int N, NodeList 
 //       child (or none, and then the residual), and the smallest margin on the way.  The walk itself is then a
 //       chain of at most K + 1 look-ups.  Every CTA of a cluster does (1) and (2) for itself: same inputs, same
 //       arithmetic, same result, nothing to exchange.
-//   (3) The terminal draw over the last node's row: the S * WT_WARPS warps of the cluster each take one segment of
-//       the vocabulary; the slice masses of the other CTAs are read through distributed shared memory by the
+//   (3) The terminal draw over the last node's row: a warp of every CTA has one segment of the vocabulary, the CTAs of the
+//       cluster share its slices; the slice masses of the other CTAs are read through distributed shared memory by the
 //       cluster's first CTA, which finishes as terminal_kernel does.  (Letting the statistics pass leave the mass
 //       of every slice of every row, so that this step reads a table and one slice, was tried: the table costs the
 //       statistics kernel as much as it saves here.)
@@ -2248,7 +2234,7 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     const int rank = S > 1 ? (int)cluster_ctarank() : 0;
     const int b = blockIdx.x / S;
     const int N = a.N, K = a.K, k = a.k;
-    const WtLayout L = wt_layout(N, K, k, TILES ? HEAD_TILE * sizeof(double) : draw_smem_bytes(a.V, S));
+    const WtLayout L = wt_layout(N, K, k, TILES ? HEAD_TILE * sizeof(double) : draw_smem_bytes(a.V));
     const WalkBuf buf = walk_buf(sh_dyn + L.stage, N, K, k);
     float *rmax = buf.rmax, *rsum = buf.rsum;
     const int32_t *ttok = buf.ttok, *cid = buf.cid;
@@ -2421,13 +2407,13 @@ static int walk_term_split(int B) {
 }
 
 // Vocabularies whose slice masses one CTA can hold.
-static bool draw_fits(int V) { return (size_t)TERM_WARPS * draw_slices(V >> 3, 1) * sizeof(double) <= (size_t)TERM_SMEM_LIMIT; }
+static bool draw_fits(int V) { return (size_t)TERM_WARPS * draw_slices(V >> 3) * sizeof(double) <= (size_t)TERM_SMEM_LIMIT; }
 
 static int launch_terminal(const TermArgs &ta, cudaStream_t st) {
     if (!draw_fits(ta.V)) return SPECROLL_ELIMIT;
     const int rc = device_setup(reinterpret_cast<const void *>(terminal_kernel), WALK_CTA_SMEM, nullptr);
     if (rc != SPECROLL_OK) return rc;
-    terminal_kernel<<<ta.B, TERM_THREADS, draw_smem_bytes(ta.V, 1), st>>>(ta);
+    terminal_kernel<<<ta.B, TERM_THREADS, draw_smem_bytes(ta.V), st>>>(ta);
     SR_LAUNCH_CHECK();
     return SPECROLL_OK;
 }
@@ -2575,7 +2561,7 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     wa.T = (double)d->temperature;
     if (truncate || lazy) {
         const int n_cta = walk_cta_split(d->B);
-        const size_t smem = walk_cta_layout(d->N, d->K, d->k, d->V, n_cta, truncate).total;
+        const size_t smem = walk_cta_layout(d->N, d->K, d->k, d->V, truncate).total;
         if (!draw_fits(d->V) || smem > (size_t)WALK_CTA_SMEM) return SPECROLL_ELIMIT;
         auto *const kern = truncate ? (lazy ? walk_cta_kernel<true, true> : walk_cta_kernel<false, true>) : walk_cta_kernel<true, false>;
         int rc_ = device_setup(reinterpret_cast<const void *>(kern), WALK_CTA_SMEM, nullptr);
@@ -2608,7 +2594,7 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
     }
     // plain verification: the walk and the terminal draw in one launch, overlapping the statistics kernel's tail
     const int S = use_runs ? 1 : walk_term_split(d->B);
-    const WtLayout L = wt_layout(d->N, d->K, d->k, draw_smem_bytes(d->V, S));
+    const WtLayout L = wt_layout(d->N, d->K, d->k, draw_smem_bytes(d->V));
     if (L.total > (size_t)WT_SMEM_LIMIT) return SPECROLL_ELIMIT;
     const int rc_ = device_setup(reinterpret_cast<const void *>(walk_term_kernel<false>), WT_SMEM_LIMIT, nullptr);
     if (rc_ != SPECROLL_OK) return rc_;
