@@ -1980,8 +1980,8 @@ nucleus_rows_kernel(const uint16_t *__restrict__ logits, int V, int N, NodeList 
 constexpr int WT_THREADS = TERM_THREADS;
 constexpr int WT_SMEM_LIMIT = 160 * 1024;
 constexpr int WT_WARPS = WT_THREADS / 32;
-constexpr int WT_STATIC_SMEM = WT_WARPS * (int)sizeof(WalkSmem) + 2048;       // (at most)
-constexpr int TILE_SMEM_LIMIT = 227 * 1024 - WT_STATIC_SMEM;                  // dynamic, of the form without stored logits
+constexpr int TILE_STATIC_SMEM = 4 * 1024;                         // (at most) of the form without stored logits
+constexpr int TILE_SMEM_LIMIT = 227 * 1024 - TILE_STATIC_SMEM;     // dynamic
 
 // Every node with children on its own.  first[u]: accepted child or -1, mm[u]: smallest margin, ovm[u, j]: the residual's
 // masses where all children were rejected.  (A warp per node took 9 k
@@ -2049,12 +2049,15 @@ __host__ __device__ inline WtLayout wt_layout(int N, int K, int k, size_t draw_b
 // shape).  They are the projection's own logits to the bit: the same tensor operations over the same slices of the
 // contraction, with the tokens as M and the hidden row as the first of N = 16.  (Sums of another order, in fp32 by all threads,
 // rounded to the neighbouring bf16 value now and then, and the draw turned or the difference fell to the tile's last token.)
-// Bound by the latency of the ring's loads, one CTA per sequence.
+// Bound by the chain of the ring's slices, one CTA per sequence: 17 us more than such sums by a cluster of eight CTAs for 16
+// sequences (210 -> 227 us with the projection of 8 nodes each), the same from 32 sequences on.  (Asking L2 for the whole tile
+// first: no change.)
 namespace dt {
 constexpr int ROWS = 16, BK = 64, UMMA_K = 16, MAX_STAGES = 8, MIN_STAGES = 2;
 constexpr int W_BYTES = HEAD_TILE * BK * 2, H_BYTES = ROWS * BK * 2, STAGE_BYTES = W_BYTES + H_BYTES;
 constexpr int TMEM_COLS = 32;
 }  // namespace dt
+static_assert(dt::MIN_STAGES * dt::STAGE_BYTES >= WT_WARPS * (int)sizeof(WalkSmem), "the walk's scratch fits the ring");
 struct TileArgs {
     CUtensorMap H, W;    // [B * N, d] in boxes of dt::ROWS rows, [V, d] in boxes of HEAD_TILE
     const float2 *mass;  // [tiles][B * N]
@@ -2106,6 +2109,7 @@ __device__ void draw_tile(const TileArgs &t, size_t row, int V, float M, float c
         x = warp_sum(x);
         if (lane == 0) seg[warp] = x;
     }
+    fence_proxy_async();  // (the walk's scratch was in the ring's place)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -2228,7 +2232,7 @@ template <bool TILES>
 __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, Topo topo, const float *__restrict__ u_fin, float c,
                                                                int S, const float2 *__restrict__ run_tab, float *__restrict__ row_max_w,
                                                                float *__restrict__ row_sum_w, const __grid_constant__ TileArgs tile) {
-    __shared__ WalkSmem sh[WT_WARPS];
+    __shared__ WalkSmem sh_static[TILES ? 1 : WT_WARPS];
     extern __shared__ __align__(16) unsigned char sh_dyn[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = S > 1 ? (int)cluster_ctarank() : 0;
@@ -2245,6 +2249,8 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     double *slices = reinterpret_cast<double *>(sh_dyn + L.slices);
     double *wp = reinterpret_cast<double *>(sh_dyn + L.p);
     const double inv_T = 1.0 / a.T;
+    // scratch of nodes examined by a warp each (TILES: in the ring's place, which is not in use yet)
+    WalkSmem *const sh = TILES ? reinterpret_cast<WalkSmem *>(sh_dyn + L.total) : sh_static;
     // (1) inputs of this call, none of them written by the kernel before this one where that is the call's own (the
     // statistics).  TILES: whatever the caller has put in front of the call may still be writing them.
     if (TILES) pdl_wait();
@@ -2729,7 +2735,7 @@ extern "C" int specroll_verify_hidden(const specroll_verify_desc *d, int32_t dim
     if (rc != SPECROLL_OK) return rc;
     // a ring as deep as fits beside the walk, with room for a second CTA on an SM where there are more sequences than SMs
     TileArgs tile;
-    const int room = (d->B > n_sm ? TILE_SMEM_LIMIT / 2 - WT_STATIC_SMEM / 2 - 1024 : TILE_SMEM_LIMIT) - (int)L.total - 1024;
+    const int room = (d->B > n_sm ? TILE_SMEM_LIMIT / 2 - TILE_STATIC_SMEM / 2 - 1024 : TILE_SMEM_LIMIT) - (int)L.total - 1024;
     tile.stages = std::max(dt::MIN_STAGES, std::min(dt::MAX_STAGES, room / dt::STAGE_BYTES));
     const size_t smem = L.total + 1024 + (size_t)tile.stages * dt::STAGE_BYTES;
     if (smem > (size_t)TILE_SMEM_LIMIT) return SPECROLL_ELIMIT;
