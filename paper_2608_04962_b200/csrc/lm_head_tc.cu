@@ -3,13 +3,15 @@
 //   logits[r, v] = Zt[r, :] . W[v, :]      r < M = B*K rows,  v < V,  contraction over d
 //
 // Persistent warp-specialised kernel, one CTA per SM:
-//   warp 0   TMA producer: 128x64 tile of Zt and 256x64 tile of W per stage, 128-byte swizzle
-//   warp 1   allocates TMEM and issues tcgen05.mma (M=128, N=256, K=16), fp32 accumulators in
+//   warp 0   TMA producer: 128x64 tile of Zt and bn x 64 tile of W per stage, 128-byte swizzle
+//   warp 1   allocates TMEM and issues tcgen05.mma (M=128, N=bn, K=16), fp32 accumulators in
 //            TMEM, two accumulator buffers so the epilogue of tile i overlaps the MMAs of tile i+1
 //   warps 2-5 epilogue: tcgen05.ld, thread = row; each thread keeps the running top list of its row
 //            in registers across all vocabulary tiles of the CTA, so logits never leave the SM
 // A CTA owns one block of 128 rows and a contiguous range of vocabulary tiles; CTAs that share a
 // vocabulary range run side by side, so each W tile is fetched from HBM once and re-read from L2.
+// The tile's width bn (a multiple of 16 up to 256) and the ring's depth come from the launch: the plan cuts the
+// vocabulary evenly over the SMs that a row block has and then each share into equal tiles.
 // Partial lists go to pval/pid[M, n_groups, k] and are merged by topk_merge_kernel.
 #include "tc05.cuh"
 
@@ -30,11 +32,17 @@ int lm_head_arm_dropped_signal() { return -1; }
 #endif
 
 namespace lmtc {
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4, UMMA_K = 16;
-constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
+constexpr int BM = 128, BN_MAX = 256, BK = 64, STAGES_MAX = 8, UMMA_K = 16;
+constexpr int A_BYTES = BM * BK * 2;
 constexpr int THREADS = 192;
 constexpr int TMEM_COLS = 512;  // two 256-column accumulator buffers
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
+constexpr int SMEM_MAX = 232448, SMEM_EXTRA = 1024 /*alignment slack*/ + 256 /*barriers*/;
+__host__ __device__ constexpr int stage_bytes(int bn) { return A_BYTES + bn * BK * 2; }
+// as many stages as fit: a narrower tile is given a deeper ring, so that the bytes in flight stay the same
+constexpr int ring_stages(int bn) {
+    const int fit = (SMEM_MAX - SMEM_EXTRA) / stage_bytes(bn);
+    return fit < STAGES_MAX ? fit : STAGES_MAX;
+}
 constexpr int KMAX = 8;
 }  // namespace lmtc
 
@@ -69,33 +77,34 @@ struct TopList8 {
 
 __global__ void __launch_bounds__(lmtc::THREADS, 1)
 lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M,
-                       int V, int d, int k, int n_mblocks, int n_groups, int tiles_per_group,
+                       int V, int d, int k, int n_mblocks, int n_groups, int tiles_per_group, int bn, int stages,
                        float *__restrict__ pval, int32_t *__restrict__ pid, int32_t *__restrict__ status) {
     using namespace lmtc;
+    const int STAGE_BYTES = stage_bytes(bn);
     extern __shared__ unsigned char smem_raw[];
     pdl_launch_dependents();
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;  // 1024-byte alignment for the 128-byte swizzle atoms
     unsigned char *aligned = smem_raw + (base - raw);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(aligned + STAGES * STAGE_BYTES);
-    // barrier slots: full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2]
-    const uint32_t bar0 = base + STAGES * STAGE_BYTES;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(aligned + stages * STAGE_BYTES);
+    // barrier slots: full[stages], empty[stages], tmem_full[2], tmem_empty[2]
+    const uint32_t bar0 = base + stages * STAGE_BYTES;
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
-    auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
-    auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + b); };
-    auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * STAGES + 2 + b); };
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * STAGES + 4);
+    auto empty_bar = [&](int s) { return bar0 + 8u * (stages + s); };
+    auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * stages + b); };
+    auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * stages + 2 + b); };
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * stages + 4);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int mb = blockIdx.x % n_mblocks, grp = blockIdx.x / n_mblocks;
     const int m0 = mb * BM;
-    const int n_tiles = (V + BN - 1) / BN;
+    const int n_tiles = (V + bn - 1) / bn;
     const int t_lo = min(n_tiles, grp * tiles_per_group), t_hi = min(n_tiles, t_lo + tiles_per_group);
     const int KB = d / BK;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < stages; ++s) {
             mbar_init(full_bar(s), 1);
             mbar_init(empty_bar(s), 1);
         }
@@ -119,11 +128,11 @@ lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     // The weights do not come from the kernels before this one in the call, which the first of them starts only when all
     // work in front of the call is complete: the first stages' W tiles are loaded while the heads' outputs are still being made; Zt follows the
     // wait.  (Asking L2 for the next 16 or 40 tiles as well made the call slower, 128 -> 133 / 148 us for two sequences.)
-    const int pre = min(STAGES, (t_hi - t_lo) * KB);
+    const int pre = min(stages, (t_hi - t_lo) * KB);
     if (threadIdx.x == 0) {
         for (int i = 0; i < pre; ++i) {
             mbar_arrive_expect_tx(full_bar(i), STAGE_BYTES);
-            tma_load_2d(base + i * STAGE_BYTES + A_BYTES, &tmB, (i % KB) * BK, (t_lo + i / KB) * BN, full_bar(i));
+            tma_load_2d(base + i * STAGE_BYTES + A_BYTES, &tmB, (i % KB) * BK, (t_lo + i / KB) * bn, full_bar(i));
         }
     }
     pdl_wait();  // set up under the tail of the kernel before; its outputs are read from here on
@@ -133,9 +142,7 @@ lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
-            int issued[STAGES];
-#pragma unroll
-            for (int s = 0; s < STAGES; ++s) issued[s] = -1;
+            int issued = 0;  // loads so far (W and Zt of one slice)
             bool ok = true;
             for (int tile = t_lo; tile < t_hi && ok; ++tile) {
                 for (int kb = 0; kb < KB; ++kb) {
@@ -147,9 +154,9 @@ lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                     const bool ahead = (tile - t_lo) * KB + kb < pre;  // (its W tile is on its way)
                     if (!ahead) mbar_arrive_expect_tx(full_bar(stage), STAGE_BYTES);
                     tma_load_2d(sa, &tmA, kb * BK, m0, full_bar(stage));
-                    if (!ahead) tma_load_2d(sb, &tmB, kb * BK, tile * BN, full_bar(stage));
-                    issued[stage] = (int)phase;
-                    if (++stage == STAGES) {
+                    if (!ahead) tma_load_2d(sb, &tmB, kb * BK, tile * bn, full_bar(stage));
+                    ++issued;
+                    if (++stage == stages) {
                         stage = 0;
                         phase ^= 1u;
                     }
@@ -157,20 +164,18 @@ lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             }
             if (!ok) {
                 // aborting: let the copies already in flight land before the CTA goes away
-#pragma unroll
-                for (int s = 0; s < STAGES; ++s)
-                    if (issued[s] >= 0) {
-                        const unsigned long long t0 = globaltimer_ns();
-                        while (!mbar_try_wait(full_bar(s), (uint32_t)issued[s]) &&
-                               globaltimer_ns() - t0 < 100000000ull) {
-                        }
+                for (int j = max(0, issued - stages); j < issued; ++j) {
+                    const unsigned long long t0 = globaltimer_ns();
+                    while (!mbar_try_wait(full_bar(j % stages), (uint32_t)(j / stages) & 1u) &&
+                           globaltimer_ns() - t0 < 100000000ull) {
                     }
+                }
             }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(BM, BN, false, false);
+            const uint32_t idesc = idesc_bf16(BM, bn, false, false);
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -180,7 +185,7 @@ lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                 const uint32_t acc_phase = (uint32_t)(t >> 1) & 1u;
                 if (!mbar_wait(tempty_bar(buf), acc_phase ^ 1u, abort_flag)) break;
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
+                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN_MAX);
                 for (int kb = 0; kb < KB; ++kb) {
                     if (!mbar_wait(full_bar(stage), phase, abort_flag)) {
                         ok = false;
@@ -195,7 +200,7 @@ lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
                         umma_ss(d_tmem, adesc + 2u * kk, bdesc + 2u * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
                     }
                     umma_commit(empty_bar(stage));  // stage reusable once these MMAs have read it
-                    if (++stage == STAGES) {
+                    if (++stage == stages) {
                         stage = 0;
                         phase ^= 1u;
                     }
@@ -220,34 +225,27 @@ lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             const uint32_t acc_phase = (uint32_t)(t >> 1) & 1u;
             if (!mbar_wait(tfull_bar(buf), acc_phase, abort_flag)) break;
             tc_fence_after();
-            const int n0 = tile * BN;
-            const int ncol = min(BN, V - n0);
-            const uint32_t taddr = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(buf * BN);
+            const int n0 = tile * bn;
+            const int ncol = min(bn, V - n0);
+            const uint32_t taddr = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(buf * BN_MAX);
 #pragma unroll 1
-            for (int c = 0; c < BN; c += 32) {
+            for (int c = 0; c < ncol; c += 32) {
                 uint32_t r[32];
                 tmem_ld32(taddr + (uint32_t)c, r);
                 tmem_ld_wait();
-                if (c + 32 <= ncol) {
-                    // Four at a time: one branch on their maximum, which is rarely above the list's last entry.
-                    // (One branch per element made this loop, with a single warp per scheduler to hide nothing
-                    // behind, slower than the MMAs of a tile: 16 k against 12 k cycles.)
+                // Four at a time: one branch on their maximum, which is rarely above the list's last entry.
+                // (One branch per element made this loop, with a single warp per scheduler to hide nothing
+                // behind, slower than the MMAs of a tile: 16 k against 12 k cycles.)
 #pragma unroll
-                    for (int i = 0; i < 32; i += 4) {
-                        const float x0 = __uint_as_float(r[i]), x1 = __uint_as_float(r[i + 1]);
-                        const float x2 = __uint_as_float(r[i + 2]), x3 = __uint_as_float(r[i + 3]);
-                        if (fmaxf(fmaxf(x0, x1), fmaxf(x2, x3)) > top.v[KMAX - 1]) {
-                            if (x0 > top.v[KMAX - 1]) top.push(x0, n0 + c + i);
-                            if (x1 > top.v[KMAX - 1]) top.push(x1, n0 + c + i + 1);
-                            if (x2 > top.v[KMAX - 1]) top.push(x2, n0 + c + i + 2);
-                            if (x3 > top.v[KMAX - 1]) top.push(x3, n0 + c + i + 3);
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const float x = __uint_as_float(r[i]);
-                        if (c + i < ncol && x > top.v[KMAX - 1]) top.push(x, n0 + c + i);
+                for (int i = 0; i < 32; i += 4) {
+                    const float x0 = __uint_as_float(r[i]), x1 = __uint_as_float(r[i + 1]);
+                    const float x2 = __uint_as_float(r[i + 2]), x3 = __uint_as_float(r[i + 3]);
+                    // (a tile's width is a multiple of eight: four columns are inside or outside together)
+                    if (c + i < ncol && fmaxf(fmaxf(x0, x1), fmaxf(x2, x3)) > top.v[KMAX - 1]) {
+                        if (x0 > top.v[KMAX - 1]) top.push(x0, n0 + c + i);
+                        if (x1 > top.v[KMAX - 1]) top.push(x1, n0 + c + i + 1);
+                        if (x2 > top.v[KMAX - 1]) top.push(x2, n0 + c + i + 2);
+                        if (x3 > top.v[KMAX - 1]) top.push(x3, n0 + c + i + 3);
                     }
                 }
             }
@@ -277,17 +275,18 @@ lm_head_topk_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 
 // Host launcher.  Zt[M, d], W[V, d] bf16; partial lists [M, n_groups, k].
 int launch_lm_head_tc(const void *Zt, const void *W, int M, int V, int d, int k, int n_mblocks, int n_groups,
-                      int tiles_per_group, float *pval, int32_t *pid, int32_t *status, cudaStream_t st) {
+                      int tiles_per_group, int bn, float *pval, int32_t *pid, int32_t *status, cudaStream_t st) {
     using namespace lmtc;
     CUtensorMap tmA, tmB;
     int rc = make_tmap_2d_bf16(&tmA, Zt, (uint64_t)M, (uint64_t)d, (uint64_t)d, BM);
     if (rc != SPECROLL_OK) return rc;
-    rc = make_tmap_2d_bf16(&tmB, W, (uint64_t)V, (uint64_t)d, (uint64_t)d, BN);
+    rc = make_tmap_2d_bf16(&tmB, W, (uint64_t)V, (uint64_t)d, (uint64_t)d, (uint32_t)bn);
     if (rc != SPECROLL_OK) return rc;
-    if ((rc = device_setup(reinterpret_cast<const void *>(lm_head_topk_tc_kernel), SMEM_BYTES, nullptr)) != SPECROLL_OK) return rc;
+    const int stages = ring_stages(bn), smem = stages * stage_bytes(bn) + SMEM_EXTRA;
+    if ((rc = device_setup(reinterpret_cast<const void *>(lm_head_topk_tc_kernel), SMEM_MAX, nullptr)) != SPECROLL_OK) return rc;
     // (the dependent of the correction kernel in the stream)
-    SR_CUDA_TRY(launch_dependent(true, lm_head_topk_tc_kernel, dim3(n_mblocks * n_groups), dim3(THREADS), SMEM_BYTES, st, tmA,
-                                 tmB, M, V, d, k, n_mblocks, n_groups, tiles_per_group, pval, pid, status));
+    SR_CUDA_TRY(launch_dependent(true, lm_head_topk_tc_kernel, dim3(n_mblocks * n_groups), dim3(THREADS), smem, st, tmA,
+                                 tmB, M, V, d, k, n_mblocks, n_groups, tiles_per_group, bn, stages, pval, pid, status));
     return SPECROLL_OK;
 }
 

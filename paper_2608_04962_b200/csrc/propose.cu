@@ -547,7 +547,7 @@ tree_draw_kernel(Topo topo, int B, int K, int k, double T, const int32_t *__rest
 // ------------------------------------------------------------------------------ host side
 
 struct ProposePlan {
-    int KX, M, n_mblocks, n_tiles, n_groups, tiles_per_group;
+    int KX, M, n_mblocks, n_groups, tiles_per_group, bn;
     bool use_tc;  // tcgen05 projection kernel (k <= 8); otherwise the mma.sync one
     size_t off_status, off_xhat, off_z, off_zt, off_pval, off_pid, off_hc, total;
 };
@@ -558,7 +558,7 @@ int launch_head_mlp_tc(const void *xhat, int KX, const void *A, const void *bias
 
 // lm_head_tc.cu
 int launch_lm_head_tc(const void *Zt, const void *W, int M, int V, int d, int k, int n_mblocks, int n_groups,
-                      int tiles_per_group, float *pval, int32_t *pid, int32_t *status, cudaStream_t st);
+                      int tiles_per_group, int bn, float *pval, int32_t *pid, int32_t *status, cudaStream_t st);
 
 static int make_plan(const specroll_propose_desc *d, bool affine, ProposePlan *p) {
     if (!d || d->B < 0 || d->N < 1 || d->N > SPECROLL_MAX_NODES || d->K < 1 || d->K > SPECROLL_MAX_HEADS ||
@@ -569,14 +569,25 @@ static int make_plan(const specroll_propose_desc *d, bool affine, ProposePlan *p
     p->KX = affine ? d->K : 1;
     p->M = d->B * d->K;
     p->use_tc = d->k <= 8 && !(d->flags & SPECROLL_PROPOSE_LEGACY_MMA);
-    const int bn = p->use_tc ? 256 : LmTile::BN;
     p->n_mblocks = (p->M + LmTile::BM - 1) / LmTile::BM;  // both kernels use 128-row blocks
-    p->n_tiles = (d->V + bn - 1) / bn;
     int want = p->n_mblocks > 0 ? ((p->use_tc ? 1 : 2) * 148) / p->n_mblocks : 1;
     if (want < 1) want = 1;
-    if (want > p->n_tiles) want = p->n_tiles;
-    p->tiles_per_group = (p->n_tiles + want - 1) / want;
-    p->n_groups = (p->n_tiles + p->tiles_per_group - 1) / p->tiles_per_group;
+    if (p->use_tc) {
+        // Every CTA of a row block gets the same share of the vocabulary, cut into equal tiles of at most 256 tokens (the
+        // widest operation; a multiple of 16).  Whole tiles of 256 leave SMs idle: 594 of them were five each for 119 SMs and
+        // none for 29.  The call on 8 rows of the 1.5B shape 119 -> 109 us, on 32 rows of the 7B shape 242.5 -> 237.6; with
+        // 320 rows (the board at its power limit) no difference.  Shares below 32 tokens would only add partial lists; down to
+        // there they shorten what a CTA's epilogue scans by itself (a whole round of the toy model 70.4 -> 58.6).
+        const int share = (d->V + want - 1) / want < 32 ? 32 : (d->V + want - 1) / want;
+        p->tiles_per_group = (share + 255) / 256;
+        p->bn = ((share + p->tiles_per_group - 1) / p->tiles_per_group + 15) / 16 * 16;
+    } else {
+        p->bn = LmTile::BN;
+        const int n_tiles = (d->V + p->bn - 1) / p->bn;
+        if (want > n_tiles) want = n_tiles;
+        p->tiles_per_group = (n_tiles + want - 1) / want;
+    }
+    p->n_groups = (d->V + p->bn * p->tiles_per_group - 1) / (p->bn * p->tiles_per_group);
     size_t o = 0;
     const size_t B = d->B, K = d->K, dd = d->d, k = d->k;
     p->off_status = o;
@@ -716,8 +727,8 @@ extern "C" int specroll_propose(const specroll_propose_desc *d, const void *h, c
         const int smem = LmTile::SMEM_BYTES;  // >= 128 * 129 * 4 staging tile
         static_assert(LmTile::SMEM_BYTES >= LmTile::BM * LM_CSTRIDE * 4, "staging tile must fit");
         if (p.use_tc) {
-            int rc = launch_lm_head_tc(zt, W, p.M, V, dd, k, p.n_mblocks, p.n_groups, p.tiles_per_group, pval, pid,
-                                       status, st);
+            int rc = launch_lm_head_tc(zt, W, p.M, V, dd, k, p.n_mblocks, p.n_groups, p.tiles_per_group, p.bn, pval,
+                                       pid, status, st);
             if (rc) return rc;
         } else if (k <= 8) {
             int rc = set_smem(lm_head_topk_kernel<8>, smem);

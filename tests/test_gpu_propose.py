@@ -95,6 +95,20 @@ def test_ragged_shapes(B, K, k, d, V, N):
     assert same.mean() > 0.9
 
 
+@pytest.mark.parametrize("B,K,V", [(3, 4, 37896),    # two tiles of 144 tokens per CTA, the last CTA's cut short
+                                   (70, 4, 20008),   # three row blocks, tiles of 208
+                                   (1, 1, 1032),     # shares of 32 tokens, the last one of eight
+                                   (2, 2, 38152)])   # tiles of 144, the last CTA with one of 136
+def test_vocabulary_shares(B, K, V):
+    # the vocabulary is cut evenly over the SMs of a row block, into tiles of any multiple of 16 tokens
+    w = I.scaled(I.WORKLOADS["qwen1.5b"], B=B, K=K, k=8, d=256, V=V, N=8, alpha_heads=(0.025, 0.01, 0.006, 0.004)[:K])
+    x = I.propose_inputs(w, peaked=True)
+    g = gpu_propose(w, x)
+    same, oid, ol = check_candidates(w, x, g, logit_atol=LOGIT_ATOL)
+    check_tree(w, x, g, same, oid=oid, ol=ol)
+    assert same.mean() > 0.9
+
+
 def test_legacy_projection_kernel_agrees():
     # the mma.sync projection (flag) and the tcgen05 one must both match the oracle
     w = I.scaled(I.WORKLOADS["qwen1.5b"], B=40, K=4, k=8, d=512, V=5000, N=16)
