@@ -135,35 +135,29 @@ struct GateArgs {
     float z_delta, mem_eps;
 };
 
-// Realised alignment of every record: a warp per record.
-__global__ void __launch_bounds__(256) align_kernel(GateArgs g) {
-    const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    pdl_wait();
-    pdl_launch_dependents();
-    if (r >= g.R) return;
-    if (g.keep && !g.keep[r]) {
-        if (lane == 0 && g.a) g.a[r] = __int_as_float(0x7fc00000);
-        return;
-    }
+// Realised alignment of record r, by a warp.
+__device__ __forceinline__ float alignment(const GateArgs &g, int r, int lane) {
     const float sv = lane < g.rank ? g.s[(size_t)r * g.rank + lane] : 0.f;
     const float xv = lane < g.rank ? g.xi[(size_t)r * g.rank + lane] : 0.f;
     const float dot = warp_sum(sv * xv), ns = sqrtf(warp_sum(sv * sv)), nx = sqrtf(warp_sum(xv * xv));
-    if (lane == 0) g.a[r] = (ns > 0.f && nx > 0.f) ? dot / (ns * nx) : 0.f;
+    return (ns > 0.f && nx > 0.f) ? dot / (ns * nx) : 0.f;
 }
 
 // A CTA per slot: its records, in order, go into the running moments; then the score and the gate, with the RMS of the
 // memory row.  Bound by latency: all threads look for the slot's records (512 at a time) and have the memory row's loads
-// in flight meanwhile (a warp per slot took 14 us for 512 slots and records of d 3584).
-__global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g, const float *__restrict__ a) {
+// in flight meanwhile (a warp per slot took 14 us for 512 slots and records of d 3584).  A record's alignment is formed by
+// the CTA of its slot, a warp per record (a kernel of its own in front of this one cost its launch and round trips).
+__global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g) {
     using namespace gt;
     __shared__ int hit[GATE_BATCH];
     __shared__ float val[GATE_BATCH];
-    __shared__ int n_hit;
+    __shared__ int lost[GATE_BATCH];
+    __shared__ int n_hit, n_lost;
     __shared__ float red[GATE_THREADS / 32];
     const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     pdl_wait();
     pdl_launch_dependents();
-    if (tid == 0) n_hit = 0;
+    if (tid == 0) n_hit = n_lost = 0;
     int n = g.n[j], nfb = g.n_fb[j];
     float mean = g.mean[j], M2 = g.M2[j];
     float ss = 0.f;
@@ -194,22 +188,40 @@ __global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g, cons
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int r = r0 + q * GATE_THREADS + tid;
-            if (sl[q] == j && r < g.R && (!g.keep || g.keep[r])) hit[atomicAdd(&n_hit, 1)] = r;
+            // (a record of no slot of this call has an alignment all the same: the first CTA's)
+            const bool stray = j == 0 && (sl[q] < 0 || sl[q] >= g.S);
+            if (r < g.R && (sl[q] == j || stray)) {
+                if (g.keep && !g.keep[r])
+                    g.a[r] = __int_as_float(0x7fc00000);
+                else if (stray)
+                    lost[atomicAdd(&n_lost, 1)] = r;
+                else
+                    hit[atomicAdd(&n_hit, 1)] = r;
+            }
         }
         __syncthreads();
-        const int nh = n_hit;
-        __syncthreads();  // (all have read it before the next records are counted)
-        if (nh == 0) continue;
+        const int nh = n_hit, nl = n_lost;
+        __syncthreads();  // (all have read them before the next records are counted)
+        if (nh + nl == 0) continue;
+        for (int e = tid >> 5; e < nl; e += GATE_THREADS / 32) {
+            const float v = alignment(g, lost[e], lane);
+            if (lane == 0) g.a[lost[e]] = v;
+        }
         // in record order
-        for (int e = tid; e < nh; e += GATE_THREADS) {
+        for (int e = tid >> 5; e < nh; e += GATE_THREADS / 32) {
             const int r = hit[e];
             int rk = 0;
-            for (int f = 0; f < nh; ++f) rk += hit[f] < r;
-            val[rk] = a[r];
+            for (int f = lane; f < nh; f += 32) rk += hit[f] < r;
+            rk = __reduce_add_sync(0xffffffffu, rk);
+            const float v = alignment(g, r, lane);
+            if (lane == 0) {
+                val[rk] = v;
+                g.a[r] = v;
+            }
         }
         __syncthreads();
         if (tid == 0) {
-            n_hit = 0;
+            n_hit = n_lost = 0;
             for (int e = 0; e < nh; ++e) {
                 n += 1;
                 const float delta = val[e] - mean;
@@ -304,7 +316,6 @@ extern "C" int specroll_reflex_gate(const specroll_gate_desc *d, const float *s,
     g.H = d->H;
     g.z_delta = d->z_delta;
     g.mem_eps = d->mem_eps;
-    if (d->R > 0) SR_CUDA_TRY(launch_dependent(true, align_kernel, dim3((unsigned)(d->R + 7) / 8), dim3(256), 0, st, g));
-    SR_CUDA_TRY(launch_dependent(true, gate_kernel, dim3((unsigned)d->S), dim3(gt::GATE_THREADS), 0, st, g, (const float *)a));
+    SR_CUDA_TRY(launch_dependent(true, gate_kernel, dim3((unsigned)d->S), dim3(gt::GATE_THREADS), 0, st, g));
     return SPECROLL_OK;
 }
