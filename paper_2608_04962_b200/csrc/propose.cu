@@ -20,6 +20,18 @@ __device__ __forceinline__ float block_sum(float v, float *sh) {
     return warp_sum(t);
 }
 
+// two sums for one pair of barriers, each formed by the additions of block_sum
+template <int THREADS>
+__device__ __forceinline__ float2 block_sum2(float a, float b, float2 *sh) {
+    a = warp_sum(a);
+    b = warp_sum(b);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane == 0) sh[warp] = make_float2(a, b);
+    __syncthreads();
+    const float2 t = lane < THREADS / 32 ? sh[lane] : make_float2(0.f, 0.f);
+    return make_float2(warp_sum(t.x), warp_sum(t.y));
+}
+
 // ------------------------------------------------------------------------------ P1 LayerNorm
 
 constexpr int LN_THREADS = 256;
@@ -29,18 +41,21 @@ __global__ void __launch_bounds__(LN_THREADS)
 layernorm_kernel(const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__restrict__ gamma,
                  const __nv_bfloat16 *__restrict__ beta, __nv_bfloat16 *__restrict__ xhat, int B, int d,
                  int KX, float eps, int32_t *__restrict__ status) {
-    extern __shared__ float row[];  // d floats
+    extern __shared__ __align__(16) float row[];  // d floats
     __shared__ float red[LN_THREADS / 32];
     pdl_launch_dependents();
     pdl_wait();
     const int b = blockIdx.x;
     if (b == 0 && threadIdx.x == 0) *status = 0;  // (of the call; a kernel behind this one may set it)
     float s = 0.f;
-    for (int i = threadIdx.x; i < d; i += LN_THREADS) {
-        const float v = __bfloat162float(h[(size_t)b * d + i]);
-        row[i] = v;
-        s += v;
+    for (int i = threadIdx.x; i < d / 8; i += LN_THREADS) {
+        const uint4 v = reinterpret_cast<const uint4 *>(h + (size_t)b * d)[i];
+        float4 *dst = reinterpret_cast<float4 *>(row + 8 * i);
+        dst[0] = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+        dst[1] = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xffff0000u), __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xffff0000u));
     }
+    __syncthreads();
+    for (int i = threadIdx.x; i < d; i += LN_THREADS) s += row[i];
     const float mu = block_sum<LN_THREADS>(s, red) / d;
     float q = 0.f;
     for (int i = threadIdx.x; i < d; i += LN_THREADS) {
@@ -99,34 +114,47 @@ constexpr int RX_THREADS = 256;
 
 // zt[r,:] = bf16(z[r,:] + coef * m[r,:]),  r = b*K + hd,
 // coef = alpha * RMS(z) / (RMS(m) + eps), shrunk so that |coef * m|_2 <= clip_c * |z|_2.
-__global__ void __launch_bounds__(RX_THREADS)
+// Bound by round trips to memory: a thread keeps its NV elements of both rows in registers (d <= NV * RX_THREADS), what the
+// call's caller wrote (memory, ratio) is read ahead of the wait, and the two sums share their barriers.  32 rows of 3584: the heads end 7.3 -> 5.8 us ahead
+// of the projection.
+template <int NV>
+__global__ void __launch_bounds__(RX_THREADS, NV <= 8 ? 7 : NV <= 24 ? 72 / NV : 1)  // (the rows of the model shapes are resident at once)
 reflex_kernel(const float *__restrict__ z, const float *__restrict__ m, const float *__restrict__ alpha,
               __nv_bfloat16 *__restrict__ zt, int d, float rms_eps, float clip_c) {
-    __shared__ float red[RX_THREADS / 32];
+    __shared__ float2 red[RX_THREADS / 32];
     pdl_launch_dependents();
+    const float a = (alpha && m) ? alpha[blockIdx.x] : 0.f;
+    const size_t at = (size_t)blockIdx.x * d + threadIdx.x;  // this thread's elements: every RX_THREADS-th of the row from here on
+    const int left = d - (int)threadIdx.x;
+    float mv[NV], zv[NV];
+    m += at;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) mv[j] = a != 0.f && j * RX_THREADS < left ? m[j * RX_THREADS] : 0.f;
     pdl_wait();
-    const size_t r = blockIdx.x;
-    const float *zr = z + r * d;
-    const float a = (alpha && m) ? alpha[r] : 0.f;
-    float coef = 0.f;
+    z += at;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) zv[j] = j * RX_THREADS < left ? z[j * RX_THREADS] : 0.f;
     if (a != 0.f) {  // uniform across the block
-        const float *mr = m + r * d;
         float sz = 0.f, sm = 0.f;
-        for (int i = threadIdx.x; i < d; i += RX_THREADS) {
-            const float zv = zr[i], mv = mr[i];
-            sz += zv * zv;
-            sm += mv * mv;
+#pragma unroll
+        for (int j = 0; j < NV; ++j) {
+            sz += zv[j] * zv[j];
+            sm += mv[j] * mv[j];
         }
-        sz = block_sum<RX_THREADS>(sz, red);
-        sm = block_sum<RX_THREADS>(sm, red);
+        const float2 t = block_sum2<RX_THREADS>(sz, sm, red);
+        sz = t.x;
+        sm = t.y;
         const float rms_z = sqrtf(sz / d), rms_m = sqrtf(sm / d);
-        coef = a * rms_z / (rms_m + rms_eps);
+        float coef = a * rms_z / (rms_m + rms_eps);
         const float nd = fabsf(coef) * sqrtf(sm), nz = sqrtf(sz);
         if (clip_c > 0.f && nd > clip_c * nz) coef *= clip_c * nz / nd;
-        for (int i = threadIdx.x; i < d; i += RX_THREADS) zt[r * d + i] = __float2bfloat16_rn(zr[i] + coef * mr[i]);
-    } else {
-        for (int i = threadIdx.x; i < d; i += RX_THREADS) zt[r * d + i] = __float2bfloat16_rn(zr[i]);
+#pragma unroll
+        for (int j = 0; j < NV; ++j) zv[j] = zv[j] + coef * mv[j];
     }
+    zt += at;
+#pragma unroll
+    for (int j = 0; j < NV; ++j)
+        if (j * RX_THREADS < left) zt[j * RX_THREADS] = __float2bfloat16_rn(zv[j]);
 }
 
 // Secondary form of the correction (SPECROLL_REFLEX_PRE_HEAD): applied to the last hidden state, one memory row
@@ -327,20 +355,22 @@ __device__ __forceinline__ void tk_insert(Top8 &L, float x, int32_t t) {
         L.i[0] = t;
     }
 }
-// the best of the lanes' current best; the lane that held it moves on to its next one (ids are distinct: one lane)
+// the best of the lanes' current best; the lane that held it moves on to its next one.  One integer reduction over the values'
+// ordered bits (-0 counts as +0), a second one over the ids only where lanes tie: the eight rounds of a merge follow one another,
+// and ten shuffles each made them half of the kernel.
 __device__ __forceinline__ void tk_pop_best(Top8 &L, float &bv, int32_t &bi) {
-    bv = L.v[0];
-    bi = L.i[0];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int32_t oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (tk_better(ov, oi, bv, bi)) {
-            bv = ov;
-            bi = oi;
-        }
+    const int lane = threadIdx.x & 31;
+    const int bits = __float_as_int(L.v[0] + 0.0f), key = bits ^ ((bits >> 31) & 0x7fffffff);
+    const bool top = key == __reduce_max_sync(0xffffffffu, key);
+    unsigned who = __ballot_sync(0xffffffffu, top);
+    if (who & (who - 1)) {
+        const int first = __reduce_min_sync(0xffffffffu, top ? L.i[0] : 0x7fffffff);
+        who = __ballot_sync(0xffffffffu, top && L.i[0] == first);
     }
-    if (L.v[0] == bv && L.i[0] == bi) {
+    const int w = __ffs(who) - 1;
+    bv = __shfl_sync(0xffffffffu, L.v[0], w);
+    bi = __shfl_sync(0xffffffffu, L.i[0], w);
+    if (lane == w) {
 #pragma unroll
         for (int i = 0; i < 7; ++i) {
             L.v[i] = L.v[i + 1];
@@ -434,11 +464,11 @@ topk_merge8_wide_kernel(const float *__restrict__ pval, const int32_t *__restric
 
 // ------------------------------------------------------------------------------ P5 tree draw
 
-constexpr int DRAW_WARPS = 8;
+constexpr int DRAW_WARPS = 16;
 
-__device__ __forceinline__ double warp_incl_scan_f64(double v, int lane) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
+// inclusive sums over the first `n` lanes (a power of two; what lies behind them is not meaningful)
+__device__ __forceinline__ double warp_incl_scan_f64(double v, int lane, int n) {
+    for (int o = 1; o < n; o <<= 1) {
         const double t = __shfl_up_sync(0xffffffffu, v, o);
         if (lane >= o) v += t;
     }
@@ -449,8 +479,9 @@ __device__ __forceinline__ double warp_incl_scan_f64(double v, int lane) {
 // drew and on nothing else, so the children of different parents are drawn at the same time and only siblings
 // wait for each other; within a draw the work over the k candidates is spread over the lanes (lane j holds
 // candidates j and j + 32): their total, the running sums of the inverse-CDF walk and the first candidate whose
-// running sum exceeds the uniform come from warp scans and ballots.  (Node after node on one warp, a draw of 48
-// nodes took 32 us: some twenty dependent fp64 operations and shuffles per node.)
+// running sum exceeds the uniform come from warp scans and ballots.  Bound by the chain over the siblings, so that
+// holds no more than it must: scans over as many lanes as there are candidates, the drawn probabilities' divisions
+// and all stores behind it (lane i keeps the i-th child's), the tree looked at ahead of the wait.
 __global__ void __launch_bounds__(DRAW_WARPS * 32)
 tree_draw_kernel(Topo topo, int B, int K, int k, double T, const int32_t *__restrict__ anchor,
                  const int32_t *__restrict__ cand_id, const float *__restrict__ cand_logit,
@@ -461,12 +492,19 @@ tree_draw_kernel(Topo topo, int B, int K, int k, double T, const int32_t *__rest
     __shared__ double sh_w[SPECROLL_MAX_HEADS][SPECROLL_MAX_TOPK];
     __shared__ int32_t sh_id[SPECROLL_MAX_HEADS][SPECROLL_MAX_TOPK];
     __shared__ float sh_u[SPECROLL_MAX_NODES];
-    __shared__ int8_t sh_parent[SPECROLL_MAX_NODES];
-    pdl_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.x;
     const int N = topo.N;
+    // (the tree and the uniforms are the caller's, complete before the call's first kernel)
+    const int par0 = lane < N ? topo.parent[lane] : -1, par1 = lane + 32 < N ? topo.parent[lane + 32] : -1;
+    unsigned long long inner = ((unsigned long long)__ballot_sync(0xffffffffu, lane + 32 < N && topo.n_child[(lane + 32) & 63] > 0) << 32) |
+                               __ballot_sync(0xffffffffu, lane < N && topo.n_child[lane] > 0);  // nodes with children
+    for (int n = threadIdx.x; n < N; n += DRAW_WARPS * 32) sh_u[n] = u_draw[(size_t)b * N + n];
+    const int32_t root = threadIdx.x == 0 ? anchor[b] : 0;
     const double inv_T = 1.0 / T;  // (the largest logit minus itself over T would be a division with a zero numerator)
+    int n_scan = 1;
+    while (n_scan < (k < 32 ? k : 32)) n_scan <<= 1;
+    pdl_wait();
     for (int hd = warp; hd < K; hd += DRAW_WARPS) {
         const float *cl = cand_logit + ((size_t)b * K + hd) * k;
         float mxf = -INFINITY;
@@ -477,39 +515,46 @@ tree_draw_kernel(Topo topo, int B, int K, int k, double T, const int32_t *__rest
             sh_id[hd][j] = cand_id[((size_t)b * K + hd) * k + j];
         }
     }
-    for (int n = threadIdx.x; n < N; n += DRAW_WARPS * 32) {
-        sh_u[n] = u_draw[(size_t)b * N + n];
-        sh_parent[n] = topo.parent[n];
-    }
     if (threadIdx.x == 0) {
-        tree_tok[(size_t)b * N] = anchor[b];
+        tree_tok[(size_t)b * N] = root;
         tree_cand[(size_t)b * N] = 255;
         slot_q[(size_t)b * N] = 1.0f;
     }
     __syncthreads();
-    int idx = 0;
-    for (int u = 0; u < N; ++u) {
-        if (topo.n_child[u] == 0) continue;
-        if ((idx++ % DRAW_WARPS) != warp) continue;
+    for (int idx = 0; inner; ++idx) {
+        const int u = __ffsll((long long)inner) - 1;
+        inner &= inner - 1;
+        if ((idx % DRAW_WARPS) != warp) continue;
         const int hd = topo.depth[u];  // the children of u are drawn by head depth(u) (0-based)
         const double *w = sh_w[hd];
-        // children of u (a child's index is larger than its parent's), in slot order
-        const unsigned cm_lo = __ballot_sync(0xffffffffu, lane > u && lane < N && sh_parent[lane < N ? lane : 0] == u);
-        const unsigned cm_hi =
-            __ballot_sync(0xffffffffu, lane + 32 > u && lane + 32 < N && sh_parent[lane + 32 < N ? lane + 32 : 0] == u);
-        unsigned long long cm = ((unsigned long long)cm_hi << 32) | cm_lo;
+        // children of u, in slot order
+        unsigned long long cm = ((unsigned long long)__ballot_sync(0xffffffffu, par1 == u) << 32) | __ballot_sync(0xffffffffu, par0 == u);
         unsigned long long taken = 0ull;
+        const double wt0 = lane < k ? w[lane] : 0.0, wt1 = lane + 32 < k ? w[lane + 32] : 0.0;
+        int count = 0, my_n = 0, my_sel = 0;
+        double my_w = 0.0, my_s = 1.0;
+        auto leave = [&]() {  // up to 32 children, one per lane
+            if (lane < count) {
+                tree_tok[(size_t)b * N + my_n] = sh_id[hd][my_sel];
+                tree_cand[(size_t)b * N + my_n] = (uint8_t)my_sel;
+                slot_q[(size_t)b * N + my_n] = (float)(my_w / my_s);
+            }
+            count = 0;
+        };
         while (cm) {
             const int n = __ffsll((long long)cm) - 1;
             cm &= cm - 1;
             const bool ok0 = lane < k && !((taken >> lane) & 1ull);
             const bool ok1 = lane + 32 < k && !((taken >> (lane + 32)) & 1ull);
-            double w0 = ok0 ? w[lane] : 0.0, w1 = ok1 ? w[lane + 32] : 0.0;
+            double w0 = ok0 ? wt0 : 0.0, w1 = ok1 ? wt1 : 0.0;
             // running sums over the remaining candidates; their total is the last one
-            double c0 = warp_incl_scan_f64(w0, lane);
-            double c1 = __shfl_sync(0xffffffffu, c0, 31);
-            if (k > 32) c1 += warp_incl_scan_f64(w1, lane);
-            double s = __shfl_sync(0xffffffffu, c1, 31);
+            double c0 = warp_incl_scan_f64(w0, lane, n_scan);
+            double s = __shfl_sync(0xffffffffu, c0, n_scan - 1);
+            double c1 = s;
+            if (k > 32) {
+                c1 += warp_incl_scan_f64(w1, lane, 32);
+                s = __shfl_sync(0xffffffffu, c1, 31);
+            }
             if (!(s > 0.0)) {
                 // every remaining weight underflowed against a taken candidate's logit: take the reference among
                 // the remaining ones instead
@@ -518,8 +563,8 @@ tree_draw_kernel(Topo topo, int B, int K, int k, double T, const int32_t *__rest
                 mxf = warp_max(mxf);
                 w0 = ok0 ? exp(((double)cl[lane] - (double)mxf) * inv_T) : 0.0;
                 w1 = ok1 ? exp(((double)cl[lane + 32] - (double)mxf) * inv_T) : 0.0;
-                c0 = warp_incl_scan_f64(w0, lane);
-                c1 = __shfl_sync(0xffffffffu, c0, 31) + warp_incl_scan_f64(w1, lane);
+                c0 = warp_incl_scan_f64(w0, lane, 32);
+                c1 = __shfl_sync(0xffffffffu, c0, 31) + warp_incl_scan_f64(w1, lane, 32);
                 s = __shfl_sync(0xffffffffu, c1, 31);
             }
             // first remaining candidate whose cumulative probability exceeds the uniform (compared as masses)
@@ -535,12 +580,15 @@ tree_draw_kernel(Topo topo, int B, int K, int k, double T, const int32_t *__rest
                 sel = v1 ? 32 + (31 - __clz(v1)) : (31 - __clz(v0));  // none: the last remaining candidate
             const double wsel = __shfl_sync(0xffffffffu, sel < 32 ? w0 : w1, sel & 31);
             taken |= 1ull << sel;
-            if (lane == 0) {
-                tree_tok[(size_t)b * N + n] = sh_id[hd][sel];
-                tree_cand[(size_t)b * N + n] = (uint8_t)sel;
-                slot_q[(size_t)b * N + n] = (float)(wsel / s);
+            if (lane == count) {
+                my_n = n;
+                my_sel = sel;
+                my_w = wsel;
+                my_s = s;
             }
+            if (++count == 32) leave();
         }
+        leave();
     }
 }
 
@@ -718,7 +766,8 @@ extern "C" int specroll_propose(const specroll_propose_desc *d, const void *h, c
         SR_LAUNCH_CHECK();
     }
 
-    SR_CUDA_TRY(launch_dependent(true, reflex_kernel, dim3(B * K), dim3(RX_THREADS), 0, st, (const float *)z,
+    auto *const reflex = dd <= 2048 ? reflex_kernel<8> : dd <= 4096 ? reflex_kernel<16> : dd <= 6144 ? reflex_kernel<24> : reflex_kernel<48>;
+    SR_CUDA_TRY(launch_dependent(true, reflex, dim3(B * K), dim3(RX_THREADS), 0, st, (const float *)z,
                                  pre_head ? (const float *)nullptr : m, pre_head ? (const float *)nullptr : alpha, zt, dd,
                                  d->rms_eps, d->clip_c));
 

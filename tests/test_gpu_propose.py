@@ -191,6 +191,22 @@ def test_tree_draw_alone_matches_exactly():
     assert np.array_equal(host(g["tree_tok"]), o["tree_tok"])
 
 
+@pytest.mark.parametrize("k,n_root,n_first", [(64, 60, 3), (33, 33, 30), (32, 32, 31), (5, 5, 4), (1, 1, 1)])
+def test_tree_draw_of_wide_nodes(k, n_root, n_first):
+    # more children than a warp has lanes (their tokens are stored in groups of 32), lists of one to 64 candidates
+    parent = np.array([-1] + [0] * n_root + [1] * n_first, np.int32)
+    B, K, N = 40, 2, parent.shape[0]
+    g = I.rng(78 + k)
+    cid = np.tile(np.arange(K * k, dtype=np.int32).reshape(1, K, k), (B, 1, 1))
+    cl = np.sort(g.standard_normal((B, K, k)).astype(np.float32), axis=-1)[..., ::-1].copy()
+    u, anchor = I.uniforms24(10, (B, N)), np.arange(B, dtype=np.int32)
+    o = ref.tree_draw(parent, anchor, cid, cl, u)
+    d = S.tree_draw(parent, dev(anchor), dev(cid), dev(cl), dev(u))
+    assert np.array_equal(host(d["tree_tok"]), o["tree_tok"])
+    assert np.array_equal(host(d["tree_cand"]), o["tree_cand"])
+    np.testing.assert_allclose(host(d["slot_q"]), o["slot_q"], rtol=1e-6)
+
+
 def test_tree_draw_with_a_candidate_that_dwarfs_the_rest():
     # One candidate of every head leads the others by more than 745 T, so that once it has been drawn the weights
     # of the rest underflow against it and the draw has to renormalise over what is left (App. B.1 Eq. "slotq":
