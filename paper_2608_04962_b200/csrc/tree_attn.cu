@@ -117,6 +117,54 @@ attn_prep_kernel(const int32_t *__restrict__ kv_indptr, const int32_t *__restric
         }
         return;
     }
+    if (B <= 32 && sorted_start) {
+        // Few sequences: one warp finds all positions in registers, a warp per sequence writes its rows.  A round of few sequences
+        // waits for this kernel, and with the scans and barriers below it took 4.6 us.
+        __shared__ int sh_seq[5][32];
+        const int warp = t >> 5, lane = t & 31;
+        if (warp == 0) {
+            int L = lane < B ? (kv_len ? kv_len[lane] : kv_indptr[lane + 1] - kv_indptr[lane]) : 0;
+#ifdef SPECROLL_CHECK
+            if (L < 0) {
+                SR_CHECK_FAIL(lane);
+                L = 0;
+            }
+#endif
+            const int kv0 = lane < B ? (kv_len ? page_indptr[lane] : kv_indptr[lane]) : 0;
+            const int tiles = (L + tile_tokens - 1) / tile_tokens;
+            const int ns = lane < B ? max(1, (tiles + chunk_tiles - 1) / chunk_tiles) : 0, cost = (tiles + max(ns, 1) - 1) / max(ns, 1);
+            int first = 0, rank = 0, at = 0, total = 0;
+            for (int o = 0; o < B; ++o) {
+                const int no = __shfl_sync(0xffffffffu, ns, o), co = __shfl_sync(0xffffffffu, cost, o);
+                const bool before = co > cost || (co == cost && o < lane);
+                first += o < lane ? no : 0;
+                rank += before;
+                at += before ? no : 0;
+                total += no;
+            }
+            if (lane < B) {
+                item_start[lane] = first;
+                seq_at_rank[rank] = lane;
+                sorted_start[rank] = at;
+                sh_seq[0][lane] = ns;
+                sh_seq[1][lane] = first;
+                sh_seq[2][lane] = at;
+                sh_seq[3][lane] = kv0;
+                sh_seq[4][lane] = L;
+            }
+            if (lane == 0) item_start[B] = sorted_start[B] = total;
+        }
+        __syncthreads();
+        if (warp < B) {
+            const int ns = sh_seq[0][warp];
+            int4 *dst = reinterpret_cast<int4 *>(unit_tab) + 2 * (size_t)sh_seq[2][warp];
+            for (int s = lane; s < ns; s += 32) {
+                dst[2 * s] = make_int4(warp, s, ns, sh_seq[1][warp]);
+                dst[2 * s + 1] = make_int4(sh_seq[3][warp], sh_seq[4][warp], 0, 0);
+            }
+        }
+        return;
+    }
     for (int b = t; b < B; b += PREP_THREADS) {
         int L = kv_len ? kv_len[b] : kv_indptr[b + 1] - kv_indptr[b];
 #ifdef SPECROLL_CHECK

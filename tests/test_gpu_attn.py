@@ -104,6 +104,15 @@ def test_sequences_cut_into_many_chunks(Hq, Hkv, D, N):
     check(o, O, lse)
 
 
+@pytest.mark.parametrize("B", [1, 31, 32, 33])
+def test_plans_of_up_to_32_sequences_and_of_more(B):
+    # up to 32 sequences are put in order by one warp; equal lengths, empty caches and one sequence that is cut
+    w = I.scaled(I.WORKLOADS["tiny"], B=B, Hq=4, Hkv=2, D=64)
+    lengths = [4000] + [(0, 130, 64, 130, 700)[i % 5] for i in range(B - 1)]
+    o, O, lse = run_both(w, I.attn_inputs(w), lengths=lengths)
+    check(o, O, lse, edge=True)
+
+
 def test_reduced_batches_of_the_large_configs():
     for name, B in (("qwen1.5b", 12), ("qwen7b", 4), ("qwen14b", 2)):
         w = I.scaled(I.WORKLOADS[name], B=B)
