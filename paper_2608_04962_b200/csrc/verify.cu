@@ -1983,26 +1983,34 @@ constexpr int WT_WARPS = WT_THREADS / 32;
 constexpr int TILE_STATIC_SMEM = 4 * 1024;                         // (at most) of the form without stored logits
 constexpr int TILE_SMEM_LIMIT = 227 * 1024 - TILE_STATIC_SMEM;     // dynamic
 
+// The nodes with children, in order, to par (by one warp); returns how many there are.  Ahead of the wait for the statistics: looked
+// for node by node behind it, they were on the walk's critical path.
+__device__ __forceinline__ int walk_parents(const Topo &topo, int N, int8_t *par) {
+    const int lane = threadIdx.x & 31;
+    int n = 0;
+    for (int u0 = 0; u0 < N; u0 += 32) {
+        const bool inner = u0 + lane < N && topo.n_child[(u0 + lane) % SPECROLL_MAX_NODES] > 0;
+        const unsigned mask = __ballot_sync(0xffffffffu, inner);
+        if (inner) par[n + __popc(mask & ((1u << lane) - 1u))] = (int8_t)(u0 + lane);
+        n += __popc(mask);
+    }
+    return n;
+}
+
 // Every node with children on its own.  first[u]: accepted child or -1, mm[u]: smallest margin, ovm[u, j]: the residual's
 // masses where all children were rejected.  (A warp per node took 9 k
 // cycles, two rounds of them where more than sixteen nodes have children: 10 us of the 66 us of 16 sequences x 48 nodes.)
-__device__ __forceinline__ void walk_nodes(const Topo &topo, int N, int k, const double *p, const float *rsum, const WalkSlots &w,
-                                           int32_t *first, float *mm, double *ovm) {
+// par: the n_par nodes with children (walk_parents).
+__device__ __forceinline__ void walk_nodes(const Topo &topo, int n_par, const int8_t *par, int k, const double *p, const float *rsum,
+                                           const WalkSlots &w, int32_t *first, float *mm, double *ovm) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int kp = 1;
     while (kp < k) kp <<= 1;
     const int per_warp = 32 / kp, grp = lane / kp, j = lane & (kp - 1);
-    int n_par = 0;
-    for (int u = 0; u < N; ++u) n_par += topo.n_child[u] > 0;
     // as few nodes per warp as give every node a place in one round
     const int share = min(per_warp, (n_par + TERM_WARPS - 1) / TERM_WARPS);
     for (int i0 = warp * share; i0 < n_par; i0 += TERM_WARPS * share) {
-        int u = -1;
-        if (grp < share && i0 + grp < n_par) {
-            int idx = 0;
-            for (int n = 0; n < N; ++n)
-                if (topo.n_child[n] > 0 && idx++ == i0 + grp) u = n;
-        }
+        const int u = grp < share && i0 + grp < n_par ? par[i0 + grp] : -1;
         double rho = u >= 0 && j < k ? p[u * k + j] : 0.0;
         float mg;
         const int child = walk_group(topo, u, k, kp, rho, w, mg);
@@ -2255,8 +2263,13 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     // statistics).  TILES: whatever the caller has put in front of the call may still be writing them.
     if (TILES) pdl_wait();
     const WalkSlots slots = walk_slots(sh_dyn + L.slots, N, k);
-    __shared__ int sh_odd;
+    __shared__ int sh_odd, sh_n_par;
+    __shared__ int8_t sh_par[SPECROLL_MAX_NODES];
     if (tid == 0) sh_odd = !L.grouped;
+    if (warp == 0) {
+        const int n = walk_parents(topo, N, sh_par);
+        if (lane == 0) sh_n_par = n;
+    }
     walk_buf_fetch(a, topo, b, buf);
     __syncthreads();
     if (L.grouped) walk_slots_fill(buf, topo, N, k, b, slots, &sh_odd);
@@ -2294,7 +2307,7 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     __syncthreads();
     // (2) every node with children on its own
     if (!sh_odd) {
-        walk_nodes(topo, N, k, wp, rsum, slots, first, mmin, ovm);
+        walk_nodes(topo, sh_n_par, sh_par, k, wp, rsum, slots, first, mmin, ovm);
     } else {
         const WalkStage stage{rmax, rsum, buf.uacc, ttok, buf.tcand, cid, buf.clog, pre, buf.parent, buf.e, wp};
         int idx = 0;
