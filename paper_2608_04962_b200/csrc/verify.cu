@@ -144,8 +144,9 @@ __device__ __forceinline__ void row_from_runs(const float2 *sh, int lane, float 
 // ring is as deep as the CTAs of an SM leave room for.  The terms of a lane's sum keep the order that the CTA-per-row form
 // (row_stats_kernel) gives them: the terminal draw follows the last bits of the runs' sums.
 constexpr int RUN_PIECE = 128;                 // vectors per copy (a group)
-constexpr int RUN_RING_MIN = 3, RUN_RING_MAX = 10;  // copies in flight per warp
-constexpr int RUN_WARPS = 4, RUN_CTAS = 8;     // warps per CTA, CTAs per SM
+constexpr int RUN_RING_MIN = 2, RUN_RING_MAX = 10;  // copies in flight per warp
+constexpr int RUN_WARPS = 4;                   // warps per CTA
+constexpr int RUN_CTAS = 8, RUN_CTAS_MORE = 11;  // CTAs per SM: the fewer, with deeper rings, or as many as give every run a warp
 // ROWS: a CTA of eight warps takes the eight runs of row blockIdx and leaves the row's own pair (up to four rows per SM).
 #ifdef SPECROLL_CHECK
 // Debug build only: when armed (specroll_check_inject(2)), the first warp of CTA 0 leaves out its first copy, once.  Its wait runs
@@ -158,8 +159,8 @@ int run_stats_arm_dropped_copy() {
 #else
 int run_stats_arm_dropped_copy() { return -1; }
 #endif
-template <bool ROWS>
-__global__ void __launch_bounds__(32 * (ROWS ? RS_WARPS : RUN_WARPS), ROWS ? 4 : RUN_CTAS)
+template <bool ROWS, int CTAS>
+__global__ void __launch_bounds__(32 * (ROWS ? RS_WARPS : RUN_WARPS), CTAS)
 run_stats_kernel(const uint16_t *__restrict__ logits, int V, float c, int n_runs, int ring_n, float2 *__restrict__ run_tab,
                  float *__restrict__ row_max, float *__restrict__ row_sum) {
     constexpr int WARPS = ROWS ? RS_WARPS : RUN_WARPS;
@@ -2520,16 +2521,22 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
         //   V 32000:  512 rows 21.3 -> 19.7, 768: 24.0 -> 23.1, 1024: 26.9 -> 26.0, 1536: 31.8 -> 37.2
         //   V 8000:   512 rows 18.8 -> 16.2, 1024: 20.3 -> 17.8, 1536: 21.6 -> 19.5
         // (20 rows of 152 k tokens from HBM 29 -> 19, 4096 rows 198 -> 234.)
-        const int n_runs = rows * RS_WARPS, most = RUN_WARPS * RUN_CTAS * n_sm, rounds = (n_runs + most - 1) / most;
+        // With more than 38 runs per SM a warp for each of them, 44 warps per SM with two copies in flight, instead of 21 or so
+        // with two runs each: too few warps keep the exponentials, the integer instructions and the waits apart.  21 warps -> 44:
+        //   V 152064: 640 rows 50.1 -> 51.5, 768: 60.0 -> 58.4, 800: 62.1 -> 58.6;  V 64000: 640 28.0 -> 29.7, 768 35.3 -> 33.1, 800 34.7 -> 33.2
+        const int n_runs = rows * RS_WARPS;
+        const bool more = n_runs > 38 * n_sm;
+        const int ctas = more ? RUN_CTAS_MORE : RUN_CTAS, most = RUN_WARPS * ctas * n_sm, rounds = (n_runs + most - 1) / most;
         if (n_runs <= 44 * n_sm) {
             // every warp the same number of runs (to one), and a CTA for each while there is room
-            const int warps = (n_runs + rounds - 1) / rounds, grid = warps <= RUN_CTAS * n_sm ? warps : RUN_CTAS * n_sm;
+            const int warps = (n_runs + rounds - 1) / rounds, grid = warps <= ctas * n_sm ? warps : ctas * n_sm;
             const int per_sm = (grid + n_sm - 1) / n_sm, piece_bytes = RUN_WARPS * RUN_PIECE * (int)sizeof(uint4);
             int ring_n = 200 * 1024 / per_sm / piece_bytes;
             ring_n = ring_n < RUN_RING_MIN ? RUN_RING_MIN : ring_n > RUN_RING_MAX ? RUN_RING_MAX : ring_n;
-            const int rc_ = device_setup(reinterpret_cast<const void *>(run_stats_kernel<false>), RUN_RING_MAX * piece_bytes, nullptr);
+            auto *const kern = more ? run_stats_kernel<false, RUN_CTAS_MORE> : run_stats_kernel<false, RUN_CTAS>;
+            const int rc_ = device_setup(reinterpret_cast<const void *>(kern), RUN_RING_MAX * piece_bytes, nullptr);
             if (rc_ != SPECROLL_OK) return rc_;
-            SR_CUDA_TRY(launch_dependent(true, run_stats_kernel<false>, dim3((unsigned)grid), dim3(32 * RUN_WARPS),
+            SR_CUDA_TRY(launch_dependent(true, kern, dim3((unsigned)grid), dim3(32 * RUN_WARPS),
                                          (size_t)ring_n * piece_bytes, st, static_cast<const uint16_t *>(logits), d->V, c, n_runs, ring_n,
                                          run_tab, (float *)nullptr, (float *)nullptr));
         } else {
@@ -2542,9 +2549,9 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
         if (per_sm <= 4) {
             int ring_n = 200 * 1024 / per_sm / piece_bytes;
             if (ring_n > RUN_RING_MAX) ring_n = RUN_RING_MAX;
-            const int rc_ = device_setup(reinterpret_cast<const void *>(run_stats_kernel<true>), RUN_RING_MAX * piece_bytes, nullptr);
+            const int rc_ = device_setup(reinterpret_cast<const void *>(run_stats_kernel<true, 4>), RUN_RING_MAX * piece_bytes, nullptr);
             if (rc_ != SPECROLL_OK) return rc_;
-            SR_CUDA_TRY(launch_dependent(true, run_stats_kernel<true>, dim3((unsigned)rows), dim3(RS_THREADS), (size_t)ring_n * piece_bytes,
+            SR_CUDA_TRY(launch_dependent(true, run_stats_kernel<true, 4>, dim3((unsigned)rows), dim3(RS_THREADS), (size_t)ring_n * piece_bytes,
                                          st, static_cast<const uint16_t *>(logits), d->V, c, rows * RS_WARPS, ring_n, (float2 *)nullptr,
                                          row_max, row_sum));
         } else {

@@ -225,6 +225,12 @@ def test_runs_by_one_warp_each_and_nodes_by_lane_groups(B, N, k, V):
     check(w, o, g, lg)
 
 
+@pytest.mark.parametrize("B,N", [(100, 7), (88, 8), (101, 8)])
+def test_a_warp_for_every_run(B, N):
+    # the last row count with two runs per warp, the first and the last with one
+    test_runs_by_one_warp_each_and_nodes_by_lane_groups(B, N, 4, 8200)
+
+
 @pytest.mark.parametrize("top_p,V", [(1.0, 40008), (0.95, 40008), (1.0, 151936), (0.95, 8200), (1.0, 32776), (1.0, 8),
                                      (1.0, 200008)])
 def test_lazy_row_statistics_do_not_follow_the_batch_size(top_p, V):
