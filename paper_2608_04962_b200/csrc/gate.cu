@@ -21,29 +21,33 @@ constexpr int GATE_THREADS = 128;
 constexpr int GATE_BATCH = 4 * GATE_THREADS;
 }  // namespace gt
 
-// y = Pi x (rank dot products of length d), then y / ||y||, for VPW records per warp; d % 4 == 0 and 16-byte aligned rows.
+// y = Pi x (rank dot products of length d), then y / ||y||; d % 4 == 0 and 16-byte aligned rows.
 // Pi is a few hundred KB that every record meets: with a CTA per record the kernel was bound by bringing it from L2 once
-// per record (512 records, d 3584, rank 24: 17-22 us).  A cluster of four CTAs takes 8 VPW records, each CTA a quarter of
+// per record (512 records, d 3584, rank 24: 17-22 us).  A cluster of four CTAs takes RECS records, each CTA a quarter of
 // the columns: it asks for its part of Pi and of the records in one go (asynchronous copies, `cols` columns of four at a
 // time), so there is one memory latency and not one per step of a loop; the partial dot products meet in distributed
-// shared memory.
-template <int VPW>
+// shared memory.  Within a CTA a warp has four records and every CS-th group of 32 columns: what the products read of shared
+// memory is what bounds them then, and with one or two records per warp that was twice to three times as much
+// (9.7 -> 9.0 us).
+template <int RECS>
 __global__ void __launch_bounds__(gt::SK_THREADS) sketch_kernel(int R, int d4, int rank, int cols, const float4 *__restrict__ X,
                                                                  const int32_t *__restrict__ rows,
                                                                  const float4 *__restrict__ Pi, float *__restrict__ sketch) {
     using namespace gt;
-    __shared__ float part[SK_WARPS * VPW][MAX_RANK];
-    extern __shared__ __align__(16) float4 sh_cols[];  // [rank + SK_WARPS * VPW][cols]
+    constexpr int QUADS = RECS / 4, CS = SK_WARPS / QUADS;
+    __shared__ float part[CS][RECS][MAX_RANK];
+    extern __shared__ __align__(16) float4 sh_cols[];  // [rank + RECS][cols]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cta = (int)cluster_ctarank();
-    const int r0 = (blockIdx.x / SK_CLUSTER) * SK_WARPS * VPW;
+    const int quad = warp % QUADS, cs = warp / QUADS;
+    const int r0 = (blockIdx.x / SK_CLUSTER) * RECS;
     const int per = (d4 + SK_CLUSTER - 1) / SK_CLUSTER, c0 = min(d4, cta * per), c1 = min(d4, c0 + per);
-    for (int e = threadIdx.x; e < SK_WARPS * VPW * MAX_RANK; e += SK_THREADS) part[e / MAX_RANK][e % MAX_RANK] = 0.f;
+    for (int e = threadIdx.x; e < CS * RECS * MAX_RANK; e += SK_THREADS) (&part[0][0][0])[e] = 0.f;
     pdl_wait();
     pdl_launch_dependents();
     for (int cb = c0; cb < c1; cb += cols) {
         const int n = min(cols, c1 - cb);
         __syncthreads();  // (part cleared; the columns before have been read)
-        for (int i = warp; i < rank + SK_WARPS * VPW; i += SK_WARPS) {
+        for (int i = warp; i < rank + RECS; i += SK_WARPS) {
             const int r = min(r0 + i - rank, R - 1);  // (beyond the last record: its copy, not written)
             const float4 *src = (i < rank ? Pi + (size_t)i * d4 : X + (size_t)(rows ? rows[r] : r) * d4) + cb;
             for (int c = lane; c < n; c += 32) cp_async16(smem_u32(sh_cols + (size_t)i * cols + c), src + c, true);
@@ -51,36 +55,35 @@ __global__ void __launch_bounds__(gt::SK_THREADS) sketch_kernel(int R, int d4, i
         cp_async_commit();
         cp_async_wait<0>();
         __syncthreads();
-        const float4 *x = sh_cols + (size_t)(rank + warp * VPW) * cols;
-        for (int i0 = 0; i0 < rank; i0 += 8) {  // eight ranks at a time: independent sums
-            float acc[VPW * 8];
+        const float4 *x = sh_cols + (size_t)(rank + quad * 4) * cols;
+        for (int i0 = 0; i0 < rank; i0 += 8) {  // eight ranks at a time: 32 independent sums
+            float acc[32];
 #pragma unroll
-            for (int q = 0; q < VPW * 8; ++q) acc[q] = 0.f;
-            for (int c = lane; c < n; c += 32) {
-                float4 xv[VPW];
+            for (int q = 0; q < 32; ++q) acc[q] = 0.f;
+            for (int c = lane + 32 * cs; c < n; c += 32 * CS) {
+                float4 xv[4];
 #pragma unroll
-                for (int v = 0; v < VPW; ++v) xv[v] = x[v * cols + c];
+                for (int v = 0; v < 4; ++v) xv[v] = x[v * cols + c];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const float4 pv = sh_cols[(size_t)min(i0 + q, rank - 1) * cols + c];
 #pragma unroll
-                    for (int v = 0; v < VPW; ++v)
+                    for (int v = 0; v < 4; ++v)
                         acc[v * 8 + q] = fmaf(pv.x, xv[v].x, fmaf(pv.y, xv[v].y, fmaf(pv.z, xv[v].z, fmaf(pv.w, xv[v].w, acc[v * 8 + q]))));
                 }
             }
-            constexpr int L = VPW == 2 ? 4 : 3;
-            const float t = warp_sum_many<L>(acc, lane);
-            const int e = lane >> (5 - L);
-            if ((lane & ((1 << (5 - L)) - 1)) == 0) part[warp * VPW + e / 8][i0 + e % 8] += t;  // (a warp's own rows)
+            part[cs][quad * 4 + lane / 8][i0 + lane % 8] += warp_sum_many<5>(acc, lane);  // (a warp's own entries)
         }
     }
     cluster_sync_all();
     // records in turn over the cluster's warps
-    for (int j = cta * SK_WARPS + warp; j < SK_WARPS * VPW && r0 + j < R; j += SK_CLUSTER * SK_WARPS) {
+    for (int j = cta * SK_WARPS + warp; j < RECS && r0 + j < R; j += SK_CLUSTER * SK_WARPS) {
         float v = 0.f;
         if (lane < rank)
 #pragma unroll
-            for (int k = 0; k < SK_CLUSTER; ++k) v += __uint_as_float(ld_dsmem_u32(&part[j][lane], k));
+            for (int k = 0; k < SK_CLUSTER; ++k)
+#pragma unroll
+                for (int q = 0; q < CS; ++q) v += __uint_as_float(ld_dsmem_u32(&part[q][j][lane], k));
         const float nrm = sqrtf(warp_sum(v * v));
         if (lane < rank) sketch[(size_t)(r0 + j) * rank + lane] = nrm > 0.f ? v / nrm : 0.f;
     }
@@ -262,10 +265,10 @@ extern "C" int specroll_reflex_sketch(int32_t R, int32_t d, int32_t rank, const 
     if (!X || !Pi || !sketch) return SPECROLL_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if ((d % 4) == 0 && aligned16(X) && aligned16(Pi)) {
-        // two records per warp halve the reads of Pi; with few records, one, for more CTAs
-        const int vpw = R > 296 ? 2 : 1, per = gt::SK_WARPS * vpw, cols_all = (d / 4 + gt::SK_CLUSTER - 1) / gt::SK_CLUSTER;
+        // sixteen records per cluster halve the reads of Pi; with few records, eight, for more CTAs
+        const int per = R > 296 ? 16 : 8, cols_all = (d / 4 + gt::SK_CLUSTER - 1) / gt::SK_CLUSTER;
         const int cols = std::min(cols_all, gt::SK_SMEM / 16 / (rank + per));
-        auto *const kern = vpw == 2 ? sketch_kernel<2> : sketch_kernel<1>;
+        auto *const kern = per == 16 ? sketch_kernel<16> : sketch_kernel<8>;
         const int rc = device_setup(reinterpret_cast<const void *>(kern), gt::SK_SMEM, nullptr);
         if (rc != SPECROLL_OK) return rc;
         SR_CUDA_TRY(launch_clusters(true, gt::SK_CLUSTER, kern, dim3((unsigned)((R + per - 1) / per * gt::SK_CLUSTER)),

@@ -154,3 +154,24 @@ def test_slots_whose_records_lie_in_later_batches(R, S_, kind):
     assert np.array_equal(host(dn), o["n"]) and np.array_equal(host(dnfb), o["n_fb"])
     np.testing.assert_allclose(host(dmean), o["mean"], rtol=0, atol=2e-5)
     np.testing.assert_allclose(host(dM2), o["M2"], rtol=2e-4, atol=2e-5)
+
+
+def test_records_of_no_slot_have_an_alignment_and_count_nowhere():
+    """Alignments are formed slot by slot; a record whose slot is not one of the call's has its alignment all the same."""
+    g = I.rng(41)
+    R, S_, rank, d = 700, 5, 24, 64
+    s, xi = (g.standard_normal((R, rank)).astype(np.float32) for _ in range(2))
+    slot = g.integers(-2, S_ + 2, size=R).astype(np.int32)
+    keep = (g.random(R) < 0.8).astype(np.uint8)
+    m = g.standard_normal((S_, d)).astype(np.float32)
+    zero, need = np.zeros(S_, np.int32), np.array([2], np.int32)
+    lo, hi = np.array([0.01], np.float32), np.array([0.025], np.float32)
+    dn, dmean, dM2, dnfb = dev(zero.copy()), dev(zero.astype(np.float32)), dev(zero.astype(np.float32)), dev(zero.copy())
+    out = S.reflex_gate(dev(s), dev(xi), dev(slot), dev(keep), dn, dmean, dM2, dnfb, dev(m), dev(zero), dev(need), dev(need),
+                        dev(lo), dev(hi))
+    a = host(out["a"])
+    assert np.array_equal(np.isnan(a), keep == 0)
+    s64, xi64 = s.astype(np.float64), xi.astype(np.float64)
+    want = (s64 * xi64).sum(1) / np.sqrt((s64 ** 2).sum(1) * (xi64 ** 2).sum(1))
+    np.testing.assert_allclose(a[keep != 0], want[keep != 0], rtol=0, atol=2e-6)   # fp32 sums of 24 terms
+    assert np.array_equal(host(dn), np.bincount(slot[(keep != 0) & (slot >= 0) & (slot < S_)], minlength=S_))
