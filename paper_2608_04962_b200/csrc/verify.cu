@@ -325,7 +325,7 @@ constexpr int NUC_THREADS = 512;
 // 15 k cycles for a row of 152 k tokens; loads a round ahead do not help, nor does a closer bound from a sample).  Where a
 // counter does not tell the values apart, or the counted mass stays below the target by rounding, the radix search over the
 // whole row gives the same result in four passes (nucleus_row_radix).  Verification of 256 sequences x 16 nodes, V 151936:
-// 590 us with a search of two passes over the tokens per row, 350 us with this one.
+// 590 us with a search of two passes over the tokens per row, 349 us with this one.
 constexpr int NUC_OCT_LO = (127 - 13) << 7;              // bf16 bits of 2^-13
 constexpr int NUC_VALUES = ((127 + 15) << 7) - NUC_OCT_LO;  // counters per sign; 0: nearer to zero than 2^-13
 constexpr int NUC_SIGN = 8192;                           // the negative values' table, 2^15 bytes behind the other: the sign bit of a
@@ -484,21 +484,20 @@ __device__ bool nucleus_cut(NucleusSmem *st, int r0, int r1, float M, float c, f
         const float e = dist(nucleus_value(r));
         return bin(e) < 256 ? (unsigned long long)n * __float2uint_rn(ex2_approx(-e) * 4294967296.0f) : 0ull;
     };
-    auto scan_u64 = [&](unsigned long long v) {
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long x = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += x;
-        }
-        return v;
+    // A warp has consecutive places, a lane every 32nd of them: beside another CTA that counts, accesses to shared memory are what
+    // this waits for.  (A thread's places next to one another, eight lanes to a bank, and one thread going through the
+    // digits took 8 us a row: verification of 8 / 64 / 256 sequences 73 / 163 / 358 us, now 70 / 160 / 349.)
+    auto sum_u64 = [&](unsigned long long v) {  // over a warp (a sum below 2^59)
+        return ((unsigned long long)__reduce_add_sync(0xffffffffu, (uint32_t)(v >> 27)) << 27) +
+               __reduce_add_sync(0xffffffffu, (uint32_t)v & 0x7ffffffu);
     };
     const unsigned long long tgt = (unsigned long long)((double)target * 4294967296.0);
     const int per = (r1 - r0 + NUC_THREADS) / NUC_THREADS;  // (<= 14)
-    const int my0 = r0 + tid * per, my1 = min(r1 + 1, my0 + per);
+    const int w0 = r0 + warp * 32 * per, w1 = min(r1 + 1, w0 + 32 * per);
     unsigned long long part = 0ull;
-    for (int r = my0; r < my1; ++r) part += fixed_at(r);
-    const unsigned long long incl = scan_u64(part);
-    if (lane == 31) st->wtot[warp] = incl;
+    for (int r = w0 + lane; r < w1; r += 32) part += fixed_at(r);
+    part = sum_u64(part);
+    if (lane == 0) st->wtot[warp] = part;
     if (tid == 0) {
         st->last = -1;
         st->inside = 0ull;
@@ -508,56 +507,59 @@ __device__ bool nucleus_cut(NucleusSmem *st, int r0, int r1, float M, float c, f
         st->p_max = -1;
     }
     __syncthreads();
-    unsigned long long before = 0ull;
-    for (int w = 0; w < warp; ++w) before += st->wtot[w];
-    const unsigned long long end = before + incl, excl = end - part;
-    const unsigned mine = __ballot_sync(0xffffffffu, excl < tgt && end >= tgt);
-    if (mine) {  // the counters of that thread, one per lane
-        const int L = __ffs(mine) - 1;
-        const unsigned long long e0 = __shfl_sync(0xffffffffu, excl, L);
-        const int f = __shfl_sync(0xffffffffu, my0, L), n = __shfl_sync(0xffffffffu, my1, L) - f;
-        const unsigned long long cum = e0 + scan_u64(lane < n ? fixed_at(f + lane) : 0ull);
-        const unsigned hit = __ballot_sync(0xffffffffu, lane < n && cum >= tgt);
-        if (hit && lane == __ffs(hit) - 1) {
-            st->last = f + lane;
-            st->upto = cum;
+    unsigned long long cum64 = sum_u64(lane < warp ? st->wtot[lane] : 0ull);
+    if (cum64 < tgt && cum64 + part >= tgt) {  // (one warp at most)
+        for (int r = w0 + lane;; r += 32) {
+            unsigned long long v = r < w1 ? fixed_at(r) : 0ull;
+            const unsigned long long all = sum_u64(v);
+            if (cum64 + all < tgt) {
+                cum64 += all;
+                continue;
+            }
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long x = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += x;
+            }
+            const unsigned hit = __ballot_sync(0xffffffffu, cum64 + v >= tgt);
+            if (lane == __ffs(hit) - 1) {
+                st->last = r;
+                st->upto = cum64 + v;
+            }
+            break;
         }
     }
     __syncthreads();
     const int last = st->last;
     if (last < 0) return false;
     const int jb = bin(dist(nucleus_value(last)));
-    // this thread's places of the bin, [b0, b1) (the bins do not fall from place to place); sums over a warp go to shared memory
-    // as one addition (near zero a bin has thousands of places, and additions to one word wait for one another)
-    int b0 = my0, b1 = my0;
-    {
+    // the places of the bin (the bins do not fall from place to place)
+    const bool here = w0 < w1 && bin(dist(nucleus_value(w0))) <= jb && bin(dist(nucleus_value(w1 - 1))) >= jb;
+    if (here) {
         unsigned long long in = 0ull;
         uint32_t lo = 0xffffu, hi = 0u;
-        for (int r = my0; r < my1; ++r) {
-            const int b = bin(dist(nucleus_value(r)));
-            if (b < jb) b0 = b1 = r + 1;
-            if (b != jb) continue;
-            b1 = r + 1;
+        int b_min = 0x7fffffff, b_max = -1;
+        for (int r = w0 + lane; r < w1; r += 32) {
+            if (bin(dist(nucleus_value(r))) != jb) continue;
+            b_min = min(b_min, r);
+            b_max = r;
             if (nucleus_count_at(st, r) == 0u) continue;
             if (r <= last) in += fixed_at(r);
             const uint32_t key = ord_key(nucleus_value(r));
             lo = min(lo, key);
             hi = max(hi, key);
         }
-        if (__any_sync(0xffffffffu, b1 > b0)) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) in += __shfl_xor_sync(0xffffffffu, in, o);
-            lo = __reduce_min_sync(0xffffffffu, lo);
-            hi = __reduce_max_sync(0xffffffffu, hi);
-            if (lane == 0) {
-                atomicAdd(&st->inside, in);
-                atomicMin(&st->k_min, lo);
-                atomicMax(&st->k_max, hi);
-            }
-            if (b1 > b0) {
-                atomicMin(&st->p_min, b0);
-                atomicMax(&st->p_max, b1 - 1);
-            }
+        in = sum_u64(in);
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        b_min = __reduce_min_sync(0xffffffffu, b_min);
+        b_max = __reduce_max_sync(0xffffffffu, b_max);
+        if (lane == 0) {
+            if (in) atomicAdd(&st->inside, in);
+            atomicMin(&st->k_min, lo);
+            atomicMax(&st->k_max, hi);
+            atomicMin(&st->p_min, b_min);
+            atomicMax(&st->p_max, b_max);
         }
     }
     __syncthreads();
@@ -565,47 +567,58 @@ __device__ bool nucleus_cut(NucleusSmem *st, int r0, int r1, float M, float c, f
     float cum = (float)((double)(st->upto - st->inside) * (1.0 / 4294967296.0));
     float keep = cum;
     uint32_t prefix = 0u;
-    // Usually the bin has a few dozen places: their masses side by side in shared memory, and one thread takes the digits'
-    // sums in falling order, about a thousand cycles (with a barrier and an addition in shared memory per digit and thread
-    // the digits took 12 k).
-    const int p0 = st->p_min, np = st->p_max - p0 + 1;
+    // Usually the bin has a few dozen places: their masses side by side in shared memory, and one warp takes the digits' sums, a
+    // lane per digit, and goes through them in falling order (with a barrier and an addition in shared memory per digit and
+    // thread the digits took 12 k cycles).
+    const int p0 = st->p_min, p1 = st->p_max + 1;
     float *const f = &st->wsum[0][0];
-    if (np <= (NUC_THREADS / 32) * 16 && (p0 > NUC_ZERO || p0 + np <= NUC_ZERO)) {  // (all of one sign)
-        for (int r = b0; r < b1; ++r)
-            f[r - p0] = (float)nucleus_count_at(st, r) * ex2_approx((bf16_bits_to_float(nucleus_value(r)) - M) * c);
+    if (p1 - p0 <= (NUC_THREADS / 32) * 16 && (p0 > NUC_ZERO || p1 <= NUC_ZERO)) {  // (all of one sign)
+        if (here)
+            for (int r = max(p0, w0) + lane; r < min(p1, w1); r += 32)
+                f[r - p0] = (float)nucleus_count_at(st, r) * ex2_approx((bf16_bits_to_float(nucleus_value(r)) - M) * c);
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0) {
             const uint32_t key0 = ord_key(nucleus_value(p0));  // (the keys fall by one from place to place)
-            int lo = 0, hi = np;
+            int lo = (int)(key0 - k_max), hi = (int)(key0 - k_min) + 1;  // (the places with tokens: at most 17 digits a level)
             for (int shift = 12; shift >= 0; shift -= 4) {
                 if (shift > 0 && ((k_min ^ k_max) >> shift) == 0u) continue;
+                const int first = (int)((key0 - lo) & ((1u << shift) - 1u)) + 1;  // (places of the first digit, at most)
+                const int i = lane == 0 ? lo : min(hi, lo + first + ((lane - 1) << shift));
+                const int j = min(hi, lo + first + (lane << shift));
+                float sum = 0.f;
+#pragma unroll 4
+                for (int q = i; q < j; ++q) sum += f[q];
+                float t[17];
+#pragma unroll
+                for (int d = 0; d < 17; ++d) t[d] = __shfl_sync(0xffffffffu, sum, d);
                 float run = cum, before = cum, tsel = 0.f;
-                int s_lo = lo, s_hi = hi;
-                for (int i = lo; i < hi;) {
-                    const int j = min(hi, i + (int)((key0 - i) & ((1u << shift) - 1u)) + 1);
-                    float sum = 0.f;
-#pragma unroll 8
-                    for (int q = i; q < j; ++q) sum += f[q];
-                    if (sum > 0.f) {
-                        s_lo = i;
-                        s_hi = j;
-                        tsel = sum;
-                        before = run;
-                        if (run + sum >= target) break;
-                        run += sum;
-                    }
-                    i = j;
+                int sel = -1;
+                bool found = false;
+#pragma unroll
+                for (int d = 0; d < 17; ++d) {
+                    if (found || !(t[d] > 0.f)) continue;
+                    sel = d;
+                    tsel = t[d];
+                    before = run;
+                    found = run + t[d] >= target;
+                    run += t[d];
                 }
                 cum = before;  // (none reached the target by rounding: the last digit with mass)
                 keep = cum + tsel;
-                lo = s_lo;
-                hi = s_hi;
+                if (sel >= 0) {
+                    hi = __shfl_sync(0xffffffffu, j, sel);
+                    lo = __shfl_sync(0xffffffffu, i, sel);
+                }
             }
-            st->prefix = key0 - lo;
-            st->keep = keep;
+            if (lane == 0) {
+                st->prefix = key0 - lo;
+                st->keep = keep;
+            }
         }
         return true;
     }
+    // this thread's places of the bin, [b0, b1)
+    const int b0 = max(p0, r0 + tid * per), b1 = min(p1, r0 + (tid + 1) * per);
     for (int level = 0; level < 4; ++level) {
         const int shift = 12 - 4 * level;
         // (one digit for all of the bin: nothing to decide, except the last one's sum)

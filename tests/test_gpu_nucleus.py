@@ -160,3 +160,19 @@ def test_rows_shared_by_one_to_eight_ctas(B, V, top_p):
     u_acc, u_fin = I.verify_uniforms(w)
     o, g = run_both(w, parent, lg, d, cid, cl, u_acc, u_fin, top_p)
     check(w, o, g)
+
+
+@pytest.mark.parametrize("a", [0.5, -0.5, 2.0, -2.0, 0.125, 0.06, -0.06, 0.0])
+@pytest.mark.parametrize("V,top_p", [(16392, 0.7), (16392, 0.3), (264, 0.5)])
+def test_cuts_where_a_bin_meets_a_digit_of_the_key(a, V, top_p):
+    """Rows of values close to a: within the cut's bin the key's upper digits change (at 0.5 and 2), the bin has hundreds of
+    values (near 0.06) or both signs (at 0), or the row has fewer values than the search has threads."""
+    w = I.scaled(I.WORKLOADS["tiny"], B=9, V=V, K=3, k=4, N=8)
+    parent = I.topology(w)
+    cid, cl = I.synthetic_candidates(w)
+    d = ref.tree_draw(parent, np.zeros(w.B, np.int32), cid, cl, I.uniforms24(5, (w.B, w.N)))
+    x = (a + 0.05 * (2 * I.rng(4100 + V).random((w.B, w.N, V)) - 1)).astype(np.float32)
+    lg = torch.from_numpy(x).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+    u_acc, u_fin = I.verify_uniforms(w)
+    o, g = run_both(w, parent, lg, d, cid, cl, u_acc, u_fin, top_p)
+    check(w, o, g)
