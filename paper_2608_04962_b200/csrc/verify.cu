@@ -2538,7 +2538,9 @@ static int run_verify(const specroll_verify_desc *d, float top_p, const void *lo
         // with two runs each: too few warps keep the exponentials, the integer instructions and the waits apart.  21 warps -> 44:
         //   V 152064: 640 rows 50.1 -> 51.5, 768: 60.0 -> 58.4, 800: 62.1 -> 58.6;  V 64000: 640 28.0 -> 29.7, 768 35.3 -> 33.1, 800 34.7 -> 33.2
         const int n_runs = rows * RS_WARPS;
-        const bool more = n_runs > 38 * n_sm;
+        // Not where a run is less than a group (V 8192) and most are empty: 800 rows of V 1024 14.9 -> 16.8, 2048 15.7 -> 14.8, 4096 14.8 ->
+        // 15.3, 8000 15.6 -> 16.0.
+        const bool more = n_runs > 38 * n_sm && d->V >= RS_WARPS * RUN_PIECE * 8;
         const int ctas = more ? RUN_CTAS_MORE : RUN_CTAS, most = RUN_WARPS * ctas * n_sm, rounds = (n_runs + most - 1) / most;
         if (n_runs <= 44 * n_sm) {
             // every warp the same number of runs (to one), and a CTA for each while there is room
