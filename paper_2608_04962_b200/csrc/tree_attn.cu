@@ -539,9 +539,13 @@ static bool merge_by_kernel(long long units, int max_ns) { return max_ns >= 5 ||
 // six shapes (4 to 40 sequences, one to four row blocks) in eight to thirteen chunk lengths each, to 5 %; the length they choose was
 // the fastest of each shape, where a unit start of 4 and a merge kernel of 8 chose 6 % slower ones, 12.6 % at most (12
 // sequences of the 14B shape 44.8 -> 40.9 us a layer, 8 of the 7B shape x 64 nodes 95.6 -> 92.9).
+// streams: the SMs share HBM's bandwidth for the whole launch (one row block, which leaves the softmax time to spare, and 40
+// tiles per SM or more), so a tile takes 1.5 us instead of 0.86 and the same costs are half as many tiles.  28 layers of 256
+// sequences of the 1.5B shape, 53 tiles per SM: 2745 us, 2770 with the costs in full, which leave the longest sequences whole;
+// 90 sequences of the 7B shape, 30 per SM, 233 us for four layers against 226 in full, 48 of the 14B shape 248 against 238.
 // limit >= 0: a plan that takes at least that long is not looked at any further.
-static long long estimate_makespan(const std::vector<int> &tiles, int ct, int copies, long long limit) {
-    constexpr int UNIT = 16, PART = 12, MERGE_CHUNK = 6, MERGE_KERNEL = 20;
+static long long estimate_makespan(const std::vector<int> &tiles, int ct, int copies, bool streams, long long limit) {
+    const int UNIT = streams ? 8 : 16, PART = streams ? 6 : 12, MERGE_CHUNK = streams ? 3 : 6, MERGE_KERNEL = streams ? 10 : 20;
     struct Chunk { int tps, cost; };
     std::vector<Chunk> chunks;
     int max_ns = 1;
@@ -639,13 +643,14 @@ static int compute_attn_plan(const specroll_attn_desc *d, const int32_t *indptr_
         for (int b = 0; b < d->B; ++b) tiles[(size_t)b] = (indptr_host[b + 1] - indptr_host[b] + TT - 1) / TT;
         std::sort(tiles.begin(), tiles.end(), std::greater<int>());
         static const int pcts[] = {100, 75, 125, 60, 150, 85, 200, 50, 300};
+        const bool streams = p->n_rb == 1 && tiles_total * ctas_per_tile >= 40LL * PLAN_SMS;
         long long best = -1;
         int seen[18], n_seen = 0;
         auto consider = [&](int c) {
             for (int i = 0; i < n_seen; ++i)
                 if (seen[i] == c) return;
             seen[n_seen++] = c;
-            const long long m = estimate_makespan(tiles, c, (int)ctas_per_tile, best);
+            const long long m = estimate_makespan(tiles, c, (int)ctas_per_tile, streams, best);
             if (best < 0 || m < best) {
                 best = m;
                 ct = c;
