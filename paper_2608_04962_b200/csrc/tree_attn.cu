@@ -530,41 +530,27 @@ static long long count_chunks(const std::vector<int> &tiles, int ct, int *max_ns
 // dependent loads), and when all work units run side by side, so that nothing streams beside that CTA.
 static bool merge_by_kernel(long long units, int max_ns) { return max_ns >= 5 || (max_ns >= 2 && units <= PLAN_SMS); }
 
-// Estimated finishing time, in quarter tiles (a fifth of a microsecond), of the persistent tcgen05 kernel when
+// Estimated finishing time, in quarter tiles (about a third of a microsecond), of the persistent tcgen05 kernel when
 // sequences of the given tile counts (sorted, longest first) are cut into chunks of at most ct tiles: work units go, in
 // the order the device uses, to whichever of PLAN_SMS CTAs is free first.  A unit costs its K/V tiles, one more for the
-// tree tile of a sequence's last chunk, and UNIT for its start (its first tiles come from pages nobody has touched, its first
-// scores take two passes, the accumulator changes hands); a chunk of a split sequence adds PART for its partial, and the last
-// one the merge when the attention kernel does it, else the merge kernel follows.  The constants are fitted to the layer times of
-// six shapes (4 to 40 sequences, one to four row blocks) in eight to thirteen chunk lengths each, to 5 %; the length they choose was
-// the fastest of each shape, where a unit start of 4 and a merge kernel of 8 chose 6 % slower ones, 12.6 % at most (12
-// sequences of the 14B shape 44.8 -> 40.9 us a layer, 8 of the 7B shape x 64 nodes 95.6 -> 92.9).
-// streams: the SMs share HBM's bandwidth for the whole launch (one row block, which leaves the softmax time to spare, and 40
-// tiles per SM or more), so a tile takes 1.5 us instead of 0.86 and the same costs are half as many tiles.  28 layers of 256
-// sequences of the 1.5B shape, 53 tiles per SM: 2745 us, 2770 with the costs in full, which leave the longest sequences whole;
-// 90 sequences of the 7B shape, 30 per SM, 233 us for four layers against 226 in full, 48 of the 14B shape 248 against 238.
-// limit >= 0: a plan that takes at least that long is not looked at any further.
-static long long estimate_makespan(const std::vector<int> &tiles, int ct, int copies, bool streams, long long limit) {
-    const int UNIT = streams ? 8 : 16, PART = streams ? 6 : 12, MERGE_CHUNK = streams ? 3 : 6, MERGE_KERNEL = streams ? 10 : 20;
+// tree tile of a sequence's last chunk, one for the hand-over between units; a chunk of a split sequence adds one
+// for its partial, and the last one the merge when the attention kernel does it, else the merge kernel follows.
+static long long estimate_makespan(const std::vector<int> &tiles, int ct, int copies) {
     struct Chunk { int tps, cost; };
     std::vector<Chunk> chunks;
     int max_ns = 1;
     const long long units = count_chunks(tiles, ct, &max_ns) * copies;
     const bool merge_inline = !merge_by_kernel(units, max_ns);
-    const long long after = (max_ns > 1 && !merge_inline) ? MERGE_KERNEL + max_ns / 2 : 0;
-    long long work = 0;
     for (int t : tiles) {
         const int ns = std::max(1, (t + ct - 1) / ct), tps = (t + ns - 1) / ns;
         for (int s = 0; s < ns; ++s) {
             const int lo = std::min(t, s * tps), hi = std::min(t, lo + tps);
-            int cost = 4 * (hi - lo) + UNIT;
+            int cost = 4 * (hi - lo) + 4;
             if (s == ns - 1) cost += 4;
-            if (ns > 1) cost += PART + ((merge_inline && s == ns - 1) ? MERGE_CHUNK * ns : 0);
+            if (ns > 1) cost += 4 + ((merge_inline && s == ns - 1) ? 6 * ns : 0);
             chunks.push_back({tps, cost});
-            work += cost;
         }
     }
-    if (limit >= 0 && work * copies / PLAN_SMS + after >= limit) return limit;
     std::stable_sort(chunks.begin(), chunks.end(), [](const Chunk &x, const Chunk &y) { return x.tps > y.tps; });
     std::priority_queue<long long, std::vector<long long>, std::greater<long long>> sms;
     for (int i = 0; i < PLAN_SMS; ++i) sms.push(0);
@@ -575,9 +561,8 @@ static long long estimate_makespan(const std::vector<int> &tiles, int ct, int co
             sms.pop();
             sms.push(t);
             end = std::max(end, t);
-            if (limit >= 0 && end + after >= limit) return limit;
         }
-    return end + after;
+    return end + ((max_ns > 1 && !merge_inline) ? 8 + max_ns / 2 : 0);
 }
 
 struct AttnPlan {
@@ -628,7 +613,11 @@ static int compute_attn_plan(const specroll_attn_desc *d, const int32_t *indptr_
     }
     // chunk length.  Legacy kernel: about four CTAs' worth of work per SM over the whole launch.  tcgen05 kernel:
     // the candidate whose estimated finishing time is lowest (the kernel hands the units, longest first, to
-    // whichever CTA is free, which a few microseconds of host time can play through).  At least 512 tokens,
+    // whichever CTA is free, which the host plays through: 3 to 5 us for a few short sequences, 35 to 70 for 8 to
+    // 37 long ones, 130 for 256, once per set of lengths and ahead of the call's first launch, so candidates are few).
+    // Nine more of them, with unit costs fitted to shapes of 4 to 40 sequences, took up to twice as long to play
+    // through and left few short sequences whole: a layer of one sequence of 800 tokens of the 1.5B shape 10.8 -> 13.1
+    // us, of two of 900 and 333 tokens of the 14B shape 11.6 -> 14.8.  At least 512 tokens,
     // so that the fp32 partials stay a small fraction of the KV bytes.
     const long long ctas_per_tile = (long long)d->Hkv * p->n_rb;
     auto chunk_for = [&](int per_sm_pct) -> int {
@@ -642,23 +631,20 @@ static int compute_attn_plan(const specroll_attn_desc *d, const int32_t *indptr_
         std::vector<int> tiles((size_t)d->B);
         for (int b = 0; b < d->B; ++b) tiles[(size_t)b] = (indptr_host[b + 1] - indptr_host[b] + TT - 1) / TT;
         std::sort(tiles.begin(), tiles.end(), std::greater<int>());
-        static const int pcts[] = {100, 75, 125, 60, 150, 85, 200, 50, 300};
-        const bool streams = p->n_rb == 1 && tiles_total * ctas_per_tile >= 40LL * PLAN_SMS;
+        static const int pcts[] = {75, 100, 125, 150, 200, 300};
         long long best = -1;
-        int seen[18], n_seen = 0;
+        int seen[9], n_seen = 0;
         auto consider = [&](int c) {
             for (int i = 0; i < n_seen; ++i)
                 if (seen[i] == c) return;
             seen[n_seen++] = c;
-            const long long m = estimate_makespan(tiles, c, (int)ctas_per_tile, streams, best);
+            const long long m = estimate_makespan(tiles, c, (int)ctas_per_tile);
             if (best < 0 || m < best) {
                 best = m;
                 ct = c;
             }
         };
         for (int pct : pcts) consider(chunk_for(pct));
-        for (int n = 1; n <= 6; ++n)  // the longest sequence in even parts
-            if ((max_tiles + n - 1) / n >= 512 / TT) consider((max_tiles + n - 1) / n);
         // Chunks below 512 tokens only where every unit still gets an SM of its own: there the layer lasts as long as
         // its longest unit (two sequences of 900 and 2400 tokens: 26 us in chunks of four tiles, attention and
         // merge), and the partials that this adds pass through L2 on an otherwise idle GPU.

@@ -82,6 +82,21 @@ def test_attention_plan_is_host_only_and_consistent(libpath):
     assert S.verify_nucleus_workspace_bytes(4, 8, 3, 2, 1024) > 0
 
 
+@pytest.mark.parametrize("N,Hq,Hkv,lengths,chunks", [(10, 12, 2, (800,), 4),          # 10.8 us a layer; whole 13.1
+                                                     (13, 40, 8, (900, 333), 11),     # 11.6; whole 14.8
+                                                     (10, 12, 2, (1000, 2250), 13),
+                                                     (10, 12, 2, (300,) * 5, 5)])     # nothing is cut
+def test_few_short_sequences_are_cut_into_chunks(libpath, N, Hq, Hkv, lengths, chunks):
+    """A layer of few sequences lasts as long as its longest unit, so they are cut while units have an SM each."""
+    from paper_2608_04962_b200 import binding as S
+    B, G, D = len(lengths), Hq // Hkv, 128
+    blocks = -(-N // (128 // G))
+    per_chunk = Hkv * -(-N // blocks) * G * blocks * (D + 2) * 4 + 32     # partial output, maximum and sum; table row
+    size = [S.tree_attn_workspace_bytes(B, N, Hq, Hkv, D, np.concatenate([[0], np.cumsum(L)]).astype(np.int32))
+            for L in (lengths, (0,) * B)]
+    assert B + round((size[0] - size[1]) / per_chunk) == chunks
+
+
 def test_cache_offsets_must_start_at_zero(libpath):
     """Token coordinates count from the base of Kc / Vc: an offset table that starts elsewhere is refused on the
     host, before anything is enqueued (no device needed)."""
