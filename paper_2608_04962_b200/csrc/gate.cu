@@ -19,6 +19,12 @@ constexpr int SK_CLUSTER = 4;   // CTAs that share the columns of their records
 constexpr int SK_SMEM = 208 * 1024;
 constexpr int GATE_THREADS = 128;
 constexpr int GATE_BATCH = 4 * GATE_THREADS;
+constexpr int GATE_RECS = 8;                // records whose alignments a warp forms at once
+// Up to so many records the gate forms their alignments itself, beyond it a kernel in front spreads them over the GPU.  A call, us,
+// in front -> itself (d 3584, rank 24): 512 records, one in each of 512 slots 14.9 -> 12.2, all in one 49 -> 43, of no slot 14.8 -> 12.2;
+// 1024 of 1024 slots 14.9 -> 12.3, of 16 slots 15.0 -> 14.5; 640 of one slot 57 -> 53, 700 of five 18.6 -> 19.9, 512 of no slot in a
+// call of one slot 14.5 -> 16.6.  Beyond: 4096 records of 16 slots 33.5 -> 35.0, of 512 slots 14.9 -> 18.6, one in each of 4096 24.7 -> 37.
+constexpr int GATE_FEW = 8 * GATE_THREADS;
 }  // namespace gt
 
 // y = Pi x (rank dot products of length d), then y / ||y||; d % 4 == 0 and 16-byte aligned rows.
@@ -138,29 +144,76 @@ struct GateArgs {
     float z_delta, mem_eps;
 };
 
-// Realised alignment of record r, by a warp.
-__device__ __forceinline__ float alignment(const GateArgs &g, int r, int lane) {
+// Realised alignments of the n records of list (the warp's own) to val (may be null) and g.a, by a warp.  The loads of GATE_RECS records
+// are in flight together; a sum is formed by the additions of warp_sum.
+__device__ __forceinline__ void alignments(const GateArgs &g, const int *list, int n, float *val, int lane) {
+    using namespace gt;
+    constexpr int LANES = 32 / GATE_RECS, L = 3;
+    static_assert(GATE_RECS == 1 << L, "records by halving");
+    for (int e0 = 0; e0 < n; e0 += GATE_RECS) {
+        float dot[GATE_RECS], ns[GATE_RECS], nx[GATE_RECS];
+#pragma unroll
+        for (int q = 0; q < GATE_RECS; ++q) {
+            const bool in = e0 + q < n && lane < g.rank;
+            const size_t at = in ? (size_t)list[e0 + q] * g.rank + lane : 0;
+            ns[q] = in ? g.s[at] : 0.f;
+            nx[q] = in ? g.xi[at] : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < GATE_RECS; ++q) {
+            dot[q] = ns[q] * nx[q];
+            ns[q] *= ns[q];
+            nx[q] *= nx[q];
+        }
+        const float d = warp_sum_many<L>(dot, lane), s = sqrtf(warp_sum_many<L>(ns, lane)), x = sqrtf(warp_sum_many<L>(nx, lane));
+        const int e = e0 + lane / LANES;
+        if (lane % LANES == 0 && e < n) {
+            const float v = (s > 0.f && x > 0.f) ? d / (s * x) : 0.f;
+            if (val) val[e] = v;
+            g.a[list[e]] = v;
+        }
+    }
+}
+
+// Realised alignment of every record, ahead of gate_kernel<false>: a warp per record.
+__global__ void __launch_bounds__(256) align_kernel(GateArgs g) {
+    const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    pdl_wait();
+    pdl_launch_dependents();
+    if (r >= g.R) return;
+    if (g.keep && !g.keep[r]) {
+        if (lane == 0) g.a[r] = __int_as_float(0x7fc00000);
+        return;
+    }
     const float sv = lane < g.rank ? g.s[(size_t)r * g.rank + lane] : 0.f;
     const float xv = lane < g.rank ? g.xi[(size_t)r * g.rank + lane] : 0.f;
     const float dot = warp_sum(sv * xv), ns = sqrtf(warp_sum(sv * sv)), nx = sqrtf(warp_sum(xv * xv));
-    return (ns > 0.f && nx > 0.f) ? dot / (ns * nx) : 0.f;
+    if (lane == 0) g.a[r] = (ns > 0.f && nx > 0.f) ? dot / (ns * nx) : 0.f;
 }
 
 // A CTA per slot: its records, in order, go into the running moments; then the score and the gate, with the RMS of the
 // memory row.  Bound by latency: all threads look for the slot's records (512 at a time) and have the memory row's loads
-// in flight meanwhile (a warp per slot took 14 us for 512 slots and records of d 3584).  A record's alignment is formed by
-// the CTA of its slot, a warp per record (a kernel of its own in front of this one cost its launch and round trips).
-__global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g) {
+// in flight meanwhile (a warp per slot took 14 us for 512 slots and records of d 3584).
+// FEW (at most GATE_FEW records, all looked at in one go): a record's alignment is formed by the warp that finds it, and those of
+// no slot are shared among the CTAs.  (Formed one at a time, and by the first CTA those of no slot: 512 in one slot 121 us, of none 68.)
+template <bool FEW>
+__global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g, int stray_mask) {
     using namespace gt;
-    __shared__ int hit[GATE_BATCH];
-    __shared__ float val[GATE_BATCH];
-    __shared__ int lost[GATE_BATCH];
-    __shared__ int n_hit, n_lost;
-    __shared__ float red[GATE_THREADS / 32];
-    const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+    constexpr int WARPS = GATE_THREADS / 32, MOST = FEW ? GATE_FEW : GATE_BATCH, PER_WARP = MOST / WARPS, GROUPS = MOST / GATE_THREADS;
+    __shared__ int hit[MOST];  // FEW: PER_WARP of every warp
+    __shared__ float val[MOST];
+    __shared__ int n_hit, n_own[WARPS];
+    __shared__ float red[WARPS];
+    const int j = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     pdl_wait();
     pdl_launch_dependents();
-    if (tid == 0) n_hit = n_lost = 0;
+    if (tid == 0) n_hit = 0;
+    int sl[GROUPS];
+    // FEW: a warp has consecutive records, the same number of groups of 32 each
+    const int groups = (g.R + GATE_THREADS - 1) / GATE_THREADS, rw = warp * groups * 32 + lane;
+    if (FEW)
+#pragma unroll
+        for (int q = 0; q < GROUPS; ++q) sl[q] = q < groups && rw + 32 * q < g.R ? g.slot[rw + 32 * q] : 0;
     int n = g.n[j], nfb = g.n_fb[j];
     float mean = g.mean[j], M2 = g.M2[j];
     float ss = 0.f;
@@ -180,63 +233,74 @@ __global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g) {
     } else {
         for (int c = tid; c < g.d; c += GATE_THREADS) ss = fmaf(mr[c], mr[c], ss);
     }
-    __syncthreads();
-    for (int r0 = 0; r0 < g.R; r0 += GATE_BATCH) {
-        int sl[4];
+    auto moment = [&](float v) {
+        n += 1;
+        const float delta = v - mean;
+        mean += delta / (float)n;
+        M2 += delta * (v - mean);
+        nfb += 1;
+    };
+    if (FEW) {
+        int *const list = hit + warp * PER_WARP;  // this slot's records in order; from the end, those of no slot
+        int own_n = 0, none_n = 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int r = r0 + q * GATE_THREADS + tid;
-            sl[q] = r < g.R ? g.slot[r] : -1;
+        for (int q = 0; q < GROUPS; ++q) {
+            const int r = rw + 32 * q;
+            const bool in = q < groups && r < g.R;
+            // (a record of no slot of this call has an alignment all the same)
+            bool own = in && sl[q] == j, none = in && (unsigned)sl[q] >= (unsigned)g.S && (r & stray_mask) == j;
+            if ((own || none) && g.keep && !g.keep[r]) {
+                g.a[r] = __int_as_float(0x7fc00000);
+                own = none = false;
+            }
+            const unsigned mo = __ballot_sync(0xffffffffu, own), mn = __ballot_sync(0xffffffffu, none), below = (1u << lane) - 1u;
+            if (own) list[own_n + __popc(mo & below)] = r;
+            if (none) list[PER_WARP - 1 - none_n - __popc(mn & below)] = r;
+            own_n += __popc(mo);
+            none_n += __popc(mn);
         }
+        __syncwarp();
+        alignments(g, list, own_n, val + warp * PER_WARP, lane);
+        alignments(g, list + PER_WARP - none_n, none_n, nullptr, lane);
+        if (lane == 0) n_own[warp] = own_n;
+        __syncthreads();
+        if (tid == 0)
+            for (int w = 0; w < WARPS; ++w)
+                for (int e = 0, ne = n_own[w]; e < ne; ++e) moment(val[w * PER_WARP + e]);
+    } else {
+        __syncthreads();
+        for (int r0 = 0; r0 < g.R; r0 += GATE_BATCH) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int r = r0 + q * GATE_THREADS + tid;
-            // (a record of no slot of this call has an alignment all the same: the first CTA's)
-            const bool stray = j == 0 && (sl[q] < 0 || sl[q] >= g.S);
-            if (r < g.R && (sl[q] == j || stray)) {
-                if (g.keep && !g.keep[r])
-                    g.a[r] = __int_as_float(0x7fc00000);
-                else if (stray)
-                    lost[atomicAdd(&n_lost, 1)] = r;
-                else
-                    hit[atomicAdd(&n_hit, 1)] = r;
+            for (int q = 0; q < 4; ++q) {
+                const int r = r0 + q * GATE_THREADS + tid;
+                sl[q] = r < g.R ? g.slot[r] : -1;
             }
-        }
-        __syncthreads();
-        const int nh = n_hit, nl = n_lost;
-        __syncthreads();  // (all have read them before the next records are counted)
-        if (nh + nl == 0) continue;
-        for (int e = tid >> 5; e < nl; e += GATE_THREADS / 32) {
-            const float v = alignment(g, lost[e], lane);
-            if (lane == 0) g.a[lost[e]] = v;
-        }
-        // in record order
-        for (int e = tid >> 5; e < nh; e += GATE_THREADS / 32) {
-            const int r = hit[e];
-            int rk = 0;
-            for (int f = lane; f < nh; f += 32) rk += hit[f] < r;
-            rk = __reduce_add_sync(0xffffffffu, rk);
-            const float v = alignment(g, r, lane);
-            if (lane == 0) {
-                val[rk] = v;
-                g.a[r] = v;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int r = r0 + q * GATE_THREADS + tid;
+                if (sl[q] == j && r < g.R && (!g.keep || g.keep[r])) hit[atomicAdd(&n_hit, 1)] = r;
             }
-        }
-        __syncthreads();
-        if (tid == 0) {
-            n_hit = n_lost = 0;
-            for (int e = 0; e < nh; ++e) {
-                n += 1;
-                const float delta = val[e] - mean;
-                mean += delta / (float)n;
-                M2 += delta * (val[e] - mean);
-                nfb += 1;
+            __syncthreads();
+            const int nh = n_hit;
+            __syncthreads();  // (all have read it before the next records are counted)
+            if (nh == 0) continue;
+            // in record order
+            for (int e = tid; e < nh; e += GATE_THREADS) {
+                const int r = hit[e];
+                int rk = 0;
+                for (int f = 0; f < nh; ++f) rk += hit[f] < r;
+                val[rk] = g.a[r];
             }
+            __syncthreads();
+            if (tid == 0) {
+                n_hit = 0;
+                for (int e = 0; e < nh; ++e) moment(val[e]);
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
     ss = warp_sum(ss);
-    if (lane == 0) red[tid >> 5] = ss;
+    if (lane == 0) red[warp] = ss;
     __syncthreads();
     if (tid == 0) {
         ss = (red[0] + red[1]) + (red[2] + red[3]);
@@ -291,7 +355,7 @@ extern "C" int specroll_reflex_gate(const specroll_gate_desc *d, const float *s,
     if (!n || !mean || !M2 || !n_fb || !m || !horizon || !n_align_min || !n_fb_min || !alpha_lo || !alpha_hi || !rel ||
         !alpha)
         return SPECROLL_EINVAL;
-    // the alignments are needed by the second kernel: without the caller's array there is nowhere to keep them
+    // more than GATE_FEW records: the alignments are needed by the second kernel, and the caller's array is where they are kept
     if (d->R > 0 && (!s || !xi || !slot || !a)) return SPECROLL_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     GateArgs g;
@@ -319,6 +383,13 @@ extern "C" int specroll_reflex_gate(const specroll_gate_desc *d, const float *s,
     g.H = d->H;
     g.z_delta = d->z_delta;
     g.mem_eps = d->mem_eps;
-    SR_CUDA_TRY(launch_dependent(true, gate_kernel, dim3((unsigned)d->S), dim3(gt::GATE_THREADS), 0, st, g));
+    if (d->R > gt::GATE_FEW) {
+        SR_CUDA_TRY(launch_dependent(true, align_kernel, dim3((unsigned)(d->R + 7) / 8), dim3(256), 0, st, g));
+        SR_CUDA_TRY(launch_dependent(true, gate_kernel<false>, dim3((unsigned)d->S), dim3(gt::GATE_THREADS), 0, st, g, 0));
+        return SPECROLL_OK;
+    }
+    int share = 1;  // CTAs that share the records of no slot: a power of two
+    while (share <= d->S / 2) share *= 2;
+    SR_CUDA_TRY(launch_dependent(true, gate_kernel<true>, dim3((unsigned)d->S), dim3(gt::GATE_THREADS), 0, st, g, share - 1));
     return SPECROLL_OK;
 }
