@@ -188,7 +188,11 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
 
 // Programmatic dependent launch: a kernel lets the next one in the stream start its prologue (pdl_launch_dependents)
 // and waits for the one before it to complete, with its memory visible (pdl_wait; returns at once in a kernel that
-// was launched the ordinary way).  Everything a kernel reads from, or writes to, global memory comes after its wait.
+// was launched the ordinary way).  Everything a kernel writes to global memory comes after its wait, and so does what it
+// reads, with one exception: the call's own inputs (weights, and what the caller's kernels left in front of the call) may
+// be read ahead of it where nothing in front of the call can still be running when the kernel starts.  That is so if
+// the call's first kernel is launched the ordinary way, or lets its dependents start only after its own wait; each early
+// read says which, and the launch that it stands on says so too.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

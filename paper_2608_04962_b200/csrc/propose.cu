@@ -115,7 +115,7 @@ constexpr int RX_THREADS = 256;
 // zt[r,:] = bf16(z[r,:] + coef * m[r,:]),  r = b*K + hd,
 // coef = alpha * RMS(z) / (RMS(m) + eps), shrunk so that |coef * m|_2 <= clip_c * |z|_2.
 // Bound by round trips to memory: a thread keeps its NV elements of both rows in registers (d <= NV * RX_THREADS), what the
-// call's caller wrote (memory, ratio) is read ahead of the wait, and the two sums share their barriers.  32 rows of 3584: it ends 6.4 -> 3.4 us
+// call's caller wrote (memory, ratio) is read ahead of the wait (the call's first kernel is an ordinary launch), and the two sums share their barriers.  32 rows of 3584: it ends 6.4 -> 3.4 us
 // behind the heads.
 template <int NV>
 __global__ void __launch_bounds__(RX_THREADS, NV <= 8 ? 7 : NV <= 24 ? 72 / NV : 1)  // (the rows of the model shapes are resident at once)
@@ -662,6 +662,7 @@ static int set_smem(Kern kern, int bytes) {
     return SPECROLL_OK;
 }
 
+// pdl: not as the first kernel of a call (the uniforms and anchors are read ahead of the kernel's wait)
 static int launch_tree_draw(bool pdl, const Topo &topo, int B, int K, int k, float T, const int32_t *anchor,
                             const int32_t *cand_id, const float *cand_logit, const float *u_draw,
                             int32_t *tree_tok, uint8_t *tree_cand, float *slot_q, cudaStream_t st) {
@@ -748,7 +749,10 @@ extern "C" int specroll_propose(const specroll_propose_desc *d, const void *h, c
 
     // From here on every kernel is launched as the programmatic dependent of the one before it: it may set itself up
     // (barriers, tensor memory, tensor-map prefetch) under the tail of its predecessor and waits for the predecessor's
-    // completion before it touches global memory.
+    // completion before it touches what the call's kernels write.  The caller's arrays are read ahead of that wait (weights,
+    // memory and ratio, anchors and uniforms), so the call's FIRST kernel has to be launched the ordinary way, behind
+    // everything in front of the call (a gate that writes the ratio lets its dependents start early): the one above,
+    // or the LayerNorm.
     SR_CUDA_TRY(launch_dependent(pre_head, layernorm_kernel, dim3(B), dim3(LN_THREADS), dd * sizeof(float), st, hb,
                                  static_cast<const __nv_bfloat16 *>(ln_gamma), static_cast<const __nv_bfloat16 *>(ln_beta),
                                  xhat, B, dd, p.KX, d->ln_eps, status));

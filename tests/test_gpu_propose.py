@@ -229,6 +229,43 @@ def test_tree_draw_with_a_candidate_that_dwarfs_the_rest():
         np.testing.assert_allclose(host(d["slot_q"]), o["slot_q"], rtol=1e-6)
 
 
+@pytest.mark.parametrize("pre_head", [False, True])
+def test_inputs_written_directly_in_front_of_a_proposal(pre_head):
+    """Ratios by the gate (which lets its dependents start early), memory, uniforms and anchors by copies, all on the stream directly in
+    front of the call: the same bits as when everything in front is complete before the call is made."""
+    w = I.scaled(I.WORKLOADS["qwen1.5b"], B=40, K=4, k=8, d=512, V=5000, N=16)
+    x = I.propose_inputs(w, peaked=True)
+    n = w.B if pre_head else w.B * w.K
+    flags = S.REFLEX_PRE_HEAD if pre_head else 0
+    fixed = [dev_bf16(x[v]) for v in ("h", "A", "bias", "W")]
+    m, anchor, u = torch.zeros((n, w.d), device="cuda"), dev(x["anchor"]), dev(x["u_draw"])
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    zero, need = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.ones(1, dtype=torch.int32, device="cuda")
+    lo = torch.full((1,), 0.05, device="cuda")
+    for _ in range(12):
+        s, new_m = torch.randn((n, 24), generator=g, device="cuda"), torch.randn((n, w.d), generator=g, device="cuda")
+        xi = s * (torch.rand((n, 1), generator=g, device="cuda") - 0.5)        # the gate opens for about half of the rows
+        new_u = torch.rand((w.B, w.N), generator=g, device="cuda")
+        new_anchor = torch.randint(0, w.V, (w.B,), generator=g, device="cuda", dtype=torch.int32)
+        outs = []
+        for apart in (True, False):
+            state = [v.clone() for v in (zero + 2, zero.float(), zero.float(), zero + 2)]
+            m.zero_(), u.zero_(), anchor.zero_()
+            torch.cuda.synchronize()
+            anchor.copy_(new_anchor), u.copy_(new_u), m.copy_(new_m)
+            alpha = S.reflex_gate(s, xi, torch.arange(n, device="cuda", dtype=torch.int32), None, *state, m, zero, need, need, lo,
+                                  2 * lo, z_delta=0.0)["alpha"]
+            if apart:
+                torch.cuda.synchronize()
+            o = S.propose(fixed[0], anchor, *fixed[1:], m if pre_head else m.view(w.B, w.K, w.d),
+                          alpha if pre_head else alpha.view(w.B, w.K), x["parent"], u, k=w.k, flags=flags)
+            torch.cuda.synchronize()
+            assert 0.2 < float((alpha > 0).float().mean()) < 0.8
+            outs.append({key: host(v) for key, v in o.items()})
+        assert all(np.array_equal(outs[0][key], outs[1][key]) for key in outs[0])
+
+
 def test_bad_arguments():
     w = I.scaled(I.WORKLOADS["tiny"], B=2)
     x = I.propose_inputs(w)
