@@ -115,10 +115,12 @@ constexpr int RX_THREADS = 256;
 // zt[r,:] = bf16(z[r,:] + coef * m[r,:]),  r = b*K + hd,
 // coef = alpha * RMS(z) / (RMS(m) + eps), shrunk so that |coef * m|_2 <= clip_c * |z|_2.
 // Bound by round trips to memory: a thread keeps its NV elements of both rows in registers (d <= NV * RX_THREADS), what the
-// call's caller wrote (memory, ratio) is read ahead of the wait (the call's first kernel is an ordinary launch), and the two sums share their barriers.  32 rows of 3584: it ends 6.4 -> 3.4 us
-// behind the heads.
+// call's caller wrote (memory, ratio) is read ahead of the wait (the call's first kernel is an ordinary launch), and the two
+// sums share their barriers.  32 rows of 3584: it ends 6.4 -> 3.4 us behind the heads.
+// CTAs per SM: what the rows' registers leave room for.  Seven at NV 8, which hold all of 1024 rows at once, spill: it ends 5.3 us behind
+// the heads for 1024 rows of 1536, 4.7 of 1024, 2.7 for 256 rows of 1536; six 4.3, 3.9 and 2.4.
 template <int NV>
-__global__ void __launch_bounds__(RX_THREADS, NV <= 8 ? 7 : NV <= 24 ? 72 / NV : 1)  // (the rows of the model shapes are resident at once)
+__global__ void __launch_bounds__(RX_THREADS, NV <= 8 ? 6 : NV <= 24 ? 72 / NV : 1)
 reflex_kernel(const float *__restrict__ z, const float *__restrict__ m, const float *__restrict__ alpha,
               __nv_bfloat16 *__restrict__ zt, int d, float rms_eps, float clip_c) {
     __shared__ float2 red[RX_THREADS / 32];
