@@ -229,6 +229,25 @@ def test_tree_draw_with_a_candidate_that_dwarfs_the_rest():
         np.testing.assert_allclose(host(d["slot_q"]), o["slot_q"], rtol=1e-6)
 
 
+@pytest.mark.parametrize("k,lead", [(33, 0), (33, 32), (40, 35), (64, 0), (64, 31), (64, 63)])
+def test_tree_draw_with_more_than_32_candidates_of_which_one_dwarfs_the_rest(k, lead):
+    # as above with lists of two candidates per lane, the leading candidate in either half; every child after a parent's first one is
+    # drawn from weights that have been renormalised
+    parent = np.array([-1] + [0] * 20 + [1] * 10 + [2] * 10, np.int32)
+    B, K, N = 32, 2, parent.shape[0]
+    g = I.rng(79 + k + lead)
+    cid = np.tile(np.arange(K * k, dtype=np.int32).reshape(1, K, k), (B, 1, 1))
+    cl = g.standard_normal((B, K, k)).astype(np.float32)
+    cl[..., lead] += 900.0
+    u, anchor = I.uniforms24(11 + lead, (B, N)), np.zeros(B, np.int32)
+    o = ref.tree_draw(parent, anchor, cid, cl, u)
+    d = S.tree_draw(parent, dev(anchor), dev(cid), dev(cl), dev(u))
+    assert (o["tree_cand"][:, [1, 21, 31]] == lead).all()
+    assert np.array_equal(host(d["tree_tok"]), o["tree_tok"])
+    assert np.array_equal(host(d["tree_cand"]), o["tree_cand"])
+    np.testing.assert_allclose(host(d["slot_q"]), o["slot_q"], rtol=1e-6)
+
+
 @pytest.mark.parametrize("pre_head", [False, True])
 def test_inputs_written_directly_in_front_of_a_proposal(pre_head):
     """Ratios by the gate (which lets its dependents start early), memory, uniforms and anchors by copies, all on the stream directly in
