@@ -225,7 +225,7 @@ def test_runs_by_one_warp_each_and_nodes_by_lane_groups(B, N, k, V):
     check(w, o, g, lg)
 
 
-@pytest.mark.parametrize("B,N", [(37, 19), (88, 8), (74, 11), (163, 5)])
+@pytest.mark.parametrize("B,N", [(100, 7), (37, 19), (88, 8), (101, 8), (74, 11), (163, 5)])
 def test_a_warp_for_every_run(B, N):
     # on 148 SMs: the last row count with two runs per warp (703), the first and the last with one (704, 814; a warp has 44 places
     # per SM), and the first with a CTA per row (815)
