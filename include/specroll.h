@@ -340,7 +340,7 @@ int specroll_reflex_feedback_ex(const specroll_feedback_desc *desc, const void *
  * inside [alpha_lo, alpha_hi] without printing the map; linear in the score is this implementation's reading.
  * Shapes (device): s, xi[R, rank] fp32; slot[R] i32 in [0, S); keep[R] u8 nullable; n, n_fb[S] i32 in/out;
  * mean, M2[S] fp32 in/out; m[S, d] fp32; horizon[S] i32 in [0, H); n_align_min, n_fb_min[H] i32; alpha_lo,
- * alpha_hi[H] fp32; outputs a[R] (nullable; NaN for records not kept), rel[S], alpha[S] fp32. */
+ * alpha_hi[H] fp32; outputs a[R] (NaN for records not kept; NULL only when R == 0), rel[S], alpha[S] fp32. */
 typedef struct {
     int32_t R, S, d, rank, H;
     float z_delta; /* paper: 0.60 */

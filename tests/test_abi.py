@@ -132,3 +132,14 @@ def test_an_empty_batch_is_valid_and_needs_no_device(libpath):
     # a malformed tree is still refused
     bad = np.array([-1, 2, 0, 1], np.int32)
     assert L.specroll_verify(C.byref(vd), null, bad.ctypes.data_as(C.c_void_p), *([null] * 15), C.c_size_t(0), null) == 1
+
+
+def test_the_gate_needs_a_place_for_the_alignments_of_its_records(libpath):
+    import ctypes as C
+    from paper_2608_04962_b200 import binding as S
+    desc = S.GateDesc(4, 2, 64, 24, 1, 0.6, 1e-12, 0)
+    some = np.zeros(64, np.float32).ctypes.data_as(C.c_void_p)     # (refused on the host: never read)
+    args = [some] * 14 + [C.c_void_p(0), some, some, C.c_void_p(0)]
+    assert S.lib().specroll_reflex_gate(C.byref(desc), *args) == 1                # SPECROLL_EINVAL
+    text = open(os.path.join(ROOT, "include", "specroll.h")).read()
+    assert "a[R] (NaN for records not kept; NULL only when R == 0)" in text
