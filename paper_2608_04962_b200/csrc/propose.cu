@@ -466,7 +466,9 @@ topk_merge8_wide_kernel(const float *__restrict__ pval, const int32_t *__restric
 
 // ------------------------------------------------------------------------------ P5 tree draw
 
-constexpr int DRAW_WARPS = 16;
+// Sixteen warps had the nodes of a wide tree side by side no sooner and left an SM half as many sequences at a time: 32 sequences x 64
+// nodes 10.0 us with eight, 10.4 with sixteen; 256 x 16 5.4 and 6.6; 1024 x 64 29 and 46; 4096 x 16 36 and 70.
+constexpr int DRAW_WARPS = 8;
 
 // inclusive sums over the first `n` lanes (a power of two; what lies behind them is not meaningful)
 __device__ __forceinline__ double warp_incl_scan_f64(double v, int lane, int n) {
