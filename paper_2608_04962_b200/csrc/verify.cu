@@ -1999,6 +1999,8 @@ constexpr int TILE_SMEM_LIMIT = 227 * 1024 - TILE_STATIC_SMEM;     // dynamic
 
 // The nodes with children, in order, to par (by one warp); returns how many there are.  Ahead of the wait for the statistics: looked
 // for node by node behind it, they were on the walk's critical path.
+// Not where there are no stored logits: nothing of that kernel runs ahead of the projection's end, and a short walk takes longer with
+// the list than it saves (1 sequence x 8 nodes 61.0 us, listed 64.3; 4 x 16 53.7 and 55.8; 32 x 32 106.7 and 107.2; 16 x 48 47.9 and 46.7).
 __device__ __forceinline__ int walk_parents(const Topo &topo, int N, int8_t *par) {
     const int lane = threadIdx.x & 31;
     int n = 0;
@@ -2014,17 +2016,31 @@ __device__ __forceinline__ int walk_parents(const Topo &topo, int N, int8_t *par
 // Every node with children on its own.  first[u]: accepted child or -1, mm[u]: smallest margin, ovm[u, j]: the residual's
 // masses where all children were rejected.  (A warp per node took 9 k
 // cycles, two rounds of them where more than sixteen nodes have children: 10 us of the 66 us of 16 sequences x 48 nodes.)
-// par: the n_par nodes with children (walk_parents).
+// LISTED: par has the n_par nodes with children (walk_parents); else they are looked for here.
+template <bool LISTED>
 __device__ __forceinline__ void walk_nodes(const Topo &topo, int n_par, const int8_t *par, int k, const double *p, const float *rsum,
                                            const WalkSlots &w, int32_t *first, float *mm, double *ovm) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int kp = 1;
     while (kp < k) kp <<= 1;
     const int per_warp = 32 / kp, grp = lane / kp, j = lane & (kp - 1);
+    if (!LISTED) {
+        n_par = 0;
+        for (int u = 0; u < topo.N; ++u) n_par += topo.n_child[u] > 0;
+    }
     // as few nodes per warp as give every node a place in one round
     const int share = min(per_warp, (n_par + TERM_WARPS - 1) / TERM_WARPS);
     for (int i0 = warp * share; i0 < n_par; i0 += TERM_WARPS * share) {
-        const int u = grp < share && i0 + grp < n_par ? par[i0 + grp] : -1;
+        int u = -1;
+        if (grp < share && i0 + grp < n_par) {
+            if (LISTED) {
+                u = par[i0 + grp];
+            } else {
+                int idx = 0;
+                for (int n = 0; n < topo.N; ++n)
+                    if (topo.n_child[n] > 0 && idx++ == i0 + grp) u = n;
+            }
+        }
         double rho = u >= 0 && j < k ? p[u * k + j] : 0.0;
         float mg;
         const int child = walk_group(topo, u, k, kp, rho, w, mg);
@@ -2278,9 +2294,9 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     if (TILES) pdl_wait();
     const WalkSlots slots = walk_slots(sh_dyn + L.slots, N, k);
     __shared__ int sh_odd, sh_n_par;
-    __shared__ int8_t sh_par[SPECROLL_MAX_NODES];
+    __shared__ int8_t sh_par[TILES ? 1 : SPECROLL_MAX_NODES];
     if (tid == 0) sh_odd = !L.grouped;
-    if (warp == 0) {
+    if (!TILES && warp == WT_WARPS - 1) {  // (the last warp has the least to fetch)
         const int n = walk_parents(topo, N, sh_par);
         if (lane == 0) sh_n_par = n;
     }
@@ -2321,7 +2337,7 @@ __global__ void __launch_bounds__(WT_THREADS, 2) walk_term_kernel(WalkArgs a, To
     __syncthreads();
     // (2) every node with children on its own
     if (!sh_odd) {
-        walk_nodes(topo, sh_n_par, sh_par, k, wp, rsum, slots, first, mmin, ovm);
+        walk_nodes<!TILES>(topo, sh_n_par, sh_par, k, wp, rsum, slots, first, mmin, ovm);
     } else {
         const WalkStage stage{rmax, rsum, buf.uacc, ttok, buf.tcand, cid, buf.clog, pre, buf.parent, buf.e, wp};
         int idx = 0;
