@@ -32,19 +32,18 @@ constexpr int GATE_FEW = 8 * GATE_THREADS;
 // per record (512 records, d 3584, rank 24: 17-22 us).  A cluster of four CTAs takes RECS records, each CTA a quarter of
 // the columns: it asks for its part of Pi and of the records in one go (asynchronous copies, `cols` columns of four at a
 // time), so there is one memory latency and not one per step of a loop; the partial dot products meet in distributed
-// shared memory.  Within a CTA a warp has four records and every CS-th group of 32 columns: what the products read of shared
-// memory is what bounds them then, and with one or two records per warp that was twice to three times as much
-// (9.7 -> 9.0 us).
-template <int RECS>
+// shared memory.  Within a CTA a warp has VPW records and every CS-th group of 32 columns: where the columns are many, what the
+// products read of shared memory bounds them, and that is the less the more records a warp has.
+template <int RECS, int VPW>
 __global__ void __launch_bounds__(gt::SK_THREADS) sketch_kernel(int R, int d4, int rank, int cols, const float4 *__restrict__ X,
                                                                  const int32_t *__restrict__ rows,
                                                                  const float4 *__restrict__ Pi, float *__restrict__ sketch) {
     using namespace gt;
-    constexpr int QUADS = RECS / 4, CS = SK_WARPS / QUADS;
+    constexpr int GROUPS = RECS / VPW, CS = SK_WARPS / GROUPS, L = VPW == 4 ? 5 : VPW == 2 ? 4 : 3;
     __shared__ float part[CS][RECS][MAX_RANK];
     extern __shared__ __align__(16) float4 sh_cols[];  // [rank + RECS][cols]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cta = (int)cluster_ctarank();
-    const int quad = warp % QUADS, cs = warp / QUADS;
+    const int grp = warp % GROUPS, cs = warp / GROUPS;
     const int r0 = (blockIdx.x / SK_CLUSTER) * RECS;
     const int per = (d4 + SK_CLUSTER - 1) / SK_CLUSTER, c0 = min(d4, cta * per), c1 = min(d4, c0 + per);
     for (int e = threadIdx.x; e < CS * RECS * MAX_RANK; e += SK_THREADS) (&part[0][0][0])[e] = 0.f;
@@ -61,24 +60,26 @@ __global__ void __launch_bounds__(gt::SK_THREADS) sketch_kernel(int R, int d4, i
         cp_async_commit();
         cp_async_wait<0>();
         __syncthreads();
-        const float4 *x = sh_cols + (size_t)(rank + quad * 4) * cols;
-        for (int i0 = 0; i0 < rank; i0 += 8) {  // eight ranks at a time: 32 independent sums
-            float acc[32];
+        const float4 *x = sh_cols + (size_t)(rank + grp * VPW) * cols;
+        for (int i0 = 0; i0 < rank; i0 += 8) {  // eight ranks at a time: 8 VPW independent sums
+            float acc[VPW * 8];
 #pragma unroll
-            for (int q = 0; q < 32; ++q) acc[q] = 0.f;
+            for (int q = 0; q < VPW * 8; ++q) acc[q] = 0.f;
             for (int c = lane + 32 * cs; c < n; c += 32 * CS) {
-                float4 xv[4];
+                float4 xv[VPW];
 #pragma unroll
-                for (int v = 0; v < 4; ++v) xv[v] = x[v * cols + c];
+                for (int v = 0; v < VPW; ++v) xv[v] = x[v * cols + c];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const float4 pv = sh_cols[(size_t)min(i0 + q, rank - 1) * cols + c];
 #pragma unroll
-                    for (int v = 0; v < 4; ++v)
+                    for (int v = 0; v < VPW; ++v)
                         acc[v * 8 + q] = fmaf(pv.x, xv[v].x, fmaf(pv.y, xv[v].y, fmaf(pv.z, xv[v].z, fmaf(pv.w, xv[v].w, acc[v * 8 + q]))));
                 }
             }
-            part[cs][quad * 4 + lane / 8][i0 + lane % 8] += warp_sum_many<5>(acc, lane);  // (a warp's own entries)
+            const float t = warp_sum_many<L>(acc, lane);
+            const int e = lane >> (5 - L);
+            if ((lane & ((1 << (5 - L)) - 1)) == 0) part[cs][grp * VPW + e / 8][i0 + e % 8] += t;  // (a warp's own entries)
         }
     }
     cluster_sync_all();
@@ -318,6 +319,34 @@ __global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g, int 
     }
 }
 
+// Records per cluster, records per warp, columns of four at a time and shared memory of a sketch.
+// us, rank 24, records per cluster x per warp:          8 x 1   8 x 2   8 x 4   16 x 2   16 x 4
+//   d 256:   64 / 296 / 1024 / 4096 records    4.4   4.1   4.6   4.9   4.7 | 4.9 4.7 5.5 4.9 4.8 | 6.5 6.8 10.7 5.9 7.1 | 22.9 21.1 29.9 14.4 17.8
+//   d 1536:  64 / 296 / 1024 / 2048            5.6   4.7   5.0   6.2   6.0 | 6.9 5.8 6.3 6.3 6.0 | 10.5 9.0 12.1 9.7 9.7 | 19.6 16.3 19.9 18.1 15.1
+//   d 3584:  64 / 264 / 272 / 512              7.6   6.2   6.2   8.9   8.1 | 9.3 6.5 6.6 9.1 8.2 | 10.8 11.4 11.6 9.0 8.2 | 11.3 12.1 12.2 9.2 8.4
+// Few records: eight per cluster, for more CTAs.  33 clusters fit side by side at a CTA per SM, and 37 where two fit an SM.
+// More: sixteen halve the reads of Pi.  Four per warp take more registers (three CTAs per SM), so where shared memory leaves room for
+// more CTAs than that, two per warp.
+struct SketchForm {
+    int per, vpw, cols, bytes;
+};
+static SketchForm sketch_form(int R, int d, int rank) {
+    using namespace gt;
+    const int cols_all = (d / 4 + SK_CLUSTER - 1) / SK_CLUSTER;
+    auto with = [&](int per, int vpw) {
+        const int cols = std::min(cols_all, SK_SMEM / 16 / (rank + per));
+        return SketchForm{per, vpw, cols, (rank + per) * cols * 16};
+    };
+    // CTAs that an SM holds: shared memory with the partial products and what the system keeps, `most` by registers
+    auto fit = [](const SketchForm &f, int most) {
+        const int parts = SK_WARPS / (f.per / f.vpw) * f.per * MAX_RANK * 4;
+        return std::min(most, 228 * 1024 / (f.bytes + parts + 1024));
+    };
+    const SketchForm few = with(8, 2), two = with(16, 2), four = with(16, 4);
+    if (R <= (fit(few, 4) >= 2 ? 8 * 37 : 8 * 33)) return few;
+    return fit(four, 3) == fit(two, 4) ? four : two;
+}
+
 }  // namespace specroll
 
 using namespace specroll;
@@ -329,14 +358,12 @@ extern "C" int specroll_reflex_sketch(int32_t R, int32_t d, int32_t rank, const 
     if (!X || !Pi || !sketch) return SPECROLL_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if ((d % 4) == 0 && aligned16(X) && aligned16(Pi)) {
-        // sixteen records per cluster halve the reads of Pi; with few records, eight, for more CTAs
-        const int per = R > 296 ? 16 : 8, cols_all = (d / 4 + gt::SK_CLUSTER - 1) / gt::SK_CLUSTER;
-        const int cols = std::min(cols_all, gt::SK_SMEM / 16 / (rank + per));
-        auto *const kern = per == 16 ? sketch_kernel<16> : sketch_kernel<8>;
+        const SketchForm f = sketch_form(R, d, rank);
+        auto *const kern = f.per == 8 ? sketch_kernel<8, 2> : f.vpw == 2 ? sketch_kernel<16, 2> : sketch_kernel<16, 4>;
         const int rc = device_setup(reinterpret_cast<const void *>(kern), gt::SK_SMEM, nullptr);
         if (rc != SPECROLL_OK) return rc;
-        SR_CUDA_TRY(launch_clusters(true, gt::SK_CLUSTER, kern, dim3((unsigned)((R + per - 1) / per * gt::SK_CLUSTER)),
-                                    dim3(gt::SK_THREADS), (size_t)(rank + per) * cols * 16, st, R, d / 4, rank, cols,
+        SR_CUDA_TRY(launch_clusters(true, gt::SK_CLUSTER, kern, dim3((unsigned)((R + f.per - 1) / f.per * gt::SK_CLUSTER)),
+                                    dim3(gt::SK_THREADS), (size_t)f.bytes, st, R, d / 4, rank, f.cols,
                                     reinterpret_cast<const float4 *>(X), rows, reinterpret_cast<const float4 *>(Pi), sketch));
         return SPECROLL_OK;
     }

@@ -127,6 +127,16 @@ def test_sketches_at_the_ends_of_the_ranges(R, d, rank):
     np.testing.assert_allclose(host(S.reflex_sketch(dev(X), dev(Pi))), ref.reflex_sketch(X, Pi), rtol=0, atol=2e-5)
 
 
+@pytest.mark.parametrize("R,d,rank", [(264, 3584, 24), (265, 3584, 24), (296, 1536, 24), (297, 1536, 24), (297, 256, 24), (310, 1536, 9),
+                                       (1, 256, 32), (11, 132, 17)])
+def test_sketches_by_every_form(R, d, rank):
+    """Eight or sixteen records per cluster, two or four per warp: the last count with eight where one CTA fits an SM and where two do,
+    ragged records, ranks and columns."""
+    g = I.rng(700 + R + d)
+    Pi, X = g.standard_normal((rank, d)).astype(np.float32), g.standard_normal((R, d)).astype(np.float32)
+    np.testing.assert_allclose(host(S.reflex_sketch(dev(X), dev(Pi))), ref.reflex_sketch(X, Pi), rtol=0, atol=2e-5)
+
+
 @pytest.mark.parametrize("R,S_,kind", [(1500, 1500, "own"), (1500, 1500, "shuffled"), (1100, 700, "last"), (1025, 3, "last")])
 def test_slots_whose_records_lie_in_later_batches(R, S_, kind):
     """A slot's records are looked for 512 at a time: slots without a record in the first batch or the first two, and slots
