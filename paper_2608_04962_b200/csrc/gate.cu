@@ -19,9 +19,9 @@ constexpr int SK_CLUSTER = 4;   // CTAs that share the columns of their records
 constexpr int SK_SMEM = 208 * 1024;
 constexpr int GATE_THREADS = 128;
 constexpr int GATE_BATCH = 4 * GATE_THREADS;
-constexpr int GATE_RECS = 8;                // records whose alignments a warp forms at once
-// Up to so many records the gate forms their alignments itself, beyond it a kernel in front spreads them over the GPU.  A call, us,
-// in front -> itself (d 3584, rank 24): 512 records, one in each of 512 slots 14.9 -> 12.2, all in one 49 -> 43, of no slot 14.8 -> 12.2;
+constexpr int GATE_RECS_LOG = 3;            // a warp forms the alignments of eight records at once
+// Up to so many records the gate forms their alignments itself, beyond it a kernel in front spreads them over the GPU.  A call, us
+// (one launch less for the host as well; in a graph 512 of 512 slots 7.8 -> 7.0, 1024 of 16 13.7 -> 14.7, 64 of one 10.7 -> 12.3), in front -> itself (d 3584, rank 24): 512 records, one in each of 512 slots 14.9 -> 12.2, all in one 49 -> 43, of no slot 14.8 -> 12.2;
 // 1024 of 1024 slots 14.9 -> 12.3, of 16 slots 15.0 -> 14.5; 640 of one slot 57 -> 53, 700 of five 18.6 -> 19.9, 512 of no slot in a
 // call of one slot 14.5 -> 16.6.  Beyond: 4096 records of 16 slots 33.5 -> 35.0, of 512 slots 14.9 -> 18.6, one in each of 4096 24.7 -> 37.
 constexpr int GATE_FEW = 8 * GATE_THREADS;
@@ -145,23 +145,22 @@ struct GateArgs {
     float z_delta, mem_eps;
 };
 
-// Realised alignments of the n records of list (the warp's own) to val (may be null) and g.a, by a warp.  The loads of GATE_RECS records
+// Realised alignments of the n records of list (the warp's own) to val (may be null) and g.a, by a warp.  The loads of 2^L records
 // are in flight together; a sum is formed by the additions of warp_sum.
+template <int L>
 __device__ __forceinline__ void alignments(const GateArgs &g, const int *list, int n, float *val, int lane) {
-    using namespace gt;
-    constexpr int LANES = 32 / GATE_RECS, L = 3;
-    static_assert(GATE_RECS == 1 << L, "records by halving");
-    for (int e0 = 0; e0 < n; e0 += GATE_RECS) {
-        float dot[GATE_RECS], ns[GATE_RECS], nx[GATE_RECS];
+    constexpr int RECS = 1 << L, LANES = 32 / RECS;
+    for (int e0 = 0; e0 < n; e0 += RECS) {
+        float dot[RECS], ns[RECS], nx[RECS];
 #pragma unroll
-        for (int q = 0; q < GATE_RECS; ++q) {
+        for (int q = 0; q < RECS; ++q) {
             const bool in = e0 + q < n && lane < g.rank;
             const size_t at = in ? (size_t)list[e0 + q] * g.rank + lane : 0;
             ns[q] = in ? g.s[at] : 0.f;
             nx[q] = in ? g.xi[at] : 0.f;
         }
 #pragma unroll
-        for (int q = 0; q < GATE_RECS; ++q) {
+        for (int q = 0; q < RECS; ++q) {
             dot[q] = ns[q] * nx[q];
             ns[q] *= ns[q];
             nx[q] *= nx[q];
@@ -247,9 +246,11 @@ __global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g, int 
 #pragma unroll
         for (int q = 0; q < GROUPS; ++q) {
             const int r = rw + 32 * q;
-            const bool in = q < groups && r < g.R;
             // (a record of no slot of this call has an alignment all the same)
-            bool own = in && sl[q] == j, none = in && (unsigned)sl[q] >= (unsigned)g.S && (r & stray_mask) == j;
+            bool own = sl[q] == j, none = (unsigned)sl[q] >= (unsigned)g.S && (r & stray_mask) == j;
+            if (q >= groups || !__any_sync(0xffffffffu, r < g.R && (own || none))) continue;
+            own = own && r < g.R;
+            none = none && r < g.R;
             if ((own || none) && g.keep && !g.keep[r]) {
                 g.a[r] = __int_as_float(0x7fc00000);
                 own = none = false;
@@ -261,8 +262,12 @@ __global__ void __launch_bounds__(gt::GATE_THREADS) gate_kernel(GateArgs g, int 
             none_n += __popc(mn);
         }
         __syncwarp();
-        alignments(g, list, own_n, val + warp * PER_WARP, lane);
-        alignments(g, list + PER_WARP - none_n, none_n, nullptr, lane);
+        if (own_n == 1) {  // (the usual case, and the shorter code: 512 records in 512 slots 7.0 us in a graph, with the general one 7.8)
+            alignments<0>(g, list, 1, val + warp * PER_WARP, lane);
+        } else if (own_n > 1) {
+            alignments<GATE_RECS_LOG>(g, list, own_n, val + warp * PER_WARP, lane);
+        }
+        if (none_n > 0) alignments<GATE_RECS_LOG>(g, list + PER_WARP - none_n, none_n, nullptr, lane);
         if (lane == 0) n_own[warp] = own_n;
         __syncthreads();
         if (tid == 0)
