@@ -223,20 +223,25 @@ def test_many_records_per_slot_and_records_of_none(R, S_, strays):
     np.testing.assert_allclose(host(y[6]), o["M2"], rtol=2e-4, atol=2e-5)
 
 
-@pytest.mark.parametrize("S_,slot", [(512, np.full(512, -1)), (512, np.full(4096, -1)), (16, np.arange(4096) % 16)])
-def test_time_does_not_hang_on_how_records_are_spread(S_, slot):
-    """Records of no slot, or of few slots, against one record in each of 512 slots.  (Measured: 1.0, 1.2 and 2.8 times as long;
-    with a slot's alignments formed one after the other, and by one CTA for the records of no slot, 5.5, 41 and 6.1.)"""
+@pytest.mark.parametrize("slot,most", [(np.full(512, -1), 4.0), (np.full(4096, -1), 4.0), (np.zeros(512), 10.0)])
+def test_time_does_not_hang_on_how_records_are_spread(slot, most):
+    """Records of no slot, or all of one of 512 slots, against one record in each, in graphs of calls.  (Measured: 1.0, 1.2 and 4.3 times
+    as long; with a slot's alignments formed one after the other, and by one CTA for the records of no slot, 6, 46 and 11.)"""
     def us(S_, slot):
         y = [v if v is None else dev(v) for v in _gate_case(len(slot), S_, slot, d=3584)]
+        S.reflex_gate(*y)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            for _ in range(20):
+                S.reflex_gate(*y)
         best = []
         for _ in range(8):
             a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
             a.record()
-            for _ in range(20):
-                S.reflex_gate(*y)
+            graph.replay()
             b.record()
             torch.cuda.synchronize()
             best.append(a.elapsed_time(b) * 50.0)
         return min(best)
-    assert us(S_, slot) < 4.0 * us(512, np.arange(512))
+    assert us(512, slot) < most * us(512, np.arange(512))
